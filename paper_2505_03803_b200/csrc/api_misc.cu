@@ -19,9 +19,30 @@ void set_last_cuda_error(cudaError_t e) {
 // Device address of the status word for the current device (kernels in other translation units
 // receive it as an argument).
 int* device_status_ptr() {
-  void* p = nullptr;
-  if (cudaGetSymbolAddress(&p, g_device_status) != cudaSuccess) return nullptr;
-  return static_cast<int*>(p);
+  static std::atomic<int*> known[kMaxDevices];
+  const int dev = current_device();
+  int* p = dev >= 0 ? known[dev].load(std::memory_order_relaxed) : nullptr;
+  if (p) return p;
+  void* q = nullptr;
+  if (cudaGetSymbolAddress(&q, g_device_status) != cudaSuccess) return nullptr;
+  p = static_cast<int*>(q);
+  if (dev >= 0) known[dev].store(p, std::memory_order_relaxed);
+  return p;
+}
+int current_device() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
+  return dev;
+}
+int sm_count() {
+  static std::atomic<int> known[kMaxDevices];
+  const int dev = current_device();
+  if (dev < 0) return 148;
+  int sms = known[dev].load(std::memory_order_relaxed);
+  if (sms > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+  known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
 }
 }  // namespace rwkvq
 

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/rwkvq.h"
 #include "format.h"
 
@@ -46,6 +48,25 @@ inline size_t matrix_aux_offset(const rwkvq_desc* d) {
 inline size_t vector_aux_offset(const rwkvq_desc* d) {
   return RWKVQ_HEADER_BYTES + round_up_sz(((size_t)(d->ic / 2) * d->bits + 7) / 8, 16);
 }
+
+constexpr int kMaxDevices = 64;
+// Ordinal of the current device, -1 if it cannot be asked or is beyond kMaxDevices.
+int current_device();
+// Multiprocessors of the current device (148 where it cannot be asked); looked up once per device.
+int sm_count();
+
+// The opt-in to more than 48 KB of dynamic shared memory holds for a kernel and a device until the process ends: it is
+// asked for once (about 1 us of host time) and not at every launch.  One object per kernel, `bytes` the same at every call.
+struct SmemOptIn {
+  std::atomic<bool> done[kMaxDevices];
+  cudaError_t operator()(const void* fn, int bytes) {
+    const int dev = current_device();
+    if (dev >= 0 && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && dev >= 0) done[dev].store(true, std::memory_order_relaxed);
+    return e;
+  }
+};
 
 void set_last_cuda_error(cudaError_t e);
 inline rwkvq_status cuda_status(cudaError_t e) {

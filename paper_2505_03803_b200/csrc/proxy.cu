@@ -1,7 +1,6 @@
 // Coarse-to-fine proxy (Section 4.1).  The paper sorts the flattened weights (Eq. 5) and works on
-// the gaps between neighbours.  For fp16 weights the sort is a counting sort over the 65 536 bit
-// patterns, so one streaming pass over the matrix (2 bytes per weight) builds a histogram and a
-// second, tiny kernel walks the occupied bins in value order:
+// the gaps between neighbours.  For 16-bit weights the sort reduces to the set of bit patterns that occur
+// (proxy_core.cuh): one streaming pass marks them and a second, tiny kernel walks the set in value order:
 //   D distinct values v_1 < ... < v_D give D-1 positive gaps; the other n-(D-1) gaps are ties (0).
 //   R = v_D - v_1 = sum of gaps;  g'_j = (v_{j+1} - v_j) / R                          (Eq. 6)
 //   P_c = ln n + sum_j g'_j ln g'_j            (Eqs. 7-9, 0 ln 0 := 0, n = oc*ic - 1)
@@ -19,180 +18,94 @@
 
 #include "../../include/rwkvq.h"
 #include "host_util.h"
+#include "proxy_core.cuh"
 #include "unpack.cuh"
 
 namespace rwkvq {
 
-constexpr int kBins = 65536;
-constexpr int kHotHalf = 24576;            // shared-memory window: |w| below fp16 pattern 0x6000 (512.0)
-constexpr int kHotBins = 2 * kHotHalf;     // 192 KB of u32 counters
-constexpr int kHotBase = 0x8000 - kHotHalf;
+constexpr size_t kMatrixBytes = 65536 * 4;   // workspace share of one matrix; its bitmap takes the first 8 KB
 
 struct ProxyResult {
   double pc, pf;
+  double variance, cv, range, mad, ie;   // the ablation's statistics of G' (Section 5.3)
   unsigned long long count;
   int distinct, nonfinite;
-  int pad[2];
-  double variance, cv, range, mad, ie;   // the ablation's statistics of G' (Section 5.3)
-  double pad2;
 };
 
-// Order-preserving key of an fp16 bit pattern: key = 0x8000 - |bits| for negative values,
-// 0x8000 + |bits| for positive ones; +0 and -0 share key 0x8000.
-__device__ __forceinline__ unsigned key_of(unsigned bits) {
-  const unsigned mag = bits & 0x7FFFu;
-  return (bits & 0x8000u) ? 0x8000u - mag : 0x8000u + mag;
-}
-// bf16 != 0: the 16 bits are a bfloat16 pattern (same sign-magnitude order, other exponent width)
-__device__ __forceinline__ double value_of_key(unsigned key, int bf16 = 0) {
-  const unsigned short bits = key >= 0x8000u ? (unsigned short)(key - 0x8000u) : (unsigned short)(0x8000u | (0x8000u - key));
-  if (bf16) return (double)__uint_as_float((unsigned)bits << 16);
-  return (double)__half2float(__ushort_as_half(bits));
-}
+struct MarkArgs {
+  static constexpr int kMost = 96;             // matrices per launch
+  const uint4* w[kMost];
+  unsigned long long n[kMost];                 // weights
+  unsigned long long start[kMost + 1];         // first 16-byte vector of each matrix in the launch's common numbering
+  int count;
+};
 
-__device__ __forceinline__ void count_one(unsigned bits, unsigned* sh, unsigned* hist, int* nonfinite, unsigned expmask) {
-  if ((bits & expmask) == expmask) { *nonfinite = 1; return; }
-  const unsigned key = key_of(bits);
-  const unsigned rel = key - (unsigned)kHotBase;
-  if (rel < (unsigned)kHotBins) atomicAdd(&sh[rel], 1u);
-  else atomicAdd(&hist[key], 1u);
-}
-
-__global__ void __launch_bounds__(1024, 1) proxy_hist_kernel(const __half* w, unsigned long long n, unsigned* hist, ProxyResult* res, int bf16) {
-  extern __shared__ unsigned sh[];
-  const unsigned expmask = bf16 ? 0x7F80u : 0x7C00u;
-  for (int j = threadIdx.x; j < kHotBins; j += blockDim.x) sh[j] = 0u;
-  __syncthreads();
-  int bad = 0;
-  const unsigned long long nvec = n / 8;
-  const uint4* wv = reinterpret_cast<const uint4*>(w);
-  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < nvec;
-       i += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint4 v = ldg_stream(wv + i);
-    const unsigned ws[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      count_one(ws[k] & 0xFFFFu, sh, hist, &bad, expmask);
-      count_one(ws[k] >> 16, sh, hist, &bad, expmask);
+// Marks the patterns of all matrices of a call.  A block takes an equal run of the matrices' vectors laid end to end, two
+// blocks of 1024 threads per SM, two vectors in flight per thread (64 KB per SM); a run that crosses into the
+// next matrix writes its bitmap out and starts a new one.  One launch instead of one per matrix, and 8 KB to clear and merge
+// per block instead of 192 KB of counters.
+__global__ void __launch_bounds__(1024, 2) proxy_mark_kernel(const __grid_constant__ MarkArgs a, uint8_t* ws) {
+  __shared__ __align__(16) uint32_t bm[kPatternWords];
+  const unsigned long long total = a.start[a.count];
+  unsigned long long at = total * blockIdx.x / gridDim.x;
+  const unsigned long long end = total * (blockIdx.x + 1) / gridDim.x;
+  int m = 0;
+  while (at < end) {
+    while (at >= a.start[m + 1]) ++m;
+    const unsigned long long stop = min(end, a.start[m + 1]);
+    for (int j = threadIdx.x; j < kPatternWords; j += 1024) bm[j] = 0u;
+    __syncthreads();
+    const uint4* w = a.w[m];
+    const unsigned long long full = a.n[m] / 8, hi = min(stop - a.start[m], full);
+    unsigned long long i = at - a.start[m] + threadIdx.x;
+    for (; i + 1024 < hi; i += 2048) {
+      const uint4 v = ldg_stream(w + i), u = ldg_stream(w + i + 1024);
+      mark_pair(bm, v.x); mark_pair(bm, v.y); mark_pair(bm, v.z); mark_pair(bm, v.w);
+      mark_pair(bm, u.x); mark_pair(bm, u.y); mark_pair(bm, u.z); mark_pair(bm, u.w);
     }
-  }
-  if (blockIdx.x == 0) {
-    for (unsigned long long i = nvec * 8 + threadIdx.x; i < n; i += blockDim.x)
-      count_one((unsigned)__half_as_ushort(w[i]), sh, hist, &bad, expmask);
-  }
-  if (bad) res->nonfinite = 1;
-  __syncthreads();
-  for (int j = threadIdx.x; j < kHotBins; j += blockDim.x) {
-    const unsigned c = sh[j];
-    if (c) atomicAdd(&hist[j + kHotBase], c);
+    if (i < hi) {
+      const uint4 v = ldg_stream(w + i);
+      mark_pair(bm, v.x); mark_pair(bm, v.y); mark_pair(bm, v.z); mark_pair(bm, v.w);
+    }
+    if (stop == a.start[m + 1] && threadIdx.x < a.n[m] % 8)      // the weights behind the last whole vector
+      mark_pattern(bm, reinterpret_cast<const unsigned short*>(w + full)[threadIdx.x]);
+    __syncthreads();
+    uint32_t* all = reinterpret_cast<uint32_t*>(ws + (size_t)m * kMatrixBytes);
+    for (int j = threadIdx.x; j < kPatternWords; j += 1024) {
+      const uint32_t v = bm[j];
+      if (v && (v & ~__ldcg(all + j))) atomicOr(all + j, v);
+    }
+    __syncthreads();
+    at = stop;
   }
 }
 
-// One block of 1024 threads per matrix; thread t owns keys [64t, 64t+64).
-__global__ void __launch_bounds__(1024, 1) proxy_reduce_kernel(const unsigned* hist_all, ProxyResult* res_all, int K, int bf16) {
-  const unsigned* hist = hist_all + (size_t)blockIdx.x * kBins;
-  ProxyResult* res = res_all + blockIdx.x;
-  __shared__ int s_last[1024];
-  __shared__ int s_first[1024];
-  __shared__ unsigned long long s_cnt[1024];
-  __shared__ int s_dist[1024];
-  __shared__ double s_red[1024];
-  const int t = threadIdx.x, k0 = t * 64;
-  int first = -1, last = -1, dist = 0;
-  unsigned long long cnt = 0;
-  for (int k = k0; k < k0 + 64; ++k) {
-    const unsigned c = hist[k];
-    if (c) { if (first < 0) first = k; last = k; ++dist; cnt += c; }
-  }
-  s_last[t] = last; s_first[t] = first; s_cnt[t] = cnt; s_dist[t] = dist;
+// One block per matrix.
+__global__ void __launch_bounds__(1024, 1) proxy_reduce_kernel(const uint8_t* ws, const __grid_constant__ MarkArgs a, ProxyResult* res_all, int K, int bf16) {
+  __shared__ __align__(16) uint32_t bm[kPatternWords];
+  __shared__ SetShared<1024> sh;
+  const uint2* all = reinterpret_cast<const uint2*>(ws + (size_t)blockIdx.x * kMatrixBytes);
+  reinterpret_cast<uint2*>(bm)[threadIdx.x] = __ldcg(all + threadIdx.x);
   __syncthreads();
-  // thread 0 turns the per-thread extremes into "previous occupied key before my segment"
-  if (t == 0) {
-    int prev = -1, mn = -1, mx = -1, D = 0;
-    unsigned long long N = 0;
-    for (int i = 0; i < 1024; ++i) {
-      const int l = s_last[i], f = s_first[i];
-      s_last[i] = prev;                       // now: predecessor key for segment i
-      if (f >= 0) { if (mn < 0) mn = f; mx = l; prev = l; }
-      D += s_dist[i]; N += s_cnt[i];
-    }
-    s_first[0] = mn; s_first[1] = mx; s_dist[0] = D; s_cnt[0] = N;
-  }
-  __syncthreads();
-  const int mn = s_first[0], mx = s_first[1], D = s_dist[0];
-  const unsigned long long N = s_cnt[0];
-  if (D < 2 || N < 2) {
-    if (t == 0) {
-      res->pc = INFINITY; res->pf = INFINITY; res->count = N; res->distinct = D;
-      res->variance = res->cv = res->range = res->mad = res->ie = INFINITY;
-    }
-    return;
-  }
-  const double R = value_of_key((unsigned)mx, bf16) - value_of_key((unsigned)mn, bf16);
-  const double n = (double)(N - 1);
-  double acc[8];  // [0] = sum g' ln g', [k-1] = sum t^k for k = 2..8
-#pragma unroll
-  for (int i = 0; i < 8; ++i) acc[i] = 0.0;
-  double abs_t = 0.0, gmax = 0.0, gmin = INFINITY;   // sum |t_j|, largest and smallest positive gap
-  int prev = s_last[t];
-  for (int k = k0; k < k0 + 64; ++k) {
-    if (hist[k] == 0u) continue;
-    if (prev >= 0) {
-      const double gp = (value_of_key((unsigned)k, bf16) - value_of_key((unsigned)prev, bf16)) / R;
-      acc[0] += gp * log(gp);
-      const double tt = n * gp - 1.0;
-      double pw = tt;
-      for (int kk = 2; kk <= K; ++kk) { pw *= tt; acc[kk - 1] += pw; }
-      abs_t += fabs(tt);
-      gmax = fmax(gmax, gp);
-      gmin = fmin(gmin, gp);
-    }
-    prev = k;
-  }
-  double tot[8];
-  for (int i = 0; i < 8; ++i) {   // fixed-shape tree: deterministic
-    __syncthreads();
-    s_red[t] = acc[i];
-    __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
-      if (t < s) s_red[t] += s_red[t + s];
-      __syncthreads();
-    }
-    tot[i] = s_red[0];
-  }
-  // three more reductions of the same shape: sum |t|, max and min positive gap
-  double extra[3];
-  for (int i = 0; i < 3; ++i) {
-    __syncthreads();
-    s_red[t] = i == 0 ? abs_t : i == 1 ? gmax : gmin;
-    __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
-      if (t < s) s_red[t] = i == 0 ? s_red[t] + s_red[t + s] : i == 1 ? fmax(s_red[t], s_red[t + s]) : fmin(s_red[t], s_red[t + s]);
-      __syncthreads();
-    }
-    extra[i] = s_red[0];
-  }
-  if (t == 0) {
-    const double ties = n - (double)(D - 1);
+  const double n = (double)(a.n[blockIdx.x] - 1ull);
+  SetStats s;
+  set_gaps<1024>(bm, bf16 != 0, n, K, sh, s);
+  if (threadIdx.x != 0) return;
+  ProxyResult r;
+  r.count = a.n[blockIdx.x]; r.distinct = s.distinct; r.nonfinite = s.nonfinite ? 1 : 0;
+  r.pc = r.pf = r.variance = r.cv = r.range = r.mad = r.ie = INFINITY;
+  if (!s.nonfinite && !s.degenerate) {
+    const double ties = n - (double)(s.distinct - 1);
     // with t = n G' - 1 (ties: t = -1):  variance = sum t^2 / n^3,  mad = sum |t| / n^2
-    res->variance = (tot[1] + ties) / (n * n * n);
-    res->cv = sqrt(res->variance) * n;
-    res->range = extra[1] - (ties > 0.0 ? 0.0 : extra[2]);
-    res->mad = (extra[0] + ties) / (n * n);
-    res->ie = -tot[0];
-    double pf = 0.0;
-    for (int kk = 2; kk <= K; ++kk) {
-      const double sign = (kk & 1) ? -1.0 : 1.0;
-      pf += fabs((tot[kk - 1] + ties * sign) / n) / (double)(kk * (kk - 1));
-    }
-    res->pc = log(n) + tot[0];
-    res->pf = pf;
-    res->count = N;
-    res->distinct = D;
+    r.variance = (s.pw[0] + ties) / (n * n * n);
+    r.cv = sqrt(r.variance) * n;
+    r.range = s.gmax - (ties > 0.0 ? 0.0 : s.gmin);
+    r.mad = (s.abs_t + ties) / (n * n);
+    r.ie = -s.sum_glng;
+    proxy_from_set(s, n, K, &r.pc, &r.pf);
   }
+  res_all[blockIdx.x] = r;
 }
-
-static size_t per_matrix_bytes() { return (size_t)kBins * 4; }
 
 }  // namespace rwkvq
 
@@ -202,7 +115,7 @@ extern "C" {
 
 size_t rwkvq_proxy_workspace_bytes(int n_mats) {
   if (n_mats <= 0) return 0;
-  return (size_t)n_mats * per_matrix_bytes() + round_up_sz((size_t)n_mats * sizeof(ProxyResult), 256);
+  return (size_t)n_mats * kMatrixBytes + round_up_sz((size_t)n_mats * sizeof(ProxyResult), 256);
 }
 
 static rwkvq_status run_proxy(const void* const* w, const int* oc, const int* ic, int n_mats, int K, void* ws,
@@ -216,23 +129,26 @@ static rwkvq_status run_proxy(const void* const* w, const int* oc, const int* ic
     if (!aligned16(w[m])) return RWKVQ_EALIGN;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  unsigned* hist = static_cast<unsigned*>(ws);
-  ProxyResult* res = reinterpret_cast<ProxyResult*>(static_cast<uint8_t*>(ws) + (size_t)n_mats * per_matrix_bytes());
-  cudaError_t e = cudaMemsetAsync(ws, 0, rwkvq_proxy_workspace_bytes(n_mats), s);
+  uint8_t* base = static_cast<uint8_t*>(ws);
+  ProxyResult* res = reinterpret_cast<ProxyResult*>(base + (size_t)n_mats * kMatrixBytes);
+  cudaError_t e = cudaMemset2DAsync(base, kMatrixBytes, 0, kPatternWords * 4, n_mats, s);
   if (e != cudaSuccess) return cuda_status(e);
-  const size_t smem = (size_t)kHotBins * 4;
-  e = cudaFuncSetAttribute(proxy_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  for (int m = 0; m < n_mats; ++m) {
-    const unsigned long long n = (unsigned long long)oc[m] * (unsigned long long)ic[m];
-    unsigned long long blocks = (n / 8 + 1023) / 1024;
-    if (blocks < 1) blocks = 1;
-    if (blocks > (unsigned long long)sms) blocks = sms;
-    proxy_hist_kernel<<<(unsigned)blocks, 1024, smem, s>>>(static_cast<const __half*>(w[m]), n, hist + (size_t)m * kBins, res + m, bf16);
+  const int sms = sm_count();
+  for (int m0 = 0; m0 < n_mats; m0 += MarkArgs::kMost) {
+    MarkArgs a;
+    a.count = std::min(n_mats - m0, MarkArgs::kMost);
+    a.start[0] = 0;
+    for (int i = 0; i < a.count; ++i) {
+      a.w[i] = static_cast<const uint4*>(w[m0 + i]);
+      a.n[i] = (unsigned long long)oc[m0 + i] * (unsigned long long)ic[m0 + i];
+      a.start[i + 1] = a.start[i] + (a.n[i] + 7) / 8;
+    }
+    // two blocks per SM, and no more than one per 1024 vectors: a block's clearing and merging should not outweigh its share
+    const unsigned long long blocks = std::min<unsigned long long>(2ull * (unsigned)sms, (a.start[a.count] + 1023) / 1024);
+    uint8_t* part = base + (size_t)m0 * kMatrixBytes;
+    proxy_mark_kernel<<<(unsigned)blocks, 1024, 0, s>>>(a, part);
+    proxy_reduce_kernel<<<a.count, 1024, 0, s>>>(part, a, res + m0, K, bf16);
   }
-  proxy_reduce_kernel<<<n_mats, 1024, 0, s>>>(hist, res, K, bf16);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e);
   out->resize(n_mats);

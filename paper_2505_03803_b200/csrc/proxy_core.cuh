@@ -1,0 +1,209 @@
+// The gaps of Eqs. 5-17 from the SET of 16-bit patterns a matrix (or a tile of one) holds.
+//
+// Neighbours in the sorted order that are equal contribute a gap of zero, so for 16-bit weights everything
+// the proxy needs is which of the 65 536 patterns occur and how many weights there are: a bitmap of 8 KB
+// instead of a sorted array or a table of 65 536 counters.  Marking is one shared-memory read per weight (and an
+// atomic only the first time a pattern is met), so a streaming pass is bound by HBM, and the walk below touches
+// 2 048 words.
+#pragma once
+#include <cuda_fp16.h>
+#include <math.h>
+#include <stdint.h>
+
+namespace rwkvq {
+
+constexpr int kPatternWords = 2048;        // bit p of the bitmap = bit (p & 31) of word p >> 5; p = raw bit pattern
+constexpr int kGapList = 2048;             // gaps evaluated per round of the walk
+
+__device__ __forceinline__ void mark_pattern(uint32_t* bm, uint32_t p) {
+  uint32_t* w = bm + (p >> 5);
+  if (!((*reinterpret_cast<volatile uint32_t*>(w) >> (p & 31u)) & 1u)) atomicOr(w, 1u << (p & 31u));
+}
+__device__ __forceinline__ void mark_pair(uint32_t* bm, uint32_t two) {
+  mark_pattern(bm, two & 0xFFFFu);
+  mark_pattern(bm, two >> 16);
+}
+
+// Value of a magnitude (the low 15 bits of a pattern).
+__device__ __forceinline__ double magnitude_value(uint32_t mag, bool bf16) {
+  return bf16 ? (double)__uint_as_float(mag << 16) : (double)__half2float(__ushort_as_half((unsigned short)mag));
+}
+
+struct SetStats {
+  double sum_glng;            // sum g' ln g' over the positive gaps
+  double pw[7];               // sum t^k for k = 2..8 over the positive gaps, t = n g' - 1
+  double abs_t, gmax, gmin;   // sum |t|, largest and smallest positive g'
+  int distinct;
+  bool nonfinite, degenerate; // degenerate: fewer than two distinct values or weights
+};
+
+template <int T>
+struct SetShared {
+  int first[T / 32], last[T / 32], count[T / 32], bad[T / 32];
+  uint32_t gaps[kGapList];    // magnitude << 16 | predecessor's magnitude
+  double red[T / 32][11];
+};
+
+// All T threads call it with the same bitmap; thread 0 receives the sums (the flags and `distinct` are valid in
+// every thread).  `n` = weights - 1.  Thread t owns 1024 / T runs of 64 consecutive patterns.  Positive and negative patterns
+// are two chains in order of magnitude, joined at zero if it occurs and by one gap across it if not.  Gaps
+// between neighbouring patterns of a run (most of them, in a dense matrix) are all one ulp of the run's binade: they
+// are counted and evaluated once; the others are collected and evaluated by all threads in turn.  All sums have a
+// fixed order, so results are reproducible.
+template <int T>
+__device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShared<T>& sh, SetStats& out) {
+  static_assert(T % 64 == 0 && T <= 1024 && 1024 % T == 0, "block size");
+  constexpr int P = 1024 / T, W = T / 32;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const bool zero = ((bm[0] | bm[kPatternWords / 2]) & 1u) != 0u;       // +0 and -0 are the same value
+  const int inf_run = bf16 ? 0x7F80 / 64 : 0x7C00 / 64;
+  int first = 0x10000, last = -1, count = 0, bad = 0;
+  uint64_t bits[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int run = t * P + i, mrun = run & 511;
+    uint64_t b = *reinterpret_cast<const uint64_t*>(bm + 2 * run);
+    if (mrun == 0) b = (b & ~1ull) | (zero ? 1ull : 0ull);
+    if (mrun >= inf_run) { bad |= b != 0ull; b = 0ull; }
+    bits[i] = b;
+    if (b) {
+      first = min(first, mrun * 64 + __ffsll((long long)b) - 1);
+      last = mrun * 64 + 63 - __clzll((long long)b);
+      count += __popcll(b);
+    }
+  }
+  // predecessor of this thread's first pattern within its side (warps 0 .. W/2 - 1 hold the positive side)
+  int prev = last, mn = first, cnt = count;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xFFFFFFFFu, prev, d);
+    if (lane >= d) prev = max(prev, v);
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    mn = min(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, d));
+    cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, d);
+  }
+  const int any_bad = __any_sync(0xFFFFFFFFu, bad);
+  if (lane == 31) { sh.last[warp] = prev; sh.first[warp] = mn; sh.count[warp] = cnt; sh.bad[warp] = any_bad; }
+  prev = __shfl_up_sync(0xFFFFFFFFu, prev, 1);
+  if (lane == 0) prev = -1;
+  __syncthreads();
+  int lo[2] = {0x10000, 0x10000}, hi[2] = {-1, -1}, distinct = zero ? -1 : 0, nf = 0;
+  for (int w = 0; w < W; ++w) {
+    const int side = w >= W / 2;
+    if (w < warp && side == (warp >= W / 2)) prev = max(prev, sh.last[w]);
+    lo[side] = min(lo[side], sh.first[w]);
+    hi[side] = max(hi[side], sh.last[w]);
+    distinct += sh.count[w];
+    nf |= sh.bad[w];
+  }
+  out.distinct = distinct; out.nonfinite = nf != 0;
+  out.degenerate = distinct < 2 || n < 1.0;
+  if (out.degenerate) return;
+  const double vmax = hi[0] >= 0 ? magnitude_value((uint32_t)hi[0], bf16) : -magnitude_value((uint32_t)lo[1], bf16);
+  const double vmin = hi[1] >= 0 ? -magnitude_value((uint32_t)hi[1], bf16) : magnitude_value((uint32_t)lo[0], bf16);
+  const double inv_R = 1.0 / (vmax - vmin);
+  double acc[11];
+#pragma unroll
+  for (int i = 0; i < 11; ++i) acc[i] = 0.0;
+  acc[10] = INFINITY;
+  auto add = [&](double gap, double times) {
+    const double gp = gap * inv_R, tt = n * gp - 1.0;
+    acc[0] += times * (gp * log(gp));
+    double pw = tt;
+#pragma unroll
+    for (int k = 2; k <= 8; ++k)
+      if (k <= K) { pw *= tt; acc[k - 1] += times * pw; }
+    acc[8] += times * fabs(tt);
+    acc[9] = fmax(acc[9], gp);
+    acc[10] = fmin(acc[10], gp);
+  };
+  // gaps of one pattern inside a run, and how many other gaps this thread has
+  uint64_t lone[P];
+  int n_lone = 0, before = prev;
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const uint64_t b = bits[i], adj = b & (b << 1);
+    const uint32_t base = (uint32_t)((t * P + i) & 511) * 64u;
+    if (adj) add(magnitude_value(base + 1u, bf16) - magnitude_value(base, bf16), (double)__popcll(adj));
+    lone[i] = b & ~adj;
+    n_lone += __popcll(lone[i]);
+  }
+  if (n_lone > 0 && before < 0) --n_lone;          // the side's smallest magnitude has no predecessor
+  if (t == 0 && !zero && hi[0] >= 0 && hi[1] >= 0) add(magnitude_value((uint32_t)lo[0], bf16) + magnitude_value((uint32_t)lo[1], bf16), 1.0);
+  // position of this thread's gaps in the common list
+  int incl = n_lone;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+    if (lane >= d) incl += v;
+  }
+  __syncthreads();                                 // sh.count is reused
+  if (lane == 31) sh.count[warp] = incl;
+  __syncthreads();
+  int pos = incl - n_lone, total = 0;
+  for (int w = 0; w < W; ++w) {
+    if (w < warp) pos += sh.count[w];
+    total += sh.count[w];
+  }
+  int next = 0;                                    // this thread's run being listed
+  for (int c0 = 0; c0 < total; c0 += kGapList) {
+    const int c1 = c0 + kGapList;
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      if (i < next) continue;
+      const uint32_t base = (uint32_t)((t * P + i) & 511) * 64u;
+      while (lone[i] && pos < c1) {
+        const int b = __ffsll((long long)lone[i]) - 1;
+        lone[i] &= lone[i] - 1ull;
+        const uint64_t below = bits[i] & ((1ull << b) - 1ull);
+        const int p = below ? (int)base + 63 - __clzll((long long)below) : before;
+        if (p >= 0) { sh.gaps[pos - c0] = ((base + (uint32_t)b) << 16) | (uint32_t)p; ++pos; }
+      }
+      if (lone[i]) break;
+      if (bits[i]) before = (int)base + 63 - __clzll((long long)bits[i]);
+      next = i + 1;
+    }
+    __syncthreads();
+    for (int j = t; j < min(kGapList, total - c0); j += T)
+      add(magnitude_value(sh.gaps[j] >> 16, bf16) - magnitude_value(sh.gaps[j] & 0xFFFFu, bf16), 1.0);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 11; ++i) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      const double o = __shfl_xor_sync(0xFFFFFFFFu, acc[i], d);
+      acc[i] = i == 9 ? fmax(acc[i], o) : i == 10 ? fmin(acc[i], o) : acc[i] + o;
+    }
+    if (lane == 0) sh.red[warp][i] = acc[i];
+  }
+  __syncthreads();
+  if (t == 0) {
+#pragma unroll
+    for (int i = 0; i < 11; ++i) acc[i] = sh.red[0][i];
+    for (int w = 1; w < W; ++w) {
+#pragma unroll
+      for (int i = 0; i < 11; ++i) {
+        const double o = sh.red[w][i];
+        acc[i] = i == 9 ? fmax(acc[i], o) : i == 10 ? fmin(acc[i], o) : acc[i] + o;
+      }
+    }
+    out.sum_glng = acc[0];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) out.pw[i] = acc[i + 1];
+    out.abs_t = acc[8]; out.gmax = acc[9]; out.gmin = acc[10];
+  }
+}
+
+// P_c of Eq. 9 and P_f of Eq. 17 from the sums; `n` = weights - 1, the n - (distinct - 1) ties have t = -1.
+__device__ __forceinline__ void proxy_from_set(const SetStats& s, double n, int K, double* pc, double* pf) {
+  const double ties = n - (double)(s.distinct - 1);
+  double f = 0.0;
+  for (int k = 2; k <= K; ++k) f += fabs((s.pw[k - 2] + ((k & 1) ? -ties : ties)) / n) / (double)(k * (k - 1));
+  *pc = log(n) + s.sum_glng;
+  *pf = f;
+}
+
+}  // namespace rwkvq

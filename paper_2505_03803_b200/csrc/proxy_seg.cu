@@ -4,9 +4,9 @@
 // inputs are the model's weights, whatever their type.  Two routes besides the fp16 histogram of
 // proxy.cu:
 //   * segments -- every seg_rows x seg_cols tile of a matrix (one output channel = a 1 x ic tile,
-//     one block = e.g. 256 x 256) is sorted by ONE thread block in shared memory (bitonic network
-//     on order-preserving integer keys: the sort of Eq. 5 literally), and the gaps between
-//     neighbours are reduced in fp64 in a fixed order (Eqs. 6-17);
+//     one block = e.g. 256 x 256) is reduced by ONE thread block in shared memory: 16-bit types through the
+//     set of patterns that occur (proxy_core.cuh), fp32 by a bitonic network on order-preserving
+//     integer keys (the sort of Eq. 5 literally), gaps reduced in fp64 in a fixed order (Eqs. 6-17);
 //   * a whole fp32 matrix too large for shared memory is sorted by the radix sort of the CUDA
 //     toolkit's CUB (a library primitive for the sort of Eq. 5), then the same gap reduction runs over
 //     the sorted array in two fixed-order passes.
@@ -24,12 +24,14 @@
 
 #include "../../include/rwkvq.h"
 #include "host_util.h"
+#include "proxy_core.cuh"
+#include "unpack.cuh"
 
 namespace rwkvq {
 namespace pseg {
 
 constexpr int kThreads = 1024;
-constexpr uint32_t kSmemKeysBytes = 131072;        // 65 536 16-bit keys or 32 768 32-bit keys
+constexpr uint32_t kSmemKeysBytes = 131072;        // a tile holds at most 65 536 16-bit or 32 768 32-bit weights
 constexpr int kMaxK = 8;
 
 struct SegResult {
@@ -38,40 +40,10 @@ struct SegResult {
   int nonfinite;
 };
 
-// Order-preserving keys.  16-bit types are sign-magnitude: key = 0x8000 -/+ magnitude (+0 and -0
-// share 0x8000).  fp32: flip all bits of negatives, the sign bit of the others.
-__device__ __forceinline__ uint16_t key16(uint16_t bits) {
-  const uint16_t mag = bits & 0x7FFFu;
-  return (bits & 0x8000u) ? (uint16_t)(0x8000u - mag) : (uint16_t)(0x8000u + mag);
-}
-__device__ __forceinline__ uint16_t bits_of_key16(uint16_t key) {
-  return key >= 0x8000u ? (uint16_t)(key - 0x8000u) : (uint16_t)(0x8000u | (0x8000u - key));
-}
+// Order-preserving keys: flip all bits of negatives, the sign bit of the others.
 __device__ __forceinline__ uint32_t key32(uint32_t bits) { return (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u); }
 __device__ __forceinline__ uint32_t bits_of_key32(uint32_t key) { return (key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key; }
-
-template <int DTYPE> struct Traits;
-template <> struct Traits<RWKVQ_F16> {
-  using Key = uint16_t; using Elem = uint16_t;
-  static constexpr Key kPad = 0xFFFFu;
-  static __device__ __forceinline__ bool finite(Elem b) { return (b & 0x7C00u) != 0x7C00u; }
-  static __device__ __forceinline__ Key key(Elem b) { return key16(b); }
-  static __device__ __forceinline__ double value(Key k) { return (double)__half2float(__ushort_as_half(bits_of_key16(k))); }
-};
-template <> struct Traits<RWKVQ_BF16> {
-  using Key = uint16_t; using Elem = uint16_t;
-  static constexpr Key kPad = 0xFFFFu;
-  static __device__ __forceinline__ bool finite(Elem b) { return (b & 0x7F80u) != 0x7F80u; }
-  static __device__ __forceinline__ Key key(Elem b) { return key16(b); }
-  static __device__ __forceinline__ double value(Key k) { return (double)__uint_as_float((uint32_t)bits_of_key16(k) << 16); }
-};
-template <> struct Traits<RWKVQ_F32> {
-  using Key = uint32_t; using Elem = uint32_t;
-  static constexpr Key kPad = 0xFFFFFFFFu;
-  static __device__ __forceinline__ bool finite(Elem b) { return (b & 0x7F800000u) != 0x7F800000u; }
-  static __device__ __forceinline__ Key key(Elem b) { return key32(b); }
-  static __device__ __forceinline__ double value(Key k) { return (double)__uint_as_float(bits_of_key32(k)); }
-};
+__device__ __forceinline__ double value_of_key32(uint32_t key) { return (double)__uint_as_float(bits_of_key32(key)); }
 
 // Block-wide sum in a fixed shape (deterministic); every thread gets the total.
 __device__ __forceinline__ double block_sum(double v, double* red) {
@@ -99,15 +71,56 @@ __device__ __forceinline__ void finish(const double (&tot)[kMaxK], double n, int
   res->pf = pf;
 }
 
-// One block per segment: tile (blockIdx.y, blockIdx.x) of seg_rows x seg_cols elements, ragged at the
+// 16-bit types: one block of T threads per tile marks the tile's patterns (8 KB) and walks them.  `wide`: rows start on
+// 16-byte boundaries and hold whole vectors of eight.  A 256 x 256 tile by the bitonic network in 128 KB of
+// shared memory took two waves of 0.4 ms; this form holds two or more tiles per SM.
+template <int T, int CTAS>
+__global__ void __launch_bounds__(T, CTAS) proxy_segment_set_kernel(const uint16_t* w, int oc, int ic, int seg_rows, int seg_cols, int wide,
+                                                                   int bf16, int K, SegResult* out) {
+  __shared__ __align__(16) uint32_t bm[kPatternWords];
+  __shared__ SetShared<T> sh;
+  const int r0 = blockIdx.y * seg_rows, c0 = blockIdx.x * seg_cols;
+  const int nr = min(seg_rows, oc - r0), nc = min(seg_cols, ic - c0);
+  for (int j = threadIdx.x; j < kPatternWords / 4; j += T) reinterpret_cast<uint4*>(bm)[j] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  const uint16_t* src = w + (size_t)r0 * ic + c0;
+  if (wide) {
+    const int per_row = nc >> 3, total = nr * per_row;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * T) {
+      uint4 v[4];
+      bool in[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * T;
+        in[u] = i < total;
+        if (in[u]) v[u] = ldg_stream(src + (size_t)(i / per_row) * ic + 8 * (i % per_row));
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (in[u]) { mark_pair(bm, v[u].x); mark_pair(bm, v[u].y); mark_pair(bm, v[u].z); mark_pair(bm, v[u].w); }
+    }
+  } else {
+    const int total = nr * nc;
+    for (int i = threadIdx.x; i < total; i += T) mark_pattern(bm, src[(size_t)(i / nc) * ic + i % nc]);
+  }
+  __syncthreads();
+  const double n = (double)(nr * nc - 1);
+  SetStats s;
+  set_gaps<T>(bm, bf16 != 0, n, K, sh, s);
+  if (threadIdx.x == 0) {
+    SegResult r;
+    r.pc = r.pf = INFINITY; r.count = (unsigned)(nr * nc); r.nonfinite = s.nonfinite ? 1 : 0;
+    if (!s.nonfinite && !s.degenerate) proxy_from_set(s, n, K, &r.pc, &r.pf);
+    out[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = r;
+  }
+}
+
+// fp32: one block per segment: tile (blockIdx.y, blockIdx.x) of seg_rows x seg_cols elements, ragged at the
 // right and bottom edges.  np2 = the power of two the padded key array has (>= the largest segment).
-template <int DTYPE>
-__global__ void __launch_bounds__(kThreads, 1) proxy_segment_kernel(const void* w, int oc, int ic, int seg_rows, int seg_cols,
-                                                                  int np2, int K, SegResult* out) {
-  using T = Traits<DTYPE>;
-  using Key = typename T::Key;
+__global__ void __launch_bounds__(kThreads, 1) proxy_segment_f32_kernel(const uint32_t* src, int oc, int ic, int seg_rows, int seg_cols,
+                                                                      int np2, int K, SegResult* out) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  Key* keys = reinterpret_cast<Key*>(smem_raw);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);
   __shared__ double red[kThreads];
   __shared__ int s_bad;
   const int r0 = blockIdx.y * seg_rows, c0 = blockIdx.x * seg_cols;
@@ -116,13 +129,12 @@ __global__ void __launch_bounds__(kThreads, 1) proxy_segment_kernel(const void* 
   SegResult* res = out + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
-  const typename T::Elem* src = static_cast<const typename T::Elem*>(w);
   int bad = 0;
   for (int i = threadIdx.x; i < np2; i += kThreads) {
-    Key k = T::kPad;
+    uint32_t k = 0xFFFFFFFFu;
     if (i < count) {
-      const typename T::Elem b = src[(size_t)(r0 + i / nc) * ic + c0 + i % nc];
-      if (!T::finite(b)) bad = 1; else k = T::key(b);
+      const uint32_t b = src[(size_t)(r0 + i / nc) * ic + c0 + i % nc];
+      if ((b & 0x7F800000u) == 0x7F800000u) bad = 1; else k = key32(b);
     }
     keys[i] = k;
   }
@@ -139,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1) proxy_segment_kernel(const void* 
         const int lo = 2 * p - (p & (stride - 1));          // index with the `stride` bit clear
         const int hi = lo + stride;
         const bool up = (lo & size) == 0;
-        const Key a = keys[lo], b = keys[hi];
+        const uint32_t a = keys[lo], b = keys[hi];
         if ((a > b) == up) { keys[lo] = b; keys[hi] = a; }
       }
       __syncthreads();
@@ -148,7 +160,7 @@ __global__ void __launch_bounds__(kThreads, 1) proxy_segment_kernel(const void* 
     if (threadIdx.x == 0) { res->pc = INFINITY; res->pf = INFINITY; res->count = (unsigned)count; res->nonfinite = 0; }
     return;
   }
-  const double vmin = T::value(keys[0]), vmax = T::value(keys[count - 1]);
+  const double vmin = value_of_key32(keys[0]), vmax = value_of_key32(keys[count - 1]);
   const double R = vmax - vmin, n = (double)(count - 1);
   if (!(R > 0.0)) {     // constant segment: G' is undefined
     if (threadIdx.x == 0) { res->pc = INFINITY; res->pf = INFINITY; res->count = (unsigned)count; res->nonfinite = 0; }
@@ -158,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1) proxy_segment_kernel(const void* 
 #pragma unroll
   for (int i = 0; i < kMaxK; ++i) acc[i] = 0.0;
   for (int i = threadIdx.x; i + 1 < count; i += kThreads)
-    gap_terms((T::value(keys[i + 1]) - T::value(keys[i])) / R, n, K, acc);
+    gap_terms((value_of_key32(keys[i + 1]) - value_of_key32(keys[i])) / R, n, K, acc);
   double tot[kMaxK];
   for (int i = 0; i < kMaxK; ++i) tot[i] = (i == 0 || i < K) ? block_sum(acc[i], red) : 0.0;
   if (threadIdx.x == 0) { finish(tot, n, K, res); res->count = (unsigned)count; res->nonfinite = 0; }
@@ -251,19 +263,24 @@ rwkvq_status rwkvq_proxy_segments(const void* w, int dtype, int oc, int ic, int 
   if (!aligned16(ws)) return RWKVQ_EALIGN;
   const int gx = (ic + seg_cols - 1) / seg_cols, gy = (oc + seg_rows - 1) / seg_rows;
   if (gy > 65535) return RWKVQ_EUNSUPPORTED;
-  const int np2 = pseg::next_pow2((int)seg_elems);
-  const size_t smem = (size_t)np2 * pseg::elem_bytes(dtype);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   pseg::SegResult* res = static_cast<pseg::SegResult*>(ws);
-  const void* fn = dtype == RWKVQ_F16 ? (const void*)pseg::proxy_segment_kernel<RWKVQ_F16>
-                 : dtype == RWKVQ_BF16 ? (const void*)pseg::proxy_segment_kernel<RWKVQ_BF16>
-                                       : (const void*)pseg::proxy_segment_kernel<RWKVQ_F32>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pseg::kSmemKeysBytes);
-  if (e != cudaSuccess) return cuda_status(e);
   const dim3 grid((unsigned)gx, (unsigned)gy, 1);
-  if (dtype == RWKVQ_F16) pseg::proxy_segment_kernel<RWKVQ_F16><<<grid, pseg::kThreads, smem, s>>>(w, oc, ic, seg_rows, seg_cols, np2, K, res);
-  else if (dtype == RWKVQ_BF16) pseg::proxy_segment_kernel<RWKVQ_BF16><<<grid, pseg::kThreads, smem, s>>>(w, oc, ic, seg_rows, seg_cols, np2, K, res);
-  else pseg::proxy_segment_kernel<RWKVQ_F32><<<grid, pseg::kThreads, smem, s>>>(w, oc, ic, seg_rows, seg_cols, np2, K, res);
+  cudaError_t e = cudaSuccess;
+  if (dtype == RWKVQ_F32) {
+    const int np2 = pseg::next_pow2((int)seg_elems);
+    static SmemOptIn opt_in;
+    e = opt_in((const void*)pseg::proxy_segment_f32_kernel, (int)pseg::kSmemKeysBytes);
+    if (e != cudaSuccess) return cuda_status(e);
+    pseg::proxy_segment_f32_kernel<<<grid, pseg::kThreads, (size_t)np2 * 4, s>>>(static_cast<const uint32_t*>(w), oc, ic, seg_rows, seg_cols, np2, K, res);
+  } else {
+    const uint16_t* w16 = static_cast<const uint16_t*>(w);
+    const int wide = ic % 8 == 0 && seg_cols % 8 == 0, bf16 = dtype == RWKVQ_BF16;
+    // small tiles (a channel of a few thousand weights): the walk over the patterns is most of the work, and more blocks of
+    // fewer threads hide its latencies; large ones: the marking is, and wants threads
+    if (seg_elems <= 16384) pseg::proxy_segment_set_kernel<256, 4><<<grid, 256, 0, s>>>(w16, oc, ic, seg_rows, seg_cols, wide, bf16, K, res);
+    else pseg::proxy_segment_set_kernel<512, 2><<<grid, 512, 0, s>>>(w16, oc, ic, seg_rows, seg_cols, wide, bf16, K, res);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e);
   const size_t nseg = (size_t)gx * gy;

@@ -187,3 +187,33 @@ def test_proxy_segments_and_typed_errors():
                 B.rwkvq_proxy_select_typed(bad, 4, 1.0, 1.0)
     with pytest.raises(B.RwkvqError):
         B.rwkvq_proxy_segments(h, 16, 16, 9, 1.0, 1.0)              # K out of range
+
+
+def _pattern_matrix(kind, dtype):
+    """Matrices of 16-bit patterns at the edges of the walk over the pattern set."""
+    if kind == "every_third":        # thousands of gaps wider than one pattern: several rounds of the gap list
+        mag = np.arange(3, 0x7800, 3, dtype=np.uint16)
+        bits = np.concatenate([mag, mag | 0x8000])
+    elif kind == "no_zero":          # the gap across zero
+        bits = np.array([0x3C00, 0x3C01, 0x8001, 0xBC00] * 40, dtype=np.uint16)
+    elif kind == "minus_zero":       # +0 and -0 are one value
+        bits = np.array([0x0000, 0x8000, 0x3C00] * 40, dtype=np.uint16)
+    elif kind == "dense":            # every finite pattern of both signs below the exponent's last binades
+        mag = np.arange(0, 0x5000, dtype=np.uint16)
+        bits = np.concatenate([mag, mag | 0x8000])
+    else:                            # one sign only
+        bits = (np.arange(0x0400, 0x0480, dtype=np.uint16) | 0x8000).repeat(3)
+    bits = bits[: bits.size // 8 * 8]
+    return torch.from_numpy(bits.view(np.int16).copy()).cuda().view(dtype).reshape(8, -1)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("kind", ["every_third", "no_zero", "minus_zero", "dense", "negative"])
+def test_proxy_pattern_sets_at_the_edges(kind, dtype):
+    w = _pattern_matrix(kind, dtype)
+    ref = orc.proxy(w.double().cpu().numpy(), K=4)
+    assert w.numel() <= 65536
+    whole = B.rwkvq_proxy_select_typed(w, 4, math.inf, math.inf)
+    tile = B.rwkvq_proxy_segments(w, w.shape[0], w.shape[1], 4, math.inf, math.inf)
+    for pc, pf in ((whole[0], whole[1]), (tile[0][0, 0], tile[1][0, 0])):
+        assert _close(pc, ref[0]) and _close(pf, ref[1], 1e-8), (pc, pf, ref)
