@@ -324,3 +324,38 @@ def test_async_quantizer_and_check():
         B.rwkvq_quantize_dev_async(torch.from_numpy(w16).cuda(), 256, 384, B.RWKVQ_SQ, 3, imgs[0], ws)
     assert B.rwkvq_quantize_check(ws) == 4
     assert B.rwkvq_quantize_check(ws) == 0        # cleared by the check
+
+
+def _edge_tile(kind):
+    rng = np.random.default_rng(77)
+    if kind == "constant":
+        return np.full((256, 256), -0.125, np.float16)
+    if kind == "few":
+        return rng.choice(np.array([-1.5, -0.0, 0.0, 2.0 ** -24, 0.75, 60000.0], np.float16), (256, 256))
+    if kind == "wide":              # magnitudes over the whole range, a few vectors far out on each side
+        return (rng.choice([-1.0, 1.0], (256, 256)) * np.exp(rng.uniform(np.log(1e-7), np.log(6e4), (256, 256)))).astype(np.float16)
+    if kind == "offset":            # all of one sign, far from zero
+        return (rng.standard_normal((256, 256)) * 0.01 + 3.0).astype(np.float16)
+    return (rng.standard_t(3, (256, 256)) * 0.01).astype(np.float16)
+
+
+@pytest.mark.parametrize("bits", [6, 8])
+@pytest.mark.parametrize("kind", ["constant", "few", "wide", "offset", "tails"])
+def test_vq_device_iterations_and_assignment_at_the_edges(kind, bits):
+    """Candidate lists and cluster sums: the assignment is the nearest centre of all, and one iteration moves the seeds to the
+    means of their members."""
+    w16 = _edge_tile(kind)
+    v = tile_vectors(w16, 0, 0)
+    books = []
+    for iters in (0, 1, 7):
+        _, img = quantize_dev(w16, B.RWKVQ_VQ, bits, seed=9, iters=iters)
+        _, codes = B.rwkvq_image_unpack(img.cpu().numpy())
+        c = np.asarray(codes["codebook"]).reshape(1 << bits, 2).astype(np.float64)
+        assert np.array_equal(np.asarray(codes["q"]).reshape(-1), orc._nearest(v, c)), (kind, iters)
+        books.append(c)
+    near = orc._nearest(v, books[0])
+    for e in range(1 << bits):
+        members = v[near == e]
+        want = members.mean(axis=0) if len(members) else books[0][e]
+        # fp16 rounding; a tie decided otherwise in fp32 moves a mean by less than that of a cluster's spread
+        assert np.all(np.abs(books[1][e] - want) <= 1e-3 * np.abs(want) + 2.0 ** -24 + 1e-2 * (np.ptp(members, axis=0) if len(members) else 0.0)), (kind, e)
