@@ -195,13 +195,15 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
-// The hint lets the hardware park the thread for up to that many nanoseconds (it is woken when
-// the phase completes), so that waiting warps do not compete for issue slots with computing ones.
+// The hardware parks the warp for a while (it is woken when the phase completes), so that waiting warps do not compete for
+// issue slots with computing ones.  Whole warps wait: from an arrival to the waiting warp's next instruction it takes about
+// 115 cycles then, 145 with a time limit as a third operand, and 750 when one lane waits while the others sit at the
+// warp's next meeting point.
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(2000u) : "memory");
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
 // The launch's poll limit sits directly behind the CTA's abort flag in the control block (Ctrl).
@@ -209,6 +211,7 @@ __device__ __forceinline__ uint32_t poll_limit_of(volatile int* abort_flag) { re
 // Bounded wait by one thread: gives up (and raises the CTA-wide abort flag) after that many polls
 // or when another role of this CTA has already given up.
 __device__ __forceinline__ bool mbar_wait_one(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  if (mbar_try_wait(bar, parity)) return true;
   const uint32_t limit = poll_limit_of(abort_flag);
   for (uint32_t it = 0; it < limit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -358,10 +361,7 @@ __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint
       const int slot = (int)(i % (uint32_t)a.n_slots);
       const uint32_t round = i / (uint32_t)a.n_slots;
       uint8_t* sl = smem + kCtrlBytes + (size_t)slot * a.slot_bytes;
-      int good = 1;
-      if (lane == 0) good = mbar_wait_one(&ctrl->empty[slot], (round & 1u) ^ 1u, abortp, a.status) ? 1 : 0;
-      good = __shfl_sync(0xFFFFFFFFu, good, 0);
-      if (!good) { ok = false; break; }
+      if (!mbar_wait_warp(&ctrl->empty[slot], (round & 1u) ^ 1u, abortp, a.status)) { ok = false; break; }
       if ((lane >> 3) == k) *reinterpret_cast<uint4*>(sl + (lane & 7) * 16) = cur;
       // fields for lane 0, by 16-byte piece of descriptor k
       const uint32_t s0l = __shfl_sync(0xFFFFFFFFu, cur.x, 8 * k), s0h = __shfl_sync(0xFFFFFFFFu, cur.y, 8 * k);
@@ -810,6 +810,9 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
   constexpr int kStagerThreads = Shape<NB>::kStagerThreads;
   const int stid = threadIdx.x - Shape<NB>::kConsumerThreads;
   const int lane = stid & 31;
+  // The grid barriers are polled by the whole first warp (one request per poll, no divergence to leave): c2 B = 1 453 -> 447 us, c3
+  // B = 8 1589 -> 1577; by one lane with two batch blocks, where it costs a little (c4 B = 16 4212 -> 4242 us).
+  constexpr int kPollLanes = NB == 1 ? 32 : 1;
   volatile int* abortp = &ctrl->abort_flag;
   uint32_t nseg = 0;          // segments staged so far
   uint32_t passed2 = 0xFFFFFFFFu;   // second-stage barrier this CTA has already passed
@@ -839,12 +842,12 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         // once the barrier opens, do this CTA's share of the new stage's pre-pass and publish it
         // through the stage's second barrier
         if (ev.barrier < (uint32_t)a.n_stages) {
-          if (ok && stid == 0) {
+          if (ok && stid < kPollLanes) {
             uint32_t it = 0;
             while ((int)(ld_acquire_gpu(a.counter + ev.barrier) - (a.target + a.wait_skew)) < 0) {
               if (++it >= (a.poll_limit << 2) || *abortp) { *abortp = 1; atomicExch(a.status, (int)RWKVQ_ETIMEOUT); ok = false; break; }
             }
-            if (ok && a.in_flag) {
+            if (ok && a.in_flag && stid == 0) {
               // the last input byte any product of the coming stage reads (x and x_prev, [B][ic] fp16 each)
               const StepMixOp* mo = a.mixops + ev.arrd.op_first;
               uint64_t last = 0;
@@ -874,7 +877,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
       // The segment is a rectangle of the stage's pre-pass output: pass the stage's second barrier
       // (once per stage), then fetch B rows and the block of sums with bulk copies.
       const uint32_t b2 = (uint32_t)a.n_stages + ev.barrier;      // counter of the second barrier of stage ev.barrier - 1
-      if (ok && stid == 0 && b2 != passed2) {
+      if (ok && stid < kPollLanes && b2 != passed2) {
         uint32_t it = 0;
         while ((int)(ld_acquire_gpu(a.counter + b2) - (a.target + a.wait_skew)) < 0) {
           if (++it >= (a.poll_limit << 2) || *abortp) { *abortp = 1; atomicExch(a.status, (int)RWKVQ_ETIMEOUT); ok = false; break; }
@@ -950,7 +953,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         *reinterpret_cast<uint4*>(xb + (size_t)b * xstride + (size_t)c8 * 16) = r;
       }
     }
-    if (ok && ev.barrier && stid == 0) {
+    if (ok && ev.barrier && stid < kPollLanes) {
       // grid-wide stage barrier: every CTA has finished (and published) the previous stage.  Each
       // barrier has its own arrival counter, so a CTA without work may run ahead and arrive at
       // later barriers without releasing this one early.
