@@ -20,16 +20,15 @@
 //     every input fragment shared by the two records.  Partial sums go to y with fp32 reductions
 //     (16 bytes per lane after a transpose among lanes) at the end of a run along K.
 //
-// For batches of four and more, and whenever a product's input is an element-wise operator on
+// For larger inputs per CTA, and whenever a product's input is an element-wise operator on
 // earlier outputs (rwkvq_input_xform: the WKV recurrence and sigmoid gate of Appendix A.1 Eqs. 23-24,
 // the squared ReLU and output gate of Eq. 27, optionally a root-mean-square normalisation), the
 // inputs of a stage are not built per CTA: after the stage barrier all CTAs together compute the
 // stage's x_mix once (mix_slice: a half-warp per 128-column group) into a scratch region of the plan,
 // publish it through a second barrier, and every CTA fetches its segments with bulk copies.
 //
-// The host plans the step once: every stage's units are dealt WHOLE to the CTAs, row of tiles by
-// row of tiles where that balances (each row gets a number of CTAs by greedy cost per CTA), else at
-// their cost midpoints, small stages in eighths of a unit (one warp's records); the plan is a per-CTA
+// The host plans the step once: every stage's units are dealt WHOLE to the CTAs, in runs of neighbouring units by the
+// smallest estimated time of the slowest CTA, along rows of tiles where that is no worse; the plan is a per-CTA
 // list of 128-byte unit descriptors plus a list of 64-byte input events (segments and barrier
 // arrivals).
 #include <cuda.h>           // types of the stream memory operations (no driver symbol is linked)
@@ -54,12 +53,12 @@ unsigned abort_epoch();     // api_misc.cu: bumped whenever rwkvq_device_status 
 enum { UF_FLUSH = 1, UF_VQ = 2, UF_BITS8 = 4 };
 
 struct StepUnit {            // 128 bytes, copied into the slot header by the producer
-  uint64_t src0, src1;       // global addresses of the first copied record of chunk A / chunk B (0 = absent)
+  uint64_t src0, src1;       // global addresses of chunk A / chunk B (0 = absent)
   uint64_t cb_src;           // VQ: codebook of the tile
-  uint32_t bytes0, bytes1;   // bytes copied from each chunk: (w1 - w0) records
+  uint32_t bytes0, bytes1;   // bytes of each chunk
   uint32_t cb_bytes;
-  uint32_t off0;             // w0 * record bytes: where the copied records sit inside a chunk
-  uint32_t flags;            // UF_* | w0 << 8 | w1 << 12: warps w0 <= w < w1 of the group have a record
+  uint32_t off0;             // unused
+  uint32_t flags;            // UF_*
   uint32_t seg;              // number, within this CTA, of the input segment the unit reads
   uint32_t stage;            // stage number (0-based)
   uint32_t xcol0;            // column of the unit's tile inside the segment
@@ -368,7 +367,7 @@ __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint
       const uint32_t s1l = __shfl_sync(0xFFFFFFFFu, cur.z, 8 * k), s1h = __shfl_sync(0xFFFFFFFFu, cur.w, 8 * k);
       const uint32_t cbl = __shfl_sync(0xFFFFFFFFu, cur.x, 8 * k + 1), cbh = __shfl_sync(0xFFFFFFFFu, cur.y, 8 * k + 1);
       const uint32_t by0 = __shfl_sync(0xFFFFFFFFu, cur.z, 8 * k + 1), by1 = __shfl_sync(0xFFFFFFFFu, cur.w, 8 * k + 1);
-      const uint32_t cbb = __shfl_sync(0xFFFFFFFFu, cur.x, 8 * k + 2), off0 = __shfl_sync(0xFFFFFFFFu, cur.y, 8 * k + 2);
+      const uint32_t cbb = __shfl_sync(0xFFFFFFFFu, cur.x, 8 * k + 2);
       const uint32_t chb = __shfl_sync(0xFFFFFFFFu, cur.z, 8 * k + 5);
       __syncwarp();
       if (lane == 0) {
@@ -379,8 +378,8 @@ __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint
         } else {
           mbar_arrive_expect_tx(full, tx);
           uint8_t* data = sl + 128;
-          if (by0) bulk_g2s(data + off0, reinterpret_cast<const void*>(((uint64_t)s0h << 32) | s0l), by0, full, policy);
-          if (by1) bulk_g2s(data + chb + off0, reinterpret_cast<const void*>(((uint64_t)s1h << 32) | s1l), by1, full, policy);
+          if (by0) bulk_g2s(data, reinterpret_cast<const void*>(((uint64_t)s0h << 32) | s0l), by0, full, policy);
+          if (by1) bulk_g2s(data + chb, reinterpret_cast<const void*>(((uint64_t)s1h << 32) | s1l), by1, full, policy);
           if (cbb) bulk_g2s(data + 2 * chb, reinterpret_cast<const void*>(((uint64_t)cbh << 32) | cbl), cbb, full, policy);
         }
       }
@@ -1173,8 +1172,6 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     const uint8_t* data = sl + 128;
     const uint8_t* xb = xbufs + (size_t)((uint32_t)held % XBufs<MIX, NB>::kCount) * XBufs<MIX, NB>::kBytes;
     const uint32_t xstride = u->xstride, nbp = u->nbp, chb = u->chunk_bytes, rb = u->rec_bytes;
-    const uint32_t w0 = (flags >> 8) & 15u, w1 = (flags >> 12) & 15u;
-    const bool active = (uint32_t)w >= w0 && (uint32_t)w < w1;
     const bool has_b = by1 != 0u;
     const uint32_t oc = u->oc, row0 = u->row0;
     float* y = reinterpret_cast<float*>(u->y);
@@ -1189,39 +1186,33 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         // 128-column groups as one stretch of code (eight tensor-core chains for the scheduler to interleave).
         uint32_t wa0[6], wb0[6], wa1[6], wb1[6];
         uint4 sza = make_uint4(0, 0, 0, 0), szb = sza;
-        if (active) {
-          sq_group_words<0>(ra, lane, wa0);
-          sq_group_words<1>(ra, lane, wa1);
-          sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
-          if (has_b) {
-            sq_group_words<0>(rbp, lane, wb0);
-            sq_group_words<1>(rbp, lane, wb1);
-            szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
-          }
+        sq_group_words<0>(ra, lane, wa0);
+        sq_group_words<1>(ra, lane, wa1);
+        sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
+        if (has_b) {
+          sq_group_words<0>(rbp, lane, wb0);
+          sq_group_words<1>(rbp, lane, wb1);
+          szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        if (active) {
-          sq_pair<NB, 0>(wa0, wb0, sza, szb, has_b, xl, acca, accb);
-          sq_pair<NB, 1>(wa1, wb1, sza, szb, has_b, xl, acca, accb);
-        }
+        sq_pair<NB, 0>(wa0, wb0, sza, szb, has_b, xl, acca, accb);
+        sq_pair<NB, 1>(wa1, wb1, sza, szb, has_b, xl, acca, accb);
       } else {
       uint32_t wa[6], wb[6];
       uint4 sza = make_uint4(0, 0, 0, 0), szb = sza;
-      if (active) {
-        sq_group_words<0>(ra, lane, wa);
-        sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
-        if (has_b) {
-          sq_group_words<0>(rbp, lane, wb);
-          szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
-        }
-        sq_pair<NB, 0>(wa, wb, sza, szb, has_b, xl, acca, accb);
-        sq_group_words<1>(ra, lane, wa);
-        if (has_b) sq_group_words<1>(rbp, lane, wb);
+      sq_group_words<0>(ra, lane, wa);
+      sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
+      if (has_b) {
+        sq_group_words<0>(rbp, lane, wb);
+        szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
       }
+      sq_pair<NB, 0>(wa, wb, sza, szb, has_b, xl, acca, accb);
+      sq_group_words<1>(ra, lane, wa);
+      if (has_b) sq_group_words<1>(rbp, lane, wb);
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctrl->empty[slot]);     // the rest of the records is in registers: free the slot
-      if (active) sq_pair<NB, 1>(wa, wb, sza, szb, has_b, xl, acca, accb);
+      sq_pair<NB, 1>(wa, wb, sza, szb, has_b, xl, acca, accb);
       }
     } else {
       // replicate the tile's codebook for conflict-free lookups (the eight warps of the group)
@@ -1237,46 +1228,40 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
       const XLane xl = make_xlane(xb + (size_t)u->xcol0 * 2, xstride, nullptr, nbp, a.B, lane);
       if (flags & UF_BITS8) {
         uint32_t va[16], vb[16];
-        if (active) {
-          vq_half_words<8, 0>(ra, lane, va); vq_half_words<8, 0>(rbp, lane, vb);
-          vq_pair<8, NB, 0>(va, vb, cb_lane, xl, acca, accb);
-          vq_half_words<8, 1>(ra, lane, va); vq_half_words<8, 1>(rbp, lane, vb);
-        }
+        vq_half_words<8, 0>(ra, lane, va); vq_half_words<8, 0>(rbp, lane, vb);
+        vq_pair<8, NB, 0>(va, vb, cb_lane, xl, acca, accb);
+        vq_half_words<8, 1>(ra, lane, va); vq_half_words<8, 1>(rbp, lane, vb);
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        if (active) vq_pair<8, NB, 1>(va, vb, cb_lane, xl, acca, accb);
+        vq_pair<8, NB, 1>(va, vb, cb_lane, xl, acca, accb);
       } else {
         uint32_t va[12], vb[12];
-        if (active) {
-          vq_half_words<6, 0>(ra, lane, va); vq_half_words<6, 0>(rbp, lane, vb);
-          vq_pair<6, NB, 0>(va, vb, cb_lane, xl, acca, accb);
-          vq_half_words<6, 1>(ra, lane, va); vq_half_words<6, 1>(rbp, lane, vb);
-        }
+        vq_half_words<6, 0>(ra, lane, va); vq_half_words<6, 0>(rbp, lane, vb);
+        vq_pair<6, NB, 0>(va, vb, cb_lane, xl, acca, accb);
+        vq_half_words<6, 1>(ra, lane, va); vq_half_words<6, 1>(rbp, lane, vb);
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        if (active) vq_pair<6, NB, 1>(va, vb, cb_lane, xl, acca, accb);
+        vq_pair<6, NB, 1>(va, vb, cb_lane, xl, acca, accb);
       }
     }
     if (flags & UF_FLUSH) {
-      if (active) {
-        {
-          // Four lanes that share t hold a 4 x 4 block (rows 4J .. 4J+3 of one row half x the accumulator's four
-          // elements): transposed, every lane owns four consecutive rows of ONE batch column and adds them
-          // with a single 16-byte reduction instead of four scattered ones.  The plan accepts only outputs
-          // that start on a 16-byte boundary, and the format only row counts that are multiples of 16.
-          const int i = g & 3;
-          const uint32_t rbase = row0 + (uint32_t)w * 16u + 8u * (uint32_t)(i >> 1) + (uint32_t)(g & ~3);
+      {
+        // Four lanes that share t hold a 4 x 4 block (rows 4J .. 4J+3 of one row half x the accumulator's four
+        // elements): transposed, every lane owns four consecutive rows of ONE batch column and adds them
+        // with a single 16-byte reduction instead of four scattered ones.  The plan accepts only outputs
+        // that start on a 16-byte boundary, and the format only row counts that are multiples of 16.
+        const int i = g & 3;
+        const uint32_t rbase = row0 + (uint32_t)w * 16u + 8u * (uint32_t)(i >> 1) + (uint32_t)(g & ~3);
 #pragma unroll
-          for (int n = 0; n < NB; ++n) {
-            const int b = n * 8 + 2 * t + (i & 1);
-            float va[4] = {acca[n][0], acca[n][1], acca[n][2], acca[n][3]};
-            transpose4_lanes(va, i);
-            if (b < a.B && rbase < oc) red_add_v4(y + (size_t)b * oc + rbase, va);
-            if (has_b) {                      // warp-uniform
-              float vb[4] = {accb[n][0], accb[n][1], accb[n][2], accb[n][3]};
-              transpose4_lanes(vb, i);
-              if (b < a.B && rbase + 128u < oc) red_add_v4(y + (size_t)b * oc + rbase + 128u, vb);
-            }
+        for (int n = 0; n < NB; ++n) {
+          const int b = n * 8 + 2 * t + (i & 1);
+          float va[4] = {acca[n][0], acca[n][1], acca[n][2], acca[n][3]};
+          transpose4_lanes(va, i);
+          if (b < a.B && rbase < oc) red_add_v4(y + (size_t)b * oc + rbase, va);
+          if (has_b) {                      // warp-uniform
+            float vb[4] = {accb[n][0], accb[n][1], accb[n][2], accb[n][3]};
+            transpose4_lanes(vb, i);
+            if (b < a.B && rbase + 128u < oc) red_add_v4(y + (size_t)b * oc + rbase + 128u, vb);
           }
         }
       }
@@ -1349,7 +1334,7 @@ static std::unordered_map<const void*, PlanInfo> g_plans;
 
 struct HostUnit {
   StepUnit u;
-  int op, tr, kt, stage, w0, w1;
+  int op, tr, kt, stage;
 };
 
 // Shared-memory footprint of an input segment: B rows of x_mix, the per-group sums (SQ) and one
@@ -1432,8 +1417,23 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   info->poll_limit = kDefaultPollLimit; info->wait_skew = 0;
   bool any_xform = false;
   for (int i = 0; i < n_ops; ++i) any_xform = any_xform || ops[i].in.kind != RWKVQ_IN_BUFFER || ops[i].in.xprev_out_fp16 != nullptr;
-  // see StepArgs::mix; the element-wise operators in front of a product exist in the stage pre-pass only
-  const bool mix = B >= 4 || any_xform;
+  // Inputs per CTA and stage: batch rows x columns of an even share of the units, averaged over the stages.
+  uint64_t share = 0, stages = 0;
+  for (int i = 0; i < n_ops; ++stages) {
+    uint64_t n = 0;
+    int j = i;
+    for (; j < n_ops && ops[j].stage == ops[i].stage; ++j) n += (uint64_t)((ops[j].W_desc.oc_pad + 255) / 256) * (uint64_t)(ops[j].W_desc.ic_pad / 256);
+    share += (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B;
+    i = j;
+  }
+  // A stage pre-pass (StepArgs::mix) costs a second barrier, about 2 us per stage whatever the sizes; without it every CTA mixes the
+  // columns it reads itself.  The line was measured with stacks of 512 to 4096 columns and batches of 2 to 16 (pre-pass / without, us): 7168 h
+  // 2048 d B=4, 1792 inputs, 232 / 176; B=8, 3584, 242 / 232; d=4096 B=3, 4608, 371 / 390; with seven stager warps d=2048 B=10, 4480, 283 /
+  // 255; B=16, 7168, 300 / 299; d=2560 B=12, 8448, 337 / 347.  The element-wise operators exist in the pre-pass only.
+  const bool mix = any_xform || share > stages * (B > 8 ? 7200u : 3600u);
+  // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
+  // take them in turn.  A segment that the CTA mixes itself weighs more.
+  const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;
   const uint32_t xbuf_bytes = XBufs<false, 1>::kBytes;
   info->mix = mix ? 1 : 0;
   const uint32_t nbp = (uint32_t)((B + 1) & ~1);
@@ -1518,11 +1518,8 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           units.push_back(h);
         }
     }
-    // contiguous, cost-balanced ranges cut at one eighth of a unit (the records of one warp).  The
-    // cost of a unit is its record count weighted by what a record of its format costs the consumer
-    // warps (measured with every product in one stage: a VQ record with 64 entries takes about 1.45
-    // times, one with 256 entries about 1.25 times as long as an SQ record), so that the CTAs that
-    // get a stage's VQ matrix do not finish last.
+    // The cost of a unit is its record count weighted by what a record of its format costs the consumer
+    // warps, so that the CTAs that get a stage's VQ matrix do not finish last.
     auto cost_of = [&](const HostUnit& h) -> uint64_t {
       const uint64_t recs = (h.u.bytes0 + h.u.bytes1) / h.u.rec_bytes;
       // in twentieths of an SQ record; the table lookups weigh more the more batch columns a record meets
@@ -1532,94 +1529,84 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       const uint64_t wgt = !(h.u.flags & UF_VQ) ? 20u : (h.u.flags & UF_BITS8) ? vq8 : vq6;
       return recs * wgt * 64u;
     };
-    // A consumer group spends about the same time on a piece of a unit as on a whole unit (the
-    // warps without a record idle), and every further input segment of a CTA costs about 1.7 us of
-    // serial staging; traces of all CTAs' barrier arrivals showed the stages waiting for the CTAs
-    // with the most pieces and segments, not for the most bytes.  So units are dealt WHOLE, and
-    // where it balances, row by row: each row of tiles (one product, one 256-row block: one input
-    // segment) gets a number of CTAs, greedily the row with the largest cost per CTA first, and
-    // its units are split into that many runs of neighbouring column tiles.  This is taken when no
-    // CTA ends up more than one unit above the even share; small stages leave some CTAs idle.
-    bool dealt = false;
-    auto push_whole = [&](int c, const HostUnit& h) {
-      HostUnit part = h;
-      part.w0 = 0; part.w1 = 8;
-      part.u.off0 = 0;
-      part.u.flags |= (0u << 8) | (8u << 12);
-      cta_units[c].push_back(part);
+    // Units are dealt WHOLE (a consumer group spends about the same time on a piece of a unit as on a whole one, the warps
+    // without a record idle), in runs of neighbouring units, by the smallest estimated time of the slowest CTA.  The estimate
+    // of a run of units: their costs, kRunCost for every row of tiles it touches, and kOddCost.  Against rows cut into whole
+    // numbers of runs alone: 14B-class stack B=16 4212 -> 4085 us (a stage of 64 rows x 16 tiles: seven units per CTA instead of
+    // eight), 7B-class B=1 1277 -> 1254.
+    const uint64_t whole = 16u * 20u * 64u;                      // an SQ unit
+    std::vector<uint64_t> before(units.size() + 1, 0);
+    for (size_t i = 0; i < units.size(); ++i) before[i + 1] = before[i] + cost_of(units[i]);
+    auto new_row = [&](size_t i) { return units[i].op != units[i - 1].op || units[i].tr != units[i - 1].tr; };
+    // most units from `first` on whose estimate stays within `limit`
+    auto take = [&](size_t first, uint64_t limit) {
+      size_t best = 0;
+      uint64_t extra = kRunCost * whole / 64u;
+      for (size_t n = 1; first + n <= units.size(); ++n) {
+        const size_t i = first + n - 1;
+        if (n > 1 && new_row(i)) extra += kRunCost * whole / 64u;
+        const uint64_t sum = before[i + 1] - before[first] + extra;
+        const uint64_t est = sum + (kGroups == 2 && (n & 1) ? cost_of(units[i]) * kOddCost / 64u : 0u);
+        if (est <= limit) best = n;
+        if (sum > limit) break;
+      }
+      return best;
     };
+    typedef std::vector<std::pair<size_t, size_t>> Deal;         // (first unit, units) of consecutive CTAs
+    auto pack = [&](uint64_t limit, Deal* deal) {
+      if (deal) deal->clear();
+      size_t i = 0;
+      for (int c = 0; c < P && i < units.size(); ++c) {
+        const size_t n = take(i, limit);
+        if (n == 0) return false;
+        if (deal) deal->push_back({i, n});
+        i += n;
+      }
+      return i == units.size();
+    };
+    // runs that ignore the ends of rows
+    uint64_t lo = 0, hi = before.back() + (uint64_t)(units.size() + 1) * (2u * whole);
+    while (lo + whole / 64u < hi) {
+      const uint64_t mid = lo + (hi - lo) / 2;
+      if (pack(mid, nullptr)) hi = mid; else lo = mid;
+    }
+    Deal deal;
+    pack(hi, &deal);
+    // rows of tiles cut into a number of runs each, greedily the row with the largest cost per CTA first: taken where it is no worse (one
+    // input segment and one flush per CTA; small stages leave some CTAs idle)
     {
-      struct Row { size_t first, count; uint64_t cost; int k; };
+      struct Row { size_t first, count; uint64_t cost; size_t k; };
       std::vector<Row> rows;
       for (size_t i = 0; i < units.size();) {
-        size_t j = i;
-        uint64_t cst = 0;
-        while (j < units.size() && units[j].op == units[i].op && units[j].tr == units[i].tr) { cst += cost_of(units[j]); ++j; }
-        rows.push_back(Row{i, j - i, cst, 1});
+        size_t j = i + 1;
+        while (j < units.size() && !new_row(j)) ++j;
+        rows.push_back(Row{i, j - i, before[j] - before[i], 1});
         i = j;
       }
-      if (!rows.empty() && rows.size() <= (size_t)P) {
-        int spare = P - (int)rows.size();
-        while (spare > 0) {
-          size_t best = rows.size();
-          uint64_t best_cost = 0;
-          for (size_t r = 0; r < rows.size(); ++r) {
-            if ((size_t)rows[r].k >= rows[r].count) continue;          // one unit per CTA at most
-            const uint64_t per = rows[r].cost / (uint64_t)rows[r].k;
-            if (per > best_cost) { best_cost = per; best = r; }
+      if (rows.size() <= (size_t)P) {
+        for (size_t spare = (size_t)P - rows.size(); spare > 0; --spare) {
+          Row* best = nullptr;
+          for (Row& r : rows)
+            if (r.k < r.count && (!best || r.cost / r.k > best->cost / best->k)) best = &r;
+          if (!best) break;
+          ++best->k;
+        }
+        Deal by_row;
+        bool fits = true;
+        for (const Row& r : rows)
+          for (size_t q = 0; q < r.k && fits; ++q) {
+            const size_t a = r.first + r.count * q / r.k, b = r.first + r.count * (q + 1) / r.k;
+            by_row.push_back({a, b - a});
+            fits = take(a, hi + whole / 64u) >= b - a;
           }
-          if (best == rows.size()) break;
-          ++rows[best].k; --spare;
-        }
-        size_t max_units = 0;
-        for (const Row& r : rows) max_units = std::max(max_units, (r.count + (size_t)r.k - 1) / (size_t)r.k);
-        const size_t even = (units.size() + (size_t)P - 1) / (size_t)P;
-        if (max_units <= even + 1) {
-          // start at a CTA that moves with the stage, so that idle CTAs are not always the same SMs
-          size_t c = ((size_t)s * 37u) % (size_t)P;
-          for (const Row& r : rows)
-            for (int q = 0; q < r.k; ++q) {
-              const size_t lo = r.count * (size_t)q / (size_t)r.k, hi = r.count * (size_t)(q + 1) / (size_t)r.k;
-              for (size_t i = lo; i < hi; ++i) push_whole((int)c, units[r.first + i]);
-              c = (c + 1) % (size_t)P;
-            }
-          dealt = true;
-        }
+        if (fits) deal.swap(by_row);
       }
     }
-    uint64_t total = 0;
-    for (const HostUnit& h : units) total += cost_of(h);
-    uint64_t run = 0;
-    auto cta_of = [&](uint64_t mid) {
-      int c = (int)((mid * (uint64_t)P) / (total ? total : 1));
-      return c >= P ? P - 1 : c;
-    };
-    const bool whole_units = units.size() >= (size_t)4 * (size_t)P;   // many units per CTA: a whole unit at its cost midpoint
-    for (const HostUnit& h : units) {
-      if (dealt) break;
-      if (whole_units) {
-        push_whole(cta_of(run + cost_of(h) / 2), h);
-        run += cost_of(h);
-        continue;
-      }
-      const uint64_t e8 = cost_of(h) / 8;
-      int w = 0;
-      while (w < 8) {
-        const int c = cta_of(run + (uint64_t)w * e8 + e8 / 2);
-        int w1 = w + 1;
-        while (w1 < 8 && cta_of(run + (uint64_t)w1 * e8 + e8 / 2) == c) ++w1;
-        HostUnit part = h;
-        part.w0 = w; part.w1 = w1;
-        const uint32_t rb = h.u.rec_bytes;
-        part.u.off0 = (uint32_t)w * rb;
-        part.u.src0 = h.u.src0 + (uint64_t)w * rb;
-        part.u.bytes0 = (uint32_t)(w1 - w) * rb;
-        if (h.u.bytes1) { part.u.src1 = h.u.src1 + (uint64_t)w * rb; part.u.bytes1 = (uint32_t)(w1 - w) * rb; }
-        part.u.flags |= ((uint32_t)w << 8) | ((uint32_t)w1 << 12);
-        cta_units[c].push_back(part);
-        w = w1;
-      }
-      run += cost_of(h);
+    // start at a CTA that moves with the stage, so that idle CTAs are not always the same SMs
+    size_t c = ((size_t)s * 37u) % (size_t)P;
+    for (const auto& d : deal) {
+      for (size_t i = d.first; i < d.first + d.second; ++i) cta_units[c].push_back(units[i]);
+      c = (c + 1) % (size_t)P;
     }
     for (int c = 0; c < P; ++c) make_arrival(c, s + 1, s + 1);
   }
@@ -1684,8 +1671,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     // a group accumulates along K in registers while its consecutive units stay on the same rows
     for (size_t i = 0; i < n; ++i) {
       const size_t j = i + (size_t)kGroups;
-      const bool same_run = j < n && L[j].stage == L[i].stage && L[j].op == L[i].op && L[j].tr == L[i].tr &&
-                            L[j].w0 == L[i].w0 && L[j].w1 == L[i].w1;
+      const bool same_run = j < n && L[j].stage == L[i].stage && L[j].op == L[i].op && L[j].tr == L[i].tr;
       if (!same_run) L[i].u.flags |= UF_FLUSH;
     }
     all_events.push_back(cta_arrivals[c][0]);
@@ -1899,8 +1885,7 @@ rwkvq_status step_run_impl(const void* plan_dev, size_t plan_bytes, void* stream
     e = cudaMemsetAsync(a.counter, 0, round_up_sz((size_t)info.n_barriers * 4, 256), s);
     if (e != cudaSuccess) return cuda_status(e);
   }
-  // batches of 4 and more use the stage pre-pass (StepArgs::mix)
-  const void* fn = !info.mix ? (const void*)step_kernel<1, false> : info.NB == 1 ? (const void*)step_kernel<1, true> : (const void*)step_kernel<2, true>;
+  const void* fn = !info.mix ? (info.NB == 1 ? (const void*)step_kernel<1, false> : (const void*)step_kernel<2, false>) : info.NB == 1 ? (const void*)step_kernel<1, true> : (const void*)step_kernel<2, true>;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
   if (e != cudaSuccess) return cuda_status(e);
   void* params[] = {&a};
@@ -1966,20 +1951,18 @@ rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, i
       const rwkvq_desc& d = ops[o].W_desc;
       const uint32_t KT = (uint32_t)d.ic_pad / 256u, slices = (uint32_t)d.oc / 16u;
       const uint8_t* payload = static_cast<const uint8_t*>(ops[o].W_image_dev) + RWKVQ_HEADER_BYTES;
-      const uint32_t w0 = (u.flags >> 8) & 15u, w1 = (u.flags >> 12) & 15u;
-      if (w0 >= w1 || w1 > 8u || u.off0 != w0 * u.rec_bytes) return RWKVQ_EINVAL;
       // the unit's chunks: warp w of the group takes record w of chunk A (and of chunk B, 128 rows below)
       const uint64_t src[2] = {u.src0, u.src1};
       const uint32_t bytes[2] = {u.bytes0, u.bytes1};
       for (int h = 0; h < 2; ++h) {
         if (!bytes[h]) continue;
-        if (bytes[h] != (w1 - w0) * u.rec_bytes) return RWKVQ_EINVAL;
-        const uint64_t rel = src[h] - (uint64_t)(uintptr_t)payload - (uint64_t)w0 * u.rec_bytes;
+        if (bytes[h] != 8u * u.rec_bytes) return RWKVQ_EINVAL;
+        const uint64_t rel = src[h] - (uint64_t)(uintptr_t)payload;
         if (rel % u.chunk_bytes) return RWKVQ_EINVAL;
         const uint64_t chunk = rel / u.chunk_bytes;       // mb * KT + kt
         const uint32_t mb = (uint32_t)(chunk / KT), kt = (uint32_t)(chunk % KT);
         if (mb * 128u != u.row0 + 128u * (uint32_t)h) return RWKVQ_EINVAL;
-        for (uint32_t w = w0; w < w1; ++w) {
+        for (uint32_t w = 0; w < 8u; ++w) {
           const uint32_t slice = mb * 8u + w;
           if (slice >= slices) continue;                  // padding rows of the last chunk
           counts_host[base[o] + (size_t)slice * KT + kt] += 1u;
