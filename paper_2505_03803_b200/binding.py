@@ -175,14 +175,32 @@ def _np_ptr(a: np.ndarray | None):
     return None if a is None else a.ctypes.data_as(C.c_void_p)
 
 
-def _stream_ptr(stream=None):
+_torch = None
+_raw_stream = None          # torch's query for the current stream's handle of a device, where this torch has it
+
+
+def _load_torch():
+    global _torch, _raw_stream
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    _torch = torch
+    if hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice"):
+        _raw_stream = torch._C._cuda_getCurrentRawStream
+    return torch
+
+
+def _stream_ptr(stream=None):
+    """cudaStream_t of `stream` (None: the current stream).  The stream object torch.cuda.current_stream builds costs more
+    than the launch of a small product, so the handle is asked for directly once CUDA is up."""
+    t = _torch or _load_torch()
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and t.cuda.is_initialized():
+        return _raw_stream(t._C._cuda_getDevice())
+    return t.cuda.current_stream().cuda_stream
 
 
 def _dev_ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 class Blob:
@@ -294,12 +312,13 @@ def rwkvq_gemv_workspace_bytes(desc: Desc, B: int) -> int:
 def rwkvq_gemv(desc: Desc, W_image, mu_desc, mu_image, x, xprev, B: int, y, workspace, stream=None):
     """rwkvq_gemv on torch tensors: W_image/mu_image uint8, x/xprev float16 [B, ic], y float32 or
     float16 [B, oc], workspace uint8 (zero-filled before first use)."""
-    import torch
-    y_dtype = RWKVQ_F32 if y.dtype == torch.float32 else RWKVQ_F16
-    _check(lib().rwkvq_gemv(C.byref(desc), _dev_ptr(W_image), None if mu_desc is None else C.byref(mu_desc),
-                            _dev_ptr(mu_image), _dev_ptr(x), _dev_ptr(xprev), B, _dev_ptr(y), y_dtype,
-                            _dev_ptr(workspace), workspace.numel() * workspace.element_size(),
-                            _stream_ptr(stream)), "rwkvq_gemv")
+    t = _torch or _load_torch()
+    status = (_lib or lib()).rwkvq_gemv(
+        desc, W_image.data_ptr(), mu_desc, None if mu_image is None else mu_image.data_ptr(), x.data_ptr(),
+        None if xprev is None else xprev.data_ptr(), B, y.data_ptr(), RWKVQ_F32 if y.dtype is t.float32 else RWKVQ_F16,
+        workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
+    if status:
+        raise RwkvqError(status, "rwkvq_gemv")
 
 
 def rwkvq_gemv_static_max_scratch_bytes() -> int:

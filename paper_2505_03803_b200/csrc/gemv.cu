@@ -4,6 +4,7 @@
 // the per-record routines below.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "../../include/rwkvq.h"
@@ -15,18 +16,28 @@ namespace rwkvq {
 // ---------------------------------------------------------------------------------------------
 // Single-product kernel.  CTA = 8 warps; block (rb, ks) covers RPC rows (128 for SQ, 256 for
 // VQ) and the column tiles [ks*nkt, min(KT, (ks+1)*nkt)).  Warp w owns record w of each chunk.
+//
+// A product of a few MB is a chain of latencies: launch, inputs and weights (one trip to memory: the first records are requested before
+// the inputs are mixed), the tensor-core steps, and the sum over the K splits.  Up to eight splits form a cluster and add
+// up in distributed shared memory; more go through global memory and a last-arriver reduction.  The launch is
+// a programmatic dependent one: its start overlaps the end of the kernel in front, which it waits for before it touches memory.
+// 512 x 512, one token, calls back to back: 10.5 -> 4.6 us a call (now the host enqueueing them).
 // ---------------------------------------------------------------------------------------------
 template <int FMT, int NB>
-__global__ void __launch_bounds__(256, 2) gemv_kernel(const GemvArgs a) {
+__global__ void __launch_bounds__(256, 2) gemv_kernel(const __grid_constant__ GemvArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int rb = blockIdx.x, ks = blockIdx.y;
   const int kt0 = ks * a.nkt, kt1 = min(a.KT, kt0 + a.nkt);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int REC = (FMT == FMT_SQ3) ? 1 : 2;
   constexpr int RPC = 128 * REC;
+  constexpr int BITS = (FMT == FMT_VQ8) ? 8 : 6;
+  constexpr int RBYTES = FMT == FMT_SQ3 ? RWKVQ_SQ_RECORD_BYTES : 64 * 32 * BITS / 8;
 
-  SmemLayout L = smem_layout<FMT>(a.nkt, a.B, a.mu ? a.mu_entries : 0, a.entries);
-  stage_input<FMT>(smem, L, a, kt0, kt1);
+  const SmemLayout L = smem_layout<FMT>(a.nkt, a.B, a.mu ? a.mu_entries : 0, a.entries);
+  const uint8_t* rec = a.payload + ((size_t)(REC * rb) * a.KT * 8 + warp) * RBYTES;      // record of tile 0; tiles 8 * RBYTES apart
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   float acc[REC][NB][4];
 #pragma unroll
@@ -37,41 +48,46 @@ __global__ void __launch_bounds__(256, 2) gemv_kernel(const GemvArgs a) {
       for (int i = 0; i < 4; ++i) acc[r][n][i] = 0.f;
 
   if constexpr (FMT == FMT_SQ3) {
-    const uint8_t* rec = a.payload + ((size_t)(rb * a.KT + kt0) * 8 + warp) * RWKVQ_SQ_RECORD_BYTES;
     SqRecord cur, nxt;
-    cur.load(rec, lane);
+    cur.load(rec + (size_t)kt0 * 8 * RBYTES, lane);
+    if (kt0 + 1 < kt1) nxt.load(rec + (size_t)(kt0 + 1) * 8 * RBYTES, lane);
+    stage_input<FMT>(smem, L, a, kt0, kt1);
     for (int kt = kt0; kt < kt1; ++kt) {
-      if (kt + 1 < kt1) nxt.load(rec + (size_t)(kt + 1 - kt0) * 8 * RWKVQ_SQ_RECORD_BYTES, lane);
       uint32_t w[12];
       cur.words(w);
+      const uint4 sz = cur.sz;
+      cur = nxt;
+      if (kt + 2 < kt1) nxt.load(rec + (size_t)(kt + 2) * 8 * RBYTES, lane);
       const XLane xl = make_xlane(smem + (size_t)(kt - kt0) * 512, L.xstride,
                                   reinterpret_cast<const float*>(smem + L.gs_off) + (size_t)(kt - kt0) * 2 * 3 * 16, 16, a.B, lane);
-      sq_record_mma<NB>(w, cur.sz, xl, acc[0]);
-      cur = nxt;
+      sq_record_mma<NB>(w, sz, xl, acc[0]);
     }
   } else {
-    constexpr int BITS = (FMT == FMT_VQ6) ? 6 : 8;
-    constexpr int RBYTES = 64 * 32 * BITS / 8;
     const int E = a.entries;
     const uint32_t* cbg = reinterpret_cast<const uint32_t*>(a.aux) + (size_t)(rb * a.KT) * E;
+    constexpr bool kEarly = !(BITS == 8 && NB == 2);      // registers suffice to request the records a tile ahead
+    VqRecord<BITS> v[REC];
+#pragma unroll
+    for (int r = 0; r < REC; ++r)
+      if (kEarly) v[r].load(rec + ((size_t)r * a.KT + kt0) * 8 * RBYTES, lane);
     stage_codebook(smem + L.cb_off, cbg + (size_t)kt0 * E, E);
+    stage_input<FMT>(smem, L, a, kt0, kt1);      // ends with a barrier
     for (int kt = kt0; kt < kt1; ++kt) {
-      __syncthreads();
+      if (kt > kt0) __syncthreads();
       if (kt + 1 < kt1)
         stage_codebook(smem + L.cb_off + (size_t)((kt + 1 - kt0) & 1) * E * 128, cbg + (size_t)(kt + 1) * E, E);
       const uint32_t* cb_lane = reinterpret_cast<const uint32_t*>(smem + L.cb_off + (size_t)((kt - kt0) & 1) * E * 128) + lane;
+      const XLane xl = make_xlane(smem + (size_t)(kt - kt0) * 512, L.xstride, nullptr, 16, a.B, lane);
 #pragma unroll
       for (int r = 0; r < REC; ++r) {
-        const uint8_t* rec = a.payload + ((size_t)((2 * rb + r) * a.KT + kt) * 8 + warp) * RBYTES;
-        VqRecord<BITS> v;
-        v.load(rec, lane);
-        const XLane xl = make_xlane(smem + (size_t)(kt - kt0) * 512, L.xstride, nullptr, 16, a.B, lane);
-        vq_record_mma<BITS, NB>(v.w, cb_lane, xl, acc[r]);
+        if (!kEarly) v[r].load(rec + ((size_t)r * a.KT + kt) * 8 * RBYTES, lane);
+        vq_record_mma<BITS, NB>(v[r].w, cb_lane, xl, acc[r]);
+        if (kEarly && kt + 1 < kt1) v[r].load(rec + ((size_t)r * a.KT + kt + 1) * 8 * RBYTES, lane);
       }
     }
   }
 
-  // ---- epilogue: direct store, or partial sums + last-arriver reduction over the K splits
+  // ---- epilogue: direct store, or partial sums + a reduction over the K splits
   const int g = lane >> 2, t = lane & 3;
   if (a.S == 1) {
 #pragma unroll
@@ -86,7 +102,8 @@ __global__ void __launch_bounds__(256, 2) gemv_kernel(const GemvArgs a) {
         }
     return;
   }
-  float* part = a.partial + ((size_t)(ks * gridDim.x + rb) * 16) * RPC;
+  float* part = a.cluster ? reinterpret_cast<float*>(smem) : a.partial + ((size_t)(ks * gridDim.x + rb) * 16) * RPC;
+  if (a.cluster) __syncthreads();      // the staged inputs are not read any more
 #pragma unroll
   for (int r = 0; r < REC; ++r)
 #pragma unroll
@@ -97,6 +114,26 @@ __global__ void __launch_bounds__(256, 2) gemv_kernel(const GemvArgs a) {
         int b = n * 8 + 2 * t + (i & 1);
         if (b < a.B) part[(size_t)b * RPC + rl] = acc[r][n][i];
       }
+  if (a.cluster) {
+    // every block of the cluster sums a share of the outputs over all S splits, in the same order
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(smem);
+    for (int idx = ks * (int)blockDim.x + threadIdx.x; idx < a.B * RPC; idx += a.S * (int)blockDim.x) {
+      float sum = 0.f;
+      for (int s = 0; s < a.S; ++s) {
+        uint32_t addr;
+        float v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine + 4u * (uint32_t)idx), "r"(s));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+        sum += v;
+      }
+      const int b = idx / RPC, row = rb * RPC + idx % RPC;
+      if (row < a.oc) store_y(a.y, a.y_dtype, (size_t)b * a.oc + row, sum);
+    }
+    // no block leaves while others may read its partial sums
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n barrier.cluster.wait.aligned;" ::: "memory");
+    return;
+  }
   __threadfence();
   __syncthreads();
   __shared__ unsigned s_last;
@@ -230,8 +267,10 @@ static int fmt_of(const rwkvq_desc* d) {
 
 struct GemvPlan {
   int fmt, NRB, KT, S, nkt;
+  bool cluster;
   size_t smem, ws_bytes, counters_bytes;
 };
+
 
 static rwkvq_status plan_gemv(const rwkvq_desc* d, int B, bool has_mu, int mu_entries, GemvPlan* p) {
   if (!d || B < 1 || B > 16) return RWKVQ_EINVAL;
@@ -242,37 +281,60 @@ static rwkvq_status plan_gemv(const rwkvq_desc* d, int B, bool has_mu, int mu_en
   const int rpc = p->fmt == FMT_SQ3 ? 128 : 256;
   p->NRB = d->oc_pad / rpc;
   p->KT = d->ic_pad / 256;
+  const int entries = has_mu ? mu_entries : 0;
+  auto smem_of = [&](int nkt) {
+    return p->fmt == FMT_SQ3 ? smem_layout<FMT_SQ3>(nkt, B, entries, d->entries).total
+         : p->fmt == FMT_VQ6 ? smem_layout<FMT_VQ6>(nkt, B, entries, d->entries).total
+                             : smem_layout<FMT_VQ8>(nkt, B, entries, d->entries).total;
+  };
   // Enough blocks for two per SM, bounded by the shared-memory footprint of the staged input.
   int want = (2 * 148 + p->NRB - 1) / p->NRB;
   int S = want < 1 ? 1 : (want > p->KT ? p->KT : want);
-  for (;; ++S) {
-    int nkt = (p->KT + S - 1) / S;
-    size_t sm = p->fmt == FMT_SQ3 ? smem_layout<FMT_SQ3>(nkt, B, has_mu ? mu_entries : 0, d->entries).total
-              : p->fmt == FMT_VQ6 ? smem_layout<FMT_VQ6>(nkt, B, has_mu ? mu_entries : 0, d->entries).total
-                                  : smem_layout<FMT_VQ8>(nkt, B, has_mu ? mu_entries : 0, d->entries).total;
-    if (sm <= 96 * 1024 || S >= p->KT) { p->nkt = nkt; p->smem = sm; break; }
+  while (S < p->KT && smem_of((p->KT + S - 1) / S) > 96 * 1024) ++S;
+  // A contraction of a few tiles is done by one block: a tile costs it less than the sum over splits does.  Where eight splits
+  // leave no block with many more tiles than that, the splits are a cluster (measured from 512 x 512 to 14336 x 4096; a VQ tile is dearer, it
+  // brings its codebook).
+  const int kTilesPerSum = p->fmt == FMT_SQ3 ? 2 : 1, kClusterTiles = p->fmt == FMT_SQ3 ? 4 : p->fmt == FMT_VQ6 ? 3 : 2;
+  const int per_cluster = (p->KT + 7) / 8;
+  p->cluster = false;
+  if (p->KT <= kTilesPerSum) {
+    S = 1;
+  } else if (S <= 8 || (per_cluster <= kClusterTiles && smem_of(per_cluster) <= 96 * 1024)) {
+    S = S < 8 ? S : 8;
+    p->cluster = true;
   }
   p->nkt = (p->KT + S - 1) / S;
   p->S = (p->KT + p->nkt - 1) / p->nkt;  // no empty splits
+  // More blocks than surely fit at once (two per SM, whole clusters within a GPC): clusters would wait for room
+  // together (14336 x 4096 VQ 28.7 us, through global memory 23.3; 9456 x 9600 SQ 22.0 and 18.4).
+  if (p->S == 1 || p->NRB * p->S > 256) p->cluster = false;
+  p->smem = smem_of(p->nkt);
+  if (p->cluster) p->smem = std::max(p->smem, (size_t)B * rpc * 4);
   p->counters_bytes = ((size_t)p->NRB * 4 + 255) / 256 * 256;
-  p->ws_bytes = p->counters_bytes + (p->S > 1 ? (size_t)p->S * p->NRB * 16 * rpc * 4 : 0);
+  p->ws_bytes = p->counters_bytes + (p->S > 1 && !p->cluster ? (size_t)p->S * p->NRB * 16 * rpc * 4 : 0);
   return RWKVQ_OK;
 }
 
+template <int FMT, int NB>
+static cudaError_t launch_gemv_as(const GemvArgs& a, const GemvPlan& p, cudaStream_t s) {
+  static SmemOptIn opt_in;
+  if (p.smem > 48 * 1024) {
+    const cudaError_t e = opt_in((const void*)gemv_kernel<FMT, NB>, 112 * 1024);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.NRB, p.S); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = p.smem; cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = p.S; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = p.cluster ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, NB>, a);
+}
 template <int FMT>
 static cudaError_t launch_gemv(const GemvArgs& a, const GemvPlan& p, cudaStream_t s) {
-  dim3 grid(p.NRB, p.S);
-  cudaError_t e;
-  if (a.B <= 8) {
-    e = cudaFuncSetAttribute(gemv_kernel<FMT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e != cudaSuccess) return e;
-    gemv_kernel<FMT, 1><<<grid, 256, p.smem, s>>>(a);
-  } else {
-    e = cudaFuncSetAttribute(gemv_kernel<FMT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e != cudaSuccess) return e;
-    gemv_kernel<FMT, 2><<<grid, 256, p.smem, s>>>(a);
-  }
-  return cudaGetLastError();
+  return a.B <= 8 ? launch_gemv_as<FMT, 1>(a, p, s) : launch_gemv_as<FMT, 2>(a, p, s);
 }
 
 }  // namespace rwkvq
@@ -308,7 +370,7 @@ static rwkvq_status run_gemv(const GemvPlan& p, const rwkvq_desc* d, const void*
                              const void* x, const void* xprev, int B, void* y, int y_dtype, void* ws, void* stream) {
   GemvArgs a;
   fill_gemv_args(&a, d, W, mud, mu, x, xprev, B, y, y_dtype);
-  a.KT = p.KT; a.S = p.S; a.nkt = p.nkt;
+  a.KT = p.KT; a.S = p.S; a.nkt = p.nkt; a.cluster = p.cluster ? 1 : 0;
   a.counters = static_cast<unsigned*>(ws);
   a.partial = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) + p.counters_bytes);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -361,8 +423,10 @@ rwkvq_status rwkvq_gemv_static(const rwkvq_desc* d, const void* W, const rwkvq_d
     g_static_scratch_addr[dev].store(ws, std::memory_order_release);
   }
   // The array keeps whatever the previous call left: the arrival counters must start at zero.
-  e = cudaMemsetAsync(ws, 0, p.counters_bytes, static_cast<cudaStream_t>(stream));
-  if (e != cudaSuccess) return cuda_status(e);
+  if (p.S > 1 && !p.cluster) {
+    e = cudaMemsetAsync(ws, 0, p.counters_bytes, static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_status(e);
+  }
   return run_gemv(p, d, W, mud, mu, x, xprev, B, y, y_dtype, ws, stream);
 }
 

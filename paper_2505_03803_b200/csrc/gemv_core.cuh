@@ -22,7 +22,7 @@ struct GemvArgs {
   void* y;
   float* partial;
   unsigned* counters;
-  int oc, ic, KT, S, nkt, entries, B, mu_bits, mu_entries, y_dtype;
+  int oc, ic, KT, S, nkt, entries, B, mu_bits, mu_entries, y_dtype, cluster;
 };
 
 struct SmemLayout {
@@ -70,66 +70,90 @@ __device__ __forceinline__ void store_w(void* out, int dtype, size_t idx, float 
 }
 
 // x_mix = x + (x_prev - x) * mu_hat for columns [kt0*256, kt1*256) of every batch row, rounded
-// to fp16 into shared memory (zeros beyond ic); then, for SQ, per 128-column group and batch
-// row the three sums the factored dequantisation needs:
+// to fp16 into shared memory (zeros beyond ic); for SQ also, per 128-column group and batch
+// row, the three sums the factored dequantisation needs:
 //    Sx  = sum x,   Bx_h = sum bias_h(col) * x   (h = 0: rows g, 1: rows g+8 of a record)
-// computed from the rounded values the tensor core will see, reduced with warp shuffles.
+// computed from the rounded values the tensor core will see.  A thread takes eight columns (16 bytes) of one
+// batch row, a half-warp one group, whose sums it reduces with shuffles; the loads of the first round are issued ahead of the
+// barrier behind which the token-shift codebook is in shared memory, so that one trip to memory covers both.
+struct MixLoad {
+  uint4 x, p;
+  uint32_t lo, hi;
+};
+__device__ __forceinline__ MixLoad mix_load(const GemvArgs& a, int b, int col) {
+  MixLoad m;
+  m.x = m.p = make_uint4(0u, 0u, 0u, 0u);
+  m.lo = m.hi = 0u;
+  if (col < a.ic) {
+    m.x = *reinterpret_cast<const uint4*>(a.x + (size_t)b * a.ic + col);
+    if (a.mu) {
+      m.p = *reinterpret_cast<const uint4*>(a.xprev + (size_t)b * a.ic + col);
+      // four indices = 4 * bits bits starting at a byte boundary (col / 2 is a multiple of 4)
+      const uint32_t byte = (uint32_t)(col >> 1) * (uint32_t)a.mu_bits >> 3;
+      const uint32_t* w = reinterpret_cast<const uint32_t*>(a.mu) + (byte >> 2);
+      m.lo = w[0];
+      m.hi = (byte & 3u) * 8u + 4u * (uint32_t)a.mu_bits > 32u ? w[1] : 0u;
+    }
+  }
+  return m;
+}
+__device__ __forceinline__ uint32_t mix_pair(uint32_t xr, uint32_t pr, uint32_t mr) {
+  const float2 xf = __half22float2(*reinterpret_cast<const __half2*>(&xr));
+  const float2 pf = __half22float2(*reinterpret_cast<const __half2*>(&pr));
+  const float2 mf = __half22float2(*reinterpret_cast<const __half2*>(&mr));
+  const __half2 v = __floats2half2_rn(fmaf(pf.x - xf.x, mf.x, xf.x), fmaf(pf.y - xf.y, mf.y, xf.y));
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
 template <int FMT>
 __device__ __forceinline__ void stage_input(uint8_t* smem, const SmemLayout& L, const GemvArgs& a, int kt0, int kt1) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   uint32_t* mucb = reinterpret_cast<uint32_t*>(smem + L.mucb_off);
+  const int nvec = (kt1 - kt0) * 32, total = a.B * nvec;      // multiples of 32
+  int b = tid / nvec, c8 = tid - b * nvec;
+  MixLoad cur = mix_load(a, b, tid < total ? kt0 * 256 + 8 * c8 : a.ic);
   if (a.mu) {
     for (int e = tid; e < a.mu_entries; e += nthr) mucb[e] = reinterpret_cast<const uint32_t*>(a.mu_aux)[e];
     __syncthreads();
   }
-  const int npairs = (kt1 - kt0) * 128;
-  for (int p = tid; p < a.B * npairs; p += nthr) {
-    const int b = p / npairs, cp = p - b * npairs;
-    const int col = kt0 * 256 + 2 * cp;
-    __half2 v = __float2half2_rn(0.f);
-    if (col < a.ic) {
-      v = *reinterpret_cast<const __half2*>(a.x + (size_t)b * a.ic + col);
-      if (a.mu) {
-        const float2 xf = __half22float2(v);
-        const float2 pf = __half22float2(*reinterpret_cast<const __half2*>(a.xprev + (size_t)b * a.ic + col));
-        const uint32_t mw = mucb[vector_index(a.mu, col >> 1, a.mu_bits)];
-        const float2 mf = __half22float2(*reinterpret_cast<const __half2*>(&mw));
-        v = __floats2half2_rn(fmaf(pf.x - xf.x, mf.x, xf.x), fmaf(pf.y - xf.y, mf.y, xf.y));
-      }
+  float* gs = reinterpret_cast<float*>(smem + L.gs_off);
+  for (int v = tid; v < total; v += nthr) {
+    if (v != tid) {
+      b = v / nvec; c8 = v - b * nvec;
+      cur = mix_load(a, b, kt0 * 256 + 8 * c8);
     }
-    *reinterpret_cast<__half2*>(smem + (size_t)b * L.xstride + (size_t)cp * 4) = v;
-  }
-  __syncthreads();
-  if constexpr (FMT == FMT_SQ3) {
-    const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
-    const int ngroups = (kt1 - kt0) * 2;
-    float* gs = reinterpret_cast<float*>(smem + L.gs_off);
-    const int o = (lane * 4) & 63;
-    const float b00 = (float)rwkvq_sq_bias(o, 0), b02 = (float)rwkvq_sq_bias(o + 2, 0);
-    const float b10 = (float)rwkvq_sq_bias(o, 1), b12 = (float)rwkvq_sq_bias(o + 2, 1);
-    for (int task = warp; task < ngroups * a.B; task += nwarps) {
-      const int grp = task / a.B, b = task - grp * a.B;
-      const uint2 raw = *reinterpret_cast<const uint2*>(smem + (size_t)b * L.xstride + (size_t)(grp * 128 + lane * 4) * 2);
-      const float2 x01 = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-      const float2 x23 = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-      const float p01 = x01.x + x01.y, p23 = x23.x + x23.y;
-      float sx = p01 + p23;
-      float s0 = fmaf(b00, p01, b02 * p23);
-      float s1 = fmaf(b10, p01, b12 * p23);
+    const int col = kt0 * 256 + 8 * c8;
+    uint4 r = cur.x;
+    if (a.mu && col < a.ic) {
+      const uint32_t bits = (uint32_t)a.mu_bits, mask = (1u << bits) - 1u;
+      const uint32_t f = __funnelshift_r(cur.lo, cur.hi, (((uint32_t)(col >> 1) * bits >> 3) & 3u) * 8u);
+      r.x = mix_pair(r.x, cur.p.x, mucb[f & mask]);
+      r.y = mix_pair(r.y, cur.p.y, mucb[(f >> bits) & mask]);
+      r.z = mix_pair(r.z, cur.p.z, mucb[(f >> (2u * bits)) & mask]);
+      r.w = mix_pair(r.w, cur.p.w, mucb[(f >> (3u * bits)) & mask]);
+    }
+    *reinterpret_cast<uint4*>(smem + (size_t)b * L.xstride + (size_t)c8 * 16) = r;
+    if constexpr (FMT == FMT_SQ3) {
+      const int o = (8 * c8) & 63;
+      auto sum2 = [](uint32_t w) { const float2 q = __half22float2(*reinterpret_cast<const __half2*>(&w)); return q.x + q.y; };
+      const float pa = sum2(r.x) + sum2(r.z), pb = sum2(r.y) + sum2(r.w);
+      float sx = pa + pb;
+      float s0 = fmaf((float)rwkvq_sq_bias(o, 0), pa, (float)rwkvq_sq_bias(o + 2, 0) * pb);
+      float s1 = fmaf((float)rwkvq_sq_bias(o, 1), pa, (float)rwkvq_sq_bias(o + 2, 1) * pb);
 #pragma unroll
-      for (int d = 16; d > 0; d >>= 1) {
+      for (int d = 8; d > 0; d >>= 1) {
         sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
         s0 += __shfl_xor_sync(0xFFFFFFFFu, s0, d);
         s1 += __shfl_xor_sync(0xFFFFFFFFu, s1, d);
       }
-      if (lane == 0) {
+      if ((tid & 15) == 0) {
+        const int grp = c8 >> 4;
         gs[(grp * 3 + 0) * 16 + b] = sx;
         gs[(grp * 3 + 1) * 16 + b] = s0;
         gs[(grp * 3 + 2) * 16 + b] = s1;
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
 }
 
 // Per-lane view of the staged input for one 256-column tile.  Lane (g, t) of a warp reads, for
@@ -403,7 +427,7 @@ inline void fill_gemv_args(GemvArgs* a, const rwkvq_desc* d, const void* W, cons
   a->xprev = static_cast<const __half*>(xprev);
   a->y = y; a->partial = nullptr; a->counters = nullptr;
   a->oc = d->oc; a->ic = d->ic; a->entries = d->entries; a->B = B; a->y_dtype = y_dtype;
-  a->KT = d->ic_pad / 256; a->S = 1; a->nkt = a->KT;
+  a->KT = d->ic_pad / 256; a->S = 1; a->nkt = a->KT; a->cluster = 0;
 }
 
 }  // namespace rwkvq

@@ -188,3 +188,37 @@ def test_sq_extreme_scales_and_fractional_zero_points(oc, ic, Bn):
     x, xp = inputs.gen_activation_pair(Bn + ic, Bn, ic, n_outliers=8)
     mu = H.pack_mu(H.random_mu_codes(ic, ic)) if Bn != 8 else None
     _check_gemv(W, mu, x.astype(np.float16), xp.astype(np.float16))
+
+
+# The ways a product's column tiles are shared out: one block, a cluster that sums in distributed shared memory, and the
+# sum through global memory (more tiles than eight blocks should take).
+@pytest.mark.parametrize("fmt,oc,ic", [("sq", 144, 512), ("sq", 144, 640), ("sq", 128, 2176), ("sq", 256, 8320), ("vq", 256, 512),
+                                       ("vq", 256, 6144), ("vq", 256, 6400)])
+@pytest.mark.parametrize("Bn", [1, 9])
+def test_splits_of_the_contraction(fmt, oc, ic, Bn):
+    W = H.pack_sq(H.random_sq_codes(oc + ic, oc, ic)) if fmt == "sq" else H.pack_vq(H.random_vq_codes(oc + ic, oc, ic, 6), 6)
+    x, xp = inputs.gen_activation_pair(Bn + ic, Bn, ic, n_outliers=8)
+    mu = H.pack_mu(H.random_mu_codes(ic + 1, ic))
+    _check_gemv(W, mu, x.astype(np.float16), xp.astype(np.float16))
+
+
+def test_products_that_feed_each_other():
+    """Calls enqueued back to back, each reading the one before's fp16 output."""
+    n, Ws = 512, []
+    for k in range(6):
+        c = H.random_sq_codes(900 + k, n, n)
+        Ws.append(H.pack_sq(c))
+    x = torch.from_numpy(inputs.gen_activation(3, 2, n, 0).astype(np.float16)).cuda()
+    ys = [torch.full((2, n), float("nan"), dtype=torch.float16, device="cuda") for _ in Ws]
+    ws = torch.zeros(max(256, max(B.rwkvq_gemv_workspace_bytes(W.desc, 2) for W in Ws)), dtype=torch.uint8, device="cuda")
+    for rep in range(20):
+        src = x
+        for W, y in zip(Ws, ys):
+            B.rwkvq_gemv(W.desc, W.dev, None, None, src, None, 2, y, ws)
+            src = y
+    torch.cuda.synchronize()
+    src = x
+    for W, y in zip(Ws, ys):
+        ref, tol = H.reference(W, None, src.cpu().numpy(), None)
+        assert (np.abs(y.double().cpu().numpy() - ref) <= tol + np.abs(ref) * 2.0 ** -10).all()
+        src = y
