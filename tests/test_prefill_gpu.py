@@ -213,3 +213,23 @@ def test_prefill_grouped_rejects_bad_groups():
         B.rwkvq_gemm_prefill_grouped([e] * 17, M)
     torch.cuda.synchronize()
     assert B.rwkvq_device_status() == 0
+
+
+@pytest.mark.parametrize("fmt,oc,ic,M,has_mu,y_dtype", [
+    ("sq", 128, 1536, 1, False, torch.float32),        # the shortest contraction that is cut: two slices of three chunks
+    ("vq6", 256, 1280, 17, True, torch.bfloat16),      # one chunk short of it
+    ("sq", 304, 9216, 203, False, torch.bfloat16),     # eight slices of 4 or 5 chunks; rows past the end of the last tile
+    ("vq8", 1024, 2048, 209, True, torch.float32),     # two token tiles of 112
+    ("vq6", 2048, 2304, 433, False, torch.float32),    # three token tiles: 48 tiles, not cut
+    ("sq", 2816, 1792, 208, True, torch.float32),      # two slices of 22 tiles
+])
+def test_prefill_sliced_contractions_and_even_token_tiles(fmt, oc, ic, M, has_mu, y_dtype):
+    """Contractions cut into slices whose sums a second launch adds, beside those that just are not; operands with a
+    token shift (pre-pass) and without (tensor map); token tiles that divide M evenly.  Twice the same bits."""
+    seed = 900 + oc + M
+    W = (H.pack_sq(H.random_sq_codes(seed, oc, ic)) if fmt == "sq"
+         else H.pack_vq(H.random_vq_codes(seed, oc, ic, 6 if fmt == "vq6" else 8), 6 if fmt == "vq6" else 8))
+    mu = H.pack_mu(H.random_mu_codes(seed + 1, ic)) if has_mu else None
+    _check(W, mu, M, seed + 2, y_dtype=y_dtype)
+    _, Xd = _bf16(inputs.gen_activation(seed + 4, M, ic, n_outliers=8))
+    assert torch.equal(_run(W, mu, Xd, None, M, y_dtype), _run(W, mu, Xd, None, M, y_dtype))
