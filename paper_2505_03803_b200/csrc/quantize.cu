@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "../../include/rwkvq.h"
 #include "format.h"
 #include "host_util.h"
@@ -302,7 +304,8 @@ __device__ __forceinline__ void join_group(ClusterSums& s, const uint32_t* vec, 
 // Seeding.  512 threads, each with the distances of 64 consecutive vectors in registers; the vectors stay in shared memory as
 // fp16 pairs (read 16 bytes at a time, the pieces of a thread's row rotated against bank conflicts).  Bound by
 // the instructions of the distance update: two conversions a vector, four packed operations per two, a minimum and a running sum.
-// Seeds are vectors of the tile, so the codebook area of the image holds them exactly until the centres are final.
+// Seeds are vectors of the tile, so the codebook area of the image holds them exactly until the centres are final.  A token-shift vector of n
+// vectors is seeded alike by one block of n / 2048 warps.
 constexpr int kVqWarps = kVqThreads / 32;
 __device__ __forceinline__ int vq_slot(int i) { return (i & ~63) | ((((i >> 2) ^ (i >> 6)) & 7) << 2) | (i & 35); }
 
@@ -312,14 +315,26 @@ struct SeedShared {
   int pick[kVqMaxE];
 };
 
+template <bool kVector>
 __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) {
+  if (kVector) asm volatile("griddepcontrol.launch_dependents;");
   extern __shared__ __align__(16) uint8_t smem[];
   uint32_t* vec = reinterpret_cast<uint32_t*>(smem);
-  SeedShared& sh = *reinterpret_cast<SeedShared*>(smem + (size_t)kVqMaxVec * 4);
+  const int n = kVector ? a.n_vec : kVqMaxVec, E = a.E, threads = kVector ? (int)blockDim.x : kVqThreads;
+  SeedShared& sh = *reinterpret_cast<SeedShared*>(smem + (size_t)threads * kVqPerThread * 4);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile = blockIdx.x, tr = tile / a.TC, tc = tile % a.TC;
-  const int n = kVqMaxVec, E = a.E;
-  {
+  if (kVector) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(a.w);
+    bool bad = false;
+    for (int i = tid; i < threads * kVqPerThread; i += threads) {
+      const uint32_t v = i < n ? __ldg(src + i) : 0u;
+      bad |= ((v & 0x7C00u) == 0x7C00u) | ((v & 0x7C000000u) == 0x7C000000u);
+      vec[vq_slot(i)] = v;
+    }
+    if (bad) atomicOr(a.flags, kFlagNonFinite);
+    if (tid < kVqWarps) sh.warp_tot[tid] = 0.f;
+  } else {
     // a warp reads 512 contiguous bytes: one row of the tile
     const uint16_t* src = a.w + (size_t)(tr * 256) * a.ic + tc * 256;
     bool bad = false;
@@ -333,8 +348,8 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
     }
     if (bad) atomicOr(a.flags, kFlagNonFinite);
   }
-  const uint64_t seed = a.seed * 0x9E3779B97F4A7C15ull + (uint64_t)tile + 1ull;
-  for (int e = tid; e < E; e += kVqThreads) {
+  const uint64_t seed = kVector ? a.seed : a.seed * 0x9E3779B97F4A7C15ull + (uint64_t)tile + 1ull;
+  for (int e = tid; e < E; e += threads) {
     sh.u01[e] = (float)unit_of(splitmix(seed, e));
     sh.pick[e] = n - 1;
   }
@@ -343,7 +358,7 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
   const int base = tid * kVqPerThread;
   float dist[kVqPerThread];
 #pragma unroll
-  for (int k = 0; k < kVqPerThread; ++k) dist[k] = INFINITY;
+  for (int k = 0; k < kVqPerThread; ++k) dist[k] = !kVector || base + k < n ? INFINITY : 0.f;
   int at = below(splitmix(seed, 0), n);
   for (int e = 0; e < E; ++e) {
     const uint32_t cv = vec[vq_slot(at)];
@@ -392,7 +407,7 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
       int pick = base;
 #pragma unroll
       for (int k = 0; k < kVqPerThread; ++k) {
-        if (acc <= target) pick = base + k;      // last vector whose running sum began at or below the target
+        if (acc <= target && (!kVector || base + k < n)) pick = base + k;      // last vector whose running sum began at or below the target
         acc += dist[k];
       }
       sh.pick[e + 1] = pick;
@@ -796,25 +811,87 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
 
 // ---- token-shift vectors ----
 //
-// One block; a vector of a few thousand elements is a few thousand two-element vectors, so every phase is spread over all
-// threads: distances live in shared memory (a run of 64 per row, padded to 68 words so that the lanes that sum runs read
-// 16 bytes each without conflicts), members are sorted by centre (stable) and every centre adds its own in vector order.
-constexpr int kVecThreads = 1024;
+// Weighted vectors are assigned by a cluster of kVecCluster, whose blocks take a part of the vectors each and
+// write what they find into the first block's shared memory; that block sorts the members by centre (stable), and every centre
+// adds its own in vector order.  Bound by the latency of the running sums: of the seeds' distances and of the longest
+// centre's members.  2048 weighted vectors, 64 centres, ten iterations: 145 us with the seeds (237 before: one block for
+// everything, seeds' distances in shared memory, two compare-and-selects for each distance, members counted and ranked
+// twice by match, sums in chains of dependent loads and conversions, the final distances all in fp64).
+constexpr int kVecThreads = 1024, kVecCluster = 8;
+// The search for the nearest centre takes the minimum over groups of eight centres, one instruction a distance, and looks for the centre only
+// in the group that wins.  One slot of padding per group: lanes that look in different groups read different banks.
+constexpr int kCentreGroup = 8;
+__host__ __device__ constexpr int centre_slot(int e) { return e + e / kCentreGroup; }
 struct VecShared {
   double cx[kVqMaxE], cy[kVqMaxE];
-  float2 cf[kVqMaxE];
-  float warp_tot[kVqThreads / 32];
-  float u01[kVqMaxE];
-  int pick[kVqMaxE];
-  float total;
-  uint16_t hist[kVecThreads / 32][kVqMaxE];   // members per warp's share and centre, then their first position
+  float4 neg[kVqMaxE + kVqMaxE / kCentreGroup];   // (-x, -x, -y, -y) of a centre, in groups, see centre_slot
+  uint16_t hist[kVecThreads / 32][kVqMaxE + 2];   // members per warp's share and centre, then those of the shares before it; a column is read by a warp
   int first[kVqMaxE + 1];
   ClusterSums sums;
+  float part_best[kVecCluster][64 * kVecThreads / 32 / kVecCluster];     // nearest centre of a part of them: distance, number
+  uint8_t part_idx[kVecCluster][64 * kVecThreads / 32 / kVecCluster];
 };
+// Up to this many vectors the first block keeps, in fp64, w * v and w of either dimension: a conversion to fp64 takes four times a
+// multiply-add's time, and a member of a centre is converted once instead of in each iteration.
+constexpr int kVecTable = 4096;
 __host__ __device__ constexpr size_t vec_smem_bytes(int n) {
-  // distances (seeding), overlaid later by the assignment (bytes) and the members sorted by centre (16-bit numbers)
-  const size_t rows = ((size_t)n + 63) / 64, d = rows * 68 * 4, s = rows * 64 * 3;
-  return (sizeof(VecShared) + 15) / 16 * 16 + (d > s ? d : s);
+  const size_t rows = ((size_t)n + 63) / 64;
+  return (sizeof(VecShared) + 15) / 16 * 16 + rows * 320 + (n <= kVecTable ? (size_t)n * 32 : 0);
+}
+
+// The cluster: barrier, and stores to the shared memory of a block of it at the address that `local` has here.
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_address(const void* local, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void peer_store8(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
+__device__ __forceinline__ void peer_store16(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory"); }
+__device__ __forceinline__ void peer_store(uint32_t at, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void peer_store(uint32_t at, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory"); }
+
+// Two vectors against all centres, distances rounded as d = w.x * (dx * dx) + (w.y * (dy * dy)) with the last product and sum in one
+// rounding (unweighted: dx * dx + (dy * dy), likewise).
+struct Nearest {
+  float best[2], second[2];     // smallest minimum of a group, and of the other groups
+  int group[2];                 // first centre of the first group with that minimum
+};
+__device__ __forceinline__ float2 pair_distance(bool weighted, float2 x, float2 y, float2 wx, float2 wy, float4 c) {
+  const float2 dx = add2(x, make_float2(c.x, c.y)), dy = add2(y, make_float2(c.z, c.w)), yy = mul2(dy, dy);
+  return weighted ? fma2(wx, mul2(dx, dx), mul2(wy, yy)) : fma2(dx, dx, yy);
+}
+__device__ __forceinline__ Nearest nearest_group(const float4* neg, int E, bool weighted, float2 x, float2 y, float2 wx, float2 wy) {
+  Nearest r;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) { r.best[q] = r.second[q] = INFINITY; r.group[q] = 0; }
+#pragma unroll 1
+  for (int e = 0; e < E; e += kCentreGroup) {
+    float2 m = make_float2(INFINITY, INFINITY);
+#pragma unroll
+    for (int k = 0; k < kCentreGroup; ++k) {
+      const float2 d = pair_distance(weighted, x, y, wx, wy, neg[centre_slot(e) + k]);
+      m = make_float2(fminf(m.x, d.x), fminf(m.y, d.y));
+    }
+    const float mm[2] = {m.x, m.y};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      r.second[q] = fminf(r.second[q], fmaxf(r.best[q], mm[q]));
+      if (mm[q] < r.best[q]) { r.best[q] = mm[q]; r.group[q] = e; }
+    }
+  }
+  return r;
+}
+__device__ __forceinline__ float one_distance(bool weighted, float x, float y, float wx, float wy, float4 c) {
+  const float dx = __fadd_rn(x, c.x), dy = __fadd_rn(y, c.z), yy = __fmul_rn(dy, dy);
+  return weighted ? __fmaf_rn(wx, __fmul_rn(dx, dx), __fmul_rn(wy, yy)) : __fmaf_rn(dx, dx, yy);
 }
 
 __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs a, const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
@@ -826,143 +903,133 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   const bool weighted = a.elem_w != nullptr;
   const uint32_t* vec = reinterpret_cast<const uint32_t*>(a.w);
   const float2* wgt = reinterpret_cast<const float2*>(a.elem_w);
-  write_header(head, image);
-  float* dist = reinterpret_cast<float*>(rest);
-  {
-    bool bad = false;
-    for (int i = tid; i < rows * 64; i += kVecThreads) {
-      if (i < n) {
-        const uint32_t v = __ldg(vec + i);
-        bad |= ((v & 0x7C00u) == 0x7C00u) | ((v & 0x7C000000u) == 0x7C000000u);
-      }
-      dist[(i >> 6) * 68 + (i & 63)] = i < n ? INFINITY : 0.f;
-    }
-    if (bad) atomicOr(a.flags, kFlagNonFinite);
-  }
-  for (int e = tid; e < E; e += kVecThreads) {
-    sh.u01[e] = (float)unit_of(splitmix(a.seed, e));
-    sh.pick[e] = n - 1;
-  }
-  __syncthreads();
-  // ---- seeding (unweighted), in the order of the kernel above: rows of 64, lanes, warps of 32 rows
-  const int row_warps = (rows + 31) / 32;
-  int at = below(splitmix(a.seed, 0), n);
-  for (int e = 0; e < E; ++e) {
-    const float2 c = vec_of(__ldg(vec + at));
-    if (tid == 0) { sh.cx[e] = (double)c.x; sh.cy[e] = (double)c.y; }
-    if (e + 1 == E) break;
-    for (int i = tid; i < n; i += kVecThreads) {
-      const float2 v = vec_of(__ldg(vec + i));
-      float* d = dist + (i >> 6) * 68 + (i & 63);
-      *d = fminf(*d, d2f(v.x, v.y, c));
-    }
-    __syncthreads();
-    float incl = 0.f, excl = 0.f;
-    const float* row = dist + tid * 68;
-    if (warp < row_warps) {
-      float local = 0.f;
-      if (tid < rows) {
-#pragma unroll
-        for (int k = 0; k < 64; k += 4) {
-          const float4 d = *reinterpret_cast<const float4*>(row + k);
-          local += d.x; local += d.y; local += d.z; local += d.w;
-        }
-      }
-      incl = local;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const float v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-        if (lane >= off) incl += v;
-      }
-      if (lane == 31) sh.warp_tot[warp] = incl;
-      excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-      if (lane == 0) excl = 0.f;
-      if (row_warps > 1) asm volatile("bar.sync 1, %0;" ::"r"(row_warps * 32) : "memory");
-      else __syncwarp();
-      float before = 0.f, total = 0.f;
-      for (int w = 0; w < row_warps; ++w) {
-        if (w == warp) before = total;
-        total += sh.warp_tot[w];
-      }
-      excl = before + excl;
-      incl = before + incl;
-      const float target = sh.u01[e + 1] * total;
-      if (tid == 0) sh.total = total;
-      if (total > 0.f && excl <= target && target < incl) {
-        float acc = excl;
-        int pick = tid * 64;
-        const int n_mine = min(64, n - tid * 64);
-#pragma unroll
-        for (int k = 0; k < 64; k += 4) {
-          const float4 d = *reinterpret_cast<const float4*>(row + k);
-          const float dd[4] = {d.x, d.y, d.z, d.w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (k + j < n_mine && acc <= target) pick = tid * 64 + k + j;
-            acc += dd[j];
-          }
-        }
-        sh.pick[e + 1] = pick;
-      }
-    }
-    __syncthreads();
-    at = sh.total > 0.f ? sh.pick[e + 1] : below(splitmix(a.seed, e + 1), n);
-  }
-  __syncthreads();
+  const uint32_t rank = cluster_rank(), peers = cluster_size();
+  const bool lead = rank == 0u;
+  if (lead) write_header(head, image);
+  for (int e = E + tid; e < (E + kCentreGroup - 1) / kCentreGroup * kCentreGroup; e += kVecThreads)      // no centre is nearer than these
+    sh.neg[centre_slot(e)] = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+  // tables of the first block, behind the assignment (bytes), the ranks of the members and the members sorted by centre (16-bit numbers)
+  const bool tables = n <= kVecTable;
+  double2* const table_wv = reinterpret_cast<double2*>(rest + (size_t)rows * 320);      // [n] w * v
+  double2* const table_w = table_wv + n;
   uint8_t* idx = rest;                                             // [rows * 64]
-  uint16_t* sorted = reinterpret_cast<uint16_t*>(rest + rows * 64);  // [rows * 64]
-  // ---- Lloyd iterations.  Warp w's share of the vectors is [w * share, (w + 1) * share), taken 32 at a time.
-  const int share = ((n + kVecThreads - 1) / kVecThreads) * 32;
-  for (int it = 0; it < a.iters; ++it) {
-    for (int e = tid; e < E; e += kVecThreads) {
-      sh.cf[e] = make_float2((float)sh.cx[e], (float)sh.cy[e]);
-#pragma unroll
-      for (int p = 0; p < 3; ++p) sh.sums.x[p][e] = sh.sums.y[p][e] = 0;
-      sh.sums.cnt[e] = 0;
+  if (lead) {
+    if (tables && weighted) {
+      for (int i = tid; i < n; i += kVecThreads) {
+        const uint32_t v = __ldg(vec + i);
+        const float2 wi = __ldg(wgt + i);
+        const double wx = (double)wi.x, wy = (double)wi.y;
+        table_w[i] = make_double2(wx, wy);
+        table_wv[i] = make_double2(wx * (double)h2f_bits(v & 0xFFFFu), wy * (double)h2f_bits(v >> 16));      // exact: 24 and 11 bits
+      }
     }
-    for (int e = lane; e < E; e += 32) sh.hist[warp][e] = 0;
+    // the seeds lie where the codebook will
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int e = tid; e < E; e += kVecThreads) {
+      const float2 c = vec_of(__ldcg(a.aux + e));
+      sh.cx[e] = (double)c.x; sh.cy[e] = (double)c.y;
+    }
     __syncthreads();
-    for (int i0 = warp * share; i0 < min(n, (warp + 1) * share); i0 += 64) {
+  }
+  uint16_t* ranks = reinterpret_cast<uint16_t*>(rest + rows * 64);   // [rows * 64]: members of the same centre before it in the warp's share
+  uint16_t* sorted = ranks + rows * 64;                             // [rows * 64]
+  // Negated centres, in fp32, to every block.
+  auto publish = [&]() {
+    for (int k = tid; k < E * (int)peers; k += kVecThreads) {
+      const int e = k % E;
+      const float cx = (float)sh.cx[e], cy = (float)sh.cy[e];
+      peer_store(peer_address(&sh.neg[centre_slot(e)], (uint32_t)(k / E)), make_float4(-cx, -cx, -cy, -cy));
+    }
+  };
+  // ---- Lloyd iterations.  Share k of the vectors is [k * share, (k + 1) * share), taken 64 at a time by the warps of block
+  // k / shares that have this share, each with a part of the centres; the first of them goes on with the nearest of all.
+  constexpr int kShares = kVecThreads / 32;
+  const int share = ((n + kVecThreads - 1) / kVecThreads) * 32, shares = kShares / (int)peers, parts = (int)peers, part = warp / shares, mine = (int)rank * shares + warp % shares;
+  const int part_e0 = E * part / parts, part_e1 = E * (part + 1) / parts;
+  const uint32_t lead_idx = peer_address(idx, 0u), lead_ranks = peer_address(ranks, 0u);
+  uint16_t* const hist = sh.hist[mine];
+  uint32_t v[2];
+  float2 wv[2] = {make_float2(1.f, 1.f), make_float2(1.f, 1.f)};
+  auto fetch = [&](int i0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = min(i0 + 32 * q + lane, n - 1);
+      v[q] = __ldg(vec + i);
+      if (weighted) wv[q] = __ldg(wgt + i);
+    }
+  };
+  fetch(mine * share);                             // a share of 64 stays in registers
+  cluster_sync();                                  // every block runs: their shared memory may be written
+  if (lead) publish();
+  for (int it = 0; it < a.iters; ++it) {
+    if (!weighted) {
+      for (int e = tid; e < E; e += kVecThreads) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p) sh.sums.x[p][e] = sh.sums.y[p][e] = 0;
+        sh.sums.cnt[e] = 0;
+      }
+    }
+    if (part == 0) for (int e = lane; e < E; e += 32) hist[e] = 0;
+    cluster_sync();
+    for (int i0 = mine * share; i0 < min(n, (mine + 1) * share); i0 += 64) {
       // two vectors per lane: the packed operations take both
       const int i[2] = {i0 + lane, i0 + 32 + lane};
-      const int stop = min(n, (warp + 1) * share);
-      uint32_t v[2];
-      float2 wv[2] = {make_float2(1.f, 1.f), make_float2(1.f, 1.f)};
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        v[q] = __ldg(vec + min(i[q], n - 1));
-        if (weighted) wv[q] = __ldg(wgt + min(i[q], n - 1));
-      }
+      const int stop = min(n, (mine + 1) * share);
+      if (share > 64) fetch(i0);
       const float2 f0 = vec_of(v[0]), f1 = vec_of(v[1]);
       const float2 x = make_float2(f0.x, f1.x), y = make_float2(f0.y, f1.y), wx = make_float2(wv[0].x, wv[1].x), wy = make_float2(wv[0].y, wv[1].y);
       float best[2] = {INFINITY, INFINITY};
-      int bi[2] = {0, 0};
-#pragma unroll 4
-      for (int e = 0; e < E; ++e) {
-        const float2 c = sh.cf[e];
-        const float2 dx = add2(x, make_float2(-c.x, -c.x)), dy = add2(y, make_float2(-c.y, -c.y));
-        const float2 yy = mul2(dy, dy);
-        const float2 d = weighted ? fma2(wx, mul2(dx, dx), mul2(wy, yy)) : fma2(dx, dx, yy);
-        if (d.x < best[0]) { best[0] = d.x; bi[0] = e; }
-        if (d.y < best[1]) { best[1] = d.y; bi[1] = e; }
+      int bi2[2] = {0, 0};
+#pragma unroll 8
+      for (int e = part_e0; e < part_e1; ++e) {
+        const float2 d = pair_distance(weighted, x, y, wx, wy, sh.neg[centre_slot(e)]);
+        if (d.x < best[0]) { best[0] = d.x; bi2[0] = e; }
+        if (d.y < best[1]) { best[1] = d.y; bi2[1] = e; }
+      }
+      if (parts > 1) {
+        const int at = (warp % shares) * 64 + lane;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) { sh.part_best[part][at + 32 * q] = best[q]; sh.part_idx[part][at + 32 * q] = (uint8_t)bi2[q]; }
+        asm volatile("bar.sync %0, %1;" ::"r"(2 + warp % shares), "r"(32 * parts) : "memory");
+        if (part == 0) {
+#pragma unroll
+          for (int k = 1; k < kVecCluster; ++k)      // parts in the order of their centres: the first of equal distances stays
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const float b = sh.part_best[k][at + 32 * q];
+              const int e = sh.part_idx[k][at + 32 * q];
+              if (b < best[q]) { best[q] = b; bi2[q] = e; }
+            }
+        }
+        if (share > 64) asm volatile("bar.sync %0, %1;" ::"r"(2 + warp % shares), "r"(32 * parts) : "memory");
+        if (part != 0) continue;
       }
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
+        const int bi = bi2[q];
         const bool in = i[q] < stop;
-        if (in) idx[i[q]] = (uint8_t)bi[q];
+        if (in) peer_store8(lead_idx + (uint32_t)i[q], (uint32_t)bi);
         if (!weighted) {
-          if (in) move_member(sh.sums, v[q], bi[q], 1);
+          if (in) move_member(sh.sums, v[q], bi, 1);
         } else {
           const unsigned live = __ballot_sync(0xFFFFFFFFu, in);
           if (in) {
-            const unsigned same = __match_any_sync(live, bi[q]);
-            if ((same & ((1u << lane) - 1u)) == 0u) sh.hist[warp][bi[q]] += (uint16_t)__popc(same);
+            const unsigned same = __match_any_sync(live, bi), below = same & ((1u << lane) - 1u);
+            const int before = hist[bi];
+            __syncwarp(live);
+            peer_store16(lead_ranks + 2u * (uint32_t)i[q], (uint32_t)(before + __popc(below)));
+            if (below == 0u) hist[bi] = (uint16_t)(before + __popc(same));
           }
           __syncwarp();
         }
       }
     }
-    __syncthreads();
+    if (weighted && !lead && part == 0) {
+      const uint32_t to = peer_address(hist, 0u);
+      for (int e = lane; e < E; e += 32) peer_store16(to + 2u * (uint32_t)e, hist[e]);
+    }
+    cluster_sync();
+    if (!lead) continue;
     if (!weighted) {
       for (int e = tid; e < E; e += kVecThreads) {
         const int cnt = sh.sums.cnt[e];
@@ -971,88 +1038,134 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     } else {
       // weighted means of Eq. 19, per dimension, members added in vector order: a stable sort by centre, then one thread
       // per centre and dimension
-      for (int e = tid; e < E; e += kVecThreads) {
-        int s = 0;
-#pragma unroll 8
-        for (int w = 0; w < kVecThreads / 32; ++w) s += sh.hist[w][e];
-        sh.first[e + 1] = s;
+      for (int e = warp; e < E; e += kVecThreads / 32) {      // lane = share
+        const int mine = sh.hist[lane][e];
+        int s = mine;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int o = __shfl_up_sync(0xFFFFFFFFu, s, off);
+          if (lane >= off) s += o;
+        }
+        sh.hist[lane][e] = (uint16_t)(s - mine);
+        if (lane == 31) sh.first[e + 1] = s;
       }
       __syncthreads();
       if (warp == 0) {
         int carry = 0;
         for (int e0 = 0; e0 < E; e0 += 32) {
-          int s = sh.first[e0 + lane + 1];
+          int s = e0 + lane < E ? sh.first[e0 + lane + 1] : 0;
 #pragma unroll
           for (int off = 1; off < 32; off <<= 1) {
             const int o = __shfl_up_sync(0xFFFFFFFFu, s, off);
             if (lane >= off) s += o;
           }
-          sh.first[e0 + lane + 1] = carry + s;
+          if (e0 + lane < E) sh.first[e0 + lane + 1] = carry + s;
           carry += __shfl_sync(0xFFFFFFFFu, s, 31);
         }
         if (lane == 0) sh.first[0] = 0;
       }
       __syncthreads();
-      for (int e = tid; e < E; e += kVecThreads) {
-        int s = sh.first[e];
-#pragma unroll 8
-        for (int w = 0; w < kVecThreads / 32; ++w) { const int c = sh.hist[w][e]; sh.hist[w][e] = (uint16_t)s; s += c; }
+      for (int i = warp * share + lane; i < min(n, (warp + 1) * share); i += 32) {
+        const int e = idx[i];
+        sorted[sh.first[e] + sh.hist[warp][e] + ranks[i]] = (uint16_t)i;
       }
       __syncthreads();
-      for (int i0 = warp * share; i0 < min(n, (warp + 1) * share); i0 += 32) {
-        const int i = i0 + lane;
-        const bool in = i < n;
-        const unsigned live = __ballot_sync(0xFFFFFFFFu, in);
-        if (in) {
-          const int e = idx[i];
-          const unsigned same = __match_any_sync(live, e);
-          const int rank = __popc(same & ((1u << lane) - 1u)), p = sh.hist[warp][e];
-          __syncwarp(live);
-          sorted[p + rank] = (uint16_t)i;
-          if (rank == 0) sh.hist[warp][e] = (uint16_t)(p + __popc(same));
+      // four threads a centre: the sums of w * v and of w, of either dimension
+      for (int k = tid; k < 4 * E; k += kVecThreads) {
+        const int e = k >> 2, dim = k & 1;
+        const bool den = (k & 2) != 0;
+        double sum = 0.0;
+        const int stop = sh.first[e + 1];
+        // eight members at a time; past the end the last one again, times zero
+        if (tables) {
+          const double* table = reinterpret_cast<const double*>(den ? table_w : table_wv) + dim;
+          for (int j = sh.first[e]; j < stop; j += 8) {
+            double v[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              v[m] = table[2 * sorted[min(j + m, stop - 1)]];
+              if (j + m >= stop) v[m] = 0.0;
+            }
+#pragma unroll
+            for (int m = 0; m < 8; ++m) sum += v[m];
+          }
+        } else {
+          for (int j = sh.first[e]; j < stop; j += 8) {
+            float wi[8], f[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              const int i = sorted[min(j + m, stop - 1)];
+              wi[m] = j + m < stop ? __ldg(a.elem_w + 2 * i + dim) : 0.f;
+              f[m] = den ? 1.f : h2f_bits(__ldg(a.w + 2 * i + dim));
+            }
+#pragma unroll
+            for (int m = 0; m < 8; ++m) sum = fma((double)wi[m], (double)f[m], sum);      // the product of 24 and 11 bits is exact
+          }
         }
-        __syncwarp();
-      }
-      __syncthreads();
-      for (int k = tid; k < 2 * E; k += kVecThreads) {
-        const int e = k >> 1, dim = k & 1;
-        double num = 0.0, den = 0.0;
-#pragma unroll 4
-        for (int j = sh.first[e]; j < sh.first[e + 1]; ++j) {
-          const int i = sorted[j];
-          const float wi = __ldg(a.elem_w + 2 * i + dim);
-          num += (double)wi * (double)h2f_bits(__ldg(a.w + 2 * i + dim));
-          den += (double)wi;
-        }
-        if (den > 0.0) (dim ? sh.cy : sh.cx)[e] = num / den;
+        const unsigned four = 0xFu << (lane & 28);
+        const double weight = __shfl_xor_sync(four, sum, 2);
+        if (!den && weight > 0.0) (dim ? sh.cy : sh.cx)[e] = sum / weight;
       }
     }
     __syncthreads();
+    publish();
   }
   // ---- centres to fp16; final assignment against the rounded centres in fp64
-  for (int e = tid; e < E; e += kVecThreads) {
-    const __half hx = __double2half(sh.cx[e]), hy = __double2half(sh.cy[e]);
-    sh.cx[e] = (double)__half2float(hx); sh.cy[e] = (double)__half2float(hy);
-    a.aux[e] = (uint32_t)__half_as_ushort(hx) | ((uint32_t)__half_as_ushort(hy) << 16);
-  }
-  __syncthreads();
-  for (int i = tid; i < n; i += kVecThreads) {
-    const float2 f = vec_of(__ldg(vec + i));
-    const double x = (double)f.x, y = (double)f.y;
-    double wx = 1.0, wy = 1.0;
-    if (weighted) { const float2 wv = __ldg(wgt + i); wx = (double)wv.x; wy = (double)wv.y; }
-    double best = INFINITY;
-    int bi = 0;
-#pragma unroll 4
-    for (int e = 0; e < E; ++e) {
-      const double dx = x - sh.cx[e], dy = y - sh.cy[e];
-      const double d = weighted ? __dadd_rn(__dmul_rn(wx, __dmul_rn(dx, dx)), __dmul_rn(wy, __dmul_rn(dy, dy)))
-                                : __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-      if (d < best) { best = d; bi = e; }
+  cluster_sync();                                  // the last centres are no longer being written
+  if (lead) {
+    for (int e = tid; e < E; e += kVecThreads) {
+      const __half hx = __double2half(sh.cx[e]), hy = __double2half(sh.cy[e]);
+      const float cx = __half2float(hx), cy = __half2float(hy);
+      a.aux[e] = (uint32_t)__half_as_ushort(hx) | ((uint32_t)__half_as_ushort(hy) << 16);
+      for (uint32_t r = 0; r < peers; ++r) {
+        peer_store(peer_address(&sh.neg[centre_slot(e)], r), make_float4(-cx, -cx, -cy, -cy));
+        peer_store(peer_address(&sh.cx[e], r), (double)cx);
+        peer_store(peer_address(&sh.cy[e], r), (double)cy);
+      }
     }
-    idx[i] = (uint8_t)bi;
   }
-  __syncthreads();
+  cluster_sync();
+  // In fp32 first: a distance is wrong by less than seven roundings there, so a centre whose distance is smallest by more than 2^-20 of it is
+  // the nearest in fp64 too, and so is one that the vector equals.  The others (and distances near the end of fp32's range) are taken in fp64.
+  const int stride = (int)peers * kVecThreads;
+  for (int i0 = (int)rank * kVecThreads + tid; i0 < n; i0 += 2 * stride) {
+    const int i[2] = {i0, i0 + stride};
+    float2 f[2], wv[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      f[q] = vec_of(__ldg(vec + min(i[q], n - 1)));
+      wv[q] = weighted ? __ldg(wgt + min(i[q], n - 1)) : make_float2(1.f, 1.f);
+    }
+    const Nearest nr = nearest_group(sh.neg, E, weighted, make_float2(f[0].x, f[1].x), make_float2(f[0].y, f[1].y), make_float2(wv[0].x, wv[1].x),
+                                     make_float2(wv[0].y, wv[1].y));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (i[q] >= n) break;
+      const float limit = nr.best[q] * (1.f + 1.f / 1048576.f);
+      const float4* c = sh.neg + centre_slot(nr.group[q]);
+      int k = 0, close = 0;
+#pragma unroll
+      for (int j = 0; j < kCentreGroup; ++j)
+        if (one_distance(weighted, f[q].x, f[q].y, wv[q].x, wv[q].y, c[j]) <= limit) { k = j; ++close; }
+      int bi = nr.group[q] + k;
+      const bool equal = f[q].x + c[k].x == 0.f && f[q].y + c[k].z == 0.f;
+      if (close != 1 || !(nr.second[q] > limit) || !(equal || (nr.best[q] > 1e-30f && nr.best[q] < 1e30f))) {
+        const double x = (double)f[q].x, y = (double)f[q].y, wx = (double)wv[q].x, wy = (double)wv[q].y;
+        double best = INFINITY;
+        bi = 0;
+#pragma unroll 4
+        for (int e = 0; e < E; ++e) {
+          const double dx = x - sh.cx[e], dy = y - sh.cy[e];
+          const double d = weighted ? __dadd_rn(__dmul_rn(wx, __dmul_rn(dx, dx)), __dmul_rn(wy, __dmul_rn(dy, dy)))
+                                    : __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+          if (d < best) { best = d; bi = e; }
+        }
+      }
+      peer_store8(lead_idx + (uint32_t)i[q], (uint32_t)bi);
+    }
+  }
+  cluster_sync();
+  if (!lead) return;
   const int bits = a.bits, n_words = (int)(((((size_t)n * bits + 7) / 8 + 15) / 16 * 16) / 4);
   for (int wi = tid; wi < n_words; wi += kVecThreads) {
     uint32_t val = 0u;
@@ -1204,17 +1317,31 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
     a.payload = img + h.off_payload;
     a.aux = reinterpret_cast<uint32_t*>(img + h.off_aux);
     a.flags = flags;
-    static SmemOptIn opt_in_seed, opt_in_64, opt_in_256, opt_in_vector;
+    static SmemOptIn opt_in_seed, opt_in_64, opt_in_256, opt_in_vector, opt_in_vector_seed;
     if (is_vector) {
-      e = opt_in_vector((const void*)vq_vector_kernel, (int)vec_smem_bytes(kVqMaxVec));
+      const int seed_threads = (a.n_vec + 2047) / 2048 * 32;
+      e = opt_in_vector_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
       if (e != cudaSuccess) return cuda_status(e);
-      vq_vector_kernel<<<1, kVecThreads, vec_smem_bytes(a.n_vec), s>>>(a, h, img);
+      vq_seed_kernel<true><<<1, seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s>>>(a);
+      e = opt_in_vector((const void*)vq_vector_kernel, (int)std::max(vec_smem_bytes(kVqMaxVec), vec_smem_bytes(kVecTable)));
+      if (e != cudaSuccess) return cuda_status(e);
+      // the exact sums of an unweighted vector are atomics in one block's shared memory
+      cudaLaunchConfig_t cfg_v = {};
+      cfg_v.gridDim = dim3(a.elem_w ? kVecCluster : 1); cfg_v.blockDim = dim3(kVecThreads); cfg_v.dynamicSmemBytes = vec_smem_bytes(a.n_vec); cfg_v.stream = s;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = cfg_v.gridDim.x; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // starts while the seeds are drawn
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg_v.attrs = attr; cfg_v.numAttrs = 2;
+      e = cudaLaunchKernelEx(&cfg_v, vq_vector_kernel, (const VqArgs)a, (const rwkvq_image_header)h, img);
+      if (e != cudaSuccess) return cuda_status(e);
     } else {
       constexpr size_t seed_smem = (size_t)kVqMaxVec * 4 + sizeof(SeedShared);
       const int tiles = (oc / 256) * (ic / 256);
-      e = opt_in_seed((const void*)vq_seed_kernel, (int)seed_smem);
+      e = opt_in_seed((const void*)vq_seed_kernel<false>, (int)seed_smem);
       if (e != cudaSuccess) return cuda_status(e);
-      vq_seed_kernel<<<tiles, kVqThreads, seed_smem, s>>>(a);
+      vq_seed_kernel<false><<<tiles, kVqThreads, seed_smem, s>>>(a);
       if (d.entries == 64) {
         e = opt_in_64((const void*)vq_lloyd_kernel<2>, (int)sizeof(LloydShared));
         if (e != cudaSuccess) return cuda_status(e);

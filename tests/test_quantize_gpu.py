@@ -243,6 +243,30 @@ def test_weighted_mu_quantizer(ic, bits):
     assert np.array_equal(out.cpu().numpy().astype(np.float64), orc.mu_decode(c.astype(np.float16), ix))
 
 
+@pytest.mark.parametrize("ic,bits", [(128, 6), (2176, 6), (8192, 6), (8448, 6), (8448, 8)])
+@pytest.mark.parametrize("weighted", [False, True])
+def test_mu_quantizer_ties_zero_weights_and_sizes(ic, bits, weighted):
+    """Sizes around the warps of the seeding, the shares of the assignment and the table of the sums; equal vectors,
+    equal distances and weights of zero: the indices are the oracle's nearest entries, lowest first."""
+    rng = np.random.default_rng(ic + bits)
+    mu16 = (rng.integers(0, 24, ic) / 16.0).astype(np.float16)
+    mu16[: ic // 2] += rng.uniform(0.0, 0.01, ic // 2).astype(np.float16)
+    wts = None
+    if weighted:
+        wts = (rng.standard_normal(ic) ** 2).astype(np.float32)
+        wts[rng.random(ic) < 0.1] = 0.0
+        wts[:8] = 0.0
+        wts[8:16] = 1e-38
+    _, img = quantize_dev(mu16, B.RWKVQ_VQ, bits, elem_weight=wts, seed=5, iters=4)
+    _, codes = B.rwkvq_image_unpack(img.cpu().numpy())
+    c = np.asarray(codes["codebook"]).reshape(1 << bits, 2).astype(np.float64)
+    w2 = None if wts is None else wts.astype(np.float64).reshape(-1, 2)
+    want = orc._nearest(mu16.astype(np.float64).reshape(-1, 2), c, w2)
+    assert np.array_equal(np.asarray(codes["q"]).reshape(-1), want)
+    _, again = quantize_dev(mu16, B.RWKVQ_VQ, bits, elem_weight=wts, seed=5, iters=4)
+    assert torch.equal(img, again)
+
+
 def test_quantize_dev_error_paths():
     w = torch.zeros((256, 256), dtype=torch.float16, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
