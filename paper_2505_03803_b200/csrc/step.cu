@@ -124,8 +124,9 @@ static_assert(sizeof(StepMixX) == 80, "pre-pass operator descriptor size");
 constexpr int kGroupWarps = 8, kGroupThreads = kGroupWarps * 32;
 // Thread layout of a CTA, by the number of batch blocks NB a record is multiplied with.
 //   NB = 1 (B <= 8): two consumer groups of eight warps, three stager warps, one producer warp: 640 threads,
-//     96 registers each at launch, re-divided at entry (consumers kConsumerRegs, the last warpgroup
-//     kStagerRegs).
+//     96 registers each, for all roles (with 104 for the consumers and 64 for the others, which the compiler takes as the limit of these
+//     roles' code, the pre-pass of a stage spilled, and behind a barrier's acquire a spilled word is a trip to L2: blocks 136 us where
+//     they take 127).
 //   NB = 2 (B > 8): the record routine wants about 150 registers, which sixteen consumer warps cannot have,
 //     and eight warps that keep everything in registers outrun sixteen that spill: ONE consumer group,
 //     seven stager warps (the stage pre-pass is theirs), one producer: 512 threads, 128 registers at
@@ -138,7 +139,7 @@ template <int NB> struct Shape {
   static constexpr int kConsumerThreads = kConsumerWarps * 32, kStagerThreads = kStagerWarps * 32;
   static constexpr int kThreads = kConsumerThreads + kStagerThreads + 32;
   static constexpr int kLaunchRegs = NB == 2 ? 128 : 96;
-  static constexpr int kConsumerRegs = NB == 2 ? 152 : 104, kStagerRegs = NB == 2 ? 104 : 64;
+  static constexpr int kConsumerRegs = NB == 2 ? 152 : 96, kStagerRegs = NB == 2 ? 104 : 96;
   static_assert(kConsumerWarps % 4 == 0 && (kStagerWarps + 1) % 4 == 0, "register re-division works on warpgroups of four warps");
   static_assert(kConsumerRegs * kConsumerThreads + kStagerRegs * (kStagerThreads + 32) <= kLaunchRegs * kThreads,
                 "register re-division exceeds the launch's pool");
@@ -278,6 +279,7 @@ struct Ctrl {
                              // stage that the barrier closes.  Per barrier, not one running total: consumer
                              // warps of a CTA without work in the coming stages may run any number of
                              // stages ahead of the stagers.
+  uint32_t mix_at[8];        // batch row | group << 16 of the item in each stager warp's MixSlot
   int abort_flag;
   int poll_limit;            // must follow abort_flag (poll_limit_of)
 };
@@ -412,78 +414,86 @@ __device__ __forceinline__ float pair_sum(uint32_t r) {
 
 constexpr int kStageUnroll = 4;
 
-__device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-x)); }
+// 1 / y for y >= 1 by Newton's correction of the approximate reciprocal with fused multiply-adds (Markstein, "Computation of elementary functions
+// on the IBM RISC System/6000 processor", 1990).  Without the general division's branch four sigmoids run side by side (200 cycles instead of 800).
+__device__ __forceinline__ float rcp_of(float y) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(y));
+  return y < 1e37f ? fmaf(r, fmaf(-y, r, 1.f), r) : r;
+}
+__device__ __forceinline__ float sigmoidf_(float x) { return rcp_of(1.f + expf(-x)); }
 __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
   const __half2 h = __floats2half2_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
-// Eight consecutive inputs of a product from the element-wise operator in front of it (Appendix A.1
+// Four consecutive inputs of a product from the element-wise operator in front of it (Appendix A.1
 // Eqs. 23, 24, 27), rounded to fp16.  e0: index of the first element in the [B][ic] fp32 arrays,
-// col: its column (index into the per-channel parameters).  `commit` false (a lane that repeats
-// another lane's group to keep the half-warp whole): the recurrence state is not written.
-__device__ __forceinline__ uint4 xform_input(const StepMixOp& mo, const StepMixX& op, size_t e0, int col, bool commit, float rstd) {
-  float s[8];
-  {
-    const float4 a = __ldcg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(op.src) + e0));
-    const float4 c = __ldcg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(op.src) + e0 + 4));
-    s[0] = a.x; s[1] = a.y; s[2] = a.z; s[3] = a.w; s[4] = c.x; s[5] = c.y; s[6] = c.z; s[7] = c.w;
-  }
-  float o[8];
+// col: its column (index into the per-channel parameters).  `commit` false (a warp that repeats
+// another's item to keep the barriers whole): the recurrence state is not written.
+__device__ __forceinline__ float4 ldcg4(uint64_t base, size_t e) { return __ldcg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + e)); }
+// The inputs themselves, asked for before anything that has to be waited for (the row statistic).
+struct XformLoads { float4 s, g; float scale; };
+__device__ __forceinline__ void xform_load(const StepMixOp& mo, const StepMixX& op, size_t e0, XformLoads& l) {
+  l.s = ldcg4(op.src, e0);
+  l.g = make_float4(0.f, 0.f, 0.f, 0.f);
+  if ((mo.kind & 0xFF) == RWKVQ_IN_F32 && op.k) l.g = ldcg4(op.k, e0);
+  l.scale = op.scale ? __ldcg(reinterpret_cast<const float*>(op.scale)) : 1.f;
+}
+__device__ __forceinline__ void spread(const float4 v, float (&o)[4]) { o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w; }
+__device__ __forceinline__ uint2 xform_input(const StepMixOp& mo, const StepMixX& op, const XformLoads& l, size_t e0, int col, bool commit, float rstd) {
   const int kind = mo.kind & 0xFF;
+  float s[4], o[4];
+  spread(l.s, s);
   if (kind == RWKVQ_IN_RELU2) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { const float m = fmaxf(s[i], 0.f); o[i] = m * m; }
+    for (int i = 0; i < 4; ++i) { const float m = fmaxf(s[i], 0.f); o[i] = m * m; }
   } else if (kind == RWKVQ_IN_F32) {
+    float g[4];
+    spread(l.g, g);
+    const bool gate = op.k != 0u;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] = s[i];
-    if (op.k) {      // gate
-      const float* g = reinterpret_cast<const float*>(op.k) + e0;
+    for (int i = 0; i < 4; ++i) o[i] = (gate ? s[i] * sigmoidf_(g[i]) : s[i]) * rstd;
+  } else {           // RWKVQ_IN_WKV: all loads ahead of the first use and of the stores
+    float k[4], vv[4], a[4], bb[4], p[4], u[4], w[4];
+    spread(ldcg4(op.k, e0), k); spread(ldcg4(op.v, e0), vv);
+    spread(ldcg4(op.state_a, e0), a); spread(ldcg4(op.state_b, e0), bb); spread(ldcg4(op.state_p, e0), p);
+    spread(__ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(op.u) + col)), u);
+    spread(__ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(op.w) + col)), w);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) o[i] *= sigmoidf_(__ldcg(g + i));
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] *= rstd;
-  } else {           // RWKVQ_IN_WKV
-    const float* kp = reinterpret_cast<const float*>(op.k) + e0;
-    const float* vp = reinterpret_cast<const float*>(op.v) + e0;
-    float* sa = reinterpret_cast<float*>(op.state_a) + e0;
-    float* sb = reinterpret_cast<float*>(op.state_b) + e0;
-    float* sp = reinterpret_cast<float*>(op.state_p) + e0;
-    const float* up = reinterpret_cast<const float*>(op.u) + col;
-    const float* wp = reinterpret_cast<const float*>(op.w) + col;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < 4; ++i) {
       // the history sums are stored as a = e^{-p} sum f v, b = e^{-p} sum f; every exponential below has
       // a non-positive argument
-      const float k = __ldcg(kp + i), vv = __ldcg(vp + i), a = __ldcg(sa + i), bb = __ldcg(sb + i), p = __ldcg(sp + i);
-      const float uk = __ldg(up + i) + k;
-      const float q = fmaxf(p, uk);
-      const float e1 = expf(p - q), e2 = expf(uk - q);
-      const float wkv = (e1 * a + e2 * vv) / (e1 * bb + e2);
+      const float uk = u[i] + k[i];
+      const float q = fmaxf(p[i], uk);
+      const float e1 = expf(p[i] - q), e2 = expf(uk - q);
+      const float wkv = (e1 * a[i] + e2 * vv[i]) / (e1 * bb[i] + e2);
       o[i] = sigmoidf_(s[i]) * wkv;
-      const float pw = p - __ldg(wp + i);
-      const float q2 = fmaxf(pw, k);
-      const float f1 = expf(pw - q2), f2 = expf(k - q2);
-      if (commit) { sa[i] = f1 * a + f2 * vv; sb[i] = f1 * bb + f2; sp[i] = q2; }
+      const float pw = p[i] - w[i];
+      const float q2 = fmaxf(pw, k[i]);
+      const float f1 = expf(pw - q2), f2 = expf(k[i] - q2);
+      a[i] = f1 * a[i] + f2 * vv[i]; bb[i] = f1 * bb[i] + f2; p[i] = q2;
+    }
+    if (commit) {
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(op.state_a) + e0) = make_float4(a[0], a[1], a[2], a[3]);
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(op.state_b) + e0) = make_float4(bb[0], bb[1], bb[2], bb[3]);
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(op.state_p) + e0) = make_float4(p[0], p[1], p[2], p[3]);
     }
   }
   if (op.scale) {
-    const float gsc = __ldcg(reinterpret_cast<const float*>(op.scale));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] *= gsc;
+    for (int i = 0; i < 4; ++i) o[i] *= l.scale;
   }
-  return make_uint4(pack_half2(o[0], o[1]), pack_half2(o[2], o[3]), pack_half2(o[4], o[5]), pack_half2(o[6], o[7]));
+  return make_uint2(pack_half2(o[0], o[1]), pack_half2(o[2], o[3]));
 }
 
-// 1 / sqrt(mean over the row of v^2 + 1e-6), v = src (* sigmoid(gate)): the sixteen lanes of a half-warp
-// read row b of the fp32 source(s) together.  Items that follow one another in a half-warp mostly share
+// 1 / sqrt(mean over the row of v^2 + 1e-6), v = src (* sigmoid(gate)): the lanes of a warp
+// read row b of the fp32 source(s) together.  Items that follow one another in a warp mostly share
 // the row, so the caller keeps the last result.
-// Called by whole warps (the shuffles name all 32 lanes); a half-warp with `active` false reads nothing.
-__device__ __forceinline__ float row_rstd(const StepMixOp& op, const StepMixX& ox, int b, int l16, bool active) {
+__device__ __noinline__ float row_rstd(const StepMixOp& op, const StepMixX& ox, int b, int lane) {
   const float* src = reinterpret_cast<const float*>(ox.src) + (size_t)b * op.ic;
   const float* gate = ox.k ? reinterpret_cast<const float*>(ox.k) + (size_t)b * op.ic : nullptr;
   float acc = 0.f;
-  for (uint32_t c = (uint32_t)l16 * 4u; active && c < op.ic; c += 64u) {
+  for (uint32_t c = (uint32_t)lane * 4u; c < op.ic; c += 128u) {
     float4 v = __ldcg(reinterpret_cast<const float4*>(src + c));
     if (gate) {
       const float4 g = __ldcg(reinterpret_cast<const float4*>(gate + c));
@@ -491,9 +501,8 @@ __device__ __forceinline__ float row_rstd(const StepMixOp& op, const StepMixX& o
     }
     acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
   }
-  __syncwarp();
 #pragma unroll
-  for (int d = 8; d > 0; d >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, d);
+  for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, d);
   return rsqrtf(acc / (float)op.ic + 1e-6f);
 }
 
@@ -572,26 +581,72 @@ __device__ void mix_warm(const StepArgs& a, const StepEvent& ev, int stid) {
   }
 }
 
-// This CTA's share of a stage's pre-pass.  A half-warp takes one (product, batch row, 128-column
-// group) at a time: it loads x (and x_prev, and decodes mu_hat), mixes, rounds to fp16, stores the
-// 128 values to the product's pre-pass rows and reduces the three sums of the group with shuffles.
+// Descriptors of a stager warp's current pre-pass item (product, batch row, 128-column group), in shared memory: taken there while the stage barrier
+// is still closed (the poll's acquire empties L1, so whatever is read behind it is a trip to L2, and a chain of four of them went by until the
+// first input was asked for); in registers they spilled, and every spilled word was such a trip too.
+struct MixSlot { StepMixOp op; StepMixX ox; };
+// Takes item r into the warp's slot; returns the lane's two mu_hat pairs.
+__device__ __forceinline__ uint2 mix_fetch(const StepArgs& a, const StepEvent& ev, uint32_t r, MixSlot* slot, uint32_t* at, int lane) {
+  const StepMixOp* ops = a.mixops + ev.arrd.op_first;
+  const int n_ops = (int)ev.arrd.op_count;
+  int k = 0;
+  uint32_t icp = __ldg(&ops[0].ic_pad);
+  while (k + 1 < n_ops && r >= (uint32_t)a.B * (icp >> 7)) { r -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
+  static_assert(sizeof(StepMixOp) == 64 && sizeof(StepMixX) == 80, "nine lanes copy a slot");
+  if (lane < 9)
+    reinterpret_cast<uint4*>(slot)[lane] = lane < 4 ? __ldg(reinterpret_cast<const uint4*>(ops + k) + lane)
+                                                    : __ldg(reinterpret_cast<const uint4*>(a.mixx + ev.arrd.op_first + k) + (lane - 4));
+  const uint32_t ng = icp >> 7, row = r / ng, grp = r % ng;
+  if (lane == 0) *at = row | grp << 16;
+  __syncwarp();
+  uint2 mu = make_uint2(0u, 0u);
+  const uint32_t col = grp * 128u + (uint32_t)lane * 4u;
+  if (slot->op.mu && col < slot->op.ic) {
+    const uint32_t bits = slot->op.mu_bits, bit = (col >> 1) * bits, sh = bit & 31u, mask = (1u << bits) - 1u;      // two indices
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(slot->op.mu) + (bit >> 5);
+    const uint32_t wlo = __ldg(w);
+    const uint32_t whi = (sh + 2u * bits > 32u) ? __ldg(w + 1) : 0u;
+    const uint32_t f = __funnelshift_r(wlo, whi, sh);
+    const uint32_t* cb = reinterpret_cast<const uint32_t*>(slot->op.mu_aux);
+    mu = make_uint2(__ldg(cb + (f & mask)), __ldg(cb + ((f >> bits) & mask)));
+  }
+  return mu;
+}
+struct MixPrep { uint2 mu; uint32_t kind; };      // of the warp's first item; of the stage's first product: what kind of stage it is
 template <int NB>
-__device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid) {
+__device__ __forceinline__ MixPrep mix_prepare(const StepArgs& a, const StepEvent& ev, int stid, MixSlot* slots, uint32_t* at) {
+  MixPrep p;
+  p.mu = make_uint2(0u, 0u);
+  p.kind = __ldg(&a.mixops[ev.arrd.op_first].kind);
+  const uint32_t lo = ev.arr.grp_lo, hi = ev.arr.grp_hi, w = (uint32_t)(stid >> 5);
+  if (lo < hi && !(p.kind & 0x800u)) p.mu = mix_fetch(a, ev, lo + w < hi ? lo + w : lo, slots + w, at + w, stid & 31);
+  return p;
+}
+
+// This CTA's share of a stage's pre-pass.  A warp takes one (product, batch row, 128-column
+// group) at a time (a quarter-warp in stages of plain inputs): it loads x (and x_prev, and decodes mu_hat), mixes, rounds to fp16, stores the
+// 128 values to the product's pre-pass rows and reduces the three sums of the group with shuffles.
+// Bound by its latency: a CTA has an item or two, and all wait.  Whole blocks, d 2048, batch 2: 10.6 us a stage before, of which the
+// pre-pass took 2 to 8.5; 7.9 with descriptors in shared memory, no spills, vector loads ahead of every wait and stores behind them
+// (the recurrence read its seven arrays element by element, each behind the stores of the one before), and sigmoids without a branch.
+template <int NB>
+__device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, const MixPrep& prep, MixSlot* slots, uint32_t* mix_at) {
   constexpr int kStagerWarps = Shape<NB>::kStagerWarps, kStagerThreads = Shape<NB>::kStagerThreads;
-  const int lane = stid & 31, l16 = lane & 15;
+  const int lane = stid & 31;
   const uint32_t lo = ev.arr.grp_lo, hi = ev.arr.grp_hi;
+  if (lo >= hi) return;      // the same for all stager warps
   const StepMixOp* ops = a.mixops + ev.arrd.op_first;
   const int n_ops = (int)ev.arrd.op_count;
   const int nbp = (a.B + 1) & ~1;
   // Row statistics first: the rows of normalised inputs that this CTA's items fall in (a few: the items
   // are consecutive groups of consecutive rows) are reduced by all stager threads together, 1.5 KB per
-  // round of loads, into a small table; rows beyond the table are reduced by the half-warp that meets them.
+  // round of loads, into a small table; rows beyond the table are reduced by the warp that meets them.
   constexpr int kRowTable = 8;
   __shared__ float s_rstd[kRowTable];
   __shared__ float s_part[kStagerWarps];
   __shared__ uint32_t s_row_end[kRowTable];      // first item behind the row of each entry
   int n_rows = 0;
-  const uint32_t stage_kind = __ldg(&ops[0].kind);
+  const uint32_t stage_kind = prep.kind;
   if (stage_kind & 0x800) {
     // Stage of plain inputs (no operator, no normalisation): a quarter-warp per item, sixteen columns per
     // lane, so that a CTA's share is done in one round of loads.
@@ -671,30 +726,41 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid) {
     }
     return;
   }
-  if (stage_kind & 0x400) {      // the planner marks the first product of a stage that has a normalised input
+  auto row_table = [&]() {
     uint32_t r = lo;
     while (r < hi && n_rows < kRowTable) {
-      uint32_t rr = r;
-      int k = 0;
-      uint32_t icp = __ldg(&ops[0].ic_pad);
-      while (k + 1 < n_ops && rr >= (uint32_t)a.B * (icp >> 7)) { rr -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
-      const StepMixOp op = ops[k];
-      const uint32_t ng = op.ic_pad >> 7;
-      const int b = (int)(rr / ng);
+      // the first row is that of the first warp's item
+      const StepMixOp* op = &slots[0].op;
+      const StepMixX* ox = &slots[0].ox;
+      uint32_t row = mix_at[0] & 0xFFFFu, left = (op->ic_pad >> 7) - (mix_at[0] >> 16);
+      if (n_rows) {
+        uint32_t rr = r;
+        int k = 0;
+        uint32_t icp = __ldg(&ops[0].ic_pad);
+        while (k + 1 < n_ops && rr >= (uint32_t)a.B * (icp >> 7)) { rr -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
+        op = ops + k; ox = a.mixx + ev.arrd.op_first + k;
+        row = rr / (icp >> 7); left = (icp >> 7) - rr % (icp >> 7);
+      }
+      const uint32_t ic = op->ic;
+      const bool norm = (op->kind & 0x100) != 0;
+      const float* src = reinterpret_cast<const float*>(ox->src) + (size_t)row * ic;
+      const float* gate = ox->k ? reinterpret_cast<const float*>(ox->k) + (size_t)row * ic : nullptr;
       float rstd = 1.f;
-      if (op.kind & 0x100) {
-        const StepMixX ox = a.mixx[ev.arrd.op_first + k];
-        const float* src = reinterpret_cast<const float*>(ox.src) + (size_t)b * op.ic;
-        const float* gate = ox.k ? reinterpret_cast<const float*>(ox.k) + (size_t)b * op.ic : nullptr;
+      if (norm) {
         float acc = 0.f;
-#pragma unroll 4
-        for (uint32_t c = (uint32_t)stid * 4u; c < op.ic; c += (uint32_t)kStagerThreads * 4u) {
-          float4 v = __ldcg(reinterpret_cast<const float4*>(src + c));
-          if (gate) {
-            const float4 g = __ldcg(reinterpret_cast<const float4*>(gate + c));
-            v.x *= sigmoidf_(g.x); v.y *= sigmoidf_(g.y); v.z *= sigmoidf_(g.z); v.w *= sigmoidf_(g.w);
-          }
-          acc += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        // two rounds of loads ahead of the one that is added up
+        constexpr uint32_t kStep = (uint32_t)kStagerThreads * 4u;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto get = [&](const float* from, uint32_t c) { return c < ic ? __ldcg(reinterpret_cast<const float4*>(from + c)) : zero; };
+        uint32_t c = (uint32_t)stid * 4u;
+        float4 v0 = get(src, c), v1 = get(src, c + kStep), g0 = zero, g1 = zero;
+        if (gate) { g0 = get(gate, c); g1 = get(gate, c + kStep); }
+#pragma unroll 1
+        for (; c < ic; c += kStep) {
+          const float4 v2 = get(src, c + 2u * kStep), g2 = gate ? get(gate, c + 2u * kStep) : zero;
+          if (gate) { v0.x *= sigmoidf_(g0.x); v0.y *= sigmoidf_(g0.y); v0.z *= sigmoidf_(g0.z); v0.w *= sigmoidf_(g0.w); }
+          acc += v0.x * v0.x + v0.y * v0.y + v0.z * v0.z + v0.w * v0.w;
+          v0 = v1; v1 = v2; g0 = g1; g1 = g2;
         }
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, d);
@@ -703,88 +769,77 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid) {
         float tot = 0.f;
 #pragma unroll
         for (int wdx = 0; wdx < kStagerWarps; ++wdx) tot += s_part[wdx];
-        rstd = rsqrtf(tot / (float)op.ic + 1e-6f);
+        rstd = rsqrtf(tot / (float)ic + 1e-6f);
         named_bar_sync(5, kStagerThreads);      // s_part is reused by the next row
       }
-      r += ng - rr % ng;                         // first item of the next row
+      r += left;                         // first item of the next row
       if (stid == 0) { s_rstd[n_rows] = rstd; s_row_end[n_rows] = r; }
       ++n_rows;
     }
     named_bar_sync(5, kStagerThreads);
-  }
-  uint64_t stat_src = 0;     // row whose statistic this half-warp computed last (rows beyond the table)
+  };
+  uint64_t stat_src = 0;     // row whose statistic this warp computed last (rows beyond the table)
   int stat_b = -1;
   float stat_rstd = 1.f;
-  for (uint32_t g0 = lo + 2u * (uint32_t)(stid >> 5); g0 < hi; g0 += 2u * (uint32_t)kStagerWarps) {
-    const uint32_t gi = g0 + (uint32_t)(lane >> 4);
+  // The planner marks the first product of a stage that has a normalised input.  In the first round, which every warp takes part in, what the items
+  // need from memory is asked for ahead of the table.
+  bool table = (stage_kind & 0x400) != 0u;
+  uint2 mu = prep.mu;
+  for (uint32_t gi = lo + (uint32_t)(stid >> 5); gi < hi || table; gi += (uint32_t)kStagerWarps) {      // a warp per item
     const bool valid = gi < hi;
-    uint32_t r = valid ? gi : lo;
-    int k = 0;
-    uint32_t icp = __ldg(&ops[0].ic_pad);
-    while (k + 1 < n_ops && r >= (uint32_t)a.B * (icp >> 7)) { r -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
-    const StepMixOp op = ops[k];
-    const uint32_t ng = op.ic_pad >> 7;
-    const int b = (int)(r / ng), grp = (int)(r % ng);
-    const int col = grp * 128 + l16 * 8;
-    StepMixX ox;
-    if (op.kind) ox = a.mixx[ev.arrd.op_first + k];
-    else { ox.src = ox.k = ox.xprev_out = ox.scale = 0; }
+    MixSlot* const slot = slots + (stid >> 5);
+    if (gi != lo + (uint32_t)(stid >> 5)) {
+      __syncwarp();
+      mu = mix_fetch(a, ev, gi, slot, mix_at + (stid >> 5), lane);
+    }
+    const StepMixOp& op = slot->op;
+    const StepMixX& ox = slot->ox;
+    const uint32_t at = mix_at[stid >> 5];
+    const int b = (int)(at & 0xFFFFu), grp = (int)(at >> 16), col = grp * 128 + lane * 4;
+    const bool in = col < (int)op.ic;
+    const size_t e0 = (size_t)b * op.ic + col;            // first of this lane's four elements
+    const bool plain = (op.kind & 0xFF) == RWKVQ_IN_BUFFER;
+    uint2 v = make_uint2(0u, 0u), pr = v;
+    XformLoads xl;
+    if (in) {
+      if (plain) v = __ldcg(reinterpret_cast<const uint2*>(reinterpret_cast<const __half*>(op.x) + e0));
+      else xform_load(op, ox, e0, xl);
+      if (op.mu) {
+        // previous token's input: read for the mix, then (where asked) replaced by this token's
+        pr = __ldcg(reinterpret_cast<const uint2*>(reinterpret_cast<const __half*>(op.xprev) + e0));
+      }
+    }
+    if (table) { row_table(); table = false; }
     float rstd = 1.f;
-    if (op.kind & 0x100) {
-      // the two half-warps of a warp hold different items: the statistic is computed by the whole warp
-      // whenever either half needs a new one
-      const bool norm = (op.kind & 0x100) != 0;
+    if (op.kind & 0x100) {      // the same for the whole warp
       const uint32_t item = valid ? gi : lo;
       int idx = 0;
       while (idx < n_rows && item >= s_row_end[idx]) ++idx;
-      const bool tabled = idx < n_rows;
-      const bool want = norm && !tabled && (stat_src != ox.src || stat_b != b);
-      if (__any_sync(0xFFFFFFFFu, want)) {
-        const float rs = row_rstd(op, ox, b, l16, want);
-        if (want) { stat_rstd = rs; stat_src = ox.src; stat_b = b; }
-      }
-      if (norm) rstd = tabled ? s_rstd[idx] : stat_rstd;
-    }
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (col < (int)op.ic) {
-      const size_t e0 = (size_t)b * op.ic + col;          // first of this lane's eight elements
-      if ((op.kind & 0xFF) == RWKVQ_IN_BUFFER) v = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const __half*>(op.x) + e0));
-      else v = xform_input(op, ox, e0, col, valid, rstd);
-      if (ox.xprev_out || op.mu) {
-        // previous token's input: read for the mix, then (where asked) replaced by this token's
-        uint4 pr = make_uint4(0u, 0u, 0u, 0u);
-        if (op.mu) pr = __ldcg(reinterpret_cast<const uint4*>(reinterpret_cast<const __half*>(op.xprev) + e0));
-        if (ox.xprev_out && valid) *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(ox.xprev_out) + e0) = v;
-        if (op.mu) {
-          const uint32_t bits = op.mu_bits, mask = (1u << bits) - 1u;
-          // four indices = 4*bits bits starting at a byte boundary (col/2 is a multiple of 4)
-          const uint32_t byte = (uint32_t)(col >> 1) * bits >> 3;
-          const uint32_t* w = reinterpret_cast<const uint32_t*>(op.mu) + (byte >> 2);
-          const uint32_t sh = (byte & 3u) * 8u;
-          const uint32_t wlo = __ldg(w);
-          const uint32_t whi = (sh + 4u * bits > 32u) ? __ldg(w + 1) : 0u;
-          const uint32_t f = __funnelshift_r(wlo, whi, sh);
-          const uint32_t* cb = reinterpret_cast<const uint32_t*>(op.mu_aux);
-          v.x = mix2(v.x, pr.x, __ldg(cb + (f & mask)));
-          v.y = mix2(v.y, pr.y, __ldg(cb + ((f >> bits) & mask)));
-          v.z = mix2(v.z, pr.z, __ldg(cb + ((f >> (2 * bits)) & mask)));
-          v.w = mix2(v.w, pr.w, __ldg(cb + ((f >> (3 * bits)) & mask)));
-        }
+      if (idx < n_rows) {
+        rstd = s_rstd[idx];
+      } else {
+        if (stat_src != ox.src || stat_b != b) { stat_rstd = row_rstd(op, ox, b, lane); stat_src = ox.src; stat_b = b; }
+        rstd = stat_rstd;
       }
     }
-    if (valid) *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(a.scratch + op.dst_x) + (size_t)b * op.ic_pad + col) = v;
-    const int o = (8 * l16) & 63;
-    const float pa = pair_sum(v.x) + pair_sum(v.z), pb = pair_sum(v.y) + pair_sum(v.w);
+    if (in) {
+      if (!plain) v = xform_input(op, ox, xl, e0, col, valid, rstd);
+      if (ox.xprev_out && valid) *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(ox.xprev_out) + e0) = v;
+      if (op.mu) { v.x = mix2(v.x, pr.x, mu.x); v.y = mix2(v.y, pr.y, mu.y); }
+    }
+    if (valid) *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(a.scratch + op.dst_x) + (size_t)b * op.ic_pad + col) = v;
+    const int o = (4 * lane) & 63;
+    const float pa = pair_sum(v.x), pb = pair_sum(v.y);
     float sx = pa + pb;
     float t0 = fmaf((float)rwkvq_sq_bias(o, 0), pa, (float)rwkvq_sq_bias(o + 2, 0) * pb);
     float t1 = fmaf((float)rwkvq_sq_bias(o, 1), pa, (float)rwkvq_sq_bias(o + 2, 1) * pb);
 #pragma unroll
-    for (int d = 8; d > 0; d >>= 1) {
+    for (int d = 16; d > 0; d >>= 1) {
       sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
       t0 += __shfl_xor_sync(0xFFFFFFFFu, t0, d);
       t1 += __shfl_xor_sync(0xFFFFFFFFu, t1, d);
     }
-    if (valid && l16 == 0 && op.sums) {
+    if (valid && lane == 0 && op.sums) {
       float* gs = reinterpret_cast<float*>(a.scratch + op.dst_sums);
       gs[(grp * 3 + 0) * nbp + b] = sx;
       gs[(grp * 3 + 1) * nbp + b] = t0;
@@ -841,6 +896,9 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         // once the barrier opens, do this CTA's share of the new stage's pre-pass and publish it
         // through the stage's second barrier
         if (ev.barrier < (uint32_t)a.n_stages) {
+          MixSlot* const slots = reinterpret_cast<MixSlot*>(mucb);      // the codebook copy of stagers that mix themselves
+          static_assert(sizeof(MixSlot) * Shape<NB>::kStagerWarps <= kMuScratch, "pre-pass slots");
+          const MixPrep prep = mix_prepare<NB>(a, ev, stid, slots, ctrl->mix_at);
           if (ok && stid < kPollLanes) {
             uint32_t it = 0;
             while ((int)(ld_acquire_gpu(a.counter + ev.barrier) - (a.target + a.wait_skew)) < 0) {
@@ -861,7 +919,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           }
           ok = named_bar_and(6, kStagerThreads, ok);   // thread 0's acquire precedes every thread's loads of x
           if (!ok) break;
-          mix_slice<NB>(a, ev, stid);
+          mix_slice<NB>(a, ev, stid, prep, slots, ctrl->mix_at);
           named_bar_sync(4, kStagerThreads);           // every thread's pre-pass stores precede thread 0's release
           if (stid == 0) red_release_gpu(a.counter + (uint32_t)a.n_stages + 1u + ev.barrier, 1u);
         }
