@@ -152,7 +152,7 @@ constexpr uint32_t kCtrlBytes = 1024, kXBufTotal = 65536, kMuScratch = 1024;
 // Input-segment buffers: two of 32 KB, one in use and one being filled.  Large segments matter more than
 // deep buffering (every hand-over of a segment costs all roles a pass through the barriers): four buffers
 // of a quarter the size, and buffers that cost the weight ring a slot or two, were measured and are slower.
-template <bool MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = kXBufTotal / kCount; };
+template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = kXBufTotal / kCount; };
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
 constexpr uint32_t kDefaultPollLimit = 1u << 22;
 
@@ -612,14 +612,67 @@ __device__ __forceinline__ uint2 mix_fetch(const StepArgs& a, const StepEvent& e
   }
   return mu;
 }
-struct MixPrep { uint2 mu; uint32_t kind; };      // of the warp's first item; of the stage's first product: what kind of stage it is
-template <int NB>
+// An item of a stage of plain inputs (no operator, no normalisation), for a quarter-warp: sixteen columns a lane, so that a CTA's share is done in
+// one round of loads.
+struct PlainItem {
+  const __half* x;          // the lane's sixteen columns
+  const __half* xprev;      // nullptr: no token shift
+  __half* dst;
+  float* sums;              // of the group, or nullptr
+  uint32_t mu[8], ic_left;  // mu_hat pairs; columns of the input from the lane's first one on (0: none)
+  int row;
+};
+__device__ __forceinline__ PlainItem plain_item(const StepArgs& a, const StepEvent& ev, uint32_t r, int l8) {
+  const StepMixOp* ops = a.mixops + ev.arrd.op_first;
+  const int n_ops = (int)ev.arrd.op_count, nbp = (a.B + 1) & ~1;
+  int k = 0;
+  uint32_t icp = __ldg(&ops[0].ic_pad);
+  while (k + 1 < n_ops && r >= (uint32_t)a.B * (icp >> 7)) { r -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
+  const StepMixOp op = load_mixop(ops + k);
+  const uint32_t ng = icp >> 7, b = r / ng, grp = r % ng, col = grp * 128u + (uint32_t)l8 * 16u;
+  const size_t e0 = (size_t)b * op.ic + col;
+  PlainItem it;
+  it.row = (int)b;
+  it.ic_left = op.ic > col ? op.ic - col : 0u;
+  it.x = reinterpret_cast<const __half*>(op.x) + e0;
+  it.xprev = op.mu ? reinterpret_cast<const __half*>(op.xprev) + e0 : nullptr;
+  it.dst = reinterpret_cast<__half*>(a.scratch + op.dst_x) + (size_t)b * op.ic_pad + col;
+  it.sums = op.sums ? reinterpret_cast<float*>(a.scratch + op.dst_sums) + (size_t)grp * 3 * nbp : nullptr;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (op.mu && it.ic_left > 8u * h) {
+      // four indices = 4*bits bits starting at a byte boundary (col/2 is a multiple of 4)
+      const uint32_t bits = op.mu_bits, mask = (1u << bits) - 1u, byte = ((col + 8u * h) >> 1) * bits >> 3, sh = (byte & 3u) * 8u;
+      const uint32_t* w = reinterpret_cast<const uint32_t*>(op.mu) + (byte >> 2);
+      const uint32_t wlo = __ldg(w);
+      const uint32_t whi = (sh + 4u * bits > 32u) ? __ldg(w + 1) : 0u;
+      const uint32_t f = __funnelshift_r(wlo, whi, sh);
+      const uint32_t* cb = reinterpret_cast<const uint32_t*>(op.mu_aux);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) it.mu[4 * h + q] = __ldg(cb + ((f >> (q * bits)) & mask));
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) it.mu[4 * h + q] = 0u;
+    }
+  }
+  return it;
+}
+struct MixPrep { PlainItem plain; uint2 mu; uint32_t kind; };      // of the warp's (lanes') first item; of the stage's first product: what kind of stage it is
+// Steps whose inputs are all plain take the whole item ahead of the barrier, steps with operators only its descriptors: with room for both in the
+// registers each spilled for the other (7B-class, batch 8: 1453 us without, 1415 with; blocks 125 and 129).
+template <int NB, bool OPS>
 __device__ __forceinline__ MixPrep mix_prepare(const StepArgs& a, const StepEvent& ev, int stid, MixSlot* slots, uint32_t* at) {
   MixPrep p;
   p.mu = make_uint2(0u, 0u);
-  p.kind = __ldg(&a.mixops[ev.arrd.op_first].kind);
+  p.kind = OPS ? (uint32_t)__ldg(&a.mixops[ev.arrd.op_first].kind) : 0x800u;
   const uint32_t lo = ev.arr.grp_lo, hi = ev.arr.grp_hi, w = (uint32_t)(stid >> 5);
-  if (lo < hi && !(p.kind & 0x800u)) p.mu = mix_fetch(a, ev, lo + w < hi ? lo + w : lo, slots + w, at + w, stid & 31);
+  if (lo >= hi) return p;
+  if constexpr (!OPS) {
+    const uint32_t gi = lo + 4u * w + (uint32_t)((stid & 31) >> 3);
+    p.plain = plain_item(a, ev, gi < hi ? gi : lo, stid & 7);
+  } else if (!(p.kind & 0x800u)) {
+    p.mu = mix_fetch(a, ev, lo + w < hi ? lo + w : lo, slots + w, at + w, stid & 31);
+  }
   return p;
 }
 
@@ -629,7 +682,7 @@ __device__ __forceinline__ MixPrep mix_prepare(const StepArgs& a, const StepEven
 // Bound by its latency: a CTA has an item or two, and all wait.  Whole blocks, d 2048, batch 2: 10.6 us a stage before, of which the
 // pre-pass took 2 to 8.5; 7.9 with descriptors in shared memory, no spills, vector loads ahead of every wait and stores behind them
 // (the recurrence read its seven arrays element by element, each behind the stores of the one before), and sigmoids without a branch.
-template <int NB>
+template <int NB, bool OPS>
 __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, const MixPrep& prep, MixSlot* slots, uint32_t* mix_at) {
   constexpr int kStagerWarps = Shape<NB>::kStagerWarps, kStagerThreads = Shape<NB>::kStagerThreads;
   const int lane = stid & 31;
@@ -648,61 +701,34 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
   int n_rows = 0;
   const uint32_t stage_kind = prep.kind;
   if (stage_kind & 0x800) {
-    // Stage of plain inputs (no operator, no normalisation): a quarter-warp per item, sixteen columns per
-    // lane, so that a CTA's share is done in one round of loads.
+    // Stage of plain inputs: a quarter-warp per item.
     const int l8 = lane & 7;
+    PlainItem it;
+    if constexpr (!OPS) it = prep.plain;
     for (uint32_t g0 = lo + 4u * (uint32_t)(stid >> 5); g0 < hi; g0 += 4u * (uint32_t)kStagerWarps) {
       const uint32_t gi = g0 + (uint32_t)(lane >> 3);
       const bool valid = gi < hi;
-      uint32_t r = valid ? gi : lo;
-      int k = 0;
-      uint32_t icp = __ldg(&ops[0].ic_pad);
-      while (k + 1 < n_ops && r >= (uint32_t)a.B * (icp >> 7)) { r -= (uint32_t)a.B * (icp >> 7); ++k; icp = __ldg(&ops[k].ic_pad); }
-      const StepMixOp op = load_mixop(ops + k);
-      const uint32_t ng = op.ic_pad >> 7;
-      const int b = (int)(r / ng), grp = (int)(r % ng);
-      const int col = grp * 128 + l8 * 16;
-      const size_t e0 = (size_t)b * op.ic + col;
-      const bool in0 = col < (int)op.ic, in1 = col + 8 < (int)op.ic;
+      if (OPS || g0 != lo + 4u * (uint32_t)(stid >> 5)) it = plain_item(a, ev, valid ? gi : lo, l8);
+      const int b = it.row;
       uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
       uint4 pr[2] = {v[0], v[0]};
-      uint32_t f[2] = {0u, 0u};
-      const __half* xs = reinterpret_cast<const __half*>(op.x) + e0;
-      if (in0) v[0] = __ldcg(reinterpret_cast<const uint4*>(xs));
-      if (in1) v[1] = __ldcg(reinterpret_cast<const uint4*>(xs + 8));
-      if (op.mu) {
-        const __half* ps = reinterpret_cast<const __half*>(op.xprev) + e0;
-        if (in0) pr[0] = __ldcg(reinterpret_cast<const uint4*>(ps));
-        if (in1) pr[1] = __ldcg(reinterpret_cast<const uint4*>(ps + 8));
-        const uint32_t bits = op.mu_bits;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h == 0 ? in0 : in1) {
-            // four indices = 4*bits bits starting at a byte boundary (col/2 is a multiple of 4)
-            const uint32_t byte = (uint32_t)((col + 8 * h) >> 1) * bits >> 3;
-            const uint32_t* w = reinterpret_cast<const uint32_t*>(op.mu) + (byte >> 2);
-            const uint32_t sh = (byte & 3u) * 8u;
-            const uint32_t wlo = __ldg(w);
-            const uint32_t whi = (sh + 4u * bits > 32u) ? __ldg(w + 1) : 0u;
-            f[h] = __funnelshift_r(wlo, whi, sh);
-          }
+      for (int h = 0; h < 2; ++h)
+        if (it.ic_left > 8u * h) {
+          v[h] = __ldcg(reinterpret_cast<const uint4*>(it.x + 8 * h));
+          if (it.xprev) pr[h] = __ldcg(reinterpret_cast<const uint4*>(it.xprev + 8 * h));
         }
-        const uint32_t mask = (1u << bits) - 1u;
-        const uint32_t* cb = reinterpret_cast<const uint32_t*>(op.mu_aux);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h == 0 ? in0 : in1) {
-            v[h].x = mix2(v[h].x, pr[h].x, __ldg(cb + (f[h] & mask)));
-            v[h].y = mix2(v[h].y, pr[h].y, __ldg(cb + ((f[h] >> bits) & mask)));
-            v[h].z = mix2(v[h].z, pr[h].z, __ldg(cb + ((f[h] >> (2 * bits)) & mask)));
-            v[h].w = mix2(v[h].w, pr[h].w, __ldg(cb + ((f[h] >> (3 * bits)) & mask)));
-          }
+      for (int h = 0; h < 2; ++h)
+        if (it.xprev && it.ic_left > 8u * h) {
+          v[h].x = mix2(v[h].x, pr[h].x, it.mu[4 * h]);
+          v[h].y = mix2(v[h].y, pr[h].y, it.mu[4 * h + 1]);
+          v[h].z = mix2(v[h].z, pr[h].z, it.mu[4 * h + 2]);
+          v[h].w = mix2(v[h].w, pr[h].w, it.mu[4 * h + 3]);
         }
-      }
       if (valid) {
-        __half* dst = reinterpret_cast<__half*>(a.scratch + op.dst_x) + (size_t)b * op.ic_pad + col;
-        *reinterpret_cast<uint4*>(dst) = v[0];
-        *reinterpret_cast<uint4*>(dst + 8) = v[1];
+        *reinterpret_cast<uint4*>(it.dst) = v[0];
+        *reinterpret_cast<uint4*>(it.dst + 8) = v[1];
       }
       // both vectors of a lane lie in one 16-column span of a triple: the same two bias values
       const int o = (16 * l8) & 63;
@@ -717,15 +743,15 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
         t0 += __shfl_xor_sync(0xFFFFFFFFu, t0, d);
         t1 += __shfl_xor_sync(0xFFFFFFFFu, t1, d);
       }
-      if (valid && l8 == 0 && op.sums) {
-        float* gs = reinterpret_cast<float*>(a.scratch + op.dst_sums);
-        gs[(grp * 3 + 0) * nbp + b] = sx;
-        gs[(grp * 3 + 1) * nbp + b] = t0;
-        gs[(grp * 3 + 2) * nbp + b] = t1;
+      if (valid && l8 == 0 && it.sums) {
+        it.sums[b] = sx;
+        it.sums[nbp + b] = t0;
+        it.sums[2 * nbp + b] = t1;
       }
     }
     return;
   }
+  if constexpr (OPS) {
   auto row_table = [&]() {
     uint32_t r = lo;
     while (r < hi && n_rows < kRowTable) {
@@ -846,6 +872,7 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
       gs[(grp * 3 + 2) * nbp + b] = t1;
     }
   }
+  }
 }
 
 // Stagers walk the CTA's event list.
@@ -858,7 +885,7 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
 //    shared memory BEFORE the stage barrier, so that only one round of vector loads of x, the
 //    mix and the sums remain behind it.  A thread owns 8 consecutive columns (16 bytes) of one
 //    batch row; a half-warp owns one 128-column group, whose three sums it reduces with shuffles.
-template <bool MIX, int NB>
+template <int MIX, int NB>
 __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_t* xbufs, uint32_t* mucb,
                             uint32_t e0, uint32_t e1) {
   constexpr int kStagerThreads = Shape<NB>::kStagerThreads;
@@ -898,7 +925,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         if (ev.barrier < (uint32_t)a.n_stages) {
           MixSlot* const slots = reinterpret_cast<MixSlot*>(mucb);      // the codebook copy of stagers that mix themselves
           static_assert(sizeof(MixSlot) * Shape<NB>::kStagerWarps <= kMuScratch, "pre-pass slots");
-          const MixPrep prep = mix_prepare<NB>(a, ev, stid, slots, ctrl->mix_at);
+          const MixPrep prep = mix_prepare<NB, MIX == 2>(a, ev, stid, slots, ctrl->mix_at);
           if (ok && stid < kPollLanes) {
             uint32_t it = 0;
             while ((int)(ld_acquire_gpu(a.counter + ev.barrier) - (a.target + a.wait_skew)) < 0) {
@@ -919,7 +946,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           }
           ok = named_bar_and(6, kStagerThreads, ok);   // thread 0's acquire precedes every thread's loads of x
           if (!ok) break;
-          mix_slice<NB>(a, ev, stid, prep, slots, ctrl->mix_at);
+          mix_slice<NB, MIX == 2>(a, ev, stid, prep, slots, ctrl->mix_at);
           named_bar_sync(4, kStagerThreads);           // every thread's pre-pass stores precede thread 0's release
           if (stid == 0) red_release_gpu(a.counter + (uint32_t)a.n_stages + 1u + ev.barrier, 1u);
         }
@@ -1127,7 +1154,7 @@ __device__ __forceinline__ void red_add_v4(float* p, const float (&v)[4]) {
 }
 
 // Consumer warp `w` of group `grp`: units grp, grp + 2, ... of the CTA's list.
-template <int NB, bool MIX>
+template <int NB, int MIX>
 __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, const uint8_t* xbufs, uint8_t* replicas,
                               uint32_t unit_base, uint32_t n_units, uint32_t ev_base, uint32_t n_events) {
   bool dead = false;
@@ -1337,7 +1364,7 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
   }
 }
 
-template <int NB, bool MIX>
+template <int NB, int MIX>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const StepArgs a) {
   constexpr int kConsumerWarps = Shape<NB>::kConsumerWarps, kStagerWarps = Shape<NB>::kStagerWarps;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -1492,8 +1519,8 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;
-  const uint32_t xbuf_bytes = XBufs<false, 1>::kBytes;
-  info->mix = mix ? 1 : 0;
+  const uint32_t xbuf_bytes = XBufs<0, 1>::kBytes;
+  info->mix = any_xform ? 2 : mix ? 1 : 0;      // the kernel's MIX
   const uint32_t nbp = (uint32_t)((B + 1) & ~1);
 
   std::vector<std::pair<int, int>> stage_ranges;  // [first op, last op) per distinct stage value
@@ -1943,7 +1970,9 @@ rwkvq_status step_run_impl(const void* plan_dev, size_t plan_bytes, void* stream
     e = cudaMemsetAsync(a.counter, 0, round_up_sz((size_t)info.n_barriers * 4, 256), s);
     if (e != cudaSuccess) return cuda_status(e);
   }
-  const void* fn = !info.mix ? (info.NB == 1 ? (const void*)step_kernel<1, false> : (const void*)step_kernel<2, false>) : info.NB == 1 ? (const void*)step_kernel<1, true> : (const void*)step_kernel<2, true>;
+  static const void* const kernels[2][3] = {{(const void*)step_kernel<1, 0>, (const void*)step_kernel<1, 1>, (const void*)step_kernel<1, 2>},
+                                            {(const void*)step_kernel<2, 0>, (const void*)step_kernel<2, 1>, (const void*)step_kernel<2, 2>}};
+  const void* fn = kernels[info.NB - 1][info.mix];
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
   if (e != cudaSuccess) return cuda_status(e);
   void* params[] = {&a};
