@@ -1512,10 +1512,11 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     i = j;
   }
   // A stage pre-pass (StepArgs::mix) costs a second barrier, about 2 us per stage whatever the sizes; without it every CTA mixes the
-  // columns it reads itself.  The line was measured with stacks of 512 to 4096 columns and batches of 2 to 16 (pre-pass / without, us): 7168 h
-  // 2048 d B=4, 1792 inputs, 232 / 176; B=8, 3584, 242 / 232; d=4096 B=3, 4608, 371 / 390; with seven stager warps d=2048 B=10, 4480, 283 /
-  // 255; B=16, 7168, 300 / 299; d=2560 B=12, 8448, 337 / 347.  The element-wise operators exist in the pre-pass only.
-  const bool mix = any_xform || share > stages * (B > 8 ? 7200u : 3600u);
+  // columns it reads itself.  The line was measured with stacks of 1024 to 4096 columns and batches of 2 to 16 (pre-pass / without, us, at
+  // `share / stages` inputs): B=6, 2688, 319 / 286 and B=3, 2688, 262 / 250; B=2, 3072, 335 / 341; B=8, 3584, 328 / 339; B=3, 4608, 338 / 370;
+  // with seven stager warps B=10, 4480, 385 / 377; B=16, 5120, 353 / 335; B=16, 7168, 406 / 443; B=12, 8448, 305 / 346.  The
+  // element-wise operators exist in the pre-pass only.
+  const bool mix = any_xform || share > stages * (B > 8 ? 5600u : 3000u);
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;

@@ -217,3 +217,25 @@ def test_step_output_rows_end_inside_a_unit(Bn):
     arr = B.make_ops([dict(desc=e["W"].desc, W=e["W"].dev, mu_desc=e["mu"].desc, mu=e["mu"].dev, x=e["xd"], xprev=e["xpd"],
                            y=bad, stage=0)])
     assert B.rwkvq_step_plan_bytes(arr, Bn) == 0
+
+
+@pytest.mark.parametrize("Bn", [5, 6, 10, 11])
+def test_step_on_both_sides_of_the_stage_pre_pass(Bn):
+    # 160 units on 148 SMs: two per CTA, 512 columns a row; 5 and 10 rows are mixed by the CTAs that read them, 6 and 11 by
+    # the pre-pass (fewer items than warps on some CTAs, a half-empty last column tile, a product without a token shift)
+    ops = []
+    for k, (fmt, oc, ic, has_mu) in enumerate([("sq", 1024, 2432, True), ("vq6", 2048, 2560, True), ("sq", 1024, 2560, False)]):
+        seed = 1000 + 10 * Bn + k
+        W = H.pack_sq(H.random_sq_codes(seed, oc, ic)) if fmt == "sq" else H.pack_vq(H.random_vq_codes(seed, oc, ic, 6), 6)
+        mu = H.pack_mu(H.random_mu_codes(seed + 3, ic, 6), 6) if has_mu else None
+        x, xp = inputs.gen_activation_pair(seed + 6, Bn, ic, n_outliers=4)
+        x16, xp16 = x.astype(np.float16), xp.astype(np.float16)
+        ops.append(dict(W=W, mu=mu, x16=x16, xp16=xp16, stage=0, xd=torch.from_numpy(x16).cuda(),
+                        xpd=torch.from_numpy(xp16).cuda() if has_mu else None,
+                        y=torch.full((Bn, oc), float("nan"), dtype=torch.float32, device="cuda")))
+    plan = _plan(ops, Bn)
+    for rep in range(2):
+        B.rwkvq_step_run(plan)
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        _check(ops, Bn)
