@@ -6,6 +6,7 @@ import re
 
 import numpy as np
 import pytest
+import torch
 
 from oracle import rwkvq_oracle as orc
 from paper_2505_03803_b200 import binding as B
@@ -282,3 +283,20 @@ def test_tau_largest_gap_separates_two_clusters():
     assert tau == 0.5 * (lo.max() + hi.min())
     with pytest.raises(B.RwkvqError):
         B.rwkvq_tau_largest_gap([1.0, float("nan")])
+
+
+class _NoStream:
+    cuda_stream = 0
+
+
+@pytest.mark.parametrize("missing,status", [("W", 1), ("x", 1), ("y", 1), ("workspace", 5)])
+def test_product_refuses_a_missing_tensor(missing, status):
+    """A tensor that is None reaches the library as a null pointer, which it refuses on the host (EINVAL; ENOMEM for the
+    workspace), before anything is enqueued."""
+    d = B.rwkvq_desc_for(128, 256, B.RWKVQ_SQ, 3)
+    t = dict(W=torch.zeros(int(d.image_bytes) + 16, dtype=torch.uint8), x=torch.zeros((1, 256), dtype=torch.float16),
+             y=torch.zeros((1, 128)), workspace=torch.zeros(4096, dtype=torch.uint8))
+    t[missing] = None
+    with pytest.raises(B.RwkvqError) as e:
+        B.rwkvq_gemv(d, t["W"], None, None, t["x"], None, 1, t["y"], t["workspace"], stream=_NoStream())
+    assert e.value.status == status
