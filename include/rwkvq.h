@@ -319,6 +319,12 @@ rwkvq_status rwkvq_step_plan_release(const void* plan_dev);
  */
 rwkvq_status rwkvq_step_set_wait(const void* plan_dev, uint32_t poll_limit, uint32_t wait_skew);
 /*
+ * out_dev[i] = 1 / y_dev[i] as the step's sigmoids take it (y = 1 + e^{-x}, so 1 <= y <= infinity; other arguments are outside its domain):
+ * equal to the correctly rounded fp32 division.  Exists so that a test can compare the two.  n at most 2^31; asynchronous on `stream`.
+ * Errors: EINVAL, EUNSUPPORTED, ECUDA.
+ */
+rwkvq_status rwkvq_step_reciprocal(const float* y_dev, float* out_dev, size_t n, void* stream);
+/*
  * Host-only check of the schedule rwkvq_step_plan would build for n_ctas CTAs (no device is
  * touched; device pointers are only stored): counts_host[n_counts] receives, product after product,
  * for every 16-row slice and every 256-column tile [oc/16][ic_pad/256] how many times the schedule

@@ -74,7 +74,7 @@ EXPORTS = [
     "rwkvq_pack", "rwkvq_blob_desc", "rwkvq_blob_nbytes", "rwkvq_blob_image", "rwkvq_blob_export_codes",
     "rwkvq_image_unpack", "rwkvq_blob_free", "rwkvq_proxy_workspace_bytes", "rwkvq_proxy_select",
     "rwkvq_gemv_workspace_bytes", "rwkvq_gemv", "rwkvq_gemv_static", "rwkvq_gemv_static_max_scratch_bytes", "rwkvq_step_plan_bytes", "rwkvq_step_plan", "rwkvq_step_run",
-    "rwkvq_step_run_host", "rwkvq_step_plan_release", "rwkvq_step_set_wait", "rwkvq_step_plan_cover",
+    "rwkvq_step_run_host", "rwkvq_step_plan_release", "rwkvq_step_set_wait", "rwkvq_step_reciprocal", "rwkvq_step_plan_cover",
     "rwkvq_prefill_workspace_bytes", "rwkvq_gemm_prefill", "rwkvq_gemm_prefill_grouped", "rwkvq_dequant", "rwkvq_device_status",
     "rwkvq_status_str", "rwkvq_last_cuda_error",
     "rwkvq_proxy_family", "rwkvq_proxy_select_bf16", "rwkvq_proxy_f32_workspace_bytes", "rwkvq_proxy_select_f32",
@@ -148,6 +148,7 @@ def lib() -> C.CDLL:
         L.rwkvq_step_run_host.argtypes = [vp, sz, vp, vp, sz, vp, vp, sz, vp]
         L.rwkvq_step_plan_release.argtypes = [vp]
         L.rwkvq_step_set_wait.argtypes = [vp, C.c_uint32, C.c_uint32]
+        L.rwkvq_step_reciprocal.argtypes = [vp, vp, sz, vp]
         L.rwkvq_step_plan_cover.argtypes = [C.POINTER(GemvOp), i32, i32, i32, C.POINTER(C.c_uint32), sz, C.POINTER(C.c_uint32)]
     if hasattr(L, "rwkvq_gemm_prefill"):
         L.rwkvq_prefill_workspace_bytes.argtypes = [C.POINTER(Desc), i32, i32]
@@ -501,6 +502,11 @@ def rwkvq_step_plan_release(plan):
 
 def rwkvq_step_set_wait(plan, poll_limit: int = 0, wait_skew: int = 0):
     _check(lib().rwkvq_step_set_wait(_dev_ptr(plan), poll_limit, wait_skew), "rwkvq_step_set_wait")
+
+
+def rwkvq_step_reciprocal(y, out, stream=None):
+    """rwkvq_step_reciprocal: out = 1 / y (float32 CUDA tensors, 1 <= y <= infinity) as the step's sigmoids take it."""
+    _check(lib().rwkvq_step_reciprocal(_dev_ptr(y), _dev_ptr(out), y.numel(), _stream_ptr(stream)), "rwkvq_step_reciprocal")
 
 
 def rwkvq_step_plan_cover(ops, B: int, n_ctas: int):

@@ -414,12 +414,16 @@ __device__ __forceinline__ float pair_sum(uint32_t r) {
 
 constexpr int kStageUnroll = 4;
 
-// 1 / y for y >= 1 by Newton's correction of the approximate reciprocal with fused multiply-adds (Markstein, "Computation of elementary functions
-// on the IBM RISC System/6000 processor", 1990).  Without the general division's branch four sigmoids run side by side (200 cycles instead of 800).
+// 1 / y for 1 <= y <= infinity, to the bit of the correctly rounded division (compared for every such y): Newton's correction of the
+// approximate reciprocal with fused multiply-adds (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990).
+// Where 1 / y is subnormal (y > 2^126) the approximation has fewer bits, and the series' second term is needed: without it five results
+// of that range are off by one in the last place.  Without the general division's branch four sigmoids run side by side: 147 cycles
+// instead of 367.
 __device__ __forceinline__ float rcp_of(float y) {
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(y));
-  return y < 1e37f ? fmaf(r, fmaf(-y, r, 1.f), r) : r;
+  const float e = fmaf(-y, r, 1.f), f = fmaf(r, fmaf(e, e, e), r);
+  return y < INFINITY ? f : r;
 }
 __device__ __forceinline__ float sigmoidf_(float x) { return rcp_of(1.f + expf(-x)); }
 __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
@@ -1364,6 +1368,12 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
   }
 }
 
+// rcp_of by itself (rwkvq_step_reciprocal).
+__global__ void __launch_bounds__(256) reciprocal_kernel(const float* y, float* out, size_t n) {
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < n) out[i] = rcp_of(y[i]);
+}
+
 template <int NB, int MIX>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const StepArgs a) {
   constexpr int kConsumerWarps = Shape<NB>::kConsumerWarps, kStagerWarps = Shape<NB>::kStagerWarps;
@@ -2012,6 +2022,13 @@ rwkvq_status rwkvq_step_set_wait(const void* plan_dev, uint32_t poll_limit, uint
   it->second.poll_limit = poll_limit ? poll_limit : kDefaultPollLimit;
   it->second.wait_skew = wait_skew;
   return RWKVQ_OK;
+}
+
+rwkvq_status rwkvq_step_reciprocal(const float* y_dev, float* out_dev, size_t n, void* stream) {
+  if (!y_dev || !out_dev || n == 0) return RWKVQ_EINVAL;
+  if (n > (size_t)1 << 31) return RWKVQ_EUNSUPPORTED;
+  reciprocal_kernel<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(y_dev, out_dev, n);
+  return cuda_status(cudaGetLastError());
 }
 
 rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, int n_ctas, uint32_t* counts_host,

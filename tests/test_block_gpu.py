@@ -199,3 +199,21 @@ def test_chained_blocks_at_7b_width_sampled(batch):
     _check_product("block 0 cm_k", type("M", (), {"w_hat": w_hat}), orc.token_shift(x_c, prev_ck0, mu_hat), by[(0, "cm_k")].y)
     w_hat, _ = _decode(st, by[(1, "cm_v")])
     _check_product("block 1 cm_v", type("M", (), {"w_hat": w_hat}), _f16(orc.relu_squared(y[(1, "cm_k")])), by[(1, "cm_v")].y)
+
+
+@pytest.mark.parametrize("exponents", [(0,), (1, 23, 24, 60), (99, 122, 123, 124, 125), (126,), (127,)])
+def test_reciprocal_of_the_sigmoids_is_the_rounded_division(exponents):
+    """The sigmoids' reciprocal against numpy's fp32 division, which IEEE rounds correctly: the same bits for every significand of
+    the binades [2^e, 2^(e+1)), among them those whose reciprocal is subnormal (from 2^126 on), and at infinity."""
+    frac = torch.arange(1 << 23, dtype=torch.int32, device="cuda")
+    for e in exponents:
+        y = (frac | ((e + 127) << 23)).view(torch.float32)
+        out = torch.empty_like(y)
+        B.rwkvq_step_reciprocal(y, out)
+        want = np.float32(1.0) / y.cpu().numpy()
+        assert np.array_equal(out.cpu().numpy().view(np.uint32), want.view(np.uint32)), e
+    ends = torch.tensor([1.0, float("inf"), float("nan"), 3.4028234e38, 2.0 ** 126, 1e37], device="cuda")
+    out = torch.empty_like(ends)
+    B.rwkvq_step_reciprocal(ends, out)
+    got = out.cpu().numpy()
+    assert got[1] == 0.0 and np.isnan(got[2]) and np.array_equal(got[[0, 3, 4, 5]], np.float32(1.0) / ends.cpu().numpy()[[0, 3, 4, 5]])
