@@ -1,4 +1,5 @@
 // Device status word and CUDA error text.
+#include <cuda.h>           // types of the driver's calls (no driver symbol is linked)
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -19,15 +20,20 @@ void set_last_cuda_error(cudaError_t e) {
 // Device address of the status word for the current device (kernels in other translation units
 // receive it as an argument).
 int* device_status_ptr() {
-  static std::atomic<int*> known[kMaxDevices];
-  const int dev = current_device();
-  int* p = dev >= 0 ? known[dev].load(std::memory_order_relaxed) : nullptr;
-  if (p) return p;
-  void* q = nullptr;
-  if (cudaGetSymbolAddress(&q, g_device_status) != cudaSuccess) return nullptr;
-  p = static_cast<int*>(q);
-  if (dev >= 0) known[dev].store(p, std::memory_order_relaxed);
-  return p;
+  static SymbolAddress address;
+  void* p = nullptr;
+  return address((const void*)&g_device_status, &p) == cudaSuccess ? static_cast<int*>(p) : nullptr;
+}
+unsigned long long context_id() {
+  typedef CUresult (*GetIdFn)(CUcontext, unsigned long long*);
+  static const GetIdFn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &f, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) f = nullptr;
+    return reinterpret_cast<GetIdFn>(f);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0ull;
 }
 int current_device() {
   int dev = 0;

@@ -5,7 +5,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "../../include/rwkvq.h"
 #include "gemv_core.cuh"
@@ -394,14 +393,11 @@ rwkvq_status rwkvq_gemv(const rwkvq_desc* d, const void* W, const rwkvq_desc* mu
 // ---------------------------------------------------------------------------------------------
 // rwkvq_gemv for callers that cannot allocate device memory: the split-K scratch lives in a
 // file-scope device array.  In host code the array's name is only a handle; its device address
-// is looked up once per device (with that device current) and cached.
+// is looked up once per device and context (with that device current).
 // ---------------------------------------------------------------------------------------------
 #define RWKVQ_STATIC_SCRATCH_BYTES (8u << 20)
 static __device__ __align__(256) unsigned char g_static_scratch[RWKVQ_STATIC_SCRATCH_BYTES];
-// One entry per device ordinal, written once; atomic because any host thread may make the first
-// call.  The address stays valid for the life of the device's primary context: after
-// cudaDeviceReset the library has to be loaded afresh (as every other device allocation).
-static std::atomic<void*> g_static_scratch_addr[64];
+static SymbolAddress g_static_scratch_address;
 
 size_t rwkvq_gemv_static_max_scratch_bytes(void) { return RWKVQ_STATIC_SCRATCH_BYTES; }
 
@@ -415,13 +411,10 @@ rwkvq_status rwkvq_gemv_static(const rwkvq_desc* d, const void* W, const rwkvq_d
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_status(e);
-  if (dev < 0 || dev >= 64) return RWKVQ_EUNSUPPORTED;
-  void* ws = g_static_scratch_addr[dev].load(std::memory_order_acquire);
-  if (!ws) {
-    e = cudaGetSymbolAddress(&ws, g_static_scratch);
-    if (e != cudaSuccess) return cuda_status(e);
-    g_static_scratch_addr[dev].store(ws, std::memory_order_release);
-  }
+  if (dev < 0 || dev >= kMaxDevices) return RWKVQ_EUNSUPPORTED;
+  void* ws = nullptr;
+  e = g_static_scratch_address((const void*)g_static_scratch, &ws);
+  if (e != cudaSuccess) return cuda_status(e);
   // The array keeps whatever the previous call left: the arrival counters must start at zero.
   if (p.S > 1 && !p.cluster) {
     e = cudaMemsetAsync(ws, 0, p.counters_bytes, static_cast<cudaStream_t>(stream));

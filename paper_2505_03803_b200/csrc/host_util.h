@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "../../include/rwkvq.h"
 #include "format.h"
@@ -55,15 +56,36 @@ int current_device();
 // Multiprocessors of the current device (148 where it cannot be asked); looked up once per device.
 int sm_count();
 
-// The opt-in to more than 48 KB of dynamic shared memory holds for a kernel and a device until the process ends: it is
-// asked for once (about 1 us of host time) and not at every launch.  One object per kernel, `bytes` the same at every call.
+// Number of the calling thread's context; 0 where it has none yet or the driver cannot be asked.  What is set or looked up in a context ends with
+// it (cudaDeviceReset), and the device's next context has another number: whatever is kept between calls is kept with this number beside it.
+unsigned long long context_id();
+
+// The opt-in to more than 48 KB of dynamic shared memory holds for a kernel as long as the context: it is asked for once (about 1 us of host
+// time) and not at every launch.  One object per kernel, `bytes` the same at every call.
 struct SmemOptIn {
-  std::atomic<bool> done[kMaxDevices];
+  std::atomic<unsigned long long> context[kMaxDevices];      // in which it was asked for
   cudaError_t operator()(const void* fn, int bytes) {
     const int dev = current_device();
-    if (dev >= 0 && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    const unsigned long long id = dev >= 0 ? context_id() : 0ull;
+    if (id != 0 && context[dev].load(std::memory_order_relaxed) == id) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && dev >= 0) done[dev].store(true, std::memory_order_relaxed);
+    if (e == cudaSuccess && id != 0) context[dev].store(id, std::memory_order_relaxed);
+    return e;
+  }
+};
+
+// Device address of a __device__ variable, looked up once per device and context.  One object per variable.
+struct SymbolAddress {
+  std::mutex mutex;
+  void* at[kMaxDevices];
+  unsigned long long context[kMaxDevices];
+  cudaError_t operator()(const void* symbol, void** out) {
+    const int dev = current_device();
+    const unsigned long long id = dev >= 0 ? context_id() : 0ull;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (id != 0 && context[dev] == id) { *out = at[dev]; return cudaSuccess; }
+    const cudaError_t e = cudaGetSymbolAddress(out, symbol);
+    if (e == cudaSuccess && id != 0) { at[dev] = *out; context[dev] = id; }
     return e;
   }
 };

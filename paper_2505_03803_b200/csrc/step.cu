@@ -2083,8 +2083,8 @@ rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, i
 }  // extern "C"
 
 namespace {
-// Streams, events and the arrival word of host-buffer runs, one set per device.  The stream memory
-// operations come from the driver through the runtime's entry-point query (no link to the driver library).
+// Streams, events and the arrival word of host-buffer runs, one set per context (context_id; what cudaDeviceReset ended
+// leaves an empty entry behind).  The stream memory operations come from the driver through the runtime's entry-point query (no link to the driver library).
 typedef CUresult (*StreamValueFn)(CUstream, CUdeviceptr, cuuint32_t, unsigned int);
 struct HostPipe {
   bool tried = false, ok = false;
@@ -2095,7 +2095,7 @@ struct HostPipe {
   StreamValueFn wait_value = nullptr, write_value = nullptr;
 };
 std::mutex g_pipe_mutex;
-std::unordered_map<int, HostPipe> g_pipes;
+std::unordered_map<unsigned long long, HostPipe> g_pipes;
 // Activations arrive in pieces of 256 KB, then twice as much each time up to 4 MB: the step begins behind the first piece (5 us instead of 80)
 // and most of the bytes go in copies long enough for the link's rate.  Outputs leave in groups of whole stages of at least a quarter
 // of what is still to come, 2 MB at most, so that little is left to copy when the step ends.  22 MB in, 44 MB out, 32 layers: 1665 us,
@@ -2109,7 +2109,9 @@ constexpr size_t kOverlapMinBytes = (size_t)512 << 10;
 HostPipe* host_pipe() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  HostPipe& hp = g_pipes[dev];
+  unsigned long long id = context_id();
+  if (id == 0 && cudaFree(nullptr) == cudaSuccess) id = context_id();      // a thread's first call
+  HostPipe& hp = g_pipes[id != 0 ? id : ~(unsigned long long)dev];
   if (hp.tried) return hp.ok ? &hp : nullptr;
   hp.tried = true;
   cudaDriverEntryPointQueryResult q1, q2;
