@@ -1919,16 +1919,11 @@ rwkvq_status rwkvq_step_plan(const rwkvq_gemv_op* ops, int n_ops, int B, void* p
 }  // extern "C"
 
 namespace {
-// Inputs that arrive while the step runs (see StepArgs::in_flag), and what the caller needs back to
-// order its output copies behind the stage barriers.
+// Inputs that arrive while the step runs (see StepArgs::in_flag).
 struct HostRun {
   const unsigned* in_flag = nullptr;
   unsigned in_base = 0, in_shift = 0;
   uint64_t in_lo = 0, in_hi = 0;
-  // out
-  unsigned* counter = nullptr;
-  unsigned target = 0;
-  PlanInfo info;
 };
 
 // Every arrival counter that is short of `target` (a run that gave up) is raised to it, so that
@@ -1938,9 +1933,22 @@ __global__ void step_finish_kernel(unsigned* counter, int n, unsigned target) {
   if (k < n && (int)(counter[k] - target) < 0) counter[k] = target;
 }
 
-rwkvq_status step_run_impl(const void* plan_dev, size_t plan_bytes, void* stream, HostRun* hr) {
+unsigned* counters_of(const void* plan_dev, const PlanInfo& info) {
+  return reinterpret_cast<unsigned*>(static_cast<uint8_t*>(const_cast<void*>(plan_dev)) + info.off_counter);
+}
+unsigned target_of(const PlanInfo& info) { return info.runs * (unsigned)info.P; }
+
+// A run that was counted but will never arrive: have the next one clear the counters.
+void forget_run(const void* plan_dev) {
+  std::lock_guard<std::mutex> lock(g_plan_mutex);
+  auto it = g_plans.find(plan_dev);
+  if (it != g_plans.end()) it->second.abort_epoch = abort_epoch() - 1u;
+}
+
+// Counts one more run of the plan and, where it is due, clears the arrival counters on the caller's stream.  Whatever waits for the counters of
+// this run on another stream is ordered behind this call.
+rwkvq_status begin_run(const void* plan_dev, size_t plan_bytes, cudaStream_t s, PlanInfo* info) {
   if (!plan_dev) return RWKVQ_EINVAL;
-  PlanInfo info;
   bool clear_counters = false;
   {
     std::lock_guard<std::mutex> lock(g_plan_mutex);
@@ -1952,49 +1960,43 @@ rwkvq_status step_run_impl(const void* plan_dev, size_t plan_bytes, void* stream
     const unsigned epoch = abort_epoch();
     if (it->second.abort_epoch != epoch) { it->second.abort_epoch = epoch; it->second.runs = 0; clear_counters = true; }
     it->second.runs += 1;
-    info = it->second;
+    *info = it->second;
   }
+  if (clear_counters) {
+    const cudaError_t e = cudaMemsetAsync(counters_of(plan_dev, *info), 0, round_up_sz((size_t)info->n_barriers * 4, 256), s);
+    if (e != cudaSuccess) { forget_run(plan_dev); return cuda_status(e); }
+  }
+  return RWKVQ_OK;
+}
+
+rwkvq_status launch_run(const void* plan_dev, const PlanInfo& info, cudaStream_t s, const HostRun* hr) {
   const uint8_t* p = static_cast<const uint8_t*>(plan_dev);
   StepArgs a;
   a.units = reinterpret_cast<const StepUnit*>(p + info.off_units);
   a.events = reinterpret_cast<const StepEvent*>(p + info.off_events);
   a.unit_off = reinterpret_cast<const uint32_t*>(p + info.off_unit_off);
   a.event_off = reinterpret_cast<const uint32_t*>(p + info.off_event_off);
-  a.counter = reinterpret_cast<unsigned*>(const_cast<uint8_t*>(p) + info.off_counter);
+  a.counter = counters_of(plan_dev, info);
   a.status = device_status_ptr();
-  if (!a.status) return RWKVQ_ECUDA;
+  if (!a.status) { forget_run(plan_dev); return RWKVQ_ECUDA; }
   a.B = info.B; a.n_slots = info.n_slots; a.n_stages = info.n_stages;
   a.mix = info.mix; a.mixops = reinterpret_cast<const StepMixOp*>(p + info.off_mixops);
   a.mixx = reinterpret_cast<const StepMixX*>(p + info.off_mixx);
   a.scratch = const_cast<uint8_t*>(p) + info.off_scratch;
   a.slot_bytes = info.slot_bytes; a.replica_bytes = info.replica_bytes;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  a.target = info.runs * (unsigned)info.P;
+  a.target = target_of(info);
   a.poll_limit = info.poll_limit; a.wait_skew = info.wait_skew;
   a.in_flag = nullptr; a.in_base = 0; a.in_shift = 0; a.in_lo = 0; a.in_hi = 0;
-  if (hr) {
-    a.in_flag = hr->in_flag; a.in_base = hr->in_base; a.in_shift = hr->in_shift; a.in_lo = hr->in_lo; a.in_hi = hr->in_hi;
-    hr->counter = a.counter; hr->target = a.target; hr->info = info;
-  }
-  cudaError_t e = cudaSuccess;
-  if (clear_counters) {
-    e = cudaMemsetAsync(a.counter, 0, round_up_sz((size_t)info.n_barriers * 4, 256), s);
-    if (e != cudaSuccess) return cuda_status(e);
-  }
+  if (hr) { a.in_flag = hr->in_flag; a.in_base = hr->in_base; a.in_shift = hr->in_shift; a.in_lo = hr->in_lo; a.in_hi = hr->in_hi; }
   static const void* const kernels[2][3] = {{(const void*)step_kernel<1, 0>, (const void*)step_kernel<1, 1>, (const void*)step_kernel<1, 2>},
                                             {(const void*)step_kernel<2, 0>, (const void*)step_kernel<2, 1>, (const void*)step_kernel<2, 2>}};
   const void* fn = kernels[info.NB - 1][info.mix];
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
-  if (e != cudaSuccess) return cuda_status(e);
   void* params[] = {&a};
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
   // Cooperative launch: all CTAs must be resident at once because they meet at the stage barrier.
-  e = cudaLaunchCooperativeKernel(fn, dim3(info.P), dim3(threads_of(info.NB)), params, info.smem_bytes, s);
-  if (e != cudaSuccess) {   // this run will never arrive: have the next one clear the counters
-    std::lock_guard<std::mutex> lock(g_plan_mutex);
-    auto it = g_plans.find(plan_dev);
-    if (it != g_plans.end()) it->second.abort_epoch = abort_epoch() - 1u;
-  }
-  if (e == cudaSuccess && hr) {
+  if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(info.P), dim3(threads_of(info.NB)), params, info.smem_bytes, s);
+  if (e != cudaSuccess) { forget_run(plan_dev); return cuda_status(e); }
+  if (hr) {
     step_finish_kernel<<<(info.n_barriers + 255u) / 256u, 256, 0, s>>>(a.counter, (int)info.n_barriers, a.target);
     e = cudaGetLastError();
   }
@@ -2005,7 +2007,9 @@ rwkvq_status step_run_impl(const void* plan_dev, size_t plan_bytes, void* stream
 extern "C" {
 
 rwkvq_status rwkvq_step_run(const void* plan_dev, size_t plan_bytes, void* stream) {
-  return step_run_impl(plan_dev, plan_bytes, stream, nullptr);
+  PlanInfo info;
+  const rwkvq_status st = begin_run(plan_dev, plan_bytes, static_cast<cudaStream_t>(stream), &info);
+  return st != RWKVQ_OK ? st : launch_run(plan_dev, info, static_cast<cudaStream_t>(stream), nullptr);
 }
 
 rwkvq_status rwkvq_step_plan_release(const void* plan_dev) {
@@ -2165,11 +2169,15 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
   HostPipe* hp = host_pipe();
   if (!hp) return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // Both side streams start behind everything already enqueued on the caller's stream.
+  PlanInfo info;
+  rwkvq_status st = begin_run(plan_dev, plan_bytes, s, &info);
+  if (st != RWKVQ_OK) return st;
+  // Both side streams start behind everything already enqueued on the caller's stream, the clearing of the counters among it: the output
+  // copies wait for this run's arrivals, which the counters of earlier runs would seem to be.
   cudaError_t e = cudaEventRecord(hp->start, s);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(hp->h2d, hp->start, 0);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(hp->d2h, hp->start, 0);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) { forget_run(plan_dev); return cuda_status(e); }
   // Activations: chunk by chunk on the copy stream; the word counts the chunks that have arrived.
   // They are enqueued BEFORE the launch: streams share a limited number of hardware queues, and a copy
   // enqueued behind the running step in the same queue would start only when the step, which waits for it, ends.
@@ -2189,15 +2197,16 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
     // Whatever happened, the word reaches its final value, so that no stager waits for a chunk in vain.
     if (e != cudaSuccess) hp->write_value(hp->h2d, (CUdeviceptr)(uintptr_t)hp->flag, hp->chunks + n_in, 0u);
     hp->chunks += n_in;
-    if (e != cudaSuccess) { cudaStreamSynchronize(hp->h2d); return cuda_status(e); }
+    if (e != cudaSuccess) { forget_run(plan_dev); cudaStreamSynchronize(hp->h2d); return cuda_status(e); }
   }
   // The step itself, on the caller's stream, at once: its stagers wait for the chunks they read.
-  rwkvq_status st = step_run_impl(plan_dev, plan_bytes, stream, &hr);
+  st = launch_run(plan_dev, info, s, &hr);
   if (st != RWKVQ_OK) { cudaStreamSynchronize(hp->h2d); return st; }
   // Outputs: stage by stage behind the stage barriers (the arrival counters of the plan), in groups of
   // whole stages, as long as the stages' outputs lie one behind the other in [y_dev, y_dev + y_bytes).
   if (y_bytes) {
-    const PlanInfo& info = hr.info;
+    unsigned* counter = counters_of(plan_dev, info);
+    const unsigned target = target_of(info);
     const uint64_t y0 = (uint64_t)(uintptr_t)y_dev, y1 = y0 + y_bytes;
     bool ordered = !info.y_lo.empty();
     uint64_t prev = y0;
@@ -2213,7 +2222,7 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
       if (!last && upto - done < std::min(kOutGroupBytes, std::max(kMinOutGroupBytes, (y_bytes - done) / 4))) continue;
       if (upto == done) continue;
       // barrier k + 1 closes stage k: every CTA has arrived behind its reductions into these outputs
-      if (hp->wait_value(hp->d2h, (CUdeviceptr)(uintptr_t)(hr.counter + (k + 1)), hr.target, CU_STREAM_WAIT_VALUE_GEQ) != CUDA_SUCCESS) { e = cudaErrorUnknown; break; }
+      if (hp->wait_value(hp->d2h, (CUdeviceptr)(uintptr_t)(counter + (k + 1)), target, CU_STREAM_WAIT_VALUE_GEQ) != CUDA_SUCCESS) { e = cudaErrorUnknown; break; }
       e = cudaMemcpyAsync(static_cast<uint8_t*>(y_host) + done, static_cast<const uint8_t*>(y_dev) + done, upto - done, cudaMemcpyDeviceToHost, hp->d2h);
       done = upto;
     }

@@ -239,3 +239,78 @@ def test_step_on_both_sides_of_the_stage_pre_pass(Bn):
         torch.cuda.synchronize()
         assert B.rwkvq_device_status() == 0
         _check(ops, Bn)
+
+
+class _HostArena:
+    """The products' activations and outputs in one buffer each on the device and in page-locked memory, `gap` bytes apart."""
+
+    def __init__(self, ops, Bn, gap):
+        self.ops, self.Bn, self.slots, act, y = ops, Bn, [], 0, 0
+        up = lambda n: (n + 255) // 256 * 256 + gap
+        for e in ops:
+            xo, po, yo = act, None, y
+            act += up(e["x16"].nbytes)
+            if e["mu"] is not None:
+                po = act
+                act += up(e["xp16"].nbytes)
+            y += up(4 * Bn * e["W"].oc)
+            self.slots.append((xo, po, yo))
+        self.act_host, self.y_host = (torch.zeros(n, dtype=torch.uint8).pin_memory() for n in (act, y))
+        self.act_dev = torch.zeros(act, dtype=torch.uint8, device="cuda")
+        self.y_dev = torch.full((y // 4,), float("nan"), dtype=torch.float32, device="cuda").view(torch.uint8)
+        for e, (xo, po, yo) in zip(ops, self.slots):
+            e["xd"] = self.act_dev[xo:xo + e["x16"].nbytes].view(torch.float16).view(Bn, -1)
+            if po is not None:
+                e["xpd"] = self.act_dev[po:po + e["xp16"].nbytes].view(torch.float16).view(Bn, -1)
+            e["y"] = self.y_dev[yo:yo + 4 * Bn * e["W"].oc].view(torch.float32).view(Bn, -1)
+        self.fill(0)
+
+    def fill(self, seed):
+        """New activations in host memory; the outputs there are cleared."""
+        an = self.act_host.numpy()
+        for k, (e, (xo, po, _)) in enumerate(zip(self.ops, self.slots)):
+            if seed:
+                x, xp = inputs.gen_activation_pair(7000 + 100 * seed + k, self.Bn, e["W"].ic, n_outliers=4)
+                e["x16"], e["xp16"] = x.astype(np.float16), xp.astype(np.float16)
+            an[xo:xo + e["x16"].nbytes] = e["x16"].reshape(-1).view(np.uint8)
+            if po is not None:
+                an[po:po + e["xp16"].nbytes] = e["xp16"].reshape(-1).view(np.uint8)
+        self.y_host.fill_(0xFF)
+
+    def run(self, plan):
+        B.rwkvq_step_run_host(plan, self.act_host, self.act_dev, self.y_dev, self.y_host)
+
+    def check(self):
+        yn = self.y_host.numpy()
+        for e, (_, _, yo) in zip(self.ops, self.slots):
+            y = yn[yo:yo + 4 * self.Bn * e["W"].oc].view(np.float32).reshape(self.Bn, -1).astype(np.float64)
+            ref, tol = H.reference(e["W"], e["mu"], e["x16"], e["xp16"])
+            assert np.isfinite(y).all() and (np.abs(y - ref) <= tol).all(), f"stage {e['stage']}"
+
+
+@pytest.mark.parametrize("Bn", [4, 16])
+def test_step_run_host_delivers_new_outputs_after_a_failed_wait(Bn):
+    """A failed wait (here: another plan's) makes the next run of every plan clear its barrier counters, which hold many runs'
+    arrivals.  The output copies wait for the arrivals of their own run, not for those: with new activations the host receives
+    new outputs."""
+    ops = _build_ops(512, 1280, 2, Bn, 6, seed=700 + Bn)
+    arena = _HostArena(ops, Bn, 3 << 20)
+    plan = _plan(ops, Bn)
+    for _ in range(3):
+        arena.run(plan)
+    torch.cuda.synchronize()
+    arena.check()
+    other = _build_ops(256, 512, 1, 1, 6, seed=60)
+    failing = _plan(other, 1)
+    for seed in (1, 2):
+        B.rwkvq_step_set_wait(failing, poll_limit=2000, wait_skew=1)
+        B.rwkvq_step_run(failing)
+        assert B.rwkvq_device_status() == 8
+        arena.fill(seed)
+        arena.run(plan)
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        arena.check()
+        arena.run(plan)
+        torch.cuda.synchronize()
+        arena.check()
