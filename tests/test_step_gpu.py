@@ -314,3 +314,19 @@ def test_step_run_host_delivers_new_outputs_after_a_failed_wait(Bn):
         arena.run(plan)
         torch.cuda.synchronize()
         arena.check()
+
+
+@pytest.mark.parametrize("Bn,gap", [(1, 24 << 10), (4, 24 << 10), (8, 50 << 10), (16, 0), (16, 100 << 10)])
+def test_step_run_host_with_copies_of_half_a_megabyte_to_eight(Bn, gap):
+    """Sizes from where the copies are overlapped on: first pieces of 256 KB and output groups of 128 KB, a few of each."""
+    ops = _build_ops(512, 1280, 3, Bn, 6, seed=800 + Bn + gap)
+    arena = _HostArena(ops, Bn, gap)
+    total = arena.act_host.numel() + arena.y_host.numel()
+    assert (512 << 10) <= total < (9 << 20)
+    plan = _plan(ops, Bn)
+    for seed in (0, 1, 2):
+        arena.fill(seed)
+        arena.run(plan)
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        arena.check()
