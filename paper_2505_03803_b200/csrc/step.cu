@@ -2097,6 +2097,8 @@ struct HostPipe {
   unsigned* flag = nullptr;      // device word: chunks arrived so far, over all runs
   unsigned chunks = 0;           // the host's copy of its final value after the last run enqueued
   StreamValueFn wait_value = nullptr, write_value = nullptr;
+  bool used = false;             // the last run came on the stream of number `user`
+  unsigned long long user = 0;
 };
 std::mutex g_pipe_mutex;
 std::unordered_map<unsigned long long, HostPipe> g_pipes;
@@ -2139,6 +2141,20 @@ HostPipe* host_pipe() {
   return &hp;
 }
 
+// Whether a run on stream s may take the copy streams: its copies must not lie behind those of another stream's run, which wait for that stream's
+// work, while its step already occupies every SM and waits for them.  Behind a run on the same stream they do not wait longer than the step.
+bool pipe_free(HostPipe& hp, cudaStream_t s) {
+  unsigned long long id = 0;
+  const bool known = cudaStreamGetId(s, &id) == cudaSuccess;
+  if (hp.used && !(known && id == hp.user)) {
+    const bool idle = cudaStreamQuery(hp.h2d) == cudaSuccess && cudaStreamQuery(hp.d2h) == cudaSuccess;
+    if (!idle) { cudaGetLastError(); return false; }
+  }
+  hp.used = true;
+  hp.user = known ? id : ~0ull;
+  return true;
+}
+
 rwkvq_status run_host_plain(const void* plan_dev, size_t plan_bytes, const void* act_host, void* act_dev, size_t act_bytes,
                             const void* y_dev, void* y_host, size_t y_bytes, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -2167,8 +2183,8 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
     return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   HostPipe* hp = host_pipe();
-  if (!hp) return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (!hp || !pipe_free(*hp, s)) return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   PlanInfo info;
   rwkvq_status st = begin_run(plan_dev, plan_bytes, s, &info);
   if (st != RWKVQ_OK) return st;

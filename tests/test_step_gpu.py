@@ -330,3 +330,36 @@ def test_step_run_host_with_copies_of_half_a_megabyte_to_eight(Bn, gap):
         torch.cuda.synchronize()
         assert B.rwkvq_device_status() == 0
         arena.check()
+
+
+def test_step_run_host_does_not_wait_for_another_streams_work():
+    """Two streams: the first holds a second of other work in front of its step.  The step of the other neither waits for that
+    work nor, occupying the SMs, keeps it from ending."""
+    arenas, plans = [], []
+    for k in range(2):
+        ops = _build_ops(512, 1280, 2, 4, 6, seed=900 + 50 * k)
+        arenas.append(_HostArena(ops, 4, 64 << 10))
+        plans.append(_plan(ops, 4))
+        arenas[k].run(plans[k])
+        torch.cuda.synchronize()
+        arenas[k].check()
+        arenas[k].fill(3 + k)
+    busy, other = torch.cuda.Stream(), torch.cuda.Stream()
+    B.rwkvq_step_set_wait(plans[1], poll_limit=20000)            # a wait for its inputs that lasts a second runs out
+    with torch.cuda.stream(busy):
+        torch.cuda._sleep(2_000_000_000)
+        arenas[0].run(plans[0])
+    with torch.cuda.stream(other):
+        arenas[1].run(plans[1])
+    other.synchronize()
+    assert not busy.query()
+    assert torch.isnan(arenas[0].y_host.view(torch.float32)).any()
+    arenas[1].check()
+    busy.synchronize()
+    arenas[0].check()
+    assert B.rwkvq_device_status() == 0
+    for k in (0, 1, 1, 0):                                       # and the copy streams are used again
+        arenas[k].fill(5 + k)
+        arenas[k].run(plans[k])
+        torch.cuda.synchronize()
+        arenas[k].check()
