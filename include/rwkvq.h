@@ -297,7 +297,8 @@ typedef struct {
  * from run to run.  rwkvq_step_plan builds the schedule on
  * the host and copies it into plan_dev (rwkvq_step_plan_bytes() bytes, caller-owned); the plan
  * embeds the pointers of `ops`, so the buffers must stay where they are.  rwkvq_step_run launches
- * it.  ops must be sorted by stage (non-decreasing).  Errors as rwkvq_gemv plus ETIMEOUT through
+ * it.  ops must be sorted by stage (non-decreasing).  A run may be captured into a graph, which may be launched any number of times, runs
+ * outside it in between (one after the other, as all runs of a plan).  Errors as rwkvq_gemv plus ETIMEOUT through
  * rwkvq_device_status.
  */
 size_t rwkvq_step_plan_bytes(const rwkvq_gemv_op* ops, int n_ops, int B);

@@ -1417,6 +1417,7 @@ struct PlanInfo {
   int P, B, NB, n_slots, n_stages, mix;
   unsigned runs;        // launches since the counters were last zero
   unsigned abort_epoch; // value of the abort epoch when the counters were last known good
+  bool captured;        // some run is part of a graph, which may be launched at any time
   uint32_t poll_limit, wait_skew;
   uint32_t slot_bytes, replica_bytes, smem_bytes;
   size_t off_unit_off, off_event_off, off_units, off_events, off_counter, off_mixops, off_mixx, off_scratch, total_bytes;
@@ -1904,6 +1905,7 @@ rwkvq_status rwkvq_step_plan(const rwkvq_gemv_op* ops, int n_ops, int B, void* p
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // `image` is a pageable temporary
   if (e != cudaSuccess) return cuda_status(e);
   info.runs = 0;
+  info.captured = false;
   info.abort_epoch = abort_epoch();   // the image just copied holds zeroed counters
   for (int i = 0; i < n_ops; ++i) {
     if (i == 0 || ops[i].stage != ops[i - 1].stage) { info.y_lo.push_back(~0ull); info.y_hi.push_back(0ull); }
@@ -1938,6 +1940,12 @@ unsigned* counters_of(const void* plan_dev, const PlanInfo& info) {
 }
 unsigned target_of(const PlanInfo& info) { return info.runs * (unsigned)info.P; }
 
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &status) != cudaSuccess) { cudaGetLastError(); return false; }      // the default stream beside another thread's capture
+  return status == cudaStreamCaptureStatusActive;
+}
+
 // A run that was counted but will never arrive: have the next one clear the counters.
 void forget_run(const void* plan_dev) {
   std::lock_guard<std::mutex> lock(g_plan_mutex);
@@ -1956,9 +1964,12 @@ rwkvq_status begin_run(const void* plan_dev, size_t plan_bytes, cudaStream_t s, 
     if (it == g_plans.end()) return RWKVQ_EINVAL;   // not a plan written by rwkvq_step_plan in this process
     if (plan_bytes < it->second.total_bytes) return RWKVQ_ENOMEM;
     // The arrival counters only ever grow: run r opens a barrier at r * CTAs arrivals, so a launch
-    // needs no clearing pass.  A run that gave up leaves them short; start over after one.
+    // needs no clearing pass.  A run that gave up leaves them short; start over after one.  A captured run is launched any number of times
+    // with the target it was captured with: it clears them itself, and so does every other run of the plan from then on, which cannot know
+    // what the graph's launches left.
     const unsigned epoch = abort_epoch();
-    if (it->second.abort_epoch != epoch) { it->second.abort_epoch = epoch; it->second.runs = 0; clear_counters = true; }
+    it->second.captured = it->second.captured || is_capturing(s);
+    if (it->second.abort_epoch != epoch || it->second.captured) { it->second.abort_epoch = epoch; it->second.runs = 0; clear_counters = true; }
     it->second.runs += 1;
     *info = it->second;
   }

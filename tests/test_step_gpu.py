@@ -363,3 +363,27 @@ def test_step_run_host_does_not_wait_for_another_streams_work():
         arenas[k].run(plans[k])
         torch.cuda.synchronize()
         arenas[k].check()
+
+
+@pytest.mark.parametrize("Bn", [1, 8, 16])
+def test_captured_step_is_launched_many_times(Bn):
+    """A step in a graph: its barriers hold in every launch of the graph and in runs between them."""
+    ops = _build_ops(512, 1280, 2, Bn, 6, seed=1100 + Bn)
+    plan = _plan(ops, Bn)
+    B.rwkvq_step_run(plan)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.rwkvq_step_run(plan)
+    for seed, launch in enumerate([graph.replay, graph.replay, lambda: B.rwkvq_step_run(plan), lambda: B.rwkvq_step_run(plan), graph.replay]):
+        for k, e in enumerate(ops):
+            x, xp = inputs.gen_activation_pair(9000 + 100 * seed + k, Bn, e["W"].ic, n_outliers=4)
+            e["x16"], e["xp16"] = x.astype(np.float16), xp.astype(np.float16)
+            e["xd"].copy_(torch.from_numpy(e["x16"]))
+            if e["mu"] is not None:
+                e["xpd"].copy_(torch.from_numpy(e["xp16"]))
+            e["y"].fill_(float("nan"))
+        launch()
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        _check(ops, Bn)
