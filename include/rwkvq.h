@@ -350,7 +350,7 @@ rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, i
  * The bytes that reach y_host are those of the plain order.  Host buffers should be page-locked,
  * otherwise the copies serialize with the host.  A size of 0 skips that copy.  A call that finds the copy
  * streams busy with another stream's call runs its three parts one after the other on `stream`, so that calls on
- * different streams do not wait for one another's work.  The environment variable RWKVQ_HOST_OVERLAP=0
+ * different streams do not wait for one another's work; so does a call that is being captured.  The environment variable RWKVQ_HOST_OVERLAP=0
  * (read at every call) keeps every step on the plain order.  Errors: as rwkvq_step_run, ECUDA.
  */
 rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const void* act_host,

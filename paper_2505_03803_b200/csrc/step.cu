@@ -2131,6 +2131,12 @@ HostPipe* host_pipe() {
   HostPipe& hp = g_pipes[id != 0 ? id : ~(unsigned long long)dev];
   if (hp.tried) return hp.ok ? &hp : nullptr;
   hp.tried = true;
+  // allocations are no concern of another thread's capture
+  struct Relaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  } relaxed;
   cudaDriverEntryPointQueryResult q1, q2;
   void *f1 = nullptr, *f2 = nullptr;
   if (cudaGetDriverEntryPoint("cuStreamWaitValue32", &f1, cudaEnableDefault, &q1) != cudaSuccess || q1 != cudaDriverEntryPointSuccess || !f1) return nullptr;
@@ -2192,9 +2198,11 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
   const char* ov = std::getenv("RWKVQ_HOST_OVERLAP");      // "0": always the plain order
   if ((ov && ov[0] == '0') || act_bytes + y_bytes < kOverlapMinBytes)
     return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
+  // A captured call stays on its stream: a graph would keep this call's numbers for the words that the overlapped order waits for.
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (is_capturing(s)) return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   HostPipe* hp = host_pipe();
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (!hp || !pipe_free(*hp, s)) return run_host_plain(plan_dev, plan_bytes, act_host, act_dev, act_bytes, y_dev, y_host, y_bytes, stream);
   PlanInfo info;
   rwkvq_status st = begin_run(plan_dev, plan_bytes, s, &info);

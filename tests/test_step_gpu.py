@@ -386,3 +386,22 @@ def test_captured_step_is_launched_many_times(Bn):
         torch.cuda.synchronize()
         assert B.rwkvq_device_status() == 0
         _check(ops, Bn)
+
+
+def test_captured_step_on_host_buffers():
+    """The whole call in a graph, at a size that is overlapped outside one: every launch takes the host's present activations."""
+    ops = _build_ops(512, 1280, 2, 4, 6, seed=1200)
+    arena = _HostArena(ops, 4, 64 << 10)
+    plan = _plan(ops, 4)
+    arena.run(plan)
+    torch.cuda.synchronize()
+    arena.check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        arena.run(plan)
+    for seed, launch in enumerate([graph.replay, graph.replay, lambda: arena.run(plan), graph.replay]):
+        arena.fill(10 + seed)
+        launch()
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        arena.check()
