@@ -64,25 +64,45 @@ __global__ void __launch_bounds__(256, 2) gemv_kernel(const __grid_constant__ Ge
   } else {
     const int E = a.entries;
     const uint32_t* cbg = reinterpret_cast<const uint32_t*>(a.aux) + (size_t)(rb * a.KT) * E;
-    constexpr bool kEarly = !(BITS == 8 && NB == 2);      // registers suffice to request the records a tile ahead
+    // registers suffice to request the first tile's records ahead of the inputs, and those of the others a tile ahead
+    constexpr bool kEarly = !(BITS == 8 && NB == 2), kAhead = NB == 1;
     VqRecord<BITS> v[REC];
 #pragma unroll
     for (int r = 0; r < REC; ++r)
       if (kEarly) v[r].load(rec + ((size_t)r * a.KT + kt0) * 8 * RBYTES, lane);
     stage_codebook(smem + L.cb_off, cbg + (size_t)kt0 * E, E);
     stage_input<FMT>(smem, L, a, kt0, kt1);      // ends with a barrier
+    // A tile's sum starts at zero and is added with a rounding of its own: the tensor core's accumulation cuts off, and its error grows with
+    // the chain (4096 x 4096, two tiles a block: 6.9e-7 of the result in one chain, 3.5e-7 like this).
+    float before[REC][NB][4] = {};
+    auto bank = [&]() {
+#pragma unroll
+      for (int r = 0; r < REC; ++r)
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) { before[r][n][i] += acc[r][n][i]; acc[r][n][i] = 0.f; }
+    };
     for (int kt = kt0; kt < kt1; ++kt) {
-      if (kt > kt0) __syncthreads();
+      if (kt > kt0) { bank(); __syncthreads(); }
       if (kt + 1 < kt1)
         stage_codebook(smem + L.cb_off + (size_t)((kt + 1 - kt0) & 1) * E * 128, cbg + (size_t)(kt + 1) * E, E);
       const uint32_t* cb_lane = reinterpret_cast<const uint32_t*>(smem + L.cb_off + (size_t)((kt - kt0) & 1) * E * 128) + lane;
       const XLane xl = make_xlane(smem + (size_t)(kt - kt0) * 512, L.xstride, nullptr, 16, a.B, lane);
 #pragma unroll
       for (int r = 0; r < REC; ++r) {
-        if (!kEarly) v[r].load(rec + ((size_t)r * a.KT + kt) * 8 * RBYTES, lane);
+        if (!kAhead && !(kEarly && kt == kt0)) v[r].load(rec + ((size_t)r * a.KT + kt) * 8 * RBYTES, lane);
         vq_record_mma<BITS, NB>(v[r].w, cb_lane, xl, acc[r]);
-        if (kEarly && kt + 1 < kt1) v[r].load(rec + ((size_t)r * a.KT + kt + 1) * 8 * RBYTES, lane);
+        if (kAhead && kt + 1 < kt1) v[r].load(rec + ((size_t)r * a.KT + kt + 1) * 8 * RBYTES, lane);
       }
+    }
+    if (kt1 - kt0 > 1) {
+#pragma unroll
+      for (int r = 0; r < REC; ++r)
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[r][n][i] += before[r][n][i];
     }
   }
 

@@ -222,3 +222,22 @@ def test_products_that_feed_each_other():
         ref, tol = H.reference(W, None, src.cpu().numpy(), None)
         assert (np.abs(y.double().cpu().numpy() - ref) <= tol + np.abs(ref) * 2.0 ** -10).all()
         src = y
+
+
+@pytest.mark.parametrize("bits,Bn", [(6, 1), (6, 16), (8, 8)])
+def test_vq_product_is_no_less_exact_than_its_tiles(bits, Bn):
+    """Sixteen column tiles in one product against sixteen products of one tile each, added in fp64.  Between the two lie roundings of
+    fp32 additions only: eight where a cluster takes two tiles a block, on partial sums that grow to the result, 1.4 * 2^-24 of it in
+    the 2-norm for independent roundings (bound: twice that); the tensor core's accumulation through all tiles is off by
+    5 * 2^-24 and more."""
+    oc, ic = 512, 4096
+    c = H.random_vq_codes(31 + bits, oc, ic, bits)
+    rng = np.random.default_rng(bits)
+    c["codebook"] = (np.abs(rng.standard_normal(c["codebook"].shape)) * 0.02).astype(np.float16)      # sums that grow: truncation is one-sided
+    x16 = np.abs(inputs.gen_activation(Bn, Bn, ic, 0)).astype(np.float16)
+    y = H.run_gemv(H.pack_vq(c, bits), None, x16, None)
+    want = np.zeros_like(y)
+    for k in range(ic // 256):
+        tile = dict(q=np.ascontiguousarray(c["q"][:, 128 * k:128 * (k + 1)]), codebook=np.ascontiguousarray(c["codebook"][:, k:k + 1]))
+        want += H.run_gemv(H.pack_vq(tile, bits), None, np.ascontiguousarray(x16[:, 256 * k:256 * (k + 1)]), None)
+    assert np.linalg.norm(y - want) <= 2.8 * 2.0 ** -24 * np.linalg.norm(want)
