@@ -29,12 +29,12 @@
 //     with the next tile.
 // (3) Long contractions with few tiles are cut into slices, which leave their sums in the workspace;
 // a third launch adds them up in order.
-// What bounds it: with many tokens the instructions of the dequantisation warps beside the tensor
-// core's 4 * NT / 2 cycles per 64-column block (about 500 cycles a block at NT = 208, where the
-// tensor pipe needs 417), and the power limit; with few tokens the same work per block (the tensor
-// pipe is nearly idle) and the launches.  Eight projections of one layer, before -> now: d 4096, 2048
-// tokens 852 -> 709 us; d 2048, 203 tokens 88.8 -> 37; d 512, 21 tokens 34 -> 16; d 640, 1783 tokens
-// 54 -> 41; d 1280, 1464 tokens 112 -> 70.
+// What bounds it: with many tokens the instructions of the dequantisation warps beside the tensor core's 4 * NT / 2 cycles per
+// 64-column block (about 500 cycles a block at NT = 208, where the tensor pipe needs 417: busy 72 % of prefill_kernel's time), and in a loop of
+// seconds the power limit (1417 instead of 1965 MHz).  With few tokens the parts around the blocks: of d 2048, 203 tokens the pre-pass takes
+// 5 us, prefill_kernel 30, of which its blocks would fill 11.5 on evenly loaded SMs, and adding up the slices 8, partly in each other's shadow.
+// Eight projections of one layer, before -> now: d 4096, 2048 tokens 991 -> 829 us in a loop, 852 -> 722 ten calls from idle;
+// d 2048, 203 tokens 88.8 -> 37; d 512, 21 tokens 34 -> 16; d 640, 1783 tokens 54 -> 41; d 1280, 1464 tokens 112 -> 70.
 // Every wait is bounded; a wait that gives up raises the device status word and all roles leave
 // through the common exit, where tensor memory is freed.
 #include <cuda.h>           // tensor map types (no driver symbol is linked)

@@ -24,8 +24,8 @@
 // earlier outputs (rwkvq_input_xform: the WKV recurrence and sigmoid gate of Appendix A.1 Eqs. 23-24,
 // the squared ReLU and output gate of Eq. 27, optionally a root-mean-square normalisation), the
 // inputs of a stage are not built per CTA: after the stage barrier all CTAs together compute the
-// stage's x_mix once (mix_slice: a half-warp per 128-column group) into a scratch region of the plan,
-// publish it through a second barrier, and every CTA fetches its segments with bulk copies.
+// stage's x_mix once (mix_slice: a quarter-warp per 128-column group of a plain input, a warp where an operator is in front)
+// into a scratch region of the plan, publish it through a second barrier, and every CTA fetches its segments with bulk copies.
 //
 // The host plans the step once: every stage's units are dealt WHOLE to the CTAs, in runs of neighbouring units by the
 // smallest estimated time of the slowest CTA, along rows of tiles where that is no worse; the plan is a per-CTA
@@ -530,10 +530,11 @@ __device__ __forceinline__ StepMixOp load_mixop(const StepMixOp* p) {
   return u.op;
 }
 
-// Everything mix_slice will read that does not depend on the stage before -- the products' descriptors,
-// the mu_hat codes of this CTA's items and the codebook entries they select -- is read once ahead of
-// time, while the consumer warps are still busy with the current stage, so that behind the barrier the
-// chain of dependent loads (descriptor -> codes -> codebook) hits in L1 and only x itself comes from L2.
+// Reads ahead, while the consumer warps are still busy with the current stage, what this CTA's items read that does not depend on
+// it: the products' descriptors, the mu_hat codes and the codebook entries they select.  A warp's first item is taken right behind the clearing of
+// the next outputs (mix_prepare) and finds this in L1; later items are taken behind the barrier, whose acquire empties L1, and find it in L2
+// instead of HBM.  The inputs that are still in HBM are requested into L2.  Without it, with it: 7B-class B=8 1427, 1398 us; 14B-class
+// B=16 3719, 3673; whole blocks, whose items are few, 123.2, 124.1.
 template <int NB>
 __device__ void mix_warm(const StepArgs& a, const StepEvent& ev, int stid) {
   constexpr int kStagerWarps = Shape<NB>::kStagerWarps;
@@ -1394,13 +1395,15 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   const uint32_t u0 = a.unit_off[blockIdx.x], u1 = a.unit_off[blockIdx.x + 1];
   const uint32_t e0 = a.event_off[blockIdx.x], e1 = a.event_off[blockIdx.x + 1];
   const int warp = threadIdx.x >> 5;
-  // Registers are re-divided at entry (see Shape): the warpgroups of stagers and producer hand part of
+  // With two batch blocks registers are re-divided at entry (see Shape): the warpgroups of stagers and producer hand part of
   // their share back and the consumer warpgroups take it, so that the record routine keeps everything
   // in registers.
-  if (warp < kConsumerWarps) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kConsumerRegs));
-  } else {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kStagerRegs));
+  if constexpr (Shape<NB>::kConsumerRegs != Shape<NB>::kLaunchRegs) {
+    if (warp < kConsumerWarps) {
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kConsumerRegs));
+    } else {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kStagerRegs));
+    }
   }
   if (warp < kConsumerWarps) {
     consumer_role<NB, MIX>(a, smem, ctrl, xbufs, replicas, u0, u1 - u0, e0, e1 - e0);
