@@ -2118,12 +2118,12 @@ std::mutex g_pipe_mutex;
 std::unordered_map<unsigned long long, HostPipe> g_pipes;
 // Activations arrive in pieces of 256 KB, then twice as much each time up to 4 MB: the step begins behind the first piece (5 us instead of 80)
 // and most of the bytes go in copies long enough for the link's rate.  Outputs leave in groups of whole stages of at least a quarter
-// of what is still to come, 2 MB at most, so that little is left to copy when the step ends.  22 MB in, 44 MB out, 32 layers: 1665 us,
-// 1860 with pieces of 4 MB and groups of 2 MB.
+// of what is still to come, 2 MB at most, so that little is left to copy when the step ends.  73 MB both ways, 32 layers: 1606 us, 1646 with
+// pieces of 4 MB and groups of 2 MB, 2795 in the plain order.
 constexpr unsigned kChunkShift = 18, kMaxChunks = 16;
 constexpr size_t kOutGroupBytes = (size_t)2 << 20, kMinOutGroupBytes = (size_t)128 << 10;
-// Steps that copy less run the plain order: overlapped, 0.4 MB took 93 us against 92, 0.9 MB 148 against 158, 2.9 MB 245 against 298, 7 MB 267
-// against 325.
+// Steps that copy less run the plain order: overlapped, 0.4 MB took 93 us against 92.  From there on it gains: 0.57 MB 147 against 150,
+// 1.1 MB 149 and 164, 2.3 MB 176 and 204, 4.6 MB 220 and 288.
 constexpr size_t kOverlapMinBytes = (size_t)512 << 10;
 
 HostPipe* host_pipe() {
