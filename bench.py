@@ -35,12 +35,12 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one step_kernel launch divided by its
-# algorithmic bytes, from an ncu capture of the 1.6B-class stack (about 0.55 GB per launch; the larger
-# stacks are beyond the size a capture should hold on the device).  The packed weights are read once
-# whatever the stack, so the traffic of a larger stack is this ratio times its algorithmic bytes.
-# None = no capture of the kernel as it stands.
-NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.0131    # 538.6 MB of DRAM traffic for 531.6 MB algorithmic
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one step_kernel launch divided by its algorithmic
+# bytes, by decode batch, from ncu captures of the kernel as it stands: the 1.6B-class stack at batch 1 (539.1 MB for
+# 532.0), the 7B-class stack at batch 8 (2 888 for 2 893) and 16 (2 963 for 2 970); the 14B-class stack is beyond the size
+# a capture should hold on the device.  The packed weights are read once whatever the stack, so the traffic of
+# a larger stack is this ratio times its algorithmic bytes.  Other batches run a kernel of which there is no capture: null.
+NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = {1: 1.0132, 8: 0.9983, 16: 0.9977}
 
 HEADLINE = ("c4_14b", 16)
 CONFIGS = (("c2_1p6b", 1), ("c3_7b", 1), ("c3_7b", 8))
@@ -383,65 +383,64 @@ def prefill_leg(reps: int = 10, M: int = 2048):
 
 
 def proxy_leg(reps: int = 10, with_oracle: bool = True):
-    """The proxy pass (Section 4.1) on fp16 matrices resident on the device: rwkvq_proxy_select over one
-    matrix at a time (histogram of the 65 536 bit patterns = the sort of Eq. 5 as a counting sort, then the
-    walk over the occupied bins, then the copy of the two numbers to the host), timed with events around
-    the call.  A 256 x 256 matrix gives the fixed cost of the call (clear, walk, copy, synchronization);
-    the large matrices minus that are the streaming pass, whose algorithmic traffic is 2 bytes per
-    weight.  The oracle's sort-and-difference on the same values is timed beside it."""
+    """The proxy pass (Section 4.1) on fp16 matrices resident on the device: rwkvq_proxy_select (the set of bit
+    patterns that occur, which is all that the sort of Eq. 5 decides; then the walk over the set, then the copy of the two numbers
+    to the host), timed with events around the call.  `call_ms` is the call for one matrix, launches, copy and
+    synchronization included.  What a further matrix costs a call -- the difference between a call for `together` matrices
+    of the shape and one for a single matrix, all in buffers of their own and larger than L2 together -- is the streaming pass, whose
+    algorithmic traffic is 2 bytes per weight.  The oracle's sort-and-difference on the same values is timed beside it."""
     import torch
     from paper_2505_03803_b200 import binding as B
     from paper_2505_03803_b200 import stack as stack_mod
     peak, kind = measured_hbm_peak()
-    ws = torch.empty(B.rwkvq_proxy_workspace_bytes(1), dtype=torch.uint8, device="cuda")
+    together = 9
+    ws = torch.empty(B.rwkvq_proxy_workspace_bytes(together), dtype=torch.uint8, device="cuda")
 
-    def timed(w):
-        B.rwkvq_proxy_select([w], 4, math.inf, math.inf, ws)
+    def timed(mats):
+        B.rwkvq_proxy_select(mats, 4, math.inf, math.inf, ws)
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
         for _ in range(reps):
-            pc, pf, _ = B.rwkvq_proxy_select([w], 4, math.inf, math.inf, ws)
+            pc, pf, _ = B.rwkvq_proxy_select(mats, 4, math.inf, math.inf, ws)
         e1.record()
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / reps, float(pc[0]), float(pf[0])
-    small = stack_mod.gen_weight_device(11, 256, 256, "gauss")
-    fixed_ms, _, _ = timed(small)
     rows = []
     for (oc, ic, kind_w) in ((4096, 4096, "gauss"), (14336, 4096, "gauss"), (4096, 4096, "student")):
-        w = stack_mod.gen_weight_device(12 + oc, oc, ic, kind_w)
-        ms, pc, pf = timed(w)
-        stream_ms = max(1e-6, ms - fixed_ms)
-        gbs = 2.0 * oc * ic / (stream_ms * 1e-3) / 1e9
-        rows.append({"matrix": f"{oc}x{ic} {kind_w}", "call_ms": ms, "histogram_ms": stream_ms, "P_c": pc, "P_f": pf,
-                     "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                                  "traffic": None, "peak_kind": f"of {kind}", "kernel": "proxy_hist_kernel",
-                                  "algorithmic_bytes_per_launch": 2 * oc * ic}})
+        mats = [stack_mod.gen_weight_device(12 + oc + i, oc, ic, kind_w) for i in range(together)]
+        ms, pc, pf = timed(mats[:1])
+        pass_ms = (timed(mats)[0] - ms) / (together - 1)
+        row = {"matrix": f"{oc}x{ic} {kind_w}", "call_ms": ms, "further_matrix_ms": pass_ms, "together": together, "P_c": pc, "P_f": pf,
+               "roofline": None}
+        if pass_ms > 0:
+            gbs = 2.0 * oc * ic / (pass_ms * 1e-3) / 1e9
+            row["roofline"] = {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": None,
+                               "peak_kind": f"of {kind}", "kernel": "proxy_mark_kernel", "algorithmic_bytes_per_matrix": 2 * oc * ic}
+        rows.append(row)
         if with_oracle and oc == 4096 and kind_w == "gauss":
             from oracle import rwkvq_oracle as orc
-            wh = w.cpu().numpy().astype(np.float64)
+            wh = mats[0].cpu().numpy().astype(np.float64)
             t0 = time.perf_counter()
             orc.proxy(wh, 4)
             rows[-1]["oracle_s"] = time.perf_counter() - t0
-        del w
-    return {"workload": "rwkvq_proxy_select on one fp16 matrix resident on the device, K = 4", "fixed_call_ms": fixed_ms,
-            "fixed_call": "256 x 256 matrix: workspace clear, proxy_reduce_kernel, copy of the results, synchronization",
-            "matrices": rows}
+        del mats
+    return {"workload": "rwkvq_proxy_select on fp16 matrices resident on the device, K = 4", "matrices": rows}
 
 
 def vq_alu_roofline(oc, ic, entries, iters, ms, sm_mhz=1965.0, sms=148):
-    """vq_kmeans_kernel against the fp32 instruction rate: an assignment pass evaluates, per (2-D vector,
-    centre) pair, two subtractions, a multiply, a fused multiply-add and a compare-and-keep = 5 thread
-    instructions; k-means++ seeding makes `entries` such passes against one new centre each (5 instructions per
-    vector and pass) and every Lloyd iteration one pass against all centres.  Peak = 128 fp32 lanes per SM per
-    clock at the maximum SM clock.  Centre updates, the scans of the seeding and the final fp64 assignment are
-    not counted, so the fraction is a lower bound on how busy the lanes are."""
+    """vq_seed_kernel + vq_lloyd_kernel against the fp32 operation rate, by the operations they cannot do without: the
+    k-means++ seeding evaluates each 2-D vector against every new centre (two differences, a product, a multiply-add, a minimum and a
+    running sum = 6 operations), and an iteration, and the final assignment, needs at least one distance per vector (two
+    differences, a product, a multiply-add, a comparison = 5; the kernel strikes out centres that cannot be nearest and compares
+    the others, a few).  Peak = 128 fp32 lanes per SM per clock at the maximum SM clock.  Building the lists of candidates, the scans
+    of the seeding, the centre updates and the fp64 assignment are not counted: the fraction is a lower bound."""
     vectors = oc * ic // 2
-    work = 5.0 * vectors * entries * (iters + 1)          # iterations against all centres + the seeding passes
+    work = 6.0 * vectors * entries + 5.0 * vectors * (iters + 1)
     achieved = work / (ms * 1e-3) / 1e12
     peak = sms * 128 * sm_mhz * 1e6 / 1e12
-    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T thread-instructions/s", "frac": achieved / peak,
-            "traffic": None, "kernel": "vq_kmeans_kernel"}
+    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T fp32 operations/s", "frac": achieved / peak,
+            "traffic": None, "kernel": "vq_seed_kernel + vq_lloyd_kernel"}
 
 
 def quantize_leg(reps: int = 5):
@@ -490,7 +489,7 @@ def quantize_leg(reps: int = 5):
     torch.cuda.synchronize()
     vq_ms = e0.elapsed_time(e1)
     return {"workload": "one 7B-class layer (8 projections, d=4096 h=14336), fp16 weights on the device -> packed images",
-            "sq_ms_per_layer": ms, "sq_weights_per_s": weights / (ms * 1e-3), "launches_per_layer": 2 * len(mats),
+            "sq_ms_per_layer": ms, "sq_weights_per_s": weights / (ms * 1e-3), "launches_per_layer": len(mats),
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak, "traffic": None,
                          "peak_kind": f"of {kind}", "kernel": "sq_quantize_kernel", "algorithmic_bytes_per_layer": nbytes,
                          "timed": "eight rwkvq_quantize_dev_async calls and one rwkvq_quantize_check (a stream "
@@ -659,9 +658,8 @@ def measure_stack(st, args, workload, K, W, world, dist, gpu_id, with_e2e=True):
     avg_launch_ms = sum(per_launch_ms) / len(per_launch_ms)
     achieved = alg_bytes / launches_per_step / (avg_launch_ms * 1e-3) / 1e9
     traffic = None
-    if (NCU_TRAFFIC_PER_ALGORITHMIC_BYTE is not None and args.mode == "step" and args.stage_group == 0
-            and args.force_method is None):
-        traffic = int(NCU_TRAFFIC_PER_ALGORITHMIC_BYTE * alg_bytes)
+    if batch in NCU_TRAFFIC_PER_ALGORITHMIC_BYTE and args.mode == "step" and args.stage_group == 0 and args.force_method is None:
+        traffic = int(NCU_TRAFFIC_PER_ALGORITHMIC_BYTE[batch] * alg_bytes)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic, "peak_kind": f"of {peak_kind}",
                 "kernel": "step_kernel" if args.mode == "step" else "gemv_kernel",
