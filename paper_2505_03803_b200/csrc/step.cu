@@ -86,12 +86,12 @@ struct StepEvent {           // 64 bytes
     // xprev = first byte of its sums, mu = 0.
     struct { uint64_t x, xprev, mu, mu_aux; } seg;
     // arrival: float ranges to clear before arriving; then this CTA's share of the stage's
-    // pre-pass: groups [grp_lo, grp_hi) of the stage's (product, batch row, 128-column group) list
+    // pre-pass: groups [grp_lo, grp_hi) of the (product, batch row, 128-column group) list that begins with product op_first
     struct { uint64_t zptr[3]; uint32_t grp_lo, grp_hi; } arr;
   };
   union {
     struct { uint32_t ic, col0, ncols; uint16_t mu_bits, mu_entries; } segd;   // copied segments: ic = bytes between rows
-    struct { uint32_t zcount[3]; uint16_t op_first, op_count; } arrd;          // products of the stage the pre-pass covers
+    struct { uint32_t zcount[3]; uint16_t op_first, op_count; } arrd;          // products this CTA's share falls in
   };
   uint32_t kind;             // EV_SEGMENT / EV_ARRIVE
   uint32_t barrier;          // segment: index + 1 of the stage barrier to pass first; arrival: index of the barrier
@@ -107,9 +107,8 @@ struct StepMixOp {           // 64 bytes
   uint64_t x, xprev, mu, mu_aux, dst_x, dst_sums;
   uint32_t ic, ic_pad;
   // kind: rwkvq_input_kind | 0x100 when the row is RMS-normalised | 0x200 when this token's input is stored
-  // (xprev_out) | 0x400 on the first product of a stage in which some input is normalised | 0x800 on the first
-  // product of a stage whose inputs are all plain buffers; a kind with any of the low ten bits set has a
-  // StepMixX beside it
+  // (xprev_out) | on every product of the stage: 0x400 where some input is normalised, 0x800 where all are
+  // plain buffers; a kind with any of the low ten bits set has a StepMixX beside it
   uint16_t mu_bits, mu_entries, sums, kind;
 };
 static_assert(sizeof(StepMixOp) == 64, "pre-pass descriptor size");
@@ -555,7 +554,7 @@ __device__ void mix_warm(const StepArgs& a, const StepEvent& ev, int stid) {
     touch_global(reinterpret_cast<const uint8_t*>(op) + 32);
     const uint64_t mu = __ldg(&op->mu);
     const uint32_t kind = __ldg(&op->kind);
-    if (kind) {
+    if (kind & 0x3FFu) {
       const uint8_t* ox = reinterpret_cast<const uint8_t*>(a.mixx + ev.arrd.op_first + k);
       touch_global(ox); touch_global(ox + 32); touch_global(ox + 64); touch_global(ox + 76);
     }
@@ -662,7 +661,7 @@ __device__ __forceinline__ PlainItem plain_item(const StepArgs& a, const StepEve
   }
   return it;
 }
-struct MixPrep { PlainItem plain; uint2 mu; uint32_t kind; };      // of the warp's (lanes') first item; of the stage's first product: what kind of stage it is
+struct MixPrep { PlainItem plain; uint2 mu; uint32_t kind; };      // of the warp's (lanes') first item; of the share's first product: what kind of stage it is
 // Steps whose inputs are all plain take the whole item ahead of the barrier, steps with operators only its descriptors: with room for both in the
 // registers each spilled for the other (7B-class, batch 8: 1453 us without, 1415 with; blocks 125 and 129).
 template <int NB, bool OPS>
@@ -812,7 +811,7 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
   uint64_t stat_src = 0;     // row whose statistic this warp computed last (rows beyond the table)
   int stat_b = -1;
   float stat_rstd = 1.f;
-  // The planner marks the first product of a stage that has a normalised input.  In the first round, which every warp takes part in, what the items
+  // The planner marks the products of a stage that has a normalised input.  In the first round, which every warp takes part in, what the items
   // need from memory is asked for ahead of the table.
   bool table = (stage_kind & 0x400) != 0u;
   uint2 mu = prep.mu;
@@ -937,7 +936,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
               if (++it >= (a.poll_limit << 2) || *abortp) { *abortp = 1; atomicExch(a.status, (int)RWKVQ_ETIMEOUT); ok = false; break; }
             }
             if (ok && a.in_flag && stid == 0) {
-              // the last input byte any product of the coming stage reads (x and x_prev, [B][ic] fp16 each)
+              // the last input byte of the products this CTA's share falls in (x and x_prev, [B][ic] fp16 each)
               const StepMixOp* mo = a.mixops + ev.arrd.op_first;
               uint64_t last = 0;
               for (uint32_t k = 0; k < ev.arrd.op_count; ++k) {
@@ -1530,7 +1529,8 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   // `share / stages` inputs): B=6, 2688, 319 / 286 and B=3, 2688, 262 / 250; B=2, 3072, 335 / 341; B=8, 3584, 328 / 339; B=3, 4608, 338 / 370;
   // with seven stager warps B=10, 4480, 385 / 377; B=16, 5120, 353 / 335; B=16, 7168, 406 / 443; B=12, 8448, 305 / 346.  The
   // element-wise operators exist in the pre-pass only.
-  const bool mix = any_xform || share > stages * (B > 8 ? 5600u : 3000u);
+  if (any_xform && n_ops > 65535) return RWKVQ_EUNSUPPORTED;      // the events count products in 16 bits
+  const bool mix = any_xform || (n_ops <= 65535 && share > stages * (B > 8 ? 5600u : 3000u));
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;
@@ -1580,9 +1580,17 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       // this CTA's share of the pre-pass of stage `barrier`
       uint64_t G = 0;
       for (int o = stage_ranges[barrier].first; o < stage_ranges[barrier].second; ++o) G += (uint64_t)B * (ops[o].W_desc.ic_pad / 128);
-      ev.arr.grp_lo = (uint32_t)(G * (uint64_t)c / P); ev.arr.grp_hi = (uint32_t)(G * (uint64_t)(c + 1) / P);
-      ev.arrd.op_first = (uint16_t)stage_ranges[barrier].first;
-      ev.arrd.op_count = (uint16_t)(stage_ranges[barrier].second - stage_ranges[barrier].first);
+      // counted from the first product that the share falls in: whoever looks for an item's product passes over those of the share only (192
+      // products in one stage, batch 1: 303 us when every item was looked for from the stage's first product)
+      const uint64_t lo = G * (uint64_t)c / P, hi = G * (uint64_t)(c + 1) / P;
+      int first = stage_ranges[barrier].first;
+      uint64_t base = 0;
+      auto groups = [&](int o) { return (uint64_t)B * (ops[o].W_desc.ic_pad / 128); };
+      while (lo < hi && lo >= base + groups(first)) base += groups(first++);
+      int end = first;
+      for (uint64_t b = base; lo < hi && b < hi; ++end) b += groups(end);
+      ev.arr.grp_lo = (uint32_t)(lo - base); ev.arr.grp_hi = (uint32_t)(lo < hi ? hi - base : lo - base);
+      ev.arrd.op_first = (uint16_t)first; ev.arrd.op_count = (uint16_t)(end - first);
     }
     cta_arrivals[c].push_back(ev);
   };
@@ -1753,10 +1761,9 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       }
       bool stage_norm = false;
       for (int o = stage_ranges[st_i].first; o < stage_ranges[st_i].second; ++o) stage_norm = stage_norm || (mixops[o].kind & 0x100);
-      if (stage_norm) mixops[stage_ranges[st_i].first].kind |= 0x400;
       bool stage_plain = true;
       for (int o = stage_ranges[st_i].first; o < stage_ranges[st_i].second; ++o) stage_plain = stage_plain && mixops[o].kind == 0;
-      if (stage_plain) mixops[stage_ranges[st_i].first].kind |= 0x800;
+      for (int o = stage_ranges[st_i].first; o < stage_ranges[st_i].second; ++o) mixops[o].kind |= (stage_norm ? 0x400 : 0) | (stage_plain ? 0x800 : 0);
       scratch_bytes = std::max(scratch_bytes, off);
     }
   }

@@ -405,3 +405,32 @@ def test_captured_step_on_host_buffers():
         torch.cuda.synchronize()
         assert B.rwkvq_device_status() == 0
         arena.check()
+
+
+@pytest.mark.parametrize("Bn", [2, 8, 11])
+def test_step_with_many_products_in_one_stage(Bn):
+    """Forty products that need not wait for one another (800 units, more inputs per CTA than it would mix itself): the CTAs' shares of
+    the pre-pass begin and end inside products of both formats, with and without a token shift.  Resident inputs, and inputs
+    that arrive from the host while the step runs."""
+    ops = []
+    for k in range(40):
+        oc, ic = (1024, 1280) if k % 4 != 1 else (1008, 1152)
+        seed = 1300 + 50 * Bn + k
+        W = H.pack_vq(H.random_vq_codes(seed, oc, ic, 6), 6) if k % 4 == 0 else H.pack_sq(H.random_sq_codes(seed, oc, ic))
+        mu = H.pack_mu(H.random_mu_codes(seed + 3, ic, 6), 6) if k % 3 else None
+        x, xp = inputs.gen_activation_pair(seed + 6, Bn, ic, n_outliers=4)
+        ops.append(dict(W=W, mu=mu, x16=x.astype(np.float16), xp16=xp.astype(np.float16), stage=0, xpd=None))
+    arena = _HostArena(ops, Bn, 8 << 10)
+    plan = _plan(ops, Bn)
+    for seed in (0, 1):
+        arena.fill(seed)
+        arena.run(plan)
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        arena.check()
+    for e in ops:
+        e["y"].fill_(float("nan"))
+    B.rwkvq_step_run(plan)
+    torch.cuda.synchronize()
+    assert B.rwkvq_device_status() == 0
+    _check(ops, Bn)
