@@ -286,7 +286,7 @@ static int fmt_of(const rwkvq_desc* d) {
 
 struct GemvPlan {
   int fmt, NRB, KT, S, nkt;
-  bool cluster;
+  bool cluster, dependent;
   size_t smem, ws_bytes, counters_bytes;
 };
 
@@ -311,22 +311,50 @@ static rwkvq_status plan_gemv(const rwkvq_desc* d, int B, bool has_mu, int mu_en
   int S = want < 1 ? 1 : (want > p->KT ? p->KT : want);
   while (S < p->KT && smem_of((p->KT + S - 1) / S) > 96 * 1024) ++S;
   // A contraction of a few tiles is done by one block: a tile costs it less than the sum over splits does.  Where eight splits
-  // leave no block with many more tiles than that, the splits are a cluster (measured from 512 x 512 to 14336 x 4096; a VQ tile is dearer, it
-  // brings its codebook).
-  const int kTilesPerSum = p->fmt == FMT_SQ3 ? 2 : 1, kClusterTiles = p->fmt == FMT_SQ3 ? 4 : p->fmt == FMT_VQ6 ? 3 : 2;
-  const int per_cluster = (p->KT + 7) / 8;
+  // leave no block with many more tiles than that, the splits are a cluster (measured from 512 x 512 to 14336 x 4096).  A VQ tile is dearer, it
+  // brings its codebook, and a sum through global memory is cheap for a few rows: tiles that a block takes more than without the cluster have to be
+  // paid for by the batch (us through global memory / cluster, one tile more: 64 entries, 512 x 4096: B=1 6.4 / 7.6, B=4 8.9 / 7.8;
+  // 4096 x 4096: B=4 9.8 / 10.2, B=6 11.2 / 10.8; 256 entries, 512 x 4096: B=8 15.5 / 17.0, B=12 18.8 / 18.5; 4096 x 4096: B=12 20.4 / 21.5, B=16
+  // 23.4 / 22.1; two tiles more, 64 entries, 512 x 6144: B=1 7.2 / 10.5, B=8 14.6 / 11.5).
+  const bool sq = p->fmt == FMT_SQ3, vq6 = p->fmt == FMT_VQ6;
+  const int kTilesPerSum = sq ? 2 : 1, kClusterTiles = sq ? 4 : vq6 ? 3 : 2;
+  const int kRowsPerTile = sq ? 0 : vq6 ? (p->NRB > 8 ? 6 : 4) : (p->NRB > 8 ? 16 : 12);
+  const int per_cluster = (p->KT + 7) / 8, more = per_cluster - (p->KT + S - 1) / S;
   p->cluster = false;
   if (p->KT <= kTilesPerSum) {
     S = 1;
-  } else if (S <= 8 || (per_cluster <= kClusterTiles && smem_of(per_cluster) <= 96 * 1024)) {
+  } else if (S <= 8 || (per_cluster <= kClusterTiles && B >= more * kRowsPerTile && smem_of(per_cluster) <= 96 * 1024)) {
     S = S < 8 ? S : 8;
     p->cluster = true;
   }
-  p->nkt = (p->KT + S - 1) / S;
-  p->S = (p->KT + p->nkt - 1) / p->nkt;  // no empty splits
+  auto blocks_of = [&](int s) { const int nkt = (p->KT + s - 1) / s; return p->NRB * ((p->KT + nkt - 1) / nkt); };      // no empty splits
   // More blocks than surely fit at once (two per SM, whole clusters within a GPC): clusters would wait for room
   // together (14336 x 4096 VQ 28.7 us, through global memory 23.3; 9456 x 9600 SQ 22.0 and 18.4).
-  if (p->S == 1 || p->NRB * p->S > 256) p->cluster = false;
+  if (blocks_of(S) == p->NRB || blocks_of(S) > 256) p->cluster = false;
+  // A few blocks more than fit at once cost a second round.  64-entry products of up to eight rows, whose blocks take half an SM's registers each, avoid
+  // it where that saves a tenth (beyond four rows, an eighth) by this estimate (in tiles; a block costs one besides its own; a round that leaves SMs
+  // with a single block takes 0.55 of the time): 10240 x 10240, one row: 320 blocks of five tiles 37.1 us, 280 of six 29.0; 9216 x 9216: 29.0 and 22.8; 23040 x 3840: 26.8
+  // and 22.8; 4096 x 14336: 20.5 and 19.1, eight rows 29.4 and 30.5; not 8192 x 14336 (30.3 and 31.8), whose second round is a short last split,
+  // nor 14336 x 4096 (17.7 and 18.1).
+  constexpr int kFit = 2 * 148;
+  if (vq6 && B <= 8 && !p->cluster && blocks_of(S) > kFit) {
+    auto estimate = [&](int s) {
+      const int nkt = (p->KT + s - 1) / s, n = blocks_of(s) / p->NRB, last = p->KT - (n - 1) * nkt;
+      double sum = 0.0;
+      for (int left = n * p->NRB; left > 0; left -= kFit)       // blocks are dealt split by split
+        sum += ((left <= p->NRB ? last : nkt) + 1) * (left <= kFit / 2 && n * p->NRB > kFit ? 0.55 : 1.0);
+      return sum;
+    };
+    int best = S;
+    for (int s = 1; s <= p->KT; ++s)
+      if (estimate(s) < estimate(best) && smem_of((p->KT + s - 1) / s) <= 96 * 1024) best = s;
+    if (estimate(best) <= (B <= 4 ? 0.9 : 0.88) * estimate(S)) S = best;
+  }
+  p->nkt = (p->KT + S - 1) / S;
+  p->S = (p->KT + p->nkt - 1) / p->nkt;
+  // A launch that starts early finds the SMs occupied by the product in front: up to a block per SM then double up on some (2048 x 4096, 64 entries, 128
+  // blocks: 7.4 us a call, plainly launched 6.8; 64 blocks 6.8 and 6.7, 32 6.4 and 6.6, 195 8.3 and 8.7, 256 7.6 and 8.2).
+  p->dependent = sq || p->cluster || p->NRB * p->S <= 74 || p->NRB * p->S > 148;
   p->smem = smem_of(p->nkt);
   if (p->cluster) p->smem = std::max(p->smem, (size_t)B * rpc * 4);
   p->counters_bytes = ((size_t)p->NRB * 4 + 255) / 256 * 256;
@@ -344,11 +372,16 @@ static cudaError_t launch_gemv_as(const GemvArgs& a, const GemvPlan& p, cudaStre
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.NRB, p.S); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = p.smem; cfg.stream = s;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = p.S; attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = p.cluster ? 2 : 1;
+  int n = 0;
+  if (p.dependent) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (p.cluster) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = 1; attr[n].val.clusterDim.y = p.S; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, NB>, a);
 }
 template <int FMT>
@@ -363,9 +396,14 @@ using namespace rwkvq;
 extern "C" {
 
 size_t rwkvq_gemv_workspace_bytes(const rwkvq_desc* d, int B) {
-  GemvPlan p;
-  if (plan_gemv(d, B, true, 256, &p) != RWKVQ_OK) return 0;
-  return p.ws_bytes;
+  // the call may come without a token shift or with one of either codebook, whose shared memory moves the splits
+  size_t most = 0;
+  for (const int mu_entries : {0, 64, 256}) {
+    GemvPlan p;
+    if (plan_gemv(d, B, mu_entries != 0, mu_entries, &p) != RWKVQ_OK) return 0;
+    most = std::max(most, p.ws_bytes);
+  }
+  return most;
 }
 
 // Every argument check of the decode product, made on the host before anything is enqueued.

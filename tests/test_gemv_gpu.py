@@ -241,3 +241,15 @@ def test_vq_product_is_no_less_exact_than_its_tiles(bits, Bn):
         tile = dict(q=np.ascontiguousarray(c["q"][:, 128 * k:128 * (k + 1)]), codebook=np.ascontiguousarray(c["codebook"][:, k:k + 1]))
         want += H.run_gemv(H.pack_vq(tile, bits), None, np.ascontiguousarray(x16[:, 256 * k:256 * (k + 1)]), None)
     assert np.linalg.norm(y - want) <= 2.8 * 2.0 ** -24 * np.linalg.norm(want)
+
+
+# Both sides of the lines between clusters and sums through global memory (batch against tiles a block takes more), launches that do not
+# start early (75 to 148 blocks), and a product whose blocks would not fit at once, cut into fewer splits.
+@pytest.mark.parametrize("bits,oc,ic,Bn", [(6, 256, 4096, 3), (6, 256, 4096, 4), (6, 256, 6144, 7), (6, 256, 6144, 8), (6, 2304, 4096, 5),
+                                           (6, 2304, 4096, 6), (8, 256, 3840, 11), (8, 256, 3840, 12), (8, 2304, 2304, 15), (8, 2304, 2304, 16),
+                                           (8, 1280, 4096, 2), (6, 25600, 1536, 1), (6, 25600, 1536, 8)])
+def test_vq_splits_by_batch_and_blocks(bits, oc, ic, Bn):
+    W = H.pack_vq(H.random_vq_codes(oc + ic, oc, ic, bits), bits)
+    x, xp = inputs.gen_activation_pair(Bn + ic, Bn, ic, n_outliers=8)
+    mu = H.pack_mu(H.random_mu_codes(ic + 1, ic)) if Bn % 2 else None
+    _check_gemv(W, mu, x.astype(np.float16), xp.astype(np.float16))
