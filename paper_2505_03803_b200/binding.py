@@ -314,11 +314,18 @@ def rwkvq_gemv(desc: Desc, W_image, mu_desc, mu_image, x, xprev, B: int, y, work
     """rwkvq_gemv on torch tensors: W_image/mu_image uint8, x/xprev float16 [B, ic], y float32 or
     float16 [B, oc], workspace uint8 (zero-filled before first use)."""
     t = _torch or _load_torch()
-    status = (_lib or lib()).rwkvq_gemv(      # a missing tensor is the library's to refuse
-        desc, None if W_image is None else W_image.data_ptr(), mu_desc, None if mu_image is None else mu_image.data_ptr(),
-        None if x is None else x.data_ptr(), None if xprev is None else xprev.data_ptr(), B, None if y is None else y.data_ptr(),
-        RWKVQ_F32 if y is None or y.dtype is t.float32 else RWKVQ_F16, None if workspace is None else workspace.data_ptr(),
-        0 if workspace is None else workspace.nbytes, _stream_ptr(stream))
+    try:
+        status = (_lib or lib()).rwkvq_gemv(
+            desc, W_image.data_ptr(), mu_desc, None if mu_image is None else mu_image.data_ptr(), x.data_ptr(),
+            None if xprev is None else xprev.data_ptr(), B, y.data_ptr(), RWKVQ_F32 if y.dtype is t.float32 else RWKVQ_F16,
+            workspace.data_ptr(), workspace.nbytes, _stream_ptr(stream))
+    except AttributeError:
+        if not any(a is None for a in (W_image, x, y, workspace)):
+            raise
+        # a missing tensor is the library's to refuse, as a null pointer
+        status = lib().rwkvq_gemv(desc, _dev_ptr(W_image), mu_desc, _dev_ptr(mu_image), _dev_ptr(x), _dev_ptr(xprev), B, _dev_ptr(y),
+                                  RWKVQ_F32 if y is None or y.dtype is t.float32 else RWKVQ_F16, _dev_ptr(workspace),
+                                  0 if workspace is None else workspace.nbytes, _stream_ptr(stream))
     if status:
         raise RwkvqError(status, "rwkvq_gemv")
 
