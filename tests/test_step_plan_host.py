@@ -64,8 +64,8 @@ def test_plan_is_built_for_benchmark_shapes(d, h, layers, Bn, bits):
 
 
 # Every record (product, 16-row slice, 256-column tile) must reach exactly one consumer warp exactly
-# once, in each of the planner's three ways of dealing a stage (row of tiles by row of tiles; whole
-# units at their cost midpoints; eighths of a unit for stages too small for either): small and large
+# once, in either of the planner's ways of dealing a stage (whole units in runs that ignore the ends of rows;
+# rows of tiles cut into whole numbers of runs): small and large
 # stages, ragged shapes (rows that end in half a unit, ic not a multiple of 256), every batch
 # regime, few and many CTAs, every product in one stage.
 @pytest.mark.parametrize("d,h,layers,Bn,bits,n_ctas,one_stage", [
