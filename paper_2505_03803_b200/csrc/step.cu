@@ -270,8 +270,11 @@ __device__ __forceinline__ uint32_t smem_add_acq_rel(uint32_t* p, uint32_t v) {
   return old;
 }
 
+// A slot's data is announced to the consumer group that takes the unit, on a barrier of that group's: with one barrier for both and an odd number of
+// slots a group would meet every second of its phases only, and while the other group's unit is still arriving in the slot, the phase before it
+// looks like the one the group waits for (waits see the parity of a phase, not its number).
 struct Ctrl {
-  uint64_t full[kMaxSlots], empty[kMaxSlots];
+  uint64_t full[2][kMaxSlots], empty[kMaxSlots];
   uint64_t xfull[4], xempty[4];
   uint32_t stage_cnt[64];    // one 8-bit count per grid barrier (four per word): how many of the parties
                              // of this CTA (every consumer warp, and the stagers as one) have reported the
@@ -337,11 +340,17 @@ __device__ __forceinline__ bool wait_inputs(const StepArgs& a, uint64_t last, vo
   return false;
 }
 
+// How often a group has had the slot of its unit before: once a round of the ring, or every second round where the ring's odd number of slots makes
+// the two groups take turns.
+template <int NB>
+__device__ __forceinline__ uint32_t slot_uses(uint32_t round, uint32_t n_slots) { return Shape<NB>::kGroups == 2 && (n_slots & 1u) ? round >> 1 : round; }
+
 // ---- roles -------------------------------------------------------------------------------------
 
 // Producer: one warp.  Four descriptors are fetched per warp-wide 16-byte load (8 lanes each) one
 // batch ahead; lane 0 waits for the slot, the owning lanes copy the descriptor into the slot
 // header, lane 0 arms the barrier and issues the bulk copies.
+template <int NB>
 __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint32_t u0, uint32_t u1) {
   const int lane = threadIdx.x & 31;
   const uint4* base = reinterpret_cast<const uint4*>(a.units);
@@ -373,7 +382,7 @@ __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint
       __syncwarp();
       if (lane == 0) {
         const uint32_t tx = by0 + by1 + cbb;
-        uint64_t* full = &ctrl->full[slot];
+        uint64_t* full = &ctrl->full[i % (uint32_t)Shape<NB>::kGroups][slot];
         if (tx == 0) {
           mbar_arrive(full);
         } else {
@@ -392,9 +401,8 @@ __device__ void producer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint
     const uint32_t first = issued > (uint32_t)a.n_slots ? issued - a.n_slots : 0;
     for (uint32_t i = first; i < issued; ++i) {
       const int slot = (int)(i % (uint32_t)a.n_slots);
-      const uint32_t parity = (i / (uint32_t)a.n_slots) & 1u;
       for (uint32_t it = 0; it < a.poll_limit; ++it)
-        if (mbar_try_wait(&ctrl->full[slot], parity)) break;
+        if (mbar_try_wait(&ctrl->full[i % (uint32_t)Shape<NB>::kGroups][slot], slot_uses<NB>(i / (uint32_t)a.n_slots, (uint32_t)a.n_slots) & 1u)) break;
     }
   }
 }
@@ -1237,7 +1245,7 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     const int slot = (int)slot_u;
     const uint8_t* sl = smem + kCtrlBytes + (size_t)slot * a.slot_bytes;
     const StepUnit* u = reinterpret_cast<const StepUnit*>(sl);
-    if (!dead && !mbar_wait_warp(&ctrl->full[slot], round & 1u, abortp, a.status)) dead = true;
+    if (!dead && !mbar_wait_warp(&ctrl->full[grp][slot], slot_uses<NB>(round, n_slots_u) & 1u, abortp, a.status)) dead = true;
     if (!dead && u->ev_index != cur_ev) {
       const uint32_t target = u->ev_index;
       pass_events(target, u->between_mask, target - cur_ev - 1u <= 32u);
@@ -1383,7 +1391,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   uint32_t* mucb = reinterpret_cast<uint32_t*>(xbufs + kXBufTotal);
   uint8_t* replicas = reinterpret_cast<uint8_t*>(mucb) + kMuScratch;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < a.n_slots; ++s) { mbar_init(&ctrl->full[s], 1); mbar_init(&ctrl->empty[s], kGroupWarps); }
+    for (int s = 0; s < a.n_slots; ++s) { mbar_init(&ctrl->full[0][s], 1); mbar_init(&ctrl->full[1][s], 1); mbar_init(&ctrl->empty[s], kGroupWarps); }
     for (int b = 0; b < 4; ++b) { mbar_init(&ctrl->xfull[b], kStagerWarps); mbar_init(&ctrl->xempty[b], kConsumerWarps); }
     for (int k = 0; k < 64; ++k) ctrl->stage_cnt[k] = 0u;
     ctrl->abort_flag = 0;
@@ -1408,7 +1416,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   } else if (warp < kConsumerWarps + kStagerWarps) {
     stager_role<MIX, NB>(a, smem, ctrl, xbufs, mucb, e0, e1);
   } else {
-    producer_role(a, smem, ctrl, u0, u1);
+    producer_role<NB>(a, smem, ctrl, u0, u1);
   }
 }
 
