@@ -434,7 +434,7 @@ rwkvq_status rwkvq_desc_for(const rwkvq_quant_cfg* cfg, int oc, int ic, rwkvq_de
  *  cfg->codes_in must be NULL.  The image carries no checksum (rwkvq_image_unpack accepts that).
  *  workspace_dev: rwkvq_quantize_workspace_bytes() bytes, 16-byte aligned, contents irrelevant.
  * The call synchronizes `stream` before it returns (it reads back a flag word).  Errors: EINVAL,
- * ESHAPE, EUNSUPPORTED, EALIGN, ENOMEM (image or workspace too small), ENONFINITE, ECUDA.
+ * ESHAPE, EUNSUPPORTED, EALIGN, ENOMEM (image or workspace too small), ENONFINITE, ECUDA, ETIMEOUT.
  */
 size_t rwkvq_quantize_workspace_bytes(void);
 rwkvq_status rwkvq_quantize_dev(const void* w_fp16_dev, int oc, int ic, const rwkvq_quant_cfg* cfg,
@@ -448,7 +448,8 @@ rwkvq_status rwkvq_quantize_dev(const void* w_fp16_dev, int oc, int ic, const rw
  * a NaN/Inf weight sets a flag in the first word of workspace_dev, which must be zero before the
  * first call and is shared by every call that uses the same workspace.  rwkvq_quantize_check
  * synchronizes `stream`, returns RWKVQ_ENONFINITE if the flag was set by any call since the last
- * check (RWKVQ_OK otherwise) and clears it.
+ * check (RWKVQ_OK otherwise) and clears it.  ETIMEOUT: a bounded wait between the blocks of a token-shift
+ * vector's kernel ran out; the images since the last check are not to be used.
  */
 rwkvq_status rwkvq_quantize_dev_async(const void* w_fp16_dev, int oc, int ic, const rwkvq_quant_cfg* cfg,
                                       const float* elem_weight_dev, void* image_dev, size_t image_bytes,

@@ -61,14 +61,18 @@ int sm_count();
 unsigned long long context_id();
 
 // The opt-in to more than 48 KB of dynamic shared memory holds for a kernel as long as the context: it is asked for once (about 1 us of host
-// time) and not at every launch.  One object per kernel, `bytes` the same at every call.
+// time) and not at every launch.  One object per kernel, `bytes` the same at every call.  `wide`: clusters of more than eight blocks as well.
 struct SmemOptIn {
   std::atomic<unsigned long long> context[kMaxDevices];      // in which it was asked for
+  const bool wide = false;
+  SmemOptIn() = default;
+  explicit SmemOptIn(bool wide_clusters) : context{}, wide(wide_clusters) {}
   cudaError_t operator()(const void* fn, int bytes) {
     const int dev = current_device();
     const unsigned long long id = dev >= 0 ? context_id() : 0ull;
     if (id != 0 && context[dev].load(std::memory_order_relaxed) == id) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && wide) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess && id != 0) context[dev].store(id, std::memory_order_relaxed);
     return e;
   }

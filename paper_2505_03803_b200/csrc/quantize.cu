@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "../../include/rwkvq.h"
 #include "format.h"
@@ -16,7 +17,7 @@
 namespace rwkvq {
 namespace {
 
-constexpr int kFlagNonFinite = 1;
+constexpr int kFlagNonFinite = 1, kFlagTimeout = 2;
 
 // The first block of a quantizer kernel also writes the image's header and clears the alignment padding behind its last section
 // (a launch and a memset of their own took as long as quantizing a small matrix).
@@ -306,7 +307,7 @@ __device__ __forceinline__ void join_group(ClusterSums& s, const uint32_t* vec, 
 // fp16 pairs (read 16 bytes at a time, the pieces of a thread's row rotated against bank conflicts).  Bound by
 // the instructions of the distance update: two conversions a vector, four packed operations per two, a minimum and a running sum.
 // Seeds are vectors of the tile, so the codebook area of the image holds them exactly until the centres are final.  A token-shift vector of n
-// vectors is seeded alike by one block of n / 2048 warps.
+// vectors, more than kVecSeeds, is seeded alike by one block of n / 2048 warps.
 constexpr int kVqWarps = kVqThreads / 32;
 __device__ __forceinline__ int vq_slot(int i) { return (i & ~63) | ((((i >> 2) ^ (i >> 6)) & 7) << 2) | (i & 35); }
 
@@ -812,371 +813,464 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
 
 // ---- token-shift vectors ----
 //
-// Weighted vectors are assigned by a cluster of kVecCluster, whose blocks take a part of the vectors each and
-// write what they find into the first block's shared memory; that block sorts the members by centre (stable), and every centre
-// adds its own in vector order.  Bound by the latency of the running sums: of the seeds' distances and of the longest
-// centre's members.  2048 weighted vectors, 64 centres, ten iterations: 145 us with the seeds (237 before: one block for
-// everything, seeds' distances in shared memory, two compare-and-selects for each distance, members counted and ranked
-// twice by match, sums in chains of dependent loads and conversions, the final distances all in fp64).
-constexpr int kVecThreads = 1024, kVecCluster = 8;
-// The search for the nearest centre takes the minimum over groups of eight centres, one instruction a distance, and looks for the centre only
-// in the group that wins.  One slot of padding per group: lanes that look in different groups read different banks.
+// One cluster a call.  Every block draws all the seeds (up to kVecSeeds vectors: sixteen a thread in registers; a longer vector is
+// seeded by vq_seed_kernel) and then keeps a part of the vectors.  An iteration: four lanes a vector, each against a quarter of the
+// centres; the members of a centre become bit masks, from which four sums a centre (of w * v and of w in either dimension; exact integers
+// without weights) are added in a fixed order; every block sends its sums to the block that has the centre, which adds up those of all blocks and sends
+// the new centre to all.  (Every block sending its sums to all saved that second trip, and took longer for the bytes.)  Bound by latency: two barriers
+// a draw (0.42 us), two barriers and two trips through the cluster an iteration (1.65 us).  2048 weighted vectors, 64 centres, ten iterations:
+// 47.6 us; 139 with one warp drawing all seeds by the chains, one block sorting the members by centre and adding them up, and a barrier of the
+// cluster at either end of it.  256 centres, 2560 vectors: 166 us, 418 then.
+constexpr int kVecThreads = 512, kVecWarps = kVecThreads / 32;
+constexpr int kVecCluster = 16;                  // blocks
+constexpr int kSeedPer = 16, kVecSeeds = 4096, kSeedWarps = kVecSeeds / (32 * kSeedPer);
+constexpr int kVecParts = 4;                     // lanes a vector
+constexpr int kVecRound = kVecThreads / kVecParts;      // vectors a block compares at a time
+constexpr int kVecGroups = 32;                   // groups of 32 vectors whose members a block adds up at a time
+// The search for the nearest centre takes the minimum over groups of eight centres, less than one instruction a distance, and looks for the
+// centre only in the group that wins.
 constexpr int kCentreGroup = 8;
-__host__ __device__ constexpr int centre_slot(int e) { return e + e / kCentreGroup; }
-struct VecShared {
-  double cx[kVqMaxE], cy[kVqMaxE];
-  float4 neg[kVqMaxE + kVqMaxE / kCentreGroup];   // (-x, -x, -y, -y) of a centre, in groups, see centre_slot
-  uint16_t hist[kVecThreads / 32][kVqMaxE + 2];   // members per warp's share and centre, then those of the shares before it; a column is read by a warp
-  int first[kVqMaxE + 1];
-  ClusterSums sums;
-  float part_best[kVecCluster][64 * kVecThreads / 32 / kVecCluster];     // nearest centre of a part of them: distance, number
-  uint8_t part_idx[kVecCluster][64 * kVecThreads / 32 / kVecCluster];
+struct VecSeeds {
+  float tot[kSeedWarps], run_tot[kVecSeeds / 2048];
+  float u01[kVqMaxE];
+  int pick[kVqMaxE];                             // -1: not decided
+  float dist[kVecSeeds / 64 * 65];               // runs of 64, each in banks of its own
+  __align__(16) uint32_t vec[kVecSeeds];
 };
-// Up to this many vectors the first block keeps, in fp64, w * v and w of either dimension: a conversion to fp64 takes four times a
-// multiply-add's time, and a member of a centre is converted once instead of in each iteration.
-constexpr int kVecTable = 4096;
-__host__ __device__ constexpr size_t vec_smem_bytes(int n) {
-  const size_t rows = ((size_t)n + 63) / 64;
-  return (sizeof(VecShared) + 15) / 16 * 16 + rows * 320 + (n <= kVecTable ? (size_t)n * 32 : 0);
-}
+constexpr int kGroupSlots = kCentreGroup / 2 + 1;      // one of padding: lanes that look in different groups read different banks
+template <int E>
+struct VecShared {
+  double c[2][E];                                // centres
+  float4 neg[E / kCentreGroup * kGroupSlots];    // (-x, -x', -y, -y') of two neighbouring centres, rounded to fp32, in groups
+  uint64_t sums_here, centres_here;              // barriers of what the other blocks send
+  double sent[E][2];                             // centres, from the block that has them
+  ulonglong2 part[kVecCluster][E / kVecCluster][2];    // (of w * v, of w) of this block's centres in either dimension, from every block
+  uint32_t seed[E];
+  __align__(16) uint32_t mask[2][E][kVecGroups + 4];   // members of a centre in each group of 32; one is cleared while the other is filled
+  uint8_t idx[kVqMaxVec / kVecCluster];
+  VecSeeds s;
+  ulonglong2 table[kVecGroups * 32][2];          // (w * v, w) in either dimension of the block's vectors, if there are no more
+};
+static_assert(sizeof(VecShared<256>) <= 232448, "shared memory of a block");
 
 // The cluster: barrier, and stores to the shared memory of a block of it at the address that `local` has here.
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ void cluster_sync() {
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t peer_address(const void* local, uint32_t rank) {
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t peer_address(uint32_t local, uint32_t rank) {
   uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void peer_store8(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
-__device__ __forceinline__ void peer_store16(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(at), "h"((uint16_t)v) : "memory"); }
-__device__ __forceinline__ void peer_store(uint32_t at, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+// A store to a block of the cluster that its barrier `bar` counts.
+__device__ __forceinline__ void peer_send(uint32_t at, ulonglong2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(at), "l"(v.x), "l"(v.y), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void peer_store(uint32_t at, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory"); }
-
-// Two vectors against all centres, distances rounded as d = w.x * (dx * dx) + (w.y * (dy * dy)) with the last product and sum in one
-// rounding (unweighted: dx * dx + (dy * dy), likewise).
-struct Nearest {
-  float best[2], second[2];     // smallest minimum of a group, and of the other groups
-  int group[2];                 // first centre of the first group with that minimum
-};
-__device__ __forceinline__ float2 pair_distance(bool weighted, float2 x, float2 y, float2 wx, float2 wy, float4 c) {
-  const float2 dx = add2(x, make_float2(c.x, c.y)), dy = add2(y, make_float2(c.z, c.w)), yy = mul2(dy, dy);
-  return weighted ? fma2(wx, mul2(dx, dx), mul2(wy, yy)) : fma2(dx, dx, yy);
+__device__ __forceinline__ void peer_send(uint32_t at, unsigned long long v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at), "l"(v), "r"(bar) : "memory");
 }
-__device__ __forceinline__ Nearest nearest_group(const float4* neg, int E, bool weighted, float2 x, float2 y, float2 wx, float2 wy) {
-  Nearest r;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) { r.best[q] = r.second[q] = INFINITY; r.group[q] = 0; }
-#pragma unroll 1
-  for (int e = 0; e < E; e += kCentreGroup) {
-    float2 m = make_float2(INFINITY, INFINITY);
-#pragma unroll
-    for (int k = 0; k < kCentreGroup; ++k) {
-      const float2 d = pair_distance(weighted, x, y, wx, wy, neg[centre_slot(e) + k]);
-      m = make_float2(fminf(m.x, d.x), fminf(m.y, d.y));
-    }
-    const float mm[2] = {m.x, m.y};
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      r.second[q] = fminf(r.second[q], fmaxf(r.best[q], mm[q]));
-      if (mm[q] < r.best[q]) { r.best[q] = mm[q]; r.group[q] = e; }
-    }
+__device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void expect_sent(uint32_t bar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Waits for a phase of a barrier of this block that stores of the cluster complete; gives up after some seconds.
+__device__ __forceinline__ bool wait_sent(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < (1 << 24); ++i) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
   }
-  return r;
-}
-__device__ __forceinline__ float one_distance(bool weighted, float x, float y, float wx, float wy, float4 c) {
-  const float dx = __fadd_rn(x, c.x), dy = __fadd_rn(y, c.z), yy = __fmul_rn(dy, dy);
-  return weighted ? __fmaf_rn(wx, __fmul_rn(dx, dx), __fmul_rn(wy, yy)) : __fmaf_rn(dx, dx, yy);
+  return false;
 }
 
+// Draws E seeds; a draw is defined as in vq_seed_kernel: distances summed in fp32 over runs of 64 vectors in order, run sums by a scan over the lanes
+// of a warp, and the last vector whose running sum begins at or below the target.  Those chains are 64 additions long, twice a draw.  So the
+// sums are taken in a tree first: with u = 2^-24, the chains' running sums are off by at most 148 u of themselves and their target by 84 u, the
+// tree's by 23 u and 20 u (its differences from the target by three more), so a vector whose running sums begin and end at least 320 u of the target away from it (and on either side)
+// is the one that the chains give.  Otherwise (one draw in 25 for 2048 vectors) the chains are walked.
+// Called by the first `threads` threads, which hold sixteen vectors each.
+__device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n, int E, uint64_t seed, int threads) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = kSeedPer * tid;
+  auto sync = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); };
+  float2 x[kSeedPer / 2], y[kSeedPer / 2];
+  float dist[kSeedPer];
+#pragma unroll
+  for (int k = 0; k < kSeedPer; k += 4) {
+    const uint4 q = *reinterpret_cast<const uint4*>(sh.vec + base + k);
+    const float2 a = vec_of(q.x), b = vec_of(q.y), c = vec_of(q.z), d = vec_of(q.w);
+    x[k / 2] = make_float2(a.x, b.x); x[k / 2 + 1] = make_float2(c.x, d.x);
+    y[k / 2] = make_float2(a.y, b.y); y[k / 2 + 1] = make_float2(c.y, d.y);
+  }
+#pragma unroll
+  for (int k = 0; k < kSeedPer; ++k) dist[k] = base + k < n ? INFINITY : 0.f;
+  uint32_t cv = sh.vec[below(splitmix(seed, 0), n)];
+  for (int e = 0;; ++e) {
+    if (tid == 0) seeds[e] = cv;
+    if (e + 1 == E) break;
+    const float u01 = sh.u01[e + 1];
+    const float2 c = vec_of(cv);
+    const float2 ncx = make_float2(-c.x, -c.x), ncy = make_float2(-c.y, -c.y);
+#pragma unroll
+    for (int k = 0; k < kSeedPer / 2; ++k) {
+      const float2 dx = add2(x[k], ncx), dy = add2(y[k], ncy), d = fma2(dx, dx, mul2(dy, dy));
+      dist[2 * k] = fminf(dist[2 * k], d.x); dist[2 * k + 1] = fminf(dist[2 * k + 1], d.y);
+    }
+    float sum[kSeedPer + 1];                       // sum[k]: of the first k
+    sum[0] = 0.f;
+    {
+      float two[kSeedPer / 2], four[kSeedPer / 4];
+#pragma unroll
+      for (int k = 0; k < kSeedPer / 2; ++k) two[k] = dist[2 * k] + dist[2 * k + 1];
+#pragma unroll
+      for (int k = 0; k < kSeedPer / 4; ++k) four[k] = two[2 * k] + two[2 * k + 1];
+      sum[4] = four[0]; sum[8] = four[0] + four[1]; sum[16] = sum[8] + (four[2] + four[3]); sum[12] = sum[8] + four[2];
+#pragma unroll
+      for (int k = 0; k < kSeedPer; k += 4) {
+        sum[k + 1] = sum[k] + dist[k];
+        sum[k + 2] = sum[k] + two[k / 2];
+        sum[k + 3] = sum[k + 2] + dist[k + 2];
+      }
+      static_assert(kSeedPer == 16, "sums of a thread");
+    }
+    float incl = sum[kSeedPer];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const float v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+      if (lane >= off) incl += v;
+    }
+    if (lane == 31) sh.tot[warp] = incl;
+    sync();
+    float t[kSeedWarps];                           // zeros behind the last warp
+#pragma unroll
+    for (int w = 0; w < kSeedWarps; w += 4) {
+      const float4 t4 = *reinterpret_cast<const float4*>(sh.tot + w);
+      t[w] = t4.x; t[w + 1] = t4.y; t[w + 2] = t4.z; t[w + 3] = t4.w;
+    }
+    float before[kSeedWarps];
+#pragma unroll
+    for (int w = 0; w < kSeedWarps; ++w) before[w] = w < warp ? t[w] : 0.f;
+#pragma unroll
+    for (int h = kSeedWarps / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int w = 0; w < h; ++w) { t[w] += t[w + h]; before[w] += before[w + h]; }
+    const float target = u01 * t[0], margin = target * (320.f / 16777216.f);
+    const float rest = target - (before[0] + (incl - sum[kSeedPer]));
+    const float under = rest - margin, over = rest + margin;
+    if (sum[0] <= under && sum[kSeedPer] > over) {
+      // the last that begins at or below, by halves
+      int at = base;
+      float win[kSeedPer + 1];
+#pragma unroll
+      for (int k = 0; k <= kSeedPer; ++k) win[k] = sum[k];
+#pragma unroll
+      for (int h = kSeedPer / 2; h > 0; h >>= 1) {
+        const bool upper = win[h] <= under;
+        at += upper ? h : 0;
+#pragma unroll
+        for (int k = 0; k <= h; ++k) win[k] = upper ? win[k + h] : win[k];
+      }
+      if (win[1] > over) sh.pick[e + 1] = at;
+    }
+    sync();
+    const int pick = sh.pick[e + 1];
+    cv = sh.vec[max(pick, 0)];
+    if (pick >= 0) continue;
+    // the chains; thread t < n / 64 has run t
+#pragma unroll
+    for (int k = 0; k < kSeedPer; ++k) sh.dist[base + k + (base >> 6)] = dist[k];
+    sync();
+    const int runs = (n + 2047) / 2048 * 32;
+    const float* run = sh.dist + 65 * tid;
+    const bool holds = tid < runs && 64 * tid < kSeedPer * threads;        // `threads` is a multiple of 32: whole runs
+    float excl = 0.f;
+    if (tid < runs) {
+      float chain = 0.f;
+      if (holds) {
+#pragma unroll 16
+        for (int k = 0; k < 64; ++k) chain += run[k];
+      }
+      incl = chain;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const float v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+        if (lane >= off) incl += v;
+      }
+      if (lane == 31) sh.run_tot[warp] = incl;
+      excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+      if (lane == 0) excl = 0.f;
+    }
+    if (tid == 0) sh.pick[e + 1] = n - 1;
+    sync();
+    const float first = warp == 1 ? sh.run_tot[0] : 0.f, total = sh.run_tot[0] + (runs > 32 ? sh.run_tot[1] : 0.f);
+    excl = first + excl;
+    incl = first + incl;
+    if (!(total > 0.f)) {
+      if (tid == 0) sh.pick[e + 1] = below(splitmix(seed, e + 1), n);
+    } else if (holds && excl <= u01 * total && u01 * total < incl) {
+      int last = 64 * tid;
+#pragma unroll 16
+      for (int k = 0; k < 64; ++k) {
+        if (excl <= u01 * total && 64 * tid + k < n) last = 64 * tid + k;
+        excl += run[k];
+      }
+      sh.pick[e + 1] = last;
+    }
+    sync();
+    cv = sh.vec[sh.pick[e + 1]];
+  }
+}
+
+// Distances of a vector to two centres, each rounded as d = w.x * (dx * dx) + (w.y * (dy * dy)) with the last product and sum in one
+// rounding (unweighted: dx * dx + (dy * dy), likewise).
+template <bool kWeighted>
+__device__ __forceinline__ float2 pair_distance(float2 f, float2 w, float4 c) {
+  const float2 dx = add2(make_float2(f.x, f.x), make_float2(c.x, c.y)), dy = add2(make_float2(f.y, f.y), make_float2(c.z, c.w)), yy = mul2(dy, dy);
+  return kWeighted ? fma2(make_float2(w.x, w.x), mul2(dx, dx), mul2(make_float2(w.y, w.y), yy)) : fma2(dx, dx, yy);
+}
+
+__device__ __forceinline__ constexpr int neg_slot(int e) { return e / kCentreGroup * kGroupSlots + e % kCentreGroup / 2; }
+template <class T> struct alignas(16) VecSums { T wv, w; };
+template <int E, bool kWeighted>
 __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs a, const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
   extern __shared__ __align__(16) uint8_t smem[];
-  VecShared& sh = *reinterpret_cast<VecShared*>(smem);
-  uint8_t* rest = smem + (sizeof(VecShared) + 15) / 16 * 16;
+  VecShared<E>& sh = *reinterpret_cast<VecShared<E>*>(smem);
+  using Sums = VecSums<typename std::conditional<kWeighted, double, long long>::type>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = a.n_vec, E = a.E, rows = (n + 63) / 64;
-  const bool weighted = a.elem_w != nullptr;
+  const int n = a.n_vec;
   const uint32_t* vec = reinterpret_cast<const uint32_t*>(a.w);
   const float2* wgt = reinterpret_cast<const float2*>(a.elem_w);
-  const uint32_t rank = cluster_rank(), peers = cluster_size();
+  const uint32_t rank = cluster_rank();
   const bool lead = rank == 0u;
   if (lead) write_header(head, image);
-  for (int e = E + tid; e < (E + kCentreGroup - 1) / kCentreGroup * kCentreGroup; e += kVecThreads)      // no centre is nearer than these
-    sh.neg[centre_slot(e)] = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-  // tables of the first block, behind the assignment (bytes), the ranks of the members and the members sorted by centre (16-bit numbers)
-  const bool tables = n <= kVecTable;
-  double2* const table_wv = reinterpret_cast<double2*>(rest + (size_t)rows * 320);      // [n] w * v
-  double2* const table_w = table_wv + n;
-  uint8_t* idx = rest;                                             // [rows * 64]
-  if (lead) {
-    if (tables && weighted) {
-      for (int i = tid; i < n; i += kVecThreads) {
-        const uint32_t v = __ldg(vec + i);
-        const float2 wi = __ldg(wgt + i);
-        const double wx = (double)wi.x, wy = (double)wi.y;
-        table_w[i] = make_double2(wx, wy);
-        table_wv[i] = make_double2(wx * (double)h2f_bits(v & 0xFFFFu), wy * (double)h2f_bits(v >> 16));      // exact: 24 and 11 bits
-      }
+  // this block's vectors: [begin, begin + 32 * groups), those below n
+  const int groups = (n + 32 * kVecCluster - 1) / (32 * kVecCluster), begin = (int)rank * groups * 32;
+  const int pass_groups = min(groups, kVecGroups);
+  const bool one_pass = groups <= kVecGroups;
+  const uint32_t sums_here = shared_address(&sh.sums_here), centres_here = shared_address(&sh.centres_here);
+  // summands of vector i in one dimension
+  auto summands = [&](int i, int dim) -> Sums {
+    const uint32_t v = __ldg(a.w + 2 * i + dim);
+    if constexpr (kWeighted) {
+      const double w = (double)__ldg(a.elem_w + 2 * i + dim);
+      return Sums{w * (double)h2f_bits(v), w};                     // the product of 24 and 11 bits is exact
+    } else {
+      return Sums{half_fixed(v), 1};
     }
+  };
+  Sums* const table = reinterpret_cast<Sums*>(sh.table);
+  if (one_pass)
+    for (int k = tid; k < groups * 64; k += kVecThreads)
+      if (begin + (k >> 1) < n) table[k] = summands(begin + (k >> 1), k & 1);
+  // neighbouring lanes compare one vector
+  const int in_four = lane & (kVecParts - 1), in_round = warp * (32 / kVecParts) + lane / kVecParts;
+  float2 f, w = make_float2(1.f, 1.f);
+  auto fetch = [&](int i0) {
+    const int i = min(i0 + in_round, n - 1);
+    f = vec_of(__ldg(vec + i));
+    if (kWeighted) w = __ldg(wgt + i);
+  };
+  fetch(begin);
+  if (tid == 0)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n mbarrier.init.shared::cta.b64 [%1], 1;\n fence.mbarrier_init.release.cluster;" ::"r"(sums_here), "r"(centres_here) : "memory");
+  if (n <= kVecSeeds) {
+    const int warps = (n + 32 * kSeedPer - 1) / (32 * kSeedPer);
+    bool bad = false;
+    for (int i = tid; i < warps * 32 * kSeedPer; i += kVecThreads) {
+      const uint32_t v = i < n ? __ldg(vec + i) : 0u;
+      bad |= ((v & 0x7C00u) == 0x7C00u) | ((v & 0x7C000000u) == 0x7C000000u);
+      sh.s.vec[i] = v;
+    }
+    if (bad && lead) atomicOr(a.flags, kFlagNonFinite);
+    if (tid < kSeedWarps) sh.s.tot[tid] = 0.f;
+    if (tid < E) { sh.s.u01[tid] = (float)unit_of(splitmix(a.seed, tid)); sh.s.pick[tid] = -1; }
+    __syncthreads();
+    if (warp < warps) draw_seeds(sh.s, sh.seed, n, E, a.seed, 32 * warps);
+  } else {
     // the seeds lie where the codebook will
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int e = tid; e < E; e += kVecThreads) {
-      const float2 c = vec_of(__ldcg(a.aux + e));
-      sh.cx[e] = (double)c.x; sh.cy[e] = (double)c.y;
-    }
-    __syncthreads();
+    if (tid < E) sh.seed[tid] = __ldcg(a.aux + tid);
   }
-  uint16_t* ranks = reinterpret_cast<uint16_t*>(rest + rows * 64);   // [rows * 64]: members of the same centre before it in the warp's share
-  uint16_t* sorted = ranks + rows * 64;                             // [rows * 64]
-  // Negated centres, in fp32, to every block.
-  auto publish = [&]() {
-    for (int k = tid; k < E * (int)peers; k += kVecThreads) {
-      const int e = k % E;
-      const float cx = (float)sh.cx[e], cy = (float)sh.cy[e];
-      peer_store(peer_address(&sh.neg[centre_slot(e)], (uint32_t)(k / E)), make_float4(-cx, -cx, -cy, -cy));
-    }
+  __syncthreads();
+  auto set_centre = [&](int e, int dim, double c) {
+    sh.c[dim][e] = c;
+    reinterpret_cast<float*>(sh.neg + neg_slot(e))[2 * dim + (e & 1)] = -(float)c;
   };
-  // ---- Lloyd iterations.  Share k of the vectors is [k * share, (k + 1) * share), taken 64 at a time by the warps of block
-  // k / shares that have this share, each with a part of the centres; the first of them goes on with the nearest of all.
-  constexpr int kShares = kVecThreads / 32;
-  const int share = ((n + kVecThreads - 1) / kVecThreads) * 32, shares = kShares / (int)peers, parts = (int)peers, part = warp / shares, mine = (int)rank * shares + warp % shares;
-  const int part_e0 = E * part / parts, part_e1 = E * (part + 1) / parts;
-  const uint32_t lead_idx = peer_address(idx, 0u), lead_ranks = peer_address(ranks, 0u);
-  uint16_t* const hist = sh.hist[mine];
-  uint32_t v[2];
-  float2 wv[2] = {make_float2(1.f, 1.f), make_float2(1.f, 1.f)};
-  auto fetch = [&](int i0) {
+  if (tid < 2 * E) set_centre(tid >> 1, tid & 1, (double)h2f_bits((sh.seed[tid >> 1] >> (16 * (tid & 1))) & 0xFFFFu));
+  auto clear_masks = [&](int which) {
+    for (int k = tid; k < E * 8; k += kVecThreads) *reinterpret_cast<uint4*>(&sh.mask[which][k >> 3][4 * (k & 7)]) = make_uint4(0u, 0u, 0u, 0u);
+  };
+  clear_masks(0);
+  cluster_arrive();                                // every block runs and has its seeds: sums may be sent
+  cluster_wait();
+  // The nearest centre of this lane's vector, the first of equally near ones, known to all four lanes.  `alone`: no other centre is within 2^-20
+  // of its distance, which is `best`.
+  auto nearest = [&](float& best, bool* alone) -> int {
+    int group = 0;
+    best = INFINITY;
+    float next = INFINITY;                         // smallest minimum of another group
+#pragma unroll 2
+    for (int g = in_four; g < E / kCentreGroup; g += kVecParts) {
+      float d[kCentreGroup];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = min(i0 + 32 * q + lane, n - 1);
-      v[q] = __ldg(vec + i);
-      if (weighted) wv[q] = __ldg(wgt + i);
+      for (int k = 0; k < kCentreGroup / 2; ++k) {
+        const float2 two = pair_distance<kWeighted>(f, w, sh.neg[g * kGroupSlots + k]);
+        d[2 * k] = two.x; d[2 * k + 1] = two.y;
+      }
+      const float m = fminf(fminf(fminf(d[0], d[1]), fminf(d[2], d[3])), fminf(fminf(d[4], d[5]), fminf(d[6], d[7])));
+      if (alone) next = fminf(next, fmaxf(best, m));
+      if (m < best) { best = m; group = g; }
     }
+#pragma unroll
+    for (int off = 1; off < kVecParts; off <<= 1) {
+      const float b = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+      const int g = __shfl_xor_sync(0xFFFFFFFFu, group, off);
+      if (alone) next = fminf(fminf(next, __shfl_xor_sync(0xFFFFFFFFu, next, off)), fmaxf(best, b));
+      if (b < best || (b == best && g < group)) { best = b; group = g; }
+    }
+    // each lane looks at two centres of the group
+    static_assert(2 * kVecParts == kCentreGroup, "a pair of centres a lane");
+    const float2 two = pair_distance<kWeighted>(f, w, sh.neg[group * kGroupSlots + in_four]);
+    int at = two.x == best ? 2 * in_four : two.y == best ? 2 * in_four + 1 : kCentreGroup;
+    int close = 0;
+    if (alone) {
+      const float limit = best * (1.f + 1.f / 1048576.f);
+      close = (two.x <= limit) + (two.y <= limit);
+      *alone = next > limit;
+    }
+#pragma unroll
+    for (int off = 1; off < kVecParts; off <<= 1) {
+      at = min(at, __shfl_xor_sync(0xFFFFFFFFu, at, off));
+      if (alone) close += __shfl_xor_sync(0xFFFFFFFFu, close, off);
+    }
+    if (alone) *alone &= close == 1;
+    return best < INFINITY ? group * kCentreGroup + at : 0;
   };
-  fetch(mine * share);                             // a share of 64 stays in registers
-  cluster_sync();                                  // every block runs: their shared memory may be written
-  if (lead) publish();
+  // Two threads add up the members of centre e in dimension `dim` (one thread, of 256 centres), two words of masks at a time; the block that has
+  // the centre, and its place there:
+  constexpr int kSplit = E == 64 ? 2 : 1;
+  const int dim = tid & 1, split = (tid >> 1) % kSplit, e = tid / (2 * kSplit);
+  constexpr int kOwn = E / kVecCluster;            // centres a block has
+  const uint32_t owner = (uint32_t)(e / kOwn), my_part = peer_address(shared_address(&sh.part[rank][e % kOwn][dim]), owner), owner_bar = peer_address(sums_here, owner);
+  // ... and kOwn * 2 * kVecCluster of them look after one of this block's centres, for one receiver each
+  const int own = tid / (2 * kVecCluster), own_dim = tid / kVecCluster % 2;
+  const uint32_t receiver = (uint32_t)(tid % kVecCluster);
+  bool lost = false;
+  int which = 0;
   for (int it = 0; it < a.iters; ++it) {
-    if (!weighted) {
-      for (int e = tid; e < E; e += kVecThreads) {
-#pragma unroll
-        for (int p = 0; p < 3; ++p) sh.sums.x[p][e] = sh.sums.y[p][e] = 0;
-        sh.sums.cnt[e] = 0;
+    Sums sum{0, 0};
+    for (int g0 = 0; g0 < groups; g0 += pass_groups) {
+      for (int r0 = 0; r0 < pass_groups * 32; r0 += kVecRound) {
+        const int i0 = begin + g0 * 32 + r0, k = r0 + in_round;
+        if (groups * 32 > kVecRound) fetch(i0);
+        if (k - lane / kVecParts >= pass_groups * 32) continue;      // the whole warp has none
+        float best;
+        const int at = nearest(best, nullptr);
+        if (in_four == 0 && k < pass_groups * 32 && g0 * 32 + k < groups * 32 && i0 + in_round < n) atomicOr(&sh.mask[which][at][k >> 5], 1u << (k & 31));
       }
-    }
-    if (part == 0) for (int e = lane; e < E; e += 32) hist[e] = 0;
-    cluster_sync();
-    for (int i0 = mine * share; i0 < min(n, (mine + 1) * share); i0 += 64) {
-      // two vectors per lane: the packed operations take both
-      const int i[2] = {i0 + lane, i0 + 32 + lane};
-      const int stop = min(n, (mine + 1) * share);
-      if (share > 64) fetch(i0);
-      const float2 f0 = vec_of(v[0]), f1 = vec_of(v[1]);
-      const float2 x = make_float2(f0.x, f1.x), y = make_float2(f0.y, f1.y), wx = make_float2(wv[0].x, wv[1].x), wy = make_float2(wv[0].y, wv[1].y);
-      float best[2] = {INFINITY, INFINITY};
-      int bi2[2] = {0, 0};
-#pragma unroll 8
-      for (int e = part_e0; e < part_e1; ++e) {
-        const float2 d = pair_distance(weighted, x, y, wx, wy, sh.neg[centre_slot(e)]);
-        if (d.x < best[0]) { best[0] = d.x; bi2[0] = e; }
-        if (d.y < best[1]) { best[1] = d.y; bi2[1] = e; }
-      }
-      if (parts > 1) {
-        const int at = (warp % shares) * 64 + lane;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) { sh.part_best[part][at + 32 * q] = best[q]; sh.part_idx[part][at + 32 * q] = (uint8_t)bi2[q]; }
-        asm volatile("bar.sync %0, %1;" ::"r"(2 + warp % shares), "r"(32 * parts) : "memory");
-        if (part == 0) {
-#pragma unroll
-          for (int k = 1; k < kVecCluster; ++k)      // parts in the order of their centres: the first of equal distances stays
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const float b = sh.part_best[k][at + 32 * q];
-              const int e = sh.part_idx[k][at + 32 * q];
-              if (b < best[q]) { best[q] = b; bi2[q] = e; }
-            }
-        }
-        if (share > 64) asm volatile("bar.sync %0, %1;" ::"r"(2 + warp % shares), "r"(32 * parts) : "memory");
-        if (part != 0) continue;
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int bi = bi2[q];
-        const bool in = i[q] < stop;
-        if (in) peer_store8(lead_idx + (uint32_t)i[q], (uint32_t)bi);
-        if (!weighted) {
-          if (in) move_member(sh.sums, v[q], bi, 1);
-        } else {
-          const unsigned live = __ballot_sync(0xFFFFFFFFu, in);
-          if (in) {
-            const unsigned same = __match_any_sync(live, bi), below = same & ((1u << lane) - 1u);
-            const int before = hist[bi];
-            __syncwarp(live);
-            peer_store16(lead_ranks + 2u * (uint32_t)i[q], (uint32_t)(before + __popc(below)));
-            if (below == 0u) hist[bi] = (uint16_t)(before + __popc(same));
-          }
-          __syncwarp();
-        }
-      }
-    }
-    if (weighted && !lead && part == 0) {
-      const uint32_t to = peer_address(hist, 0u);
-      for (int e = lane; e < E; e += 32) peer_store16(to + 2u * (uint32_t)e, hist[e]);
-    }
-    cluster_sync();
-    if (!lead) continue;
-    if (!weighted) {
-      for (int e = tid; e < E; e += kVecThreads) {
-        const int cnt = sh.sums.cnt[e];
-        if (cnt) { sh.cx[e] = mean_of_pieces(sh.sums.x, e, cnt); sh.cy[e] = mean_of_pieces(sh.sums.y, e, cnt); }
-      }
-    } else {
-      // weighted means of Eq. 19, per dimension, members added in vector order: a stable sort by centre, then one thread
-      // per centre and dimension
-      for (int e = warp; e < E; e += kVecThreads / 32) {      // lane = share
-        const int mine = sh.hist[lane][e];
-        int s = mine;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int o = __shfl_up_sync(0xFFFFFFFFu, s, off);
-          if (lane >= off) s += o;
-        }
-        sh.hist[lane][e] = (uint16_t)(s - mine);
-        if (lane == 31) sh.first[e + 1] = s;
-      }
+      clear_masks(which ^ 1);
       __syncthreads();
-      if (warp == 0) {
-        int carry = 0;
-        for (int e0 = 0; e0 < E; e0 += 32) {
-          int s = e0 + lane < E ? sh.first[e0 + lane + 1] : 0;
-#pragma unroll
-          for (int off = 1; off < 32; off <<= 1) {
-            const int o = __shfl_up_sync(0xFFFFFFFFu, s, off);
-            if (lane >= off) s += o;
-          }
-          if (e0 + lane < E) sh.first[e0 + lane + 1] = carry + s;
-          carry += __shfl_sync(0xFFFFFFFFu, s, 31);
-        }
-        if (lane == 0) sh.first[0] = 0;
-      }
-      __syncthreads();
-      for (int i = warp * share + lane; i < min(n, (warp + 1) * share); i += 32) {
-        const int e = idx[i];
-        sorted[sh.first[e] + sh.hist[warp][e] + ranks[i]] = (uint16_t)i;
-      }
-      __syncthreads();
-      // four threads a centre: the sums of w * v and of w, of either dimension
-      for (int k = tid; k < 4 * E; k += kVecThreads) {
-        const int e = k >> 2, dim = k & 1;
-        const bool den = (k & 2) != 0;
-        double sum = 0.0;
-        const int stop = sh.first[e + 1];
-        // eight members at a time; past the end the last one again, times zero
-        if (tables) {
-          const double* table = reinterpret_cast<const double*>(den ? table_w : table_wv) + dim;
-          for (int j = sh.first[e]; j < stop; j += 8) {
-            double v[8];
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-              v[m] = table[2 * sorted[min(j + m, stop - 1)]];
-              if (j + m >= stop) v[m] = 0.0;
+      if (tid < 2 * E * kSplit) {
+        auto add_members = [&](auto member) {
+          for (int g = 2 * split; g < pass_groups; g += 2 * kSplit) {
+            uint2 m = *reinterpret_cast<const uint2*>(&sh.mask[which][e][g]);
+            while (m.x | m.y) {
+              const int kx = 31 - __clz((int)m.x), ky = 31 - __clz((int)m.y);       // -1: none left
+              Sums x{0, 0}, y{0, 0};
+              if (kx >= 0) x = member(32 * g + kx);
+              if (ky >= 0) y = member(32 * g + 32 + ky);
+              m.x &= ~(1u << (kx & 31)); m.y &= ~(1u << (ky & 31));
+              sum.wv += x.wv + y.wv; sum.w += x.w + y.w;
             }
-#pragma unroll
-            for (int m = 0; m < 8; ++m) sum += v[m];
           }
-        } else {
-          for (int j = sh.first[e]; j < stop; j += 8) {
-            float wi[8], f[8];
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-              const int i = sorted[min(j + m, stop - 1)];
-              wi[m] = j + m < stop ? __ldg(a.elem_w + 2 * i + dim) : 0.f;
-              f[m] = den ? 1.f : h2f_bits(__ldg(a.w + 2 * i + dim));
-            }
-#pragma unroll
-            for (int m = 0; m < 8; ++m) sum = fma((double)wi[m], (double)f[m], sum);      // the product of 24 and 11 bits is exact
-          }
-        }
-        const unsigned four = 0xFu << (lane & 28);
-        const double weight = __shfl_xor_sync(four, sum, 2);
-        if (!den && weight > 0.0) (dim ? sh.cy : sh.cx)[e] = sum / weight;
+        };
+        if (one_pass) add_members([&](int k) { return table[2 * k + dim]; });
+        else add_members([&](int k) { return summands(begin + g0 * 32 + k, dim); });
       }
+      if (!one_pass) __syncthreads();
+      which ^= 1;
+    }
+    if (kSplit == 2) { sum.wv += __shfl_xor_sync(0xFFFFFFFFu, sum.wv, 2); sum.w += __shfl_xor_sync(0xFFFFFFFFu, sum.w, 2); }
+    if (tid == 0) { expect_sent(sums_here, (int)sizeof(sh.part)); expect_sent(centres_here, (int)sizeof(sh.sent)); }
+    if (tid < 2 * E * kSplit && split == 0) {
+      ulonglong2 bits;
+      if constexpr (kWeighted) bits = make_ulonglong2((unsigned long long)__double_as_longlong(sum.wv), (unsigned long long)__double_as_longlong(sum.w));
+      else bits = make_ulonglong2((unsigned long long)sum.wv, (unsigned long long)sum.w);
+      peer_send(my_part, bits, owner_bar);
+    }
+    // A block sends its next sums when it has the centres of all blocks, and a block its next centres when it has the next sums of all: neither place is
+    // written again before it has been read.
+    if (tid < 2 * kOwn * kVecCluster) {
+      lost |= !wait_sent(sums_here, (uint32_t)it & 1u);
+      Sums s[kVecCluster];
+#pragma unroll
+      for (int r = 0; r < kVecCluster; ++r) s[r] = reinterpret_cast<const Sums&>(sh.part[r][own][own_dim]);
+#pragma unroll
+      for (int h = 1; h < kVecCluster; h <<= 1)
+#pragma unroll
+        for (int r = 0; r < kVecCluster; r += 2 * h) { s[r].wv += s[r + h].wv; s[r].w += s[r + h].w; }
+      double c = sh.c[own_dim][rank * kOwn + own];
+      __syncwarp();                                // all sixteen threads of a centre have read
+      if (s[0].w > 0) {
+        if constexpr (kWeighted) c = s[0].wv / s[0].w;
+        else c = (double)s[0].wv * (1.0 / 16777216.0) / (double)s[0].w;
+      }
+      peer_send(peer_address(shared_address(&sh.sent[rank * kOwn + own][own_dim]), receiver), (unsigned long long)__double_as_longlong(c), peer_address(centres_here, receiver));
+    }
+    if (tid < 2 * E) {
+      lost |= !wait_sent(centres_here, (uint32_t)it & 1u);
+      set_centre(tid >> 1, tid & 1, sh.sent[tid >> 1][tid & 1]);
     }
     __syncthreads();
-    publish();
   }
+  cluster_arrive();                                // before the end: no block leaves while another might send to it
+  if (lost) atomicOr(a.flags, kFlagTimeout);
   // ---- centres to fp16; final assignment against the rounded centres in fp64
-  cluster_sync();                                  // the last centres are no longer being written
-  if (lead) {
-    for (int e = tid; e < E; e += kVecThreads) {
-      const __half hx = __double2half(sh.cx[e]), hy = __double2half(sh.cy[e]);
-      const float cx = __half2float(hx), cy = __half2float(hy);
-      a.aux[e] = (uint32_t)__half_as_ushort(hx) | ((uint32_t)__half_as_ushort(hy) << 16);
-      for (uint32_t r = 0; r < peers; ++r) {
-        peer_store(peer_address(&sh.neg[centre_slot(e)], r), make_float4(-cx, -cx, -cy, -cy));
-        peer_store(peer_address(&sh.cx[e], r), (double)cx);
-        peer_store(peer_address(&sh.cy[e], r), (double)cy);
-      }
-    }
+  if (tid < 2 * E) {
+    const __half h = __double2half(sh.c[tid & 1][tid >> 1]);
+    if (lead) reinterpret_cast<uint16_t*>(a.aux)[tid] = __half_as_ushort(h);
+    set_centre(tid >> 1, tid & 1, (double)__half2float(h));
   }
-  cluster_sync();
+  __syncthreads();
   // In fp32 first: a distance is wrong by less than seven roundings there, so a centre whose distance is smallest by more than 2^-20 of it is
   // the nearest in fp64 too, and so is one that the vector equals.  The others (and distances near the end of fp32's range) are taken in fp64.
-  const int stride = (int)peers * kVecThreads;
-  for (int i0 = (int)rank * kVecThreads + tid; i0 < n; i0 += 2 * stride) {
-    const int i[2] = {i0, i0 + stride};
-    float2 f[2], wv[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      f[q] = vec_of(__ldg(vec + min(i[q], n - 1)));
-      wv[q] = weighted ? __ldg(wgt + min(i[q], n - 1)) : make_float2(1.f, 1.f);
-    }
-    const Nearest nr = nearest_group(sh.neg, E, weighted, make_float2(f[0].x, f[1].x), make_float2(f[0].y, f[1].y), make_float2(wv[0].x, wv[1].x),
-                                     make_float2(wv[0].y, wv[1].y));
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (i[q] >= n) break;
-      const float limit = nr.best[q] * (1.f + 1.f / 1048576.f);
-      const float4* c = sh.neg + centre_slot(nr.group[q]);
-      int k = 0, close = 0;
-#pragma unroll
-      for (int j = 0; j < kCentreGroup; ++j)
-        if (one_distance(weighted, f[q].x, f[q].y, wv[q].x, wv[q].y, c[j]) <= limit) { k = j; ++close; }
-      int bi = nr.group[q] + k;
-      const bool equal = f[q].x + c[k].x == 0.f && f[q].y + c[k].z == 0.f;
-      if (close != 1 || !(nr.second[q] > limit) || !(equal || (nr.best[q] > 1e-30f && nr.best[q] < 1e30f))) {
-        const double x = (double)f[q].x, y = (double)f[q].y, wx = (double)wv[q].x, wy = (double)wv[q].y;
-        double best = INFINITY;
-        bi = 0;
+  for (int r0 = 0; r0 < groups * 32; r0 += kVecRound) {
+    const int k = r0 + in_round, i = begin + k;
+    if (groups * 32 > kVecRound) fetch(begin + r0);
+    if (k - lane / kVecParts >= groups * 32) continue;
+    float best;
+    bool alone;
+    int at = nearest(best, &alone);
+    const float* neg = reinterpret_cast<const float*>(sh.neg + neg_slot(at)) + (at & 1);
+    const bool equal = f.x + neg[0] == 0.f && f.y + neg[2] == 0.f;
+    if (!alone || !(equal || (best > 1e-30f && best < 1e30f))) {
+      const double x = (double)f.x, y = (double)f.y, wx = (double)w.x, wy = (double)w.y;
+      double lowest = INFINITY;
+      at = 0;
 #pragma unroll 4
-        for (int e = 0; e < E; ++e) {
-          const double dx = x - sh.cx[e], dy = y - sh.cy[e];
-          const double d = weighted ? __dadd_rn(__dmul_rn(wx, __dmul_rn(dx, dx)), __dmul_rn(wy, __dmul_rn(dy, dy)))
-                                    : __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
-          if (d < best) { best = d; bi = e; }
-        }
+      for (int c = 0; c < E; ++c) {
+        const double dx = x - sh.c[0][c], dy = y - sh.c[1][c];
+        const double d = kWeighted ? __dadd_rn(__dmul_rn(wx, __dmul_rn(dx, dx)), __dmul_rn(wy, __dmul_rn(dy, dy)))
+                                   : __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+        if (d < lowest) { lowest = d; at = c; }
       }
-      peer_store8(lead_idx + (uint32_t)i[q], (uint32_t)bi);
     }
+    if (in_four == 0 && k < groups * 32 && i < n) sh.idx[k] = (uint8_t)at;
   }
-  cluster_sync();
-  if (!lead) return;
-  const int bits = a.bits, n_words = (int)(((((size_t)n * bits + 7) / 8 + 15) / 16 * 16) / 4);
-  for (int wi = tid; wi < n_words; wi += kVecThreads) {
+  __syncthreads();
+  // 32 indices are whole words of the bit stream; the last block also writes what it is padded with
+  constexpr int kBits = E == 64 ? 6 : 8;
+  const int n_words = (int)(((((size_t)n * kBits + 7) / 8 + 15) / 16 * 16) / 4);
+  const int stop = rank == kVecCluster - 1 ? n_words : min(n_words, (begin + 32 * groups) / 32 * kBits);
+  for (int wi = begin / 32 * kBits + tid; wi < stop; wi += kVecThreads) {
     uint32_t val = 0u;
     const int lo_bit = 32 * wi;
-    for (int nn = lo_bit / bits; nn < n && nn * bits < lo_bit + 32; ++nn) {
-      const int shft = nn * bits - lo_bit;
-      val |= shft >= 0 ? (uint32_t)idx[nn] << shft : (uint32_t)idx[nn] >> (-shft);
+    for (int nn = lo_bit / kBits; nn < n && nn * kBits < lo_bit + 32; ++nn) {
+      const int shft = nn * kBits - lo_bit;
+      val |= shft >= 0 ? (uint32_t)sh.idx[nn - begin] << shft : (uint32_t)sh.idx[nn - begin] >> (-shft);
     }
     reinterpret_cast<uint32_t*>(a.payload)[wi] = val;
   }
+  cluster_wait();
 }
 
 // ---- representative activation (Section 4.2) -----------------------------------------------------
@@ -1268,6 +1362,22 @@ __global__ void __launch_bounds__(256) representative_kernel(const RepArgs a) {
   }
 }
 
+template <int E, bool kWeighted>
+cudaError_t launch_vector(const VqArgs& a, const rwkvq_image_header& h, uint8_t* img, cudaStream_t s) {
+  static SmemOptIn opt_in(true);
+  cudaError_t e = opt_in((const void*)vq_vector_kernel<E, kWeighted>, (int)sizeof(VecShared<E>));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kVecCluster); cfg.blockDim = dim3(kVecThreads); cfg.dynamicSmemBytes = sizeof(VecShared<E>); cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kVecCluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // starts while vq_seed_kernel draws the seeds
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = a.n_vec > kVecSeeds ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, vq_vector_kernel<E, kWeighted>, a, h, img);
+}
+
 }  // namespace
 }  // namespace rwkvq
 
@@ -1318,24 +1428,16 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
     a.payload = img + h.off_payload;
     a.aux = reinterpret_cast<uint32_t*>(img + h.off_aux);
     a.flags = flags;
-    static SmemOptIn opt_in_seed, opt_in_64, opt_in_256, opt_in_vector, opt_in_vector_seed;
+    static SmemOptIn opt_in_seed, opt_in_64, opt_in_256, opt_in_vector_seed;
     if (is_vector) {
-      const int seed_threads = (a.n_vec + 2047) / 2048 * 32;
-      e = opt_in_vector_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
-      if (e != cudaSuccess) return cuda_status(e);
-      vq_seed_kernel<true><<<1, seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s>>>(a);
-      e = opt_in_vector((const void*)vq_vector_kernel, (int)std::max(vec_smem_bytes(kVqMaxVec), vec_smem_bytes(kVecTable)));
-      if (e != cudaSuccess) return cuda_status(e);
-      // the exact sums of an unweighted vector are atomics in one block's shared memory
-      cudaLaunchConfig_t cfg_v = {};
-      cfg_v.gridDim = dim3(a.elem_w ? kVecCluster : 1); cfg_v.blockDim = dim3(kVecThreads); cfg_v.dynamicSmemBytes = vec_smem_bytes(a.n_vec); cfg_v.stream = s;
-      cudaLaunchAttribute attr[2];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = cfg_v.gridDim.x; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // starts while the seeds are drawn
-      attr[1].val.programmaticStreamSerializationAllowed = 1;
-      cfg_v.attrs = attr; cfg_v.numAttrs = 2;
-      e = cudaLaunchKernelEx(&cfg_v, vq_vector_kernel, (const VqArgs)a, (const rwkvq_image_header)h, img);
+      if (a.n_vec > kVecSeeds) {
+        const int seed_threads = (a.n_vec + 2047) / 2048 * 32;
+        e = opt_in_vector_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
+        if (e != cudaSuccess) return cuda_status(e);
+        vq_seed_kernel<true><<<1, seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s>>>(a);
+      }
+      e = d.entries == 64 ? (a.elem_w ? launch_vector<64, true>(a, h, img, s) : launch_vector<64, false>(a, h, img, s))
+                          : (a.elem_w ? launch_vector<256, true>(a, h, img, s) : launch_vector<256, false>(a, h, img, s));
       if (e != cudaSuccess) return cuda_status(e);
     } else {
       constexpr size_t seed_smem = (size_t)kVqMaxVec * 4 + sizeof(SeedShared);
@@ -1369,7 +1471,7 @@ rwkvq_status rwkvq_quantize_check(void* workspace_dev, void* stream) {
   if (e == cudaSuccess) e = cudaMemsetAsync(workspace_dev, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
-  return (host_flags & kFlagNonFinite) ? RWKVQ_ENONFINITE : RWKVQ_OK;
+  return (host_flags & kFlagTimeout) ? RWKVQ_ETIMEOUT : (host_flags & kFlagNonFinite) ? RWKVQ_ENONFINITE : RWKVQ_OK;
 }
 
 rwkvq_status rwkvq_quantize_dev_async(const void* w_dev, int oc, int ic, const rwkvq_quant_cfg* cfg, const float* elem_weight_dev,

@@ -267,6 +267,66 @@ def test_mu_quantizer_ties_zero_weights_and_sizes(ic, bits, weighted):
     assert torch.equal(img, again)
 
 
+def _drawn_seeds(v16, entries, seed):
+    """k-means++ draws as the device defines them: fp32 distances summed over runs of 64 vectors in order, run sums by a scan over
+    32 lanes and then warp by warp; a draw takes the last vector whose running sum begins at or below the target."""
+    f32, mask, n = np.float32, (1 << 64) - 1, len(v16)
+
+    def unit(k):
+        z = (seed + (k + 1) * 0x9E3779B97F4A7C15) & mask
+        z = ((z ^ (z >> 30)) * 0xBF58476D1CE4E5B9) & mask
+        z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) & mask
+        return ((z ^ (z >> 31)) >> 11) * 2.0 ** -53
+
+    lanes = -(-n // 2048) * 32
+    v = v16.astype(f32)
+    dist = np.zeros(lanes * 64, f32)
+    dist[:n] = np.inf
+    at, picks = int(unit(0) * n) % n, []
+    for e in range(entries):
+        picks.append(at)
+        if e + 1 == entries:
+            return v16[picks]
+        d = v - v[at]
+        # one rounding of dx * dx + (dy * dy): exact enough in the long type
+        dist[:n] = np.minimum(dist[:n], (d[:, 0].astype(np.longdouble) ** 2 + (d[:, 1] * d[:, 1]).astype(np.longdouble)).astype(f32))
+        local = np.cumsum(dist.reshape(lanes, 64), axis=1, dtype=f32)[:, -1]
+        incl = local.reshape(-1, 32).copy()
+        for off in (1, 2, 4, 8, 16):
+            step = incl.copy()
+            step[:, off:] += incl[:, :-off]
+            incl = step
+        before = np.concatenate([[f32(0)], np.cumsum(incl[:, -1], dtype=f32)])
+        total = before[-1]
+        excl = (before[:-1, None] + np.concatenate([np.zeros((len(incl), 1), f32), incl[:, :-1]], axis=1)).reshape(-1)
+        incl = (before[:-1, None] + incl).reshape(-1)
+        target = f32(f32(unit(e + 1)) * total)
+        at = n - 1
+        if not total > 0:
+            at = int(unit(e + 1) * n) % n
+        hit = np.flatnonzero((excl <= target) & (target < incl))
+        if total > 0 and len(hit):
+            acc, run = excl[hit[0]], int(hit[0]) * 64
+            at = run
+            for k in range(run, min(run + 64, n)):
+                if acc <= target:
+                    at = k
+                acc = f32(acc + dist[k])
+
+
+@pytest.mark.parametrize("ic,bits", [(2, 6), (126, 6), (1024, 8), (1026, 6), (4096, 8), (4098, 6), (8190, 8), (8192, 8), (8194, 6)])
+@pytest.mark.parametrize("kind", ["uniform", "ties"])
+def test_mu_seeds_are_the_draws_of_the_definition(ic, bits, kind):
+    """Vectors whose seeds are found from sums in a tree, with the chains behind them, up to 4096 of them (around the ends of runs, warps and of that
+    range), against the chains; ties and zeros among the distances included."""
+    rng = np.random.default_rng(ic + bits)
+    mu16 = rng.uniform(0.0, 1.0, ic).astype(np.float16) if kind == "uniform" else (rng.integers(0, 9, ic) / 8.0).astype(np.float16)
+    _, img = quantize_dev(mu16, B.RWKVQ_VQ, bits, seed=7, iters=0)
+    _, codes = B.rwkvq_image_unpack(img.cpu().numpy())
+    got = np.asarray(codes["codebook"]).reshape(1 << bits, 2).view(np.uint16)
+    assert np.array_equal(got, _drawn_seeds(mu16.reshape(-1, 2), 1 << bits, 7).view(np.uint16))
+
+
 def test_quantize_dev_error_paths():
     w = torch.zeros((256, 256), dtype=torch.float16, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
