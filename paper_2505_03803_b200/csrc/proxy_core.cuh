@@ -29,6 +29,35 @@ __device__ __forceinline__ double magnitude_value(uint32_t mag, bool bf16) {
   return bf16 ? (double)__uint_as_float(mag << 16) : (double)__half2float(__ushort_as_half((unsigned short)mag));
 }
 
+// Natural logarithm of a positive normal number by table, after P. T. P. Tang, "Table-driven implementation of the logarithm function in
+// IEEE floating-point arithmetic" (1990): with v = 2^e m and 1/c the table's reciprocal of the middle of m's interval (one of 128),
+//   ln v = e ln 2 - ln(1/c) + ln(1 + r),   r = m (1/c) - 1 (one rounding), |r| <= 2^-8,
+// and the series of ln(1 + r) up to r^7 leaves 2^-67.  Off by at most 2^-52 of the result or of ln 2, whichever is larger.  A gap's
+// logarithm was most of its fp64 work: 25 operations a gap instead of about 90.
+constexpr int kLogEntries = 128;
+struct LogTable {
+  double inv[kLogEntries], neg_log[kLogEntries];
+};
+__device__ __forceinline__ void fill_log_table(LogTable& t) {
+  for (int i = threadIdx.x; i < kLogEntries; i += blockDim.x) {
+    const double inv = 1.0 / (1.0 + ((double)i + 0.5) / kLogEntries);
+    t.inv[i] = inv;
+    t.neg_log[i] = -log(inv);
+  }
+}
+__device__ __forceinline__ double log_by(const LogTable& t, double v) {
+  const int hi = __double2hiint(v), i = (hi >> 13) & (kLogEntries - 1);
+  const double m = __hiloint2double((hi & 0x000FFFFF) | 0x3FF00000, __double2loint(v));
+  const double e = __hiloint2double(0x43300000, (int)((uint32_t)((hi >> 20) - 1023) ^ 0x80000000u)) - 4503601774854144.0;      // 2^52 + 2^31
+  const double r = fma(m, t.inv[i], -1.0);
+  double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+  q = fma(r, q, 0.2);
+  q = fma(r, q, -0.25);
+  q = fma(r, q, 1.0 / 3.0);
+  q = fma(r, q, -0.5);
+  return fma(e, 0.6931471805599453094, t.neg_log[i] + fma(r * r, q, r));
+}
+
 struct SetStats {
   double sum_glng;            // sum g' ln g' over the positive gaps
   double pw[7];               // sum t^k for k = 2..8 over the positive gaps, t = n g' - 1
@@ -39,6 +68,7 @@ struct SetStats {
 
 template <int T>
 struct SetShared {
+  LogTable logs;
   int first[T / 32], last[T / 32], count[T / 32], bad[T / 32];
   uint32_t gaps[kGapList];    // magnitude << 16 | predecessor's magnitude
   double red[T / 32][11];
@@ -49,12 +79,13 @@ struct SetShared {
 // are two chains in order of magnitude, joined at zero if it occurs and by one gap across it if not.  Gaps
 // between neighbouring patterns of a run (most of them, in a dense matrix) are all one ulp of the run's binade: they
 // are counted and evaluated once; the others are collected and evaluated by all threads in turn.  All sums have a
-// fixed order, so results are reproducible.
-template <int T>
+// fixed order, so results are reproducible.  kFamily: also sum |t| and the extreme gaps.
+template <int T, bool kFamily = true>
 __device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShared<T>& sh, SetStats& out) {
   static_assert(T % 64 == 0 && T <= 1024 && 1024 % T == 0, "block size");
   constexpr int P = 1024 / T, W = T / 32;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  fill_log_table(sh.logs);
   const bool zero = ((bm[0] | bm[kPatternWords / 2]) & 1u) != 0u;       // +0 and -0 are the same value
   const int inf_run = bf16 ? 0x7F80 / 64 : 0x7C00 / 64;
   int first = 0x10000, last = -1, count = 0, bad = 0;
@@ -110,14 +141,16 @@ __device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShar
   acc[10] = INFINITY;
   auto add = [&](double gap, double times) {
     const double gp = gap * inv_R, tt = n * gp - 1.0;
-    acc[0] += times * (gp * log(gp));
+    acc[0] += times * (gp * log_by(sh.logs, gp));
     double pw = tt;
 #pragma unroll
     for (int k = 2; k <= 8; ++k)
       if (k <= K) { pw *= tt; acc[k - 1] += times * pw; }
-    acc[8] += times * fabs(tt);
-    acc[9] = fmax(acc[9], gp);
-    acc[10] = fmin(acc[10], gp);
+    if (kFamily) {
+      acc[8] += times * fabs(tt);
+      acc[9] = fmax(acc[9], gp);
+      acc[10] = fmin(acc[10], gp);
+    }
   };
   // gaps of one pattern inside a run, and how many other gaps this thread has
   uint64_t lone[P];
@@ -172,6 +205,8 @@ __device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShar
   }
 #pragma unroll
   for (int i = 0; i < 11; ++i) {
+    if (i >= (kFamily ? 11 : 8)) break;
+    if (i >= K && i < 8) continue;                 // sums of powers that are not asked for
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) {
       const double o = __shfl_xor_sync(0xFFFFFFFFu, acc[i], d);
@@ -182,10 +217,11 @@ __device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShar
   __syncthreads();
   if (t == 0) {
 #pragma unroll
-    for (int i = 0; i < 11; ++i) acc[i] = sh.red[0][i];
+    for (int i = 0; i < (kFamily ? 11 : 8); ++i) acc[i] = i >= K && i < 8 ? 0.0 : sh.red[0][i];
     for (int w = 1; w < W; ++w) {
 #pragma unroll
-      for (int i = 0; i < 11; ++i) {
+      for (int i = 0; i < (kFamily ? 11 : 8); ++i) {
+        if (i >= K && i < 8) continue;
         const double o = sh.red[w][i];
         acc[i] = i == 9 ? fmax(acc[i], o) : i == 10 ? fmin(acc[i], o) : acc[i] + o;
       }

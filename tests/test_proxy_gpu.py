@@ -217,3 +217,28 @@ def test_proxy_pattern_sets_at_the_edges(kind, dtype):
     tile = B.rwkvq_proxy_segments(w, w.shape[0], w.shape[1], 4, math.inf, math.inf)
     for pc, pf in ((whole[0], whole[1]), (tile[0][0, 0], tile[1][0, 0])):
         assert _close(pc, ref[0]) and _close(pf, ref[1], 1e-8), (pc, pf, ref)
+
+
+@pytest.mark.parametrize("count", [2, 255, 4095, 4096, 4097, 16384, 16385, 32768])
+@pytest.mark.parametrize("kind", ["gauss", "255 equal", "256 equal", "octaves", "around one"])
+def test_proxy_fp32_tiles_at_the_edges_of_the_sort(count, kind):
+    """Block sizes and buckets of the fp32 tile sort: full buckets and one more key than they take, both zeros, magnitudes beyond the
+    buckets' sixteen octaves, all keys in one bucket."""
+    rng = np.random.default_rng(count)
+    a = rng.standard_normal((2, count)).astype(np.float32) * 0.02
+    if kind.endswith("equal"):
+        same = min(int(kind.split()[0]), count - 1)
+        a[:, :same] = np.float32(0.0123)
+        a[1, same // 2:same] = np.float32(-0.0123)
+        a[0, -1] = -0.0
+    elif kind == "octaves":
+        a = (np.sign(a) * np.exp(rng.uniform(-40.0, 40.0, a.shape))).astype(np.float32)
+    elif kind == "around one":
+        a = 1.0 + a * np.float32(1e-3)
+    vals, dev = _typed(a, torch.float32)
+    pc, pf, _ = B.rwkvq_proxy_segments(dev, 1, count, 4, 3.0, 1e30)
+    rpc, rpf = orc.proxy_segments(vals, 1, count, K=4)
+    _close_arr(pc, rpc, 1e-9)
+    assert np.all(np.abs(pf - rpf) <= 1e-8 * np.maximum(1.0, np.abs(rpf)))
+    again = B.rwkvq_proxy_segments(dev, 1, count, 4, 3.0, 1e30)
+    assert np.array_equal(pc, again[0]) and np.array_equal(pf, again[1])
