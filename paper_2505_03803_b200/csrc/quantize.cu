@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256, 2) sq_quantize_kernel(const uint16_t* __r
 
 // ---- vector quantizer ------------------------------------------------------------------------
 //
-// k-means++ seeding and Lloyd iterations in fp32 with exact integer cluster sums, one block per codebook.  Two kernels:
+// k-means++ seeding and Lloyd iterations in fp32 with exact integer cluster sums, one cluster of blocks per codebook.  Two kinds:
 // a 256 x 256 tile (32 768 two-element vectors, vector i = 128 * row + pair) and a token-shift vector (ic / 2 vectors,
 // optionally weighted).  Both draw the same seeds: the distances are summed over runs of 64 consecutive vectors in
 // order, the run sums by a scan over the lanes of a warp and then warp by warp, all in fp32, and a draw falls on
@@ -255,10 +255,12 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 // Exact cluster sums with native 32-bit shared-memory atomics (a 64-bit one is a compare-and-swap loop): the fixed-point
 // value is added as signed pieces of 13, 13 and 14 bits; 32 768 of them stay below 2^29.  The last piece is zero for
 // |w| < 4 and then skipped.  Layout [piece][centre].
+template <int E>
 struct ClusterSums {
-  int x[3][kVqMaxE], y[3][kVqMaxE], cnt[kVqMaxE];
+  int x[3][E], y[3][E], cnt[E];
 };
-__device__ __forceinline__ void add_sum(int (*sum)[kVqMaxE], int e, long long v) {
+template <int E>
+__device__ __forceinline__ void add_sum(int (*sum)[E], int e, long long v) {
   const int sg = v < 0 ? -1 : 1;
   const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
   atomicAdd(&sum[0][e], sg * (int)(m & 0x1FFFu));
@@ -266,60 +268,267 @@ __device__ __forceinline__ void add_sum(int (*sum)[kVqMaxE], int e, long long v)
   if (p1) atomicAdd(&sum[1][e], sg * p1);
   if (p2) atomicAdd(&sum[2][e], sg * p2);
 }
-__device__ __forceinline__ double mean_of_pieces(const int (*sum)[kVqMaxE], int e, int cnt) {
-  const long long s = (long long)sum[0][e] + ((long long)sum[1][e] << 13) + ((long long)sum[2][e] << 26);
+__device__ __forceinline__ double mean_of_pieces(int p0, int p1, int p2, int cnt) {
+  const long long s = (long long)p0 + ((long long)p1 << 13) + ((long long)p2 << 26);
   return (double)s * (1.0 / 16777216.0) / (double)cnt;
 }
-__device__ __forceinline__ void move_member(ClusterSums& s, uint32_t bits, int e, int sign) {
-  add_sum(s.x, e, sign * half_fixed(bits & 0xFFFFu));
-  add_sum(s.y, e, sign * half_fixed(bits >> 16));
-  atomicAdd(&s.cnt[e], sign);
+// Numbers below 4 in magnitude are 26-bit integers times 2^-24: two pieces, without 64-bit arithmetic.
+constexpr float kTwoPieces = 4.f;
+struct Pieces { int lo, hi; };
+__device__ __forceinline__ Pieces two_pieces(float v) {
+  const int q = __float2int_rn(v * 16777216.f);
+  return Pieces{q & 0x1FFF, q >> 13};
 }
-
-// The first assignment: a thread adds up the 32 vectors of a group for the two centres it meets first, the few others go one by one.  (One
-// by one, all lanes would meet at the same addresses; summed over warps with redux, this took 47 us a tile.)
-__device__ __forceinline__ void join_group(ClusterSums& s, const uint32_t* vec, const uint8_t* idx, int lane) {
-  int e[2] = {-1, -1}, cnt[2] = {0, 0};
-  long long x[2] = {0, 0}, y[2] = {0, 0};
-  for (int k = 0; k < 32; ++k) {
-    const int i = (k + lane) & 31;
-    const uint32_t v = vec[i];
-    const int c = idx[i];
-    if (e[0] < 0) e[0] = c;
-    else if (e[1] < 0 && c != e[0]) e[1] = c;
-    if (c == e[0] || c == e[1]) {
-      const long long vx = half_fixed(v & 0xFFFFu), vy = half_fixed(v >> 16);
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-        if (c == e[j]) { x[j] += vx; y[j] += vy; ++cnt[j]; }
-    } else {
-      move_member(s, v, c, 1);
-    }
+// A vector leaves centre `from` and joins `to`.
+template <int E>
+__device__ __forceinline__ void move_member(ClusterSums<E>& s, uint32_t bits, int from, int to) {
+  const float2 f = vec_of(bits);
+  if (fmaxf(fabsf(f.x), fabsf(f.y)) < kTwoPieces) {
+    const Pieces x = two_pieces(f.x), y = two_pieces(f.y);
+    atomicAdd(&s.x[0][from], -x.lo); atomicAdd(&s.x[1][from], -x.hi); atomicAdd(&s.y[0][from], -y.lo); atomicAdd(&s.y[1][from], -y.hi);
+    atomicAdd(&s.x[0][to], x.lo); atomicAdd(&s.x[1][to], x.hi); atomicAdd(&s.y[0][to], y.lo); atomicAdd(&s.y[1][to], y.hi);
+  } else {
+    const long long x = half_fixed(bits & 0xFFFFu), y = half_fixed(bits >> 16);
+    add_sum(s.x, from, -x); add_sum(s.y, from, -y);
+    add_sum(s.x, to, x); add_sum(s.y, to, y);
   }
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-    if (cnt[j]) { add_sum(s.x, e[j], x[j]); add_sum(s.y, e[j], y[j]); atomicAdd(&s.cnt[e[j]], cnt[j]); }
+  atomicAdd(&s.cnt[from], -1);
+  atomicAdd(&s.cnt[to], 1);
 }
 
-// ---- tiles ----
+// All 64 vectors of a group (two a lane) join one centre.
+template <int E>
+__device__ __forceinline__ void join_group(ClusterSums<E>& s, uint32_t v0, uint32_t v1, int e) {
+  const float2 f0 = vec_of(v0), f1 = vec_of(v1);
+  const bool small = fmaxf(fmaxf(fabsf(f0.x), fabsf(f0.y)), fmaxf(fabsf(f1.x), fabsf(f1.y))) < kTwoPieces;
+  if (__all_sync(0xFFFFFFFFu, small)) {
+    const Pieces x0 = two_pieces(f0.x), y0 = two_pieces(f0.y), x1 = two_pieces(f1.x), y1 = two_pieces(f1.y);
+    const int xl = __reduce_add_sync(0xFFFFFFFFu, x0.lo + x1.lo), xh = __reduce_add_sync(0xFFFFFFFFu, x0.hi + x1.hi);
+    const int yl = __reduce_add_sync(0xFFFFFFFFu, y0.lo + y1.lo), yh = __reduce_add_sync(0xFFFFFFFFu, y0.hi + y1.hi);
+    if ((threadIdx.x & 31) == 0) { atomicAdd(&s.x[0][e], xl); atomicAdd(&s.x[1][e], xh); atomicAdd(&s.y[0][e], yl); atomicAdd(&s.y[1][e], yh); }
+  } else {
+    add_sum(s.x, e, half_fixed(v0 & 0xFFFFu)); add_sum(s.y, e, half_fixed(v0 >> 16));
+    add_sum(s.x, e, half_fixed(v1 & 0xFFFFu)); add_sum(s.y, e, half_fixed(v1 >> 16));
+  }
+  if ((threadIdx.x & 31) == 0) atomicAdd(&s.cnt[e], 64);
+}
+
+// Clusters: barrier, and accesses to the shared memory of a block at the address that `local` has here.
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t peer_address(uint32_t local, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+  return r;
+}
+// A store to a block of the cluster that its barrier `bar` counts.
+__device__ __forceinline__ void peer_send(uint32_t at, ulonglong2 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(at), "l"(v.x), "l"(v.y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void peer_send(uint32_t at, unsigned long long v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at), "l"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void expect_sent(uint32_t bar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void peer_send(uint32_t at, uint32_t v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(at), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void peer_store(uint32_t at, uint32_t v0, uint32_t v1) { asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(v0), "r"(v1) : "memory"); }
+__device__ __forceinline__ uint32_t peer_load(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 peer_load4(uint32_t at) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+  return v;
+}
+// Waits for a phase of a barrier of this block that stores of the cluster complete; gives up after some seconds.
+__device__ __forceinline__ bool wait_sent(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < (1 << 24); ++i) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// ---- seeds ----
 //
-// Seeding.  512 threads, each with the distances of 64 consecutive vectors in registers; the vectors stay in shared memory as
-// fp16 pairs (read 16 bytes at a time, the pieces of a thread's row rotated against bank conflicts).  Bound by
-// the instructions of the distance update: two conversions a vector, four packed operations per two, a minimum and a running sum.
-// Seeds are vectors of the tile, so the codebook area of the image holds them exactly until the centres are final.  A token-shift vector of n
-// vectors, more than kVecSeeds, is seeded alike by one block of n / 2048 warps.
-constexpr int kVqWarps = kVqThreads / 32;
+// A thread has the distances of 64 consecutive vectors in registers; the vectors stay in shared memory as fp16 pairs (read 16 bytes at a time,
+// the pieces of a thread's row rotated against bank conflicts).  Seeds are vectors of the tile, so the codebook area of the image holds them
+// exactly until the centres are final.
 __device__ __forceinline__ int vq_slot(int i) { return (i & ~63) | ((((i >> 2) ^ (i >> 6)) & 7) << 2) | (i & 35); }
 
+// v - c with the fp16 pair v widened and each difference rounded once.
+__device__ __forceinline__ void sub_pair(uint32_t v, float cx, float cy, float& dx, float& dy) {
+  asm("{\n .reg .b16 x, y;\n mov.b32 {x, y}, %2;\n sub.rn.f32.f16 %0, x, %3;\n sub.rn.f32.f16 %1, y, %4;\n}" : "=f"(dx), "=f"(dy) : "r"(v), "f"(cx), "f"(cy));
+}
+// Distances to one more centre for a thread's 64 vectors; their sum in order.
+__device__ __forceinline__ float nearer(float (&dist)[kVqPerThread], const uint32_t* vec, int base, uint32_t centre) {
+  const float2 c = vec_of(centre);
+  float local = 0.f;
+#pragma unroll
+  for (int k = 0; k < kVqPerThread; k += 4) {
+    const uint4 q = *reinterpret_cast<const uint4*>(vec + vq_slot(base + k));
+    float2 dxa, dya, dxb, dyb;
+    sub_pair(q.x, c.x, c.y, dxa.x, dya.x); sub_pair(q.y, c.x, c.y, dxa.y, dya.y);
+    sub_pair(q.z, c.x, c.y, dxb.x, dyb.x); sub_pair(q.w, c.x, c.y, dxb.y, dyb.y);
+    const float2 da = fma2(dxa, dxa, mul2(dya, dya)), db = fma2(dxb, dxb, mul2(dyb, dyb));
+    dist[k] = fminf(dist[k], da.x); dist[k + 1] = fminf(dist[k + 1], da.y);
+    dist[k + 2] = fminf(dist[k + 2], db.x); dist[k + 3] = fminf(dist[k + 3], db.y);
+    local += dist[k]; local += dist[k + 1]; local += dist[k + 2]; local += dist[k + 3];
+  }
+  return local;
+}
+// Sums over the lanes of a warp up to and including this one.
+__device__ __forceinline__ float sum_to_lane(float v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const float o = __shfl_up_sync(0xFFFFFFFFu, v, off);
+    if (lane >= off) v += o;
+  }
+  return v;
+}
+// Sums of all warps, and of those in front of number `warp`.
+__device__ __forceinline__ void warp_sums(const float* tot, int warp, float& before, float& total) {
+  before = total = 0.f;
+#pragma unroll
+  for (int w4 = 0; w4 < kVqMaxVec / 2048 / 4; ++w4) {
+    const float4 t4 = *reinterpret_cast<const float4*>(tot + 4 * w4);
+    const float tt[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (4 * w4 + k == warp) before = total;
+      total += tt[k];
+    }
+  }
+}
+// Last vector of a thread's run whose running sum, from `acc` on, begins at or below the target.
+__device__ __forceinline__ int last_at_or_below(const float (&dist)[kVqPerThread], float acc, float target, int base, int n) {
+  int pick = base;
+#pragma unroll
+  for (int k = 0; k < kVqPerThread; ++k) {
+    if (acc <= target && base + k < n) pick = base + k;
+    acc += dist[k];
+  }
+  return pick;
+}
+
+// Rows of a tile to their slots; a warp reads 512 contiguous bytes, one row.
+__device__ __forceinline__ void load_rows(uint32_t* vec, const uint16_t* src, int ic, int rows, int warps, int* flags) {
+  const int lane = threadIdx.x & 31;
+  bool bad = false;
+#pragma unroll 4
+  for (int r = threadIdx.x >> 5; r < rows; r += warps) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(src + (size_t)r * ic) + lane);
+    const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bad |= ((v[k] & 0x7C00u) == 0x7C00u) | ((v[k] & 0x7C000000u) == 0x7C000000u);
+    *reinterpret_cast<uint4*>(vec + vq_slot(r * 128 + lane * 4)) = q;
+  }
+  if (bad) atomicOr(flags, kFlagNonFinite);
+}
+__device__ __forceinline__ uint64_t tile_seed(uint64_t seed, int tile) { return seed * 0x9E3779B97F4A7C15ull + (uint64_t)tile + 1ull; }
+
+// Few tiles: a cluster of four blocks each, 64 rows (four warps) a block.  A draw hands over twice: every warp's sum goes to all blocks, and the
+// drawn vector from the block that has it.  Bound by the latency of a draw (0.97 us: half of it the two trips, a quarter the distances).  64 entries: 62 us
+// for up to 33 tiles, 79 for 64, 95 for 100; a block a tile, bound by the instructions of the distances (six a vector), 92 in every case (117 with the
+// fp16 numbers converted before the difference was taken).
+constexpr int kTileBlocks = 4, kPartVec = kVqMaxVec / kTileBlocks, kSeedThreads = kPartVec / kVqPerThread;
+struct TileSeeds {
+  uint32_t vec[kPartVec];
+  float tot[2][kVqMaxVec / 2048];                // sums of the tile's warps, for every other draw
+  float u01[kVqMaxE];
+  uint64_t tot_here[2], pick_here;
+  uint32_t pick;
+};
+__global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  extern __shared__ __align__(16) uint8_t smem[];
+  TileSeeds& sh = *reinterpret_cast<TileSeeds*>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, E = a.E;
+  const uint32_t rank = cluster_rank();
+  const int tile = blockIdx.x / kTileBlocks, tr = tile / a.TC, tc = tile % a.TC;
+  const uint32_t tot_here = shared_address(&sh.tot_here[0]), pick_here = shared_address(&sh.pick_here);
+  if (tid == 0)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n mbarrier.init.shared::cta.b64 [%1], 1;\n mbarrier.init.shared::cta.b64 [%2], 1;\n fence.mbarrier_init.release.cluster;"
+                 ::"r"(tot_here), "r"(tot_here + 8), "r"(pick_here) : "memory");
+  load_rows(sh.vec, a.w + (size_t)(tr * 256 + (int)rank * (256 / kTileBlocks)) * a.ic + tc * 256, a.ic, 256 / kTileBlocks, kSeedThreads / 32, a.flags);
+  const uint64_t seed = tile_seed(a.seed, tile);
+  for (int e = tid; e < E; e += kSeedThreads) sh.u01[e] = (float)unit_of(splitmix(seed, e));
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();
+  const int base = tid * kVqPerThread, tile_warp = (int)rank * (kSeedThreads / 32) + warp;
+  float dist[kVqPerThread];
+#pragma unroll
+  for (int k = 0; k < kVqPerThread; ++k) dist[k] = INFINITY;
+  uint32_t* aux = a.aux + (size_t)tile * E;
+  bool lost = false;
+  // the block with vector `at` sends it to all
+  auto send = [&](int at) {
+    const uint32_t v = sh.vec[vq_slot(at)];
+#pragma unroll
+    for (uint32_t r = 0; r < kTileBlocks; ++r) peer_send(peer_address(shared_address(&sh.pick), r), v, peer_address(pick_here, r));
+  };
+  auto receive = [&](int e) -> uint32_t {
+    if (tid == 0) expect_sent(pick_here, 4);
+    lost |= !wait_sent(pick_here, (uint32_t)e & 1u);
+    return sh.pick;
+  };
+  const int first = below(splitmix(seed, 0), kVqMaxVec);
+  if (tid == 0 && first / kPartVec == (int)rank) send(first % kPartVec);
+  for (int e = 0;; ++e) {
+    // A block sends its next draw when it has the next sums of all warps, and a warp its next sums when it has this draw; the sums of two draws
+    // are under way at once, to places and barriers of their own.
+    const uint32_t cv = receive(e);
+    if (tid == 0 && rank == 0u) aux[e] = cv;
+    if (e + 1 == E) break;
+    const float local = nearer(dist, sh.vec, base, cv);
+    const float incl = sum_to_lane(local);
+    const uint32_t bar = tot_here + 8 * (e & 1);
+    if (tid == 0) expect_sent(bar, (int)sizeof(sh.tot[0]));
+    if (lane == 31) {
+#pragma unroll
+      for (uint32_t r = 0; r < kTileBlocks; ++r)
+        peer_send(peer_address(shared_address(&sh.tot[e & 1][tile_warp]), r), __float_as_uint(incl), peer_address(bar, r));
+    }
+    float excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+    if (lane == 0) excl = 0.f;
+    lost |= !wait_sent(bar, (uint32_t)(e >> 1) & 1u);
+    float before, total;
+    warp_sums(sh.tot[e & 1], tile_warp, before, total);
+    const float target = sh.u01[e + 1] * total;
+    if (!(total > 0.f) || !(target < total)) {       // no distance left, or nothing behind the target
+      const int at = total > 0.f ? kVqMaxVec - 1 : below(splitmix(seed, e + 1), kVqMaxVec);
+      if (tid == 0 && at / kPartVec == (int)rank) send(at % kPartVec);
+    } else if (before <= target && target < before + sh.tot[e & 1][tile_warp]) {      // one warp: the sums in front of the warps do not fall
+      const uint32_t hit = __ballot_sync(0xFFFFFFFFu, before + excl <= target && target < before + incl);
+      if (hit != 0u && lane == __ffs((int)hit) - 1) send(last_at_or_below(dist, before + excl, target, base, kPartVec));
+    }
+  }
+  if (lost) atomicOr(a.flags, kFlagTimeout);
+  cluster_arrive();
+  cluster_wait();
+}
+
+// One block: a tile, where there are enough of them for every SM (hand-overs cost less inside a block), or a token-shift vector of n vectors, more
+// than kVecSeeds, with n / 2048 warps.
+constexpr int kVqWarps = kVqThreads / 32;
 struct SeedShared {
   float warp_tot[kVqWarps];
   float u01[kVqMaxE];
   int pick[kVqMaxE];
 };
-
 template <bool kVector>
 __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) {
-  if (kVector) asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.launch_dependents;");
   extern __shared__ __align__(16) uint8_t smem[];
   uint32_t* vec = reinterpret_cast<uint32_t*>(smem);
   const int n = kVector ? a.n_vec : kVqMaxVec, E = a.E, threads = kVector ? (int)blockDim.x : kVqThreads;
@@ -337,20 +546,9 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
     if (bad) atomicOr(a.flags, kFlagNonFinite);
     if (tid < kVqWarps) sh.warp_tot[tid] = 0.f;
   } else {
-    // a warp reads 512 contiguous bytes: one row of the tile
-    const uint16_t* src = a.w + (size_t)(tr * 256) * a.ic + tc * 256;
-    bool bad = false;
-#pragma unroll 4
-    for (int r = warp; r < 256; r += kVqWarps) {
-      const uint4 q = __ldg(reinterpret_cast<const uint4*>(src + (size_t)r * a.ic) + lane);
-      const uint32_t v[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) bad |= ((v[k] & 0x7C00u) == 0x7C00u) | ((v[k] & 0x7C000000u) == 0x7C000000u);
-      *reinterpret_cast<uint4*>(vec + vq_slot(r * 128 + lane * 4)) = q;
-    }
-    if (bad) atomicOr(a.flags, kFlagNonFinite);
+    load_rows(vec, a.w + (size_t)(tr * 256) * a.ic + tc * 256, a.ic, 256, kVqWarps, a.flags);
   }
-  const uint64_t seed = kVector ? a.seed : a.seed * 0x9E3779B97F4A7C15ull + (uint64_t)tile + 1ull;
+  const uint64_t seed = kVector ? a.seed : tile_seed(a.seed, tile);
   for (int e = tid; e < E; e += threads) {
     sh.u01[e] = (float)unit_of(splitmix(seed, e));
     sh.pick[e] = n - 1;
@@ -364,97 +562,84 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
   int at = below(splitmix(seed, 0), n);
   for (int e = 0; e < E; ++e) {
     const uint32_t cv = vec[vq_slot(at)];
-    const float2 c = vec_of(cv);
     if (tid == 0) aux[e] = cv;
     if (e + 1 == E) break;
-    float local = 0.f;
-    const float2 ncx = make_float2(-c.x, -c.x), ncy = make_float2(-c.y, -c.y);
-#pragma unroll
-    for (int k = 0; k < kVqPerThread; k += 4) {
-      const uint4 q = *reinterpret_cast<const uint4*>(vec + vq_slot(base + k));
-      const float2 v0 = vec_of(q.x), v1 = vec_of(q.y), v2 = vec_of(q.z), v3 = vec_of(q.w);
-      const float2 dxa = add2(make_float2(v0.x, v1.x), ncx), dya = add2(make_float2(v0.y, v1.y), ncy);
-      const float2 dxb = add2(make_float2(v2.x, v3.x), ncx), dyb = add2(make_float2(v2.y, v3.y), ncy);
-      const float2 da = fma2(dxa, dxa, mul2(dya, dya)), db = fma2(dxb, dxb, mul2(dyb, dyb));
-      dist[k] = fminf(dist[k], da.x); dist[k + 1] = fminf(dist[k + 1], da.y);
-      dist[k + 2] = fminf(dist[k + 2], db.x); dist[k + 3] = fminf(dist[k + 3], db.y);
-      local += dist[k]; local += dist[k + 1]; local += dist[k + 2]; local += dist[k + 3];
-    }
-    float incl = local;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const float v = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-      if (lane >= off) incl += v;
-    }
+    const float local = nearer(dist, vec, base, cv);
+    float incl = sum_to_lane(local);
     if (lane == 31) sh.warp_tot[warp] = incl;
     float excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
     if (lane == 0) excl = 0.f;
     __syncthreads();
-    float before = 0.f, total = 0.f;
-#pragma unroll
-    for (int w4 = 0; w4 < kVqThreads / 128; ++w4) {
-      const float4 t4 = *reinterpret_cast<const float4*>(sh.warp_tot + 4 * w4);
-      const float tt[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (4 * w4 + k == warp) before = total;
-        total += tt[k];
-      }
-    }
+    float before, total;
+    warp_sums(sh.warp_tot, warp, before, total);
     excl = before + excl;
     incl = before + incl;
     const float target = sh.u01[e + 1] * total;
-    if (total > 0.f && excl <= target && target < incl) {
-      float acc = excl;
-      int pick = base;
-#pragma unroll
-      for (int k = 0; k < kVqPerThread; ++k) {
-        if (acc <= target && (!kVector || base + k < n)) pick = base + k;      // last vector whose running sum began at or below the target
-        acc += dist[k];
-      }
-      sh.pick[e + 1] = pick;
-    }
+    if (total > 0.f && excl <= target && target < incl) sh.pick[e + 1] = last_at_or_below(dist, excl, target, base, n);
     __syncthreads();
     at = total > 0.f ? sh.pick[e + 1] : below(splitmix(seed, e + 1), n);
   }
 }
 
+// ---- tiles ----
+//
 // Lloyd iterations.  The assignment takes the nearest centre of all E, but looks at a few: the vectors are sorted once along
-// a Hilbert curve over 64 x 64 cells and every 32 neighbours form a group with a box around them.  In every iteration each thread
-// strikes out, for one group, the centres that cannot be nearest to any point of its box: those the box lies wholly on the
+// a Hilbert curve over 64 x 64 cells and every 64 neighbours form a group with a box around them.  In every iteration two threads
+// strike out, for one group, the centres that cannot be nearest to any point of its box: those the box lies wholly on the
 // far side of, at their bisector with one centre near the box, by a margin far above the rounding of the fp32 (and fp64)
 // distances.  The assignment found among the others, lowest index first, is therefore the one that all E centres would give,
 // bit for bit.  Then the groups are dealt over the warps in turn (the long lists lie together, in the tails), all lanes of a
-// warp testing the same candidates for 32 neighbours: nothing diverges and no two lanes read different centres.  (Candidate lists per
+// warp testing the same candidates for two neighbours each, two to an instruction: nothing diverges and no two lanes read different centres.  (Candidate lists per
 // cell of a grid, read by vectors in any order, took three times as long an iteration for bank conflicts and divergence; lists built
 // from a warp's common shortlist waited for the warps in the tails, whose shortlists were all E centres.)  A group that lay
 // and still lies wholly with one centre is passed over; cluster sums change only by the vectors that moved.
-constexpr int kLloydThreads = 1024, kLloydWarps = kLloydThreads / 32, kCells = 64, kMoveQueue = 64;
-constexpr int kGroups = kVqMaxVec / 32, kListMax = 15;
-static_assert(kGroups == kLloydThreads, "a group per thread");
-constexpr uint32_t kListAll = 255u, kListSame = 0u;
-struct LloydShared {
-  uint32_t vec[kVqMaxVec];
-  union {
-    struct { uint16_t pos[kVqMaxVec]; int place[kCells * kCells]; uint16_t curve[kCells * kCells]; float red[2][kLloydWarps]; int tot[kLloydWarps]; } sort;
-    struct {
-      uint8_t idx[kVqMaxVec];
-      uint4 list[kGroups];                    // up to fifteen candidates in ascending order, padded with the last one to an even number; last byte: their
-                                              // number, kListAll (more: take every centre), kListSame (nothing to do)
-      double cx[kVqMaxE], cy[kVqMaxE];        // centres
-      float4 cf[kVqMaxE];                     // x, y rounded to fp32 for the assignment; their squared length less a margin
-      ClusterSums sums;
-      uint32_t moves[kLloydWarps][kMoveQueue];   // vector << 16 | old centre << 8 | new centre
-      int moved;
-      __device__ __forceinline__ void set_centre(int e, float x, float y) {
-        const float l = fmaf(x, x, y * y);
-        cf[e] = make_float4(x, y, l - 1e-5f * l, l);
-      }
-      __device__ __forceinline__ float2 centre(uint32_t e) const { return *reinterpret_cast<const float2*>(cf + e); }
-    } it;
-  };
+// A tile is one block's, or a cluster of four sorts it together, deals its groups out and adds up all blocks' sums after an iteration (`LloydOf`).
+// Bound by instructions (190 a group, iteration and warp; 55 % of the issue slots).  A block with 144 tiles, ten iterations: 281 us (283 with
+// groups of 32 dealt out beforehand and the first members added up by one thread a group; seeds 93 us instead of 117).
+constexpr int kCells = 64, kMoveQueue = 64, kGroupVec = 64, kListMax = 15;
+template <int kBlocks>
+struct LloydOf {
+  static constexpr int kVec = kVqMaxVec / kBlocks, kThreads = kVec / 32, kWarps = kThreads / 32, kGroups = kVec / kGroupVec, kTurns = kGroups / kWarps;
+  static constexpr int kRows = 256 / kBlocks;      // of the matrix
+  static_assert(2 * kGroups == kThreads && kTurns <= 32, "two threads a group, a turn a lane");
 };
-static_assert(sizeof(LloydShared) <= 232448, "shared memory of a tile");
+constexpr uint32_t kListAll = 255u, kListSame = 0u;
+// Vectors and their numbers as the sort leaves them, sent from all blocks; before that the cells' counts and the curve.
+template <int kBlocks>
+struct SortedVectors { uint2 both[LloydOf<kBlocks>::kVec]; };
+template <>
+struct SortedVectors<1> { uint32_t vec[kVqMaxVec]; uint16_t pos[kVqMaxVec]; };
+template <int E, int kBlocks>
+union LloydShared {
+  using L = LloydOf<kBlocks>;
+  struct {
+    SortedVectors<kBlocks> to;
+    uint32_t place[kCells * kCells / 2];          // next place of a cell, two to a word
+    float red[2][L::kWarps], mean[2];
+    int tot[L::kWarps];
+  } sort;
+  struct {
+    uint32_t vec[L::kVec];                        // at last the indices in the order of the matrix, those of the whole tile
+    uint8_t idx[L::kVec];                         // at last those of the block's rows
+    uint4 list[L::kGroups];                       // up to fifteen candidates in ascending order, padded with the last one to an even number; last byte: their
+                                                  // number, kListAll (more: take every centre), kListSame (nothing to do)
+    double cx[E], cy[E];                          // centres
+    float4 cf[E + 1];                             // x, y rounded to fp32; their squared length less a margin, and as it is; see cf_slot
+    float4 neg[E];                                // -x, -x, -y, -y for the assignment
+    ClusterSums<E> sums;                          // of the block's members
+    uint32_t moves[L::kWarps][kMoveQueue];        // vector << 16 | old centre << 8 | new centre
+    int moved, next[2];                           // group to be taken next, for every other iteration
+    // a place of padding between the halves: the two threads of a group read different banks
+    static __device__ __forceinline__ int cf_slot(int e) { return e + (e >= E / 2 ? 1 : 0); }
+    __device__ __forceinline__ void set_centre(int e, float x, float y) {
+      const float l = fmaf(x, x, y * y);
+      cf[cf_slot(e)] = make_float4(x, y, l - 1e-5f * l, l);
+      neg[e] = make_float4(-x, -x, -y, -y);
+    }
+    __device__ __forceinline__ float2 centre(int e) const { return *reinterpret_cast<const float2*>(cf + cf_slot(e)); }
+  } it;
+};
+static_assert(3 * (sizeof(LloydShared<256, 4>) + 1024) <= 233472 && sizeof(LloydShared<256, 1>) <= 232448, "three blocks an SM, or one");
 
 // Cell of a coordinate: eight per doubling of |x| + mean for the first two octaves, then four, so that a heavy-tailed tile is resolved as well as
 // a Gaussian one.  Only the sorting order depends on it.
@@ -487,66 +672,83 @@ struct Box {
   }
 };
 
-// The list of this thread's group.  `near`: a centre near the middle of the box (-1: to be looked for), the one that strikes others out;
+// The list of a group, by two neighbouring threads with half of the centres each (`half`: 0 or 1); they have the same box, `near` and
+// `owner`.  `near`: a centre near the middle of the box (-1: to be looked for), the one that strikes others out;
 // replaced by the nearest for the next time.  `owner`: the only centre of the group in the iteration before, -1 if it had
 // several; `skip_same` writes kListSame where that has not changed.
 //   |p - c|^2 - |p - b|^2 is linear in p: over the box its minimum is  |c|^2 - 2 m c - (|b|^2 - 2 m b) - 2 |c - b| h  per dimension,
 // six operations a centre; what it has to exceed is a margin of 1e-5 (|c|^2 + |b|^2 + |m|^2 + |h|^2).
-template <int EW>
-__device__ __forceinline__ void build_list(LloydShared& sh, const Box& box, int group, int& near, int& owner, bool skip_same) {
+template <int EW, int kBlocks>
+__device__ __forceinline__ void build_list(LloydShared<EW * 32, kBlocks>& sh, const Box& box, int group, int half, int& near, int& owner, bool skip_same) {
   auto& s = sh.it;
-  if (near < 0) {
+  constexpr int W = EW / 2;                      // words of a half
+  const int first = half * W * 32;
+  auto nearer_of_both = [&](float best, int at) -> int {
+    const float other = __shfl_xor_sync(0xFFFFFFFFu, best, 1);
+    const int other_at = __shfl_xor_sync(0xFFFFFFFFu, at, 1);
+    return other < best || (other == best && other_at < at) ? other_at : at;
+  };
+  if (__any_sync(0xFFFFFFFFu, near < 0)) {
     float best = INFINITY;
-    near = 0;
+    int at = first;
 #pragma unroll 8
-    for (int e = 0; e < EW * 32; ++e) {
+    for (int e = first; e < first + W * 32; ++e) {
       const float d = d2f(box.mx, box.my, s.centre(e));
-      if (d < best) { best = d; near = e; }
+      if (d < best) { best = d; at = e; }
     }
+    at = nearer_of_both(best, at);
+    if (near < 0) near = at;
   }
-  const float4 b = s.cf[near];
+  const float4 b = s.cf[s.cf_slot(near)];
   const float mx2 = -2.f * box.mx, my2 = -2.f * box.my, hx2 = -2.f * box.hx, hy2 = -2.f * box.hy;
   const float limit = fmaf(mx2, b.x, fmaf(my2, b.y, b.w)) + 1e-5f * (b.w + box.mx * box.mx + box.my * box.my + box.hx * box.hx + box.hy * box.hy);
-  uint32_t mask[EW];
+  uint32_t mask[W];
+  int count = 0;
 #pragma unroll
-  for (int i = 0; i < EW; ++i) {
+  for (int i = 0; i < W; ++i) {
     uint32_t m = 0u;
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-      const float4 c = s.cf[i * 32 + k];
+      const float4 c = s.cf[first + half + i * 32 + k];
       float t = fmaf(mx2, c.x, fmaf(my2, c.y, c.z));
       t = fmaf(hx2, fabsf(c.x - b.x), t);
       t = fmaf(hy2, fabsf(c.y - b.y), t);
       if (!(t > limit)) m |= 1u << k;
     }
+    if (((near - first) >> 5) == i) m |= 1u << (near & 31);
     mask[i] = m;
+    count += __popc(m);
   }
-  mask[0] |= near < 32 ? 1u << (near & 31) : 0u;
-#pragma unroll
-  for (int i = 1; i < EW; ++i) mask[i] |= (near >> 5) == i ? 1u << (near & 31) : 0u;
-  int count = 0;
-#pragma unroll
-  for (int i = 0; i < EW; ++i) count += __popc(mask[i]);
+  const int others = __shfl_xor_sync(0xFFFFFFFFu, count, 1), all = count + others;
   uint8_t* list = reinterpret_cast<uint8_t*>(s.list + group);
   int now = -1;
-  if (count <= kListMax) {
+  if (__any_sync(0xFFFFFFFFu, all <= kListMax)) {
     float best = INFINITY;
-    int n = 0, last = 0, nearest = near;
+    int nearest = near, n = half ? others : 0, last = -1;
+    if (all <= kListMax) {
 #pragma unroll
-    for (int i = 0; i < EW; ++i)
-      for (uint32_t m = mask[i]; m; m &= m - 1u) {
-        last = i * 32 + __ffs((int)m) - 1;
-        list[n++] = (uint8_t)last;
-        const float d = d2f(box.mx, box.my, s.centre(last));
-        if (d < best) { best = d; nearest = last; }
-      }
-    if (n & 1) list[n] = (uint8_t)last;          // at fifteen: overwritten below, and over_list repeats the last one
-    near = nearest;
-    if (count == 1) now = last;
+      for (int i = 0; i < W; ++i)
+        for (uint32_t m = mask[i]; m; m &= m - 1u) {
+          last = first + i * 32 + __ffs((int)m) - 1;
+          list[n++] = (uint8_t)last;
+          const float d = d2f(box.mx, box.my, s.centre(last));
+          if (d < best) { best = d; nearest = last; }
+        }
+    }
+    nearest = nearer_of_both(best, nearest);
+    last = max(last, __shfl_xor_sync(0xFFFFFFFFu, last, 1));
+    if (all <= kListMax) {
+      if ((all & 1) && half == 0) list[all] = (uint8_t)last;          // at fifteen: overwritten below, and over_list repeats the last one
+      near = nearest;
+      if (all == 1) now = last;
+    } else {
+      near = -1;
+    }
   } else {
     near = -1;
   }
-  list[15] = (uint8_t)(skip_same && now >= 0 && now == owner ? kListSame : count <= kListMax ? (uint32_t)count : kListAll);
+  __syncwarp();
+  if (half == 0) list[15] = (uint8_t)(skip_same && now >= 0 && now == owner ? kListSame : all <= kListMax ? (uint32_t)all : kListAll);
   owner = now;
 }
 
@@ -592,21 +794,25 @@ __device__ __forceinline__ void vq_pack_lane(const uint8_t* idx, int rec, int g,
     *reinterpret_cast<uint4*>(out + p * 512 + L * 16) = make_uint4(words[4 * p], words[4 * p + 1], words[4 * p + 2], words[4 * p + 3]);
 }
 
-template <int EW>
-__global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs a, const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
+template <int EW, int kBlocks>
+__global__ void __launch_bounds__(LloydOf<kBlocks>::kThreads, kBlocks == 1 ? 1 : 3) vq_lloyd_kernel(const VqArgs a, const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
   extern __shared__ __align__(16) uint8_t smem[];
-  LloydShared& sh = *reinterpret_cast<LloydShared*>(smem);
-  constexpr int E = EW * 32;
+  using L = LloydOf<kBlocks>;
+  constexpr int E = EW * 32, kThreads = L::kThreads, kVec = L::kVec;
+  LloydShared<E, kBlocks>& sh = *reinterpret_cast<LloydShared<E, kBlocks>*>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tile = blockIdx.x, tr = tile / a.TC, tc = tile % a.TC;
-  if (tile == 0) write_header(head, image);
-  uint32_t pos[kVqMaxVec / kLloydThreads / 2];        // numbers of this lane's vectors, group after group, two to a word
+  const uint32_t rank = cluster_rank();
+  const int tile = blockIdx.x / kBlocks, tr = tile / a.TC, tc = tile % a.TC;
+  if (blockIdx.x == 0) write_header(head, image);
+  uint32_t pos[kVec / kThreads / 2];         // numbers of the vectors tid, tid + kThreads, ..., two to a word
   {
-    constexpr int kRows = 256 / kLloydWarps;
+    constexpr int kRows = L::kRows / L::kWarps, kCounts = kCells * kCells / 2;
+    uint32_t* const counts = reinterpret_cast<uint32_t*>(&sh.sort.to);      // of the cells, two to a word
+    uint16_t* const curve = reinterpret_cast<uint16_t*>(counts + kCounts);
     uint4 q[kRows];
-    const uint16_t* src = a.w + (size_t)(tr * 256) * a.ic + tc * 256;
+    const uint16_t* src = a.w + (size_t)(tr * 256 + (int)rank * L::kRows) * a.ic + tc * 256;
 #pragma unroll
-    for (int j = 0; j < kRows; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(warp + j * kLloydWarps) * a.ic) + lane);
+    for (int j = 0; j < kRows; ++j) q[j] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(warp + j * L::kWarps) * a.ic) + lane);
     float ax = 0.f, ay = 0.f;
 #pragma unroll
     for (int j = 0; j < kRows; ++j) {
@@ -617,30 +823,71 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) { ax += __shfl_xor_sync(0xFFFFFFFFu, ax, off); ay += __shfl_xor_sync(0xFFFFFFFFu, ay, off); }
     if (lane == 0) { sh.sort.red[0][warp] = ax; sh.sort.red[1][warp] = ay; }
-    for (int i = tid; i < kCells * kCells; i += kLloydThreads) {
-      sh.sort.place[i] = 0;
-      sh.sort.curve[i] = (uint16_t)hilbert(i % kCells, i / kCells);
-    }
+    for (int i = tid; i < kCounts; i += kThreads) counts[i] = 0u;
+    for (int i = tid; i < kCells * kCells; i += kThreads) curve[i] = (uint16_t)hilbert(i % kCells, i / kCells);
     __syncthreads();
-    ax = sh.sort.red[0][lane]; ay = sh.sort.red[1][lane];
+    if (tid < 2) {
+      float sum = 0.f;
+      for (int w = 0; w < L::kWarps; ++w) sum += sh.sort.red[tid][w];
+      sh.sort.mean[tid] = sum;
+    }
+    cluster_arrive();
+    cluster_wait();
+    ax = ay = 0.f;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) { ax += __shfl_xor_sync(0xFFFFFFFFu, ax, off); ay += __shfl_xor_sync(0xFFFFFFFFu, ay, off); }
+    for (uint32_t r = 0; r < kBlocks; ++r) {
+      ax += __uint_as_float(peer_load(peer_address(shared_address(&sh.sort.mean[0]), r)));
+      ay += __uint_as_float(peer_load(peer_address(shared_address(&sh.sort.mean[1]), r)));
+    }
     ax = ax > 1e-25f && ax < 1e25f ? ax * (1.f / kVqMaxVec) : 1.f;
     ay = ay > 1e-25f && ay < 1e25f ? ay * (1.f / kVqMaxVec) : 1.f;
-    auto place_of = [&](uint32_t v) {
+    auto cell_of = [&](uint32_t v) -> uint32_t {
       const float2 f = vec_of(v);
-      return sh.sort.place + sh.sort.curve[axis_cell(f.y, ay) * kCells + axis_cell(f.x, ax)];
+      return curve[axis_cell(f.y, ay) * kCells + axis_cell(f.x, ax)];
     };
+    uint32_t cells[kRows][2];                         // of a row's four vectors, two to a word
 #pragma unroll
     for (int j = 0; j < kRows; ++j) {
-      atomicAdd(place_of(q[j].x), 1); atomicAdd(place_of(q[j].y), 1); atomicAdd(place_of(q[j].z), 1); atomicAdd(place_of(q[j].w), 1);
+      cells[j][0] = cell_of(q[j].x) | cell_of(q[j].y) << 16;
+      cells[j][1] = cell_of(q[j].z) | cell_of(q[j].w) << 16;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t c = (cells[j][k / 2] >> (16 * (k & 1))) & 0xFFFFu;
+        atomicAdd(counts + (c >> 1), c & 1u ? 0x10000u : 1u);      // 32 768 at most: no carry into the other half
+      }
     }
-    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
     {
-      constexpr int kPer = kCells * kCells / kLloydThreads;
-      int4 c = *reinterpret_cast<int4*>(sh.sort.place + tid * kPer);
-      static_assert(kPer == 4, "cells per thread");
-      const int sum = c.x + c.y + c.z + c.w;
+      // a thread's cells: their counts in all blocks, and in the blocks in front
+      constexpr int kPer = kCounts / kThreads;
+      static_assert(kPer % 2 == 0, "cells per thread");
+      uint32_t all[kPer], front[kPer];
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) all[i] = front[i] = 0u;
+#pragma unroll
+      for (uint32_t r = 0; r < kBlocks; ++r) {
+        const uint32_t at = peer_address(shared_address(counts + tid * kPer), r);
+        uint32_t c[kPer];
+        if constexpr (kPer % 4 == 0) {
+#pragma unroll
+          for (int i = 0; i < kPer; i += 4) {
+            const uint4 v = peer_load4(at + 4 * i);
+            c[i] = v.x; c[i + 1] = v.y; c[i + 2] = v.z; c[i + 3] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < kPer; ++i) c[i] = peer_load(at + 4 * i);
+        }
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          if (r < rank) front[i] += c[i];
+          all[i] += c[i];
+        }
+      }
+      int sum = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) sum += (int)(all[i] & 0xFFFFu) + (int)(all[i] >> 16);
       int incl = sum;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -649,59 +896,86 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
       }
       if (lane == 31) sh.sort.tot[warp] = incl;
       __syncthreads();
-      int before = sh.sort.tot[lane];
-      before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? before : 0);
-      before += incl - sum;
-      const int4 f = make_int4(before, before + c.x, before + c.x + c.y, before + c.x + c.y + c.z);
-      *reinterpret_cast<int4*>(sh.sort.place + tid * kPer) = f;
+      int at = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? sh.sort.tot[lane] : 0) + incl - sum;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int lo = (int)(all[i] & 0xFFFFu), hi = (int)(all[i] >> 16);
+        sh.sort.place[tid * kPer + i] = (uint32_t)at + (uint32_t)(at + lo) * 0x10000u + front[i];
+        at += lo + hi;
+      }
     }
-    __syncthreads();
+    cluster_arrive();                                 // the counts have been read, the curve has been used: their place may be written
+    cluster_wait();
 #pragma unroll
     for (int j = 0; j < kRows; ++j) {
       const uint32_t v[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int p = atomicAdd(place_of(v[k]), 1);      // the order within a cell does not matter: sums are exact
-        sh.vec[p] = v[k];
-        sh.sort.pos[p] = (uint16_t)((warp + j * kLloydWarps) * 128 + lane * 4 + k);
+        const uint32_t c = (cells[j][k / 2] >> (16 * (k & 1))) & 0xFFFFu;
+        const uint32_t old = atomicAdd(sh.sort.place + (c >> 1), c & 1u ? 0x10000u : 1u);      // the order within a cell does not matter: sums are exact
+        const uint32_t p = c & 1u ? old >> 16 : old & 0xFFFFu, number = (uint32_t)(((int)rank * L::kRows + warp + j * L::kWarps) * 128 + lane * 4 + k);
+        if constexpr (kBlocks == 1) {
+          sh.sort.to.vec[p] = v[k];
+          sh.sort.to.pos[p] = (uint16_t)number;
+        } else {
+          // the groups go to the blocks in turn: their lists are longest at either end of the curve
+          const uint32_t group = p / kGroupVec;
+          peer_store(peer_address(shared_address(sh.sort.to.both + group / kBlocks * kGroupVec + p % kGroupVec), group % kBlocks), v[k], number);
+        }
+      }
+    }
+    cluster_arrive();
+    cluster_wait();
+    // `vec` lies over the first half of `both`
+    constexpr int kStep = 8;
+#pragma unroll
+    for (int i0 = 0; i0 < kVec / kThreads; i0 += kStep) {
+      uint2 t[kStep];
+#pragma unroll
+      for (int i = 0; i < kStep; ++i) {
+        if constexpr (kBlocks == 1) t[i].y = sh.sort.to.pos[(i0 + i) * kThreads + tid];
+        else t[i] = sh.sort.to.both[(i0 + i) * kThreads + tid];
+      }
+      if (kBlocks > 1) __syncthreads();
+#pragma unroll
+      for (int i = 0; i < kStep; ++i) {
+        if (kBlocks > 1) sh.it.vec[(i0 + i) * kThreads + tid] = t[i].x;
+        if (i & 1) pos[(i0 + i) / 2] |= t[i].y << 16; else pos[(i0 + i) / 2] = t[i].y;
       }
     }
     __syncthreads();
-#pragma unroll
-    for (int g = 0; g < 32; g += 2) pos[g / 2] = sh.sort.pos[warp * 1024 + g * 32 + lane] | (uint32_t)sh.sort.pos[warp * 1024 + (g + 1) * 32 + lane] << 16;
-    __syncthreads();
   }
-  Box box;                                       // of group number tid
+  const int my_group = tid >> 1, my_half = tid & 1;
+  Box box;                                       // of this thread's group
   {
     float x0 = INFINITY, x1 = -INFINITY, y0 = INFINITY, y1 = -INFINITY;
 #pragma unroll 8
     for (int k = 0; k < 32; ++k) {
-      const float2 f = vec_of(sh.vec[tid * 32 + ((k + lane) & 31)]);
+      const float2 f = vec_of(sh.it.vec[tid * 32 + ((k + lane) & 31)]);
       x0 = fminf(x0, f.x); x1 = fmaxf(x1, f.x); y0 = fminf(y0, f.y); y1 = fmaxf(y1, f.y);
     }
+    x0 = fminf(x0, __shfl_xor_sync(0xFFFFFFFFu, x0, 1)); x1 = fmaxf(x1, __shfl_xor_sync(0xFFFFFFFFu, x1, 1));
+    y0 = fminf(y0, __shfl_xor_sync(0xFFFFFFFFu, y0, 1)); y1 = fmaxf(y1, __shfl_xor_sync(0xFFFFFFFFu, y1, 1));
     box.set(x0, x1, y0, y1);
   }
   uint32_t* aux = a.aux + (size_t)tile * E;
   auto& s = sh.it;
-  for (int e = tid; e < kVqMaxE; e += kLloydThreads) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");      // the seeds
+  for (int e = tid; e < E; e += kThreads) {
 #pragma unroll
     for (int p = 0; p < 3; ++p) s.sums.x[p][e] = s.sums.y[p][e] = 0;
     s.sums.cnt[e] = 0;
-    if (e < E) {
-      const float2 c = vec_of(aux[e]);
-      s.cx[e] = (double)c.x; s.cy[e] = (double)c.y;
-      s.set_centre(e, c.x, c.y);
-    }
+    const float2 c = vec_of(__ldcg(aux + e));
+    s.cx[e] = (double)c.x; s.cy[e] = (double)c.y;
+    s.set_centre(e, c.x, c.y);
   }
-  if (tid == 0) s.moved = 0;
+  if (tid == 0) s.moved = s.next[0] = s.next[1] = 0;
   __syncthreads();
   int near = -1, owner = -1;
   for (int it = 0; it < a.iters; ++it) {
-    build_list<EW>(sh, box, tid, near, owner, it > 0);
+    build_list<EW, kBlocks>(sh, box, my_group, my_half, near, owner, it > 0);
     __syncthreads();
-    // lane j holds the list of the j-th group of this warp's turn
-    const uint4 entry = s.list[lane * kLloydWarps + warp];
-    uint32_t todo = __ballot_sync(0xFFFFFFFFu, (entry.w >> 24) != kListSame);
+    if (it > 0) cluster_wait();                  // the sums have been read
     bool moved = it == 0;
     int queued = 0;                              // moves of this warp not yet in the sums
     uint32_t* queue = s.moves[warp];
@@ -709,37 +983,20 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
       __syncwarp();
       if (lane < count) {
         const uint32_t m = queue[lane];
-        const uint32_t v = sh.vec[m >> 16];
-        move_member(s.sums, v, (int)((m >> 8) & 0xFFu), -1);
-        move_member(s.sums, v, (int)(m & 0xFFu), 1);
+        const uint32_t v = s.vec[m >> 16];
+        move_member(s.sums, v, (int)((m >> 8) & 0xFFu), (int)(m & 0xFFu));
       }
       __syncwarp();
     };
-    for (; todo; todo &= todo - 1u) {
-      const int j = __ffs((int)todo) - 1, g = j * kLloydWarps + warp, p = g * 32 + lane;
-      const uint32_t q = sh.vec[p];
-      const int was = it > 0 ? (int)s.idx[p] : 0;
-      const float2 f = vec_of(q);
-      float best = INFINITY;
-      int bi = 0;
-      const uint4 e16 = make_uint4(__shfl_sync(0xFFFFFFFFu, entry.x, j), __shfl_sync(0xFFFFFFFFu, entry.y, j), __shfl_sync(0xFFFFFFFFu, entry.z, j), __shfl_sync(0xFFFFFFFFu, entry.w, j));
-      over_list<E>(e16, [&](uint32_t e0, uint32_t e1) {
-        const float d0 = d2f(f.x, f.y, s.centre(e0)), d1 = d2f(f.x, f.y, s.centre(e1));
-        if (d0 < best) { best = d0; bi = (int)e0; }
-        if (d1 < best) { best = d1; bi = (int)e1; }
-      });
-      if (it == 0) {
-        s.idx[p] = (uint8_t)bi;
-        continue;
-      }
-      // the vectors that moved are queued and taken 32 at a time: a few lanes of every warp would otherwise walk
-      // the whole update for every group
-      const uint32_t who = __ballot_sync(0xFFFFFFFFu, bi != was);
-      if (who == 0u) continue;
+    // the vectors that moved are queued and taken 32 at a time: a few lanes of every warp would otherwise walk
+    // the whole update for every group
+    auto move = [&](int p, uint32_t was, uint32_t now) {
+      const uint32_t who = __ballot_sync(0xFFFFFFFFu, now != was);
+      if (who == 0u) return;
       moved = true;
-      if (bi != was) {
-        s.idx[p] = (uint8_t)bi;
-        queue[queued + __popc(who & ((1u << lane) - 1u))] = (uint32_t)p << 16 | (uint32_t)was << 8 | (uint32_t)bi;
+      if (now != was) {
+        s.idx[p] = (uint8_t)now;
+        queue[queued + __popc(who & ((1u << lane) - 1u))] = (uint32_t)p << 16 | was << 8 | now;
       }
       queued += __popc(who);
       if (queued >= 32) {
@@ -749,66 +1006,170 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
         __syncwarp();
         if (lane < queued) queue[lane] = m;
       }
+    };
+    // a warp takes the next group when it is done with one: their lists differ
+    auto take = [&]() -> int { return lane == 0 ? atomicAdd(&s.next[it & 1], 1) : 0; };
+    int ahead = take();
+    for (;;) {
+      const int g = __shfl_sync(0xFFFFFFFFu, ahead, 0), p = g * kGroupVec + lane;
+      if (g >= L::kGroups) break;
+      ahead = take();
+      const uint4 entry = s.list[g];
+      if ((entry.w >> 24) == kListSame) continue;
+      const uint32_t v0 = s.vec[p], v1 = s.vec[p + 32];
+      const float2 f0 = vec_of(v0), f1 = vec_of(v1);
+      const float2 x = make_float2(f0.x, f1.x), y = make_float2(f0.y, f1.y);
+      float best0 = INFINITY, best1 = INFINITY;
+      uint32_t at0 = 0u, at1 = 0u;
+      auto compare = [&](uint32_t e) {
+        const float4 c = s.neg[e];
+        const float2 dx = add2(x, make_float2(c.x, c.y)), dy = add2(y, make_float2(c.z, c.w)), d = fma2(dx, dx, mul2(dy, dy));
+        if (d.x < best0) { best0 = d.x; at0 = e; }
+        if (d.y < best1) { best1 = d.y; at1 = e; }
+      };
+      over_list<E>(entry, [&](uint32_t e0, uint32_t e1) { compare(e0); compare(e1); });
+      uint32_t was0, was1;
+      if (it == 0) {
+        // all join the centre of one of them, and most others' centres: the rest moves on
+        const uint32_t a8 = __shfl_sync(0xFFFFFFFFu, at0, 8), a24 = __shfl_sync(0xFFFFFFFFu, at1, 24);
+        const int n8 = __popc(__ballot_sync(0xFFFFFFFFu, at0 == a8)) + __popc(__ballot_sync(0xFFFFFFFFu, at1 == a8));
+        const int n24 = __popc(__ballot_sync(0xFFFFFFFFu, at0 == a24)) + __popc(__ballot_sync(0xFFFFFFFFu, at1 == a24));
+        was0 = was1 = n8 >= n24 ? a8 : a24;
+        s.idx[p] = s.idx[p + 32] = (uint8_t)was0;
+        join_group(s.sums, v0, v1, (int)was0);
+      } else {
+        was0 = s.idx[p]; was1 = s.idx[p + 32];
+      }
+      move(p, was0, at0);
+      move(p + 32, was1, at1);
     }
     flush(queued);
-    if (it == 0) {
-      __syncthreads();
-      join_group(s.sums, sh.vec + tid * 32, s.idx + tid * 32, lane);
-    }
+    if (tid == 0) s.next[(it + 1) & 1] = 0;
     if (moved && lane == 0) s.moved = it + 1;
-    __syncthreads();
-    if (s.moved != it + 1) break;                // the centres would stay as they are in every further iteration
-    for (int e = tid; e < E; e += kLloydThreads) {
-      const int cnt = s.sums.cnt[e];
-      if (cnt) {
-        s.cx[e] = mean_of_pieces(s.sums.x, e, cnt); s.cy[e] = mean_of_pieces(s.sums.y, e, cnt);
-        s.set_centre(e, (float)s.cx[e], (float)s.cy[e]);
+    cluster_arrive();
+    cluster_wait();
+    bool any = false;
+#pragma unroll
+    for (uint32_t r = 0; r < kBlocks; ++r) any |= (int)peer_load(peer_address(shared_address(&s.moved), r)) == it + 1;
+    if (any) {
+      // four neighbouring lanes a centre, one for each block's sums
+#pragma unroll
+      for (int k = tid; k < kBlocks * E; k += kThreads) {
+        const int e = k / kBlocks;
+        const uint32_t from = (uint32_t)(k % kBlocks);
+        int v[7];
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          v[p] = (int)peer_load(peer_address(shared_address(&s.sums.x[p][e]), from));
+          v[3 + p] = (int)peer_load(peer_address(shared_address(&s.sums.y[p][e]), from));
+        }
+        v[6] = (int)peer_load(peer_address(shared_address(&s.sums.cnt[e]), from));
+#pragma unroll
+        for (int p = 0; p < 7; ++p) {
+#pragma unroll
+          for (int off = 1; off < kBlocks; off <<= 1) v[p] += __shfl_xor_sync(0xFFFFFFFFu, v[p], off);
+        }
+        if (from == 0u && v[6]) {
+          const double x = mean_of_pieces(v[0], v[1], v[2], v[6]), y = mean_of_pieces(v[3], v[4], v[5], v[6]);
+          s.cx[e] = x; s.cy[e] = y;
+          s.set_centre(e, (float)x, (float)y);
+        }
       }
     }
+    cluster_arrive();
+    if (!any) {                                  // the centres would stay as they are in every further iteration
+      cluster_wait();
+      break;
+    }
+    if (it + 1 == a.iters) cluster_wait();
     __syncthreads();
   }
   // ---- centres to fp16; final assignment against the rounded centres in fp64 (exact differences,
   // products and sum each rounded once, in this order; the lowest index wins ties)
-  for (int e = tid; e < E; e += kLloydThreads) {
+  for (int e = tid; e < E; e += kThreads) {
     const __half hx = __double2half(s.cx[e]), hy = __double2half(s.cy[e]);
     s.cx[e] = (double)__half2float(hx); s.cy[e] = (double)__half2float(hy);
     s.set_centre(e, __half2float(hx), __half2float(hy));
-    aux[e] = (uint32_t)__half_as_ushort(hx) | ((uint32_t)__half_as_ushort(hy) << 16);
+    if (rank == 0u) aux[e] = (uint32_t)__half_as_ushort(hx) | ((uint32_t)__half_as_ushort(hy) << 16);
   }
   __syncthreads();
-  build_list<EW>(sh, box, tid, near, owner, false);
+  build_list<EW, kBlocks>(sh, box, my_group, my_half, near, owner, false);
   __syncthreads();
-  for (int g = warp; g < kGroups; g += kLloydWarps) {
-    const int p = g * 32 + lane;
-    const float2 f = vec_of(sh.vec[p]);
+  // In fp32 first: a distance is wrong by less than seven roundings there, so a centre whose distance is smallest by more than 2^-20 of it is
+  // the nearest in fp64 too, and so is one that the vector equals.  The others (and distances near the end of fp32's range) are taken in fp64.
+  for (int g = warp; g < L::kGroups; g += L::kWarps) {
     const uint4 entry = s.list[g];
-    int bi = (int)(entry.x & 0xFFu);
+    const int p = g * kGroupVec + lane;
+    const float2 f[2] = {vec_of(s.vec[p]), vec_of(s.vec[p + 32])};
+    const float2 x = make_float2(f[0].x, f[1].x), y = make_float2(f[0].y, f[1].y);
+    float best[2] = {INFINITY, INFINITY}, next[2] = {INFINITY, INFINITY};
+    uint32_t at[2] = {entry.x & 0xFFu, entry.x & 0xFFu}, last = kListAll + 1u;
     if ((entry.w >> 24) != 1u) {
-      const double x = (double)f.x, y = (double)f.y;
-      double best = INFINITY;
-      over_list<E>(entry, [&](uint32_t e0, uint32_t e1) {
-        const double dx0 = x - s.cx[e0], dy0 = y - s.cy[e0], dx1 = x - s.cx[e1], dy1 = y - s.cy[e1];
-        const double d0 = __dadd_rn(__dmul_rn(dx0, dx0), __dmul_rn(dy0, dy0)), d1 = __dadd_rn(__dmul_rn(dx1, dx1), __dmul_rn(dy1, dy1));
-        if (d0 < best) { best = d0; bi = (int)e0; }
-        if (d1 < best) { best = d1; bi = (int)e1; }
-      });
+      auto compare = [&](uint32_t e) {
+        if (e == last) return;                   // the padding of a list is no second centre
+        last = e;
+        const float4 c = s.neg[e];
+        const float2 dx = add2(x, make_float2(c.x, c.y)), dy = add2(y, make_float2(c.z, c.w)), d = fma2(dx, dx, mul2(dy, dy));
+        next[0] = fminf(next[0], fmaxf(best[0], d.x)); next[1] = fminf(next[1], fmaxf(best[1], d.y));
+        if (d.x < best[0]) { best[0] = d.x; at[0] = e; }
+        if (d.y < best[1]) { best[1] = d.y; at[1] = e; }
+      };
+      over_list<E>(entry, [&](uint32_t e0, uint32_t e1) { compare(e0); compare(e1); });
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float4 c = s.neg[at[k]];
+        const bool equal = f[k].x + c.x == 0.f && f[k].y + c.z == 0.f;
+        if (next[k] > best[k] * (1.f + 1.f / 1048576.f) && (equal || (best[k] > 1e-30f && best[k] < 1e30f))) continue;
+        const double dx = (double)f[k].x, dy = (double)f[k].y;
+        double nearest = INFINITY;
+        over_list<E>(entry, [&](uint32_t e0, uint32_t e1) {
+          const double dx0 = dx - s.cx[e0], dy0 = dy - s.cy[e0], dx1 = dx - s.cx[e1], dy1 = dy - s.cy[e1];
+          const double d0 = __dadd_rn(__dmul_rn(dx0, dx0), __dmul_rn(dy0, dy0)), d1 = __dadd_rn(__dmul_rn(dx1, dx1), __dmul_rn(dy1, dy1));
+          if (d0 < nearest) { nearest = d0; at[k] = e0; }
+          if (d1 < nearest) { nearest = d1; at[k] = e1; }
+        });
+      }
     }
-    s.idx[p] = (uint8_t)bi;
+    s.idx[p] = (uint8_t)at[0]; s.idx[p + 32] = (uint8_t)at[1];
   }
   __syncthreads();
-  // back to the order of the matrix; the vectors are not needed any more
-  uint8_t* idx = reinterpret_cast<uint8_t*>(sh.vec);
+  // back to the order of the matrix; the vectors are not needed any more.  A block writes its indices into an empty tile, and takes its rows
+  // of all blocks' tiles.  (Bytes stored to the block that has the row took 16 000 cycles instead of 8 000.)
+  uint8_t* const tile_idx = reinterpret_cast<uint8_t*>(s.vec);
+  if (kBlocks > 1) {
 #pragma unroll
-  for (int g = 0; g < 32; ++g) idx[(pos[g / 2] >> (16 * (g & 1))) & 0xFFFFu] = s.idx[warp * 1024 + g * 32 + lane];
+    for (int i = 0; i < kVqMaxVec / 16 / kThreads; ++i) reinterpret_cast<uint4*>(tile_idx)[i * kThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < kVec / kThreads; ++i) tile_idx[(pos[i / 2] >> (16 * (i & 1))) & 0xFFFFu] = s.idx[i * kThreads + tid];
+  if constexpr (kBlocks > 1) {
+    cluster_arrive();
+    cluster_wait();
+#pragma unroll
+    for (int i = 0; i < kVec / 16 / kThreads; ++i) {
+      const int at = i * kThreads + tid;
+      uint4 all = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (uint32_t r = 0; r < kBlocks; ++r) {
+        const uint4 v = peer_load4(peer_address(shared_address(tile_idx + rank * kVec + at * 16), r));
+        all.x |= v.x; all.y |= v.y; all.z |= v.z; all.w |= v.w;
+      }
+      reinterpret_cast<uint4*>(s.idx)[at] = all;
+    }
+    cluster_arrive();                            // the others have read this block's tile
+  }
   __syncthreads();
   // ---- bit packing (format.h)
-  if (warp < 16) {
-    const int gr = lane >> 2, t = lane & 3;
+  constexpr int kRecords = 16 / kBlocks;
+  if (warp < kRecords) {
+    const int gr = lane >> 2, t = lane & 3, rec = (int)rank * kRecords + warp;
     constexpr int kBits = EW == 2 ? 6 : 8;
-    const int mb = tr * 2 + (warp >> 3), rt = warp & 7;
+    const int mb = tr * 2 + (rec >> 3), rt = rec & 7;
     uint8_t* out = a.payload + (((size_t)mb * a.TC + tc) * 8 + rt) * rwkvq_vq_record_bytes(kBits);
-    vq_pack_lane<kBits>(idx, warp, gr, t, lane, out);
+    vq_pack_lane<kBits>(kBlocks > 1 ? s.idx : tile_idx, warp, gr, t, lane, out);
   }
+  if (kBlocks > 1) cluster_wait();
 }
 
 // ---- token-shift vectors ----
@@ -821,7 +1182,7 @@ __global__ void __launch_bounds__(kLloydThreads, 1) vq_lloyd_kernel(const VqArgs
 // a draw (0.42 us), two barriers and two trips through the cluster an iteration (1.65 us).  2048 weighted vectors, 64 centres, ten iterations:
 // 47.6 us; 139 with one warp drawing all seeds by the chains, one block sorting the members by centre and adding them up, and a barrier of the
 // cluster at either end of it.  256 centres, 2560 vectors: 166 us, 418 then.
-constexpr int kVecThreads = 512, kVecWarps = kVecThreads / 32;
+constexpr int kVecThreads = 512;
 constexpr int kVecCluster = 16;                  // blocks
 constexpr int kSeedPer = 16, kVecSeeds = 4096, kSeedWarps = kVecSeeds / (32 * kSeedPer);
 constexpr int kVecParts = 4;                     // lanes a vector
@@ -852,36 +1213,6 @@ struct VecShared {
   ulonglong2 table[kVecGroups * 32][2];          // (w * v, w) in either dimension of the block's vectors, if there are no more
 };
 static_assert(sizeof(VecShared<256>) <= 232448, "shared memory of a block");
-
-// The cluster: barrier, and stores to the shared memory of a block of it at the address that `local` has here.
-__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ uint32_t peer_address(uint32_t local, uint32_t rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
-// A store to a block of the cluster that its barrier `bar` counts.
-__device__ __forceinline__ void peer_send(uint32_t at, ulonglong2 v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(at), "l"(v.x), "l"(v.y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void peer_send(uint32_t at, unsigned long long v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at), "l"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ uint32_t shared_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void expect_sent(uint32_t bar, int bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Waits for a phase of a barrier of this block that stores of the cluster complete; gives up after some seconds.
-__device__ __forceinline__ bool wait_sent(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 24); ++i) {
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
 
 // Draws E seeds; a draw is defined as in vq_seed_kernel: distances summed in fp32 over runs of 64 vectors in order, run sums by a scan over the lanes
 // of a warp, and the last vector whose running sum begins at or below the target.  Those chains are 64 additions long, twice a draw.  So the
@@ -1362,20 +1693,41 @@ __global__ void __launch_bounds__(256) representative_kernel(const RepArgs a) {
   }
 }
 
+// Up to this many tiles are a cluster's of four blocks each, more a block's.  104 clusters run at once; iterations and seeds, 64 entries, ten iterations:
+// 16 tiles 200 us (a block each: 343), 33 tiles 220 (343), 64 tiles 273 (347), 100 tiles 343 (371), 144 tiles 569 (376).
+constexpr unsigned kSpreadTiles = 100;
+// Blocks of a cluster are put on as few SMs as take them.  Shared memory that a block asks for beyond its need keeps others away while there are SMs
+// enough: 33 clusters of four fit one block an SM, 66 two (36 tiles: 308 us as they come, 252 so).
+constexpr int kSmemAlone = 118 * 1024, kSmemTwo = 80 * 1024;
+size_t smem_to_spread(unsigned tiles) { return tiles <= 33 ? kSmemAlone : tiles <= 66 ? kSmemTwo : 0; }
+// `early`: may start while the kernel before it runs, which this library launched in the same call.
+template <class... Args>
+cudaError_t launch_cluster(void (*fn)(Args...), unsigned blocks, unsigned cluster, unsigned threads, size_t smem, bool early, cudaStream_t s, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = early ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
 template <int E, bool kWeighted>
 cudaError_t launch_vector(const VqArgs& a, const rwkvq_image_header& h, uint8_t* img, cudaStream_t s) {
   static SmemOptIn opt_in(true);
-  cudaError_t e = opt_in((const void*)vq_vector_kernel<E, kWeighted>, (int)sizeof(VecShared<E>));
+  const cudaError_t e = opt_in((const void*)vq_vector_kernel<E, kWeighted>, (int)sizeof(VecShared<E>));
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kVecCluster); cfg.blockDim = dim3(kVecThreads); cfg.dynamicSmemBytes = sizeof(VecShared<E>); cfg.stream = s;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kVecCluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // starts while vq_seed_kernel draws the seeds
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = a.n_vec > kVecSeeds ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, vq_vector_kernel<E, kWeighted>, a, h, img);
+  return launch_cluster(vq_vector_kernel<E, kWeighted>, kVecCluster, kVecCluster, kVecThreads, sizeof(VecShared<E>), a.n_vec > kVecSeeds, s, a, h, img);
+}
+template <int EW, int kBlocks>
+cudaError_t launch_lloyd(const VqArgs& a, const rwkvq_image_header& h, uint8_t* img, unsigned tiles, cudaStream_t s) {
+  using Shared = LloydShared<EW * 32, kBlocks>;
+  static SmemOptIn opt_in;
+  const cudaError_t e = opt_in((const void*)vq_lloyd_kernel<EW, kBlocks>, kBlocks == 1 ? (int)sizeof(Shared) : kSmemAlone);
+  if (e != cudaSuccess) return e;
+  const size_t smem = kBlocks == 1 ? sizeof(Shared) : std::max(sizeof(Shared), smem_to_spread(tiles));
+  return launch_cluster(vq_lloyd_kernel<EW, kBlocks>, tiles * kBlocks, kBlocks, LloydOf<kBlocks>::kThreads, smem, true, s, a, h, img);
 }
 
 }  // namespace
@@ -1428,33 +1780,33 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
     a.payload = img + h.off_payload;
     a.aux = reinterpret_cast<uint32_t*>(img + h.off_aux);
     a.flags = flags;
-    static SmemOptIn opt_in_seed, opt_in_64, opt_in_256, opt_in_vector_seed;
     if (is_vector) {
       if (a.n_vec > kVecSeeds) {
+        static SmemOptIn opt_in_seed;
         const int seed_threads = (a.n_vec + 2047) / 2048 * 32;
-        e = opt_in_vector_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
+        e = opt_in_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
         if (e != cudaSuccess) return cuda_status(e);
         vq_seed_kernel<true><<<1, seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s>>>(a);
       }
       e = d.entries == 64 ? (a.elem_w ? launch_vector<64, true>(a, h, img, s) : launch_vector<64, false>(a, h, img, s))
                           : (a.elem_w ? launch_vector<256, true>(a, h, img, s) : launch_vector<256, false>(a, h, img, s));
-      if (e != cudaSuccess) return cuda_status(e);
     } else {
-      constexpr size_t seed_smem = (size_t)kVqMaxVec * 4 + sizeof(SeedShared);
-      const int tiles = (oc / 256) * (ic / 256);
-      e = opt_in_seed((const void*)vq_seed_kernel<false>, (int)seed_smem);
-      if (e != cudaSuccess) return cuda_status(e);
-      vq_seed_kernel<false><<<tiles, kVqThreads, seed_smem, s>>>(a);
-      if (d.entries == 64) {
-        e = opt_in_64((const void*)vq_lloyd_kernel<2>, (int)sizeof(LloydShared));
-        if (e != cudaSuccess) return cuda_status(e);
-        vq_lloyd_kernel<2><<<tiles, kLloydThreads, sizeof(LloydShared), s>>>(a, h, img);
+      const unsigned tiles = (unsigned)(oc / 256) * (unsigned)(ic / 256);
+      const bool spread = tiles <= kSpreadTiles;
+      if (spread) {
+        static SmemOptIn opt_in_seed;
+        e = opt_in_seed((const void*)vq_tile_seed_kernel, kSmemAlone);
+        if (e == cudaSuccess) e = launch_cluster(vq_tile_seed_kernel, tiles * kTileBlocks, kTileBlocks, kSeedThreads, std::max(sizeof(TileSeeds), smem_to_spread(tiles)), false, s, (const VqArgs)a);
       } else {
-        e = opt_in_256((const void*)vq_lloyd_kernel<8>, (int)sizeof(LloydShared));
-        if (e != cudaSuccess) return cuda_status(e);
-        vq_lloyd_kernel<8><<<tiles, kLloydThreads, sizeof(LloydShared), s>>>(a, h, img);
+        static SmemOptIn opt_in_seed;
+        constexpr size_t seed_smem = (size_t)kVqMaxVec * 4 + sizeof(SeedShared);
+        e = opt_in_seed((const void*)vq_seed_kernel<false>, (int)seed_smem);
+        if (e == cudaSuccess) vq_seed_kernel<false><<<tiles, kVqThreads, seed_smem, s>>>(a);
       }
+      if (e == cudaSuccess) e = d.entries == 64 ? (spread ? launch_lloyd<2, 4>(a, h, img, tiles, s) : launch_lloyd<2, 1>(a, h, img, tiles, s))
+                                             : (spread ? launch_lloyd<8, 4>(a, h, img, tiles, s) : launch_lloyd<8, 1>(a, h, img, tiles, s));
     }
+    if (e != cudaSuccess) return cuda_status(e);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e);

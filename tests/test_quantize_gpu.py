@@ -443,3 +443,27 @@ def test_vq_device_iterations_and_assignment_at_the_edges(kind, bits):
         want = members.mean(axis=0) if len(members) else books[0][e]
         # fp16 rounding; a tie decided otherwise in fp32 moves a mean by less than that of a cluster's spread
         assert np.all(np.abs(books[1][e] - want) <= 1e-3 * np.abs(want) + 2.0 ** -24 + 1e-2 * (np.ptp(members, axis=0) if len(members) else 0.0)), (kind, e)
+
+
+@pytest.mark.parametrize("bits", [6, 8])
+@pytest.mark.parametrize("few", [1, 33, 34, 66, 67, 100])
+def test_vq_tiles_alike_in_one_block_and_in_a_cluster(few, bits):
+    """101 tiles are taken by a block each, up to 100 by clusters of four (at 33 and 66 with other blocks on an SM): the first tiles of a wide
+    matrix come out alike, with weights beyond the two-piece sums and many equal ones among them, and as the oracle assigns them."""
+    rng = np.random.default_rng(few)
+    w16 = (rng.standard_t(3, (256, 101 * 256)) * 0.01).astype(np.float16)
+    w16[:, 256:512] *= np.float16(900.0)              # around four in magnitude, on both sides
+    w16[:, 512:768] = rng.choice(np.array([-0.5, 0.0, 2.0 ** -24, 3.0], np.float16), (256, 256))
+    _, wide = quantize_dev(w16, B.RWKVQ_VQ, bits, seed=11, iters=4)
+    _, part = quantize_dev(w16[:, :few * 256], B.RWKVQ_VQ, bits, seed=11, iters=4)
+    E = 1 << bits
+    books, index = [], []
+    for img, tiles in ((wide, 101), (part, few)):
+        _, codes = B.rwkvq_image_unpack(img.cpu().numpy())
+        books.append(np.asarray(codes["codebook"]).reshape(tiles, E, 2)[:few])
+        index.append(np.asarray(codes["q"]).reshape(256, tiles * 128)[:, :few * 128])
+    assert np.array_equal(books[0].view(np.uint16), books[1].view(np.uint16))
+    assert np.array_equal(index[0], index[1])
+    for t in range(min(few, 3)):
+        v = w16[:, t * 256:(t + 1) * 256].astype(np.float64).reshape(-1, 2)
+        assert np.array_equal(index[1][:, t * 128:(t + 1) * 128].reshape(-1), orc._nearest(v, books[1][t].astype(np.float64)))
