@@ -25,42 +25,61 @@ __device__ __forceinline__ void write_header(const rwkvq_image_header& h, uint8_
   const uint32_t* src = reinterpret_cast<const uint32_t*>(&h);
   if (threadIdx.x < RWKVQ_HEADER_BYTES / 4) reinterpret_cast<uint32_t*>(image)[threadIdx.x] = src[threadIdx.x];
   const uint64_t used = h.off_aux + h.aux_bytes;
-  if (threadIdx.x < h.image_bytes - used) image[used + threadIdx.x] = 0;       // less than 256 bytes
+  for (uint64_t i = used + threadIdx.x; i < h.image_bytes; i += blockDim.x) image[i] = 0;
+}
+
+// Two fp32 operations in one instruction, each rounded as the single one is.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mul.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z, w;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;\n}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
 }
 
 // ---- scalar quantizer ------------------------------------------------------------------------
 //
-// One warp per record (16 rows x 256 columns), one block of eight warps per chunk.  A lane keeps its eight columns of all sixteen
+// One warp per record (16 rows x 256 columns).  A lane keeps its eight columns of all sixteen
 // rows in registers (lanes 0..15 have group 0, lanes 16..31 group 1), so that the matrix is read once, sixteen 16-byte loads in flight.
 // The (row, group) minima and maxima are reduced sixteen rows at once: each step exchanges half of the rows that a lane still
 // has, 15 shuffles in all, and lane r + 16 h ends with (row r, group h), whose (s, z) it derives
 // in fp64 exactly as Eq. 2 prescribes.
 //
-// The codes need no division.  q = clamp(round(w / s) + z, 0, 7) counts the k in 1..7 with
-// round(w / s) >= k - z, and round(x) >= m (ties to even) holds iff x > m - 1/2, or x = m - 1/2
-// with m even.  (m - 1/2) * s is exact in fp32 (4 bits times 11 bits), so each k has an exact
-// fp16 threshold T_k -- the smallest fp16 number that is >= (or >) that product -- and
-// q = #{k : w >= T_k}.  The T_k do not fall with k, so three packed comparisons, each against the threshold that the ones before it
-// choose, find q for two weights: ten instructions instead of the fourteen of seven comparisons.  Bound by these instructions;
-// 14336 x 4096: 46.5 us (49.5 with two passes over the rows, a shuffle tree per row and seven comparisons).
+// A code is clamp(round(w / s) + z, 0, 7), ties to even before z is added.  The quotient by Markstein's correction of w * (1/s) with fused
+// multiply-adds ("Computation of elementary functions on the IBM RISC System/6000 processor", 1990): an m + 1/2 comes out exact, and any other
+// quotient below 8 is at least 2^-13 away from one (w and s have 11 bits) while the correction leaves 2^-21.  Then (w / s + z) / 8, saturated
+// to [0, 1], plus 1.5 * 2^20, whose last place is 1/8: the addition rounds, and the code is in the low bits.  An odd z would turn the ties; with
+// one more in the constant they fall as they should, and the code is one more, too.  Eight, where the largest quotient rounds up,
+// becomes seven for four codes at once.  These are multiply-adds beside the integer pipe, which holds this kernel (minima and maxima, codes, bit
+// packing): choosing among seven exact thresholds by three packed comparisons kept it busy half as long again.  Twenty warps an SM in blocks of four: with
+// sixteen in blocks of eight, 1792 chunks are seven rounds of 6.05, with sixteen in blocks of four 37.1 us, with twenty-four (spilled) 40.
+// 14336 x 4096: 35.1 us (45.4 with the comparisons, 40.6 without them), 4096 x 4096: 14.6 (18.2).
+constexpr int kSqWarps = 4;              // of a block; twenty on an SM
 constexpr int kSqRowStride = 256 + 16;   // bytes per row of the code staging area: conflict-free lane reads
 
 __device__ __forceinline__ float h2f_bits(uint32_t h) { return __half2float(__ushort_as_half((unsigned short)h)); }
 __device__ __forceinline__ __half2 as_h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 __device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
-__device__ __forceinline__ uint32_t ge_mask(uint32_t x, uint32_t t) { return __hge2_mask(as_h2(x), as_h2(t)); }
-__device__ __forceinline__ uint32_t choose(uint32_t mask, uint32_t a, uint32_t b) { return (mask & a) | (~mask & b); }
-
-__global__ void __launch_bounds__(256, 2) sq_quantize_kernel(const uint16_t* __restrict__ w, int oc, int ic, int KT,
+__global__ void __launch_bounds__(32 * kSqWarps, 20 / kSqWarps) sq_quantize_kernel(const uint16_t* __restrict__ w, int oc, int ic, int KT,
                                                              uint8_t* __restrict__ payload, int* __restrict__ flags,
                                                              const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
-  __shared__ __align__(16) uint8_t codes_all[8][16 * kSqRowStride];
-  __shared__ __align__(16) uint32_t thr_all[8][2][16][8];     // [warp][group][row][k]: (T_k, T_k) as half2, k = 1..7 in 0..6
+  __shared__ __align__(16) uint8_t codes_all[kSqWarps][16 * kSqRowStride];
+  __shared__ float4 code_all[kSqWarps][2][16];                     // [warp][group][row]: -s, 1/s, z / 8, 1.5 * 2^20 (+ 1/8 for an odd z)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (blockIdx.x == 0) write_header(head, image);
-  const int mb = blockIdx.x / KT, kt = blockIdx.x % KT;
-  const int r0 = mb * 128 + warp * 16, c0 = kt * 256;
+  const unsigned record = blockIdx.x * kSqWarps + warp, chunk = record >> 3;
+  const int mb = (int)(chunk / (unsigned)KT), kt = (int)(chunk % (unsigned)KT);
+  const int r0 = mb * 128 + (int)(record & 7u) * 16, c0 = kt * 256;
   uint8_t* codes = codes_all[warp];
   const int half = lane >> 4;
   const int col = c0 + 8 * lane;
@@ -98,56 +117,48 @@ __global__ void __launch_bounds__(256, 2) sq_quantize_kernel(const uint16_t* __r
     const double mn = (double)my_mn, mx = (double)my_mx;
     const __half s16 = __double2half((mx - mn) / 7.0);
     const double s = (double)__half2float(s16);
-    uint32_t* thr = thr_all[warp][half][lane & 15];
-    const uint32_t kNever = 0x7C007C00u, kAlways = 0xFC00FC00u;     // +inf, -inf
+    float inv, add;
     if (mx == mn || s == 0.0) {
       my_s = mn == 0.0 ? 1.f : fabsf(my_mn);
       my_z = mn < 0.0 ? 1.f : 0.f;
-      thr[0] = mn > 0.0 ? kAlways : kNever;
-#pragma unroll
-      for (int k = 1; k < 7; ++k) thr[k] = kNever;
+      inv = 0.f;                                   // the same code for all
+      add = mn > 0.0 ? 1.f : 0.f;
     } else {
       my_s = (float)s;
       my_z = (float)fmin(7.0, fmax(0.0, rint(-mn / s)));
-#pragma unroll
-      for (int k = 1; k <= 7; ++k) {
-        const float m = (float)k - my_z;
-        const float theta = (m - 0.5f) * my_s;                  // exact
-        __half t16 = __float2half_ru(theta);                   // smallest fp16 >= theta (+inf / -65504 beyond the range)
-        if (((int)m & 1) && __half2float(t16) == theta) {       // m odd: the tie rounds down, so w must exceed theta
-          const unsigned short hb = __half_as_ushort(t16);
-          t16 = __ushort_as_half((hb & 0x7FFFu) == 0 ? (unsigned short)1 : (hb & 0x8000u) ? (unsigned short)(hb - 1) : (unsigned short)(hb + 1));
-        }
-        const uint32_t tb = __half_as_ushort(t16);
-        thr[k - 1] = tb | (tb << 16);
-      }
+      inv = 1.f / my_s;
+      add = my_z;
     }
-    thr[7] = 0u;
+    code_all[warp][half][lane & 15] = make_float4(-my_s, inv, add * 0.125f, 1572864.f + (((int)add & 1) ? 0.125f : 0.f));
   }
   __syncwarp();
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
     const bool inside = col_in && (r0 + r) < oc;
-    const uint4 ta = *reinterpret_cast<const uint4*>(thr_all[warp][half][r]);          // T_1 .. T_4
-    const uint4 tb = *reinterpret_cast<const uint4*>(thr_all[warp][half][r] + 4);      // T_5 .. T_7
+    const float4 c = code_all[warp][half][r];
+    const float2 neg_s = make_float2(c.x, c.x), inv = make_float2(c.y, c.y), magic = make_float2(c.w, c.w);
+    const uint32_t odd = (__float_as_uint(c.w) & 1u) * 0x01010101u;
     const uint32_t words[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-    uint32_t qw[4];
+    uint32_t bits[8];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const uint32_t x = words[k];
-      const uint32_t m4 = ge_mask(x, ta.w);
-      const uint32_t m2 = ge_mask(x, choose(m4, tb.y, ta.y));
-      const uint32_t m1 = ge_mask(x, choose(m2, choose(m4, tb.z, ta.z), choose(m4, tb.x, ta.x)));
-      qw[k] = (m4 & 0x00040004u) | (m2 & 0x00020002u) | (m1 & 0x00010001u);
+      const float2 x = __half22float2(as_h2(words[k]));
+      const float2 q0 = mul2(x, inv), q1 = fma2(fma2(q0, neg_s, x), inv, q0);
+      const float2 sum = add2(make_float2(__saturatef(fmaf(q1.x, 0.125f, c.z)), __saturatef(fmaf(q1.y, 0.125f, c.z))), magic);
+      bits[2 * k] = __float_as_uint(sum.x); bits[2 * k + 1] = __float_as_uint(sum.y);
     }
-    const uint2 out = make_uint2(__byte_perm(qw[0], qw[1], 0x6420u), __byte_perm(qw[2], qw[3], 0x6420u));
+    uint2 out;
+    out.x = __byte_perm(__byte_perm(bits[0], bits[1], 0x0040u), __byte_perm(bits[2], bits[3], 0x0040u), 0x5410u) - odd;
+    out.y = __byte_perm(__byte_perm(bits[4], bits[5], 0x0040u), __byte_perm(bits[6], bits[7], 0x0040u), 0x5410u) - odd;
+    out.x -= (out.x >> 3) & 0x01010101u;
+    out.y -= (out.y >> 3) & 0x01010101u;
     *reinterpret_cast<uint2*>(codes + r * kSqRowStride + 8 * lane) = inside ? out : make_uint2(0u, 0u);
   }
   __syncwarp();
   // Bit packing of format.h: lane (g, t) owns rows g and g + 8 and, in every tensor-core step,
   // the four columns 4t .. 4t+3 (one 32-bit read of the staging area = registers R and R + 2).
   const int g = lane >> 2, t = lane & 3;
-  uint8_t* rec = payload + ((size_t)blockIdx.x * 8 + warp) * RWKVQ_SQ_RECORD_BYTES;
+  uint8_t* rec = payload + (size_t)record * RWKVQ_SQ_RECORD_BYTES;
   uint32_t wd[12];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -234,24 +245,6 @@ __device__ __forceinline__ float d2f(float x, float y, float2 c) {
   return fmaf(dx, dx, dy * dy);
 }
 __device__ __forceinline__ float2 vec_of(uint32_t v) { return make_float2(h2f_bits(v & 0xFFFFu), h2f_bits(v >> 16)); }
-// Two fp32 operations in one instruction, each rounded as the single one is.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  float2 r;
-  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  float2 r;
-  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mul.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return r;
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  float2 r;
-  asm("{\n .reg .b64 x, y, z, w;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;\n}"
-      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return r;
-}
-
 // Exact cluster sums with native 32-bit shared-memory atomics (a 64-bit one is a compare-and-swap loop): the fixed-point
 // value is added as signed pieces of 13, 13 and 14 bits; 32 768 of them stay below 2^29.  The last piece is zero for
 // |w| < 4 and then skipped.  Layout [piece][centre].
@@ -1767,7 +1760,7 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
   }
   if (d.method == RWKVQ_SQ) {
     const int MB = d.oc_pad / 128, KT = d.ic_pad / 256;
-    sq_quantize_kernel<<<MB * KT, 256, 0, s>>>(static_cast<const uint16_t*>(w_dev), oc, ic, KT, img + h.off_payload, flags, h, img);
+    sq_quantize_kernel<<<MB * KT * (8 / kSqWarps), 32 * kSqWarps, 0, s>>>(static_cast<const uint16_t*>(w_dev), oc, ic, KT, img + h.off_payload, flags, h, img);
   } else {
     VqArgs a;
     a.w = static_cast<const uint16_t*>(w_dev);
