@@ -134,8 +134,7 @@ def lib() -> C.CDLL:
         L.rwkvq_proxy_select_f32.argtypes = [vp, i32, i32, i32, dbl, dbl, C.POINTER(dbl), C.POINTER(dbl), C.POINTER(i32), vp, sz, vp]
         L.rwkvq_proxy_segments_workspace_bytes.argtypes = [i32, i32, i32, i32]
         L.rwkvq_proxy_segments_workspace_bytes.restype = sz
-        L.rwkvq_proxy_segments.argtypes = [vp, i32, i32, i32, i32, i32, i32, dbl, dbl, C.POINTER(dbl), C.POINTER(dbl),
-                                           C.POINTER(i32), vp, sz, vp]
+        L.rwkvq_proxy_segments.argtypes = [vp, i32, i32, i32, i32, i32, i32, dbl, dbl, vp, vp, vp, vp, sz, vp]
     if hasattr(L, "rwkvq_quant_error"):
         L.rwkvq_quant_error_workspace_bytes.argtypes = [C.POINTER(Desc)]
         L.rwkvq_quant_error_workspace_bytes.restype = sz
@@ -379,7 +378,7 @@ def rwkvq_proxy_select(mats, K: int, tau_c: float, tau_f: float, workspace, stre
 
 
 def _torch_dtype_code(t):
-    import torch
+    torch = _torch or _load_torch()
     return {torch.float32: RWKVQ_F32, torch.float16: RWKVQ_F16, torch.bfloat16: RWKVQ_BF16}[t.dtype]
 
 
@@ -405,17 +404,15 @@ def rwkvq_proxy_select_typed(w, K: int, tau_c: float, tau_f: float, stream=None)
 def rwkvq_proxy_segments(w, seg_rows: int, seg_cols: int, K: int, tau_c: float, tau_f: float, stream=None):
     """rwkvq_proxy_segments on a CUDA tensor [oc, ic] (float16, bfloat16 or float32).  Returns (P_c, P_f, phi)
     numpy arrays of shape [ceil(oc / seg_rows), ceil(ic / seg_cols)]."""
-    import torch
+    t, L = _torch or _load_torch(), _lib or lib()
     oc, ic = int(w.shape[0]), int(w.shape[1])
     sr, sc = min(seg_rows, oc), min(seg_cols, ic)
-    gy, gx = (oc + sr - 1) // sr, (ic + sc - 1) // sc
-    pc, pf, phi = np.empty(gy * gx, np.float64), np.empty(gy * gx, np.float64), np.empty(gy * gx, np.int32)
-    ws = torch.empty(max(256, int(lib().rwkvq_proxy_segments_workspace_bytes(oc, ic, sr, sc))), dtype=torch.uint8, device=w.device)
-    _check(lib().rwkvq_proxy_segments(_dev_ptr(w), _torch_dtype_code(w), oc, ic, seg_rows, seg_cols, K, tau_c, tau_f,
-                                      pc.ctypes.data_as(C.POINTER(C.c_double)), pf.ctypes.data_as(C.POINTER(C.c_double)),
-                                      phi.ctypes.data_as(C.POINTER(C.c_int)), _dev_ptr(ws), ws.numel(), _stream_ptr(stream)),
-           "rwkvq_proxy_segments")
-    return pc.reshape(gy, gx), pf.reshape(gy, gx), phi.reshape(gy, gx)
+    shape = ((oc + sr - 1) // sr, (ic + sc - 1) // sc)
+    pc, pf, phi = np.empty(shape, np.float64), np.empty(shape, np.float64), np.empty(shape, np.int32)
+    ws = t.empty(max(256, L.rwkvq_proxy_segments_workspace_bytes(oc, ic, sr, sc)), dtype=t.uint8, device=w.device)
+    _check(L.rwkvq_proxy_segments(w.data_ptr(), _torch_dtype_code(w), oc, ic, seg_rows, seg_cols, K, tau_c, tau_f, pc.ctypes.data,
+                                  pf.ctypes.data, phi.ctypes.data, ws.data_ptr(), ws.nbytes, _stream_ptr(stream)), "rwkvq_proxy_segments")
+    return pc, pf, phi
 
 
 def rwkvq_proxy_family(mats, workspace, stream=None):

@@ -50,6 +50,36 @@ int sm_count() {
   known[dev].store(sms, std::memory_order_relaxed);
   return sms;
 }
+void* pinned_results(size_t bytes) {
+  constexpr size_t kLeast = 64 << 10, kMost = 1 << 20;
+  struct Buffer { void* p; size_t bytes; unsigned long long context; };
+  struct Buffers {
+    Buffer of[kMaxDevices];
+    ~Buffers() {
+      for (Buffer& b : of)
+        if (b.p) cudaFreeHost(b.p);
+    }
+  };
+  static thread_local Buffers buffers;
+  const int dev = current_device();
+  const unsigned long long id = dev >= 0 ? context_id() : 0ull;
+  if (id == 0 || bytes > kMost) return nullptr;
+  Buffer& b = buffers.of[dev];
+  if (b.p && b.context == id && b.bytes >= bytes) return b.p;
+  // another thread may be capturing a graph, in which an allocation has no part
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+  if (b.p && b.context == id) cudaFreeHost(b.p);      // a context that has ended took its buffer with it
+  b = Buffer{nullptr, 0, id};
+  size_t want = kLeast;
+  while (want < bytes) want *= 2;
+  void* p = nullptr;
+  const cudaError_t e = cudaHostAlloc(&p, want, cudaHostAllocDefault);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  b.p = p; b.bytes = want;
+  return p;
+}
 }  // namespace rwkvq
 
 extern "C" {

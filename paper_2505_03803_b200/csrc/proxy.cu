@@ -130,7 +130,8 @@ static rwkvq_status run_proxy(const void* const* w, const int* oc, const int* ic
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* base = static_cast<uint8_t*>(ws);
-  ProxyResult* res = reinterpret_cast<ProxyResult*>(base + (size_t)n_mats * kMatrixBytes);
+  ProxyResult* const pinned = static_cast<ProxyResult*>(pinned_results((size_t)n_mats * sizeof(ProxyResult)));
+  ProxyResult* const res = pinned ? pinned : reinterpret_cast<ProxyResult*>(base + (size_t)n_mats * kMatrixBytes);
   cudaError_t e = cudaMemset2DAsync(base, kMatrixBytes, 0, kPatternWords * 4, n_mats, s);
   if (e != cudaSuccess) return cuda_status(e);
   const int sms = sm_count();
@@ -152,9 +153,10 @@ static rwkvq_status run_proxy(const void* const* w, const int* oc, const int* ic
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e);
   out->resize(n_mats);
-  e = cudaMemcpyAsync(out->data(), res, (size_t)n_mats * sizeof(ProxyResult), cudaMemcpyDeviceToHost, s);
+  if (!pinned) e = cudaMemcpyAsync(out->data(), res, (size_t)n_mats * sizeof(ProxyResult), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
+  if (pinned) std::copy(pinned, pinned + n_mats, out->begin());
   for (int m = 0; m < n_mats; ++m)
     if ((*out)[m].nonfinite) return RWKVQ_ENONFINITE;
   return RWKVQ_OK;

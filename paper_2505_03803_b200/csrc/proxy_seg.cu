@@ -390,7 +390,9 @@ rwkvq_status rwkvq_proxy_segments(const void* w, int dtype, int oc, int ic, int 
   const int gx = (ic + seg_cols - 1) / seg_cols, gy = (oc + seg_rows - 1) / seg_rows;
   if (gy > 65535) return RWKVQ_EUNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  pseg::SegResult* res = static_cast<pseg::SegResult*>(ws);
+  const size_t nseg = (size_t)gx * gy;
+  pseg::SegResult* const pinned = static_cast<pseg::SegResult*>(pinned_results(nseg * sizeof(pseg::SegResult)));
+  pseg::SegResult* const res = pinned ? pinned : static_cast<pseg::SegResult*>(ws);
   const dim3 grid((unsigned)gx, (unsigned)gy, 1);
   cudaError_t e = cudaSuccess;
   if (dtype == RWKVQ_F32) {
@@ -410,9 +412,13 @@ rwkvq_status rwkvq_proxy_segments(const void* w, int dtype, int oc, int ic, int 
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_status(e);
-  const size_t nseg = (size_t)gx * gy;
-  std::vector<pseg::SegResult> host(nseg);
-  e = cudaMemcpyAsync(host.data(), res, nseg * sizeof(pseg::SegResult), cudaMemcpyDeviceToHost, s);
+  std::vector<pseg::SegResult> copy;
+  const pseg::SegResult* host = pinned;
+  if (!pinned) {
+    copy.resize(nseg);
+    e = cudaMemcpyAsync(copy.data(), res, nseg * sizeof(pseg::SegResult), cudaMemcpyDeviceToHost, s);
+    host = copy.data();
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
   rwkvq_status st = RWKVQ_OK;

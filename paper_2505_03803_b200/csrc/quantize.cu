@@ -1811,11 +1811,13 @@ rwkvq_status rwkvq_quantize_check(void* workspace_dev, void* stream) {
   using namespace rwkvq;
   if (!workspace_dev) return RWKVQ_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int host_flags = 0;
-  cudaError_t e = cudaMemcpyAsync(&host_flags, workspace_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+  int copy = 0;
+  volatile int* const pinned = static_cast<int*>(pinned_results(sizeof(int)));
+  cudaError_t e = cudaMemcpyAsync(pinned ? (void*)pinned : &copy, workspace_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(workspace_dev, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e);
+  const int host_flags = pinned ? *pinned : copy;
   return (host_flags & kFlagTimeout) ? RWKVQ_ETIMEOUT : (host_flags & kFlagNonFinite) ? RWKVQ_ENONFINITE : RWKVQ_OK;
 }
 
