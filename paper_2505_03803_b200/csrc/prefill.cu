@@ -793,12 +793,17 @@ struct HostProduct {
 // Slices of a product's contraction: where it has so few tiles that its long contraction would be what the others wait for, about four
 // chunks each (a slice costs its sums in the workspace, about a chunk's time), not more in all than leave room for other products.  Of limits from
 // 48 to 296 and lengths from 3 to 7, 64 to 74 and 4 were the best over 22 layers (d 2048, 203 tokens: 53.6 us with whole tiles, 37 with
-// slices; d 768, 48 tokens: 22.6, 14.4; d 640, 1368 tokens, limit 64: no slices, 32.8 where two each took 36.9).  A function of the
+// slices; d 768, 48 tokens: 22.6, 14.4; d 640, 1368 tokens, limit 64: no slices, 32.8 where two each took 36.9).  Short contractions, whose slices
+// are a chunk or two shorter than the whole, not where their sums (tiles x tokens of a tile) are many: d 512, 1000 tokens (4160): two slices 26.8 us,
+// one 22.8; d 768, 400 tokens (2496): three 24.5, two 20.7; d 2048, 400 tokens (6656): two 62.8, one 56.2; 203 tokens (3328): two 34.9, one 37.2;
+// of twelve chunks they are worth it again (d 896, 400 tokens: three 26.6, two 28.7).  A function of the
 // product and M alone, so that a product gives the same bits in every group.
-int slices_of(int KT, long long tiles) {
-  constexpr int kMinChunks = 6, kSliceChunks = 4, kMaxSlicedTiles = 64;
+int slices_of(int KT, long long tiles, int NT) {
+  constexpr int kMinChunks = 6, kSliceChunks = 4, kMaxSlicedTiles = 64, kShortChunks = 11, kMaxShortSums = 7000;
   if (KT < kMinChunks) return 1;
-  return (int)std::min<long long>({(long long)pf::kMaxSlices, (long long)((KT + kSliceChunks / 2) / kSliceChunks), std::max<long long>(1, kMaxSlicedTiles / tiles)});
+  long long most = kMaxSlicedTiles / tiles;
+  if (KT <= kShortChunks) most = std::min(most, kMaxShortSums / (tiles * NT));
+  return (int)std::min<long long>({(long long)pf::kMaxSlices, (long long)((KT + kSliceChunks / 2) / kSliceChunks), std::max<long long>(1, most)});
 }
 
 // A product's workspace: operand tiles, the ticket, sums of the slices.
@@ -808,7 +813,7 @@ Layout layout_of(const rwkvq_desc* d, int M) {
   l.MT = (M + pf::kTileTokens - 1) / pf::kTileTokens;
   l.NT = ((M + l.MT - 1) / l.MT + 15) / 16 * 16;
   const size_t KB = (size_t)d->ic_pad / pf::kKBlock, tiles = (size_t)(d->oc_pad / 128) * l.MT;
-  l.S = slices_of((int)(KB / 4), (long long)tiles);
+  l.S = slices_of((int)(KB / 4), (long long)tiles, l.NT);
   l.off_ticket = round_up_sz((size_t)l.MT * KB * l.NT * 128, 256);
   l.off_pieces = l.off_ticket + pf::kTicketBytes;
   l.bytes = l.off_pieces + (l.S > 1 ? tiles * l.S * l.NT * 512 : 0);
