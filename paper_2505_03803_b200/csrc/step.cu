@@ -1133,14 +1133,6 @@ __device__ __forceinline__ void sq_group_words(const uint8_t* rec, int lane, uin
   }
 }
 
-// One 128-column group of the two records of a warp: the input fragments are loaded once and shared
-// by both records, whose tensor-core chains run interleaved.
-template <int NB, int GRP>
-__device__ __forceinline__ void sq_pair(const uint32_t (&wa)[6], const uint32_t (&wb)[6], const uint4 sza, const uint4 szb,
-                                        bool has_b, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
-  sq_group_mma2<NB, GRP>(wa, wb, sza, szb, has_b, xl, acca, accb);
-}
-
 template <int BITS, int NB, int HALF>
 __device__ __forceinline__ void vq_pair(const uint32_t (&wa)[2 * BITS], const uint32_t (&wb)[2 * BITS], const uint32_t* cb_lane,
                                         const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
@@ -1282,34 +1274,32 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         // Registers suffice for the whole record pair: take all of it, free the slot, then run both
         // 128-column groups as one stretch of code (eight tensor-core chains for the scheduler to interleave).
         uint32_t wa0[6], wb0[6], wa1[6], wb1[6];
-        uint4 sza = make_uint4(0, 0, 0, 0), szb = sza;
+        uint4 sza, szb;
         sq_group_words<0>(ra, lane, wa0);
         sq_group_words<1>(ra, lane, wa1);
         sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
-        if (has_b) {
-          sq_group_words<0>(rbp, lane, wb0);
-          sq_group_words<1>(rbp, lane, wb1);
-          szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
-        }
+        const uint8_t* second = has_b ? rbp : ra;      // no second record: the first one again, whose results are dropped
+        sq_group_words<0>(second, lane, wb0);
+        sq_group_words<1>(second, lane, wb1);
+        szb = *reinterpret_cast<const uint4*>(second + RWKVQ_SQ_CODE_BYTES + g * 16);
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        sq_pair<NB, 0>(wa0, wb0, sza, szb, has_b, xl, acca, accb);
-        sq_pair<NB, 1>(wa1, wb1, sza, szb, has_b, xl, acca, accb);
+        sq_group_mma2<NB, 0>(wa0, wb0, sza, szb, xl, acca, accb);
+        sq_group_mma2<NB, 1>(wa1, wb1, sza, szb, xl, acca, accb);
       } else {
       uint32_t wa[6], wb[6];
-      uint4 sza = make_uint4(0, 0, 0, 0), szb = sza;
+      uint4 sza, szb;
       sq_group_words<0>(ra, lane, wa);
       sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
-      if (has_b) {
-        sq_group_words<0>(rbp, lane, wb);
-        szb = *reinterpret_cast<const uint4*>(rbp + RWKVQ_SQ_CODE_BYTES + g * 16);
-      }
-      sq_pair<NB, 0>(wa, wb, sza, szb, has_b, xl, acca, accb);
+      const uint8_t* second = has_b ? rbp : ra;
+      sq_group_words<0>(second, lane, wb);
+      szb = *reinterpret_cast<const uint4*>(second + RWKVQ_SQ_CODE_BYTES + g * 16);
+      sq_group_mma2<NB, 0>(wa, wb, sza, szb, xl, acca, accb);
       sq_group_words<1>(ra, lane, wa);
-      if (has_b) sq_group_words<1>(rbp, lane, wb);
+      sq_group_words<1>(second, lane, wb);
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctrl->empty[slot]);     // the rest of the records is in registers: free the slot
-      sq_pair<NB, 1>(wa, wb, sza, szb, has_b, xl, acca, accb);
+      sq_group_mma2<NB, 1>(wa, wb, sza, szb, xl, acca, accb);
       }
     } else {
       // replicate the tile's codebook for conflict-free lookups (the eight warps of the group)
