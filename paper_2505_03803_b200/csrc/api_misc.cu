@@ -56,8 +56,15 @@ void* pinned_results(size_t bytes) {
   struct Buffers {
     Buffer of[kMaxDevices];
     ~Buffers() {
-      for (Buffer& b : of)
-        if (b.p) cudaFreeHost(b.p);
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;      // as below
+      bool relaxed = false;
+      for (int d = 0; d < kMaxDevices; ++d) {
+        if (!of[d].p) continue;
+        if (!relaxed && cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+        relaxed = true;
+        // a context that has ended took its buffer with it, and the address may be another allocation's by now
+        if ((current_device() == d || cudaSetDevice(d) == cudaSuccess) && context_id() == of[d].context) cudaFreeHost(of[d].p);
+      }
     }
   };
   static thread_local Buffers buffers;

@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqA
   };
   auto receive = [&](int e) -> uint32_t {
     if (tid == 0) expect_sent(pick_here, 4);
-    lost |= !wait_sent(pick_here, (uint32_t)e & 1u);
+    lost = lost || !wait_sent(pick_here, (uint32_t)e & 1u);
     return sh.pick;
   };
   const int first = below(splitmix(seed, 0), kVqMaxVec);
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqA
     }
     float excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
     if (lane == 0) excl = 0.f;
-    lost |= !wait_sent(bar, (uint32_t)(e >> 1) & 1u);
+    lost = lost || !wait_sent(bar, (uint32_t)(e >> 1) & 1u);
     float before, total;
     warp_sums(sh.tot[e & 1], tile_warp, before, total);
     const float target = sh.u01[e + 1] * total;
@@ -1524,7 +1524,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     // A block sends its next sums when it has the centres of all blocks, and a block its next centres when it has the next sums of all: neither place is
     // written again before it has been read.
     if (tid < 2 * kOwn * kVecCluster) {
-      lost |= !wait_sent(sums_here, (uint32_t)it & 1u);
+      lost = lost || !wait_sent(sums_here, (uint32_t)it & 1u);
       Sums s[kVecCluster];
 #pragma unroll
       for (int r = 0; r < kVecCluster; ++r) s[r] = reinterpret_cast<const Sums&>(sh.part[r][own][own_dim]);
@@ -1541,7 +1541,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
       peer_send(peer_address(shared_address(&sh.sent[rank * kOwn + own][own_dim]), receiver), (unsigned long long)__double_as_longlong(c), peer_address(centres_here, receiver));
     }
     if (tid < 2 * E) {
-      lost |= !wait_sent(centres_here, (uint32_t)it & 1u);
+      lost = lost || !wait_sent(centres_here, (uint32_t)it & 1u);
       set_centre(tid >> 1, tid & 1, sh.sent[tid >> 1][tid & 1]);
     }
     __syncthreads();

@@ -5,6 +5,7 @@ import os
 import subprocess
 import sys
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -54,8 +55,35 @@ def test_results_up_to_and_beyond_the_buffer(rows):
     assert np.allclose(pc[pick], rpc, rtol=1e-9, atol=1e-9) and np.allclose(pf[pick], rpf, rtol=1e-8, atol=1e-8)
 
 
-def test_results_after_a_device_reset():
-    r = subprocess.run([sys.executable, "-m", "tests.test_host_results_gpu"], cwd=ROOT, capture_output=True, text=True, timeout=300)
+def test_a_thread_may_end_while_another_captures():
+    import torch
+    from paper_2505_03803_b200 import binding as B
+    w = torch.randn((256, 512), device="cuda").half()
+    called, end = threading.Event(), threading.Event()
+
+    def work():
+        B.rwkvq_proxy_segments(w, 16, 128, 4, 3.0, math.inf)
+        called.set()
+        end.wait(60)
+
+    t = threading.Thread(target=work)
+    t.start()
+    assert called.wait(60)
+    x, graph = torch.zeros(64, device="cuda"), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, capture_error_mode="global"):
+        end.set()
+        t.join()
+        time.sleep(0.2)             # the system's thread ends a little after the interpreter's
+        x += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 64
+
+
+@pytest.mark.parametrize("what", ["calls", "thread"])
+def test_results_after_a_device_reset(what):
+    r = subprocess.run([sys.executable, "-m", "tests.test_host_results_gpu", what], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.split()[-1] == "same", r.stdout + r.stderr
 
 
@@ -66,11 +94,33 @@ if __name__ == "__main__":
     from tests.test_context_reset_gpu import _Cuda
     cu, out = _Cuda(), []
     w16 = np.random.default_rng(1).standard_normal((64, 256)).astype(np.float16)
-    for _ in range(3):
+
+    def call():
         w, n = cu.put(w16), int(B.lib().rwkvq_proxy_segments_workspace_bytes(64, 256, 1, 256))
         pc, pf, phi = np.empty(64), np.empty(64), np.empty(64, np.int32)
         cu.ok(B.lib().rwkvq_proxy_segments(w, B.RWKVQ_F16, 64, 256, 1, 256, 4, 3.0, math.inf, pc.ctypes.data, pf.ctypes.data, phi.ctypes.data, cu.zeros(n), n, None))
         out.append((pc, pf, phi))
+
+    if sys.argv[1] == "calls":
+        for _ in range(3):
+            call()
+            cu.ok(cu.rt.cudaDeviceReset())
+        assert all(np.array_equal(a, b) for o in out[1:] for a, b in zip(out[0], o)) and np.isfinite(out[0][0]).all()
+    else:
+        # a thread ends in a later context than its buffer's: what lies at the buffer's address by then stays
+        called, end = threading.Event(), threading.Event()
+        t = threading.Thread(target=lambda: (call(), called.set(), end.wait(60)))
+        t.start()
+        assert called.wait(60)
         cu.ok(cu.rt.cudaDeviceReset())
-    assert all(np.array_equal(a, b) for o in out[1:] for a, b in zip(out[0], o)) and np.isfinite(out[0][0]).all()
+        later = []
+        for _ in range(4):
+            p = C.c_void_p()
+            cu.ok(cu.rt.cudaMallocHost(C.byref(p), 64 << 10))
+            later.append(p)
+        end.set()
+        t.join()
+        time.sleep(0.2)
+        for p in later:
+            cu.ok(cu.rt.cudaFreeHost(p))
     print("same")
