@@ -147,11 +147,12 @@ template <int NB> struct Shape {
 constexpr int groups_of(int NB) { return NB == 2 ? 1 : 2; }
 constexpr int threads_of(int NB) { return NB == 2 ? Shape<2>::kThreads : Shape<1>::kThreads; }
 constexpr int kMaxSlots = 12;
-constexpr uint32_t kCtrlBytes = 1024, kXBufTotal = 65536, kMuScratch = 1024;
+constexpr uint32_t kCtrlBytes = 1024, kMuScratch = 1024;
 // Input-segment buffers: two of 32 KB, one in use and one being filled.  Large segments matter more than
 // deep buffering (every hand-over of a segment costs all roles a pass through the barriers): four buffers
 // of a quarter the size, and buffers that cost the weight ring a slot or two, were measured and are slower.
-template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = kXBufTotal / kCount; };
+constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 32768u : 32768u; }
+template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = xbuf_bytes_of(NB); };
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
 constexpr uint32_t kDefaultPollLimit = 1u << 22;
 
@@ -1133,10 +1134,34 @@ __device__ __forceinline__ void sq_group_words(const uint8_t* rec, int lane, uin
   }
 }
 
-template <int BITS, int NB, int HALF>
-__device__ __forceinline__ void vq_pair(const uint32_t (&wa)[2 * BITS], const uint32_t (&wb)[2 * BITS], const uint32_t* cb_lane,
-                                        const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
-  vq_half_mma2<BITS, NB, HALF>(wa, wb, cb_lane, xl, acca, accb);
+// A pair of VQ records.  The tile's codebook is copied 32 times for lookups without bank conflicts by the eight warps of the group, an eighth of its
+// entries each, sixteen bytes a lane and store: in steps of four bytes, one behind the other, the copies of 256 entries took a fifth of the time.
+// Bound by the lookups, 1024 of the 1750 reads and writes of shared memory that a unit takes (at batch 1 its pipe is busy 70 to 76 % of the time).
+template <int BITS, int NB>
+__device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, const uint32_t* codebook, uint8_t* rep, int w, int lane, int bar,
+                                        uint64_t* empty, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
+  constexpr int kStores = (1 << BITS) / 32;        // of a warp, four entries each
+  uint32_t entry[kStores];
+#pragma unroll
+  for (int i = 0; i < kStores; ++i) entry[i] = codebook[(w * kStores + i) * 4 + (lane >> 3)];
+  named_bar_sync(bar, kGroupThreads);              // the group's previous lookups are done
+#pragma unroll
+  for (int i = 0; i < kStores; ++i) *reinterpret_cast<uint4*>(rep + (w * kStores + i) * 512 + lane * 16) = make_uint4(entry[i], entry[i], entry[i], entry[i]);
+  uint32_t va[2 * BITS], vb[2 * BITS];
+  vq_half_words<BITS, 0>(ra, lane, va); vq_half_words<BITS, 0>(rb, lane, vb);
+  named_bar_sync(bar, kGroupThreads);
+  const uint32_t* cb_lane = reinterpret_cast<const uint32_t*>(rep) + lane;
+  // A unit's sums start at zero and are added with a rounding of their own: the tensor core's accumulation cuts off, and its error grows with the chain.
+  float ca[NB][4] = {}, cb[NB][4] = {};
+  vq_half_mma2<BITS, NB, 0>(va, vb, cb_lane, xl, ca, cb);
+  vq_half_words<BITS, 1>(ra, lane, va); vq_half_words<BITS, 1>(rb, lane, vb);
+  __syncwarp();
+  if (lane == 0) mbar_arrive(empty);               // the rest of the records is in registers: free the slot
+  vq_half_mma2<BITS, NB, 1>(va, vb, cb_lane, xl, ca, cb);
+#pragma unroll
+  for (int n = 0; n < NB; ++n)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { acca[n][k] += ca[n][k]; accb[n][k] += cb[n][k]; }
 }
 
 // c[k] of the four lanes whose row index g differs in its two low bits (lanes 4 apart) -> lane i (= g & 3)
@@ -1302,34 +1327,12 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
       sq_group_mma2<NB, 1>(wa, wb, sza, szb, xl, acca, accb);
       }
     } else {
-      // replicate the tile's codebook for conflict-free lookups (the eight warps of the group)
-      const uint32_t E = u->entries;
-      named_bar_sync(1 + grp, kGroupThreads);          // the group's previous lookups are done
-      {
-        const uint32_t* cbraw = reinterpret_cast<const uint32_t*>(data + 2 * chb);
-        uint32_t* rp = reinterpret_cast<uint32_t*>(rep);
-        for (uint32_t idx = (uint32_t)(w * 32 + lane); idx < E * 32u; idx += kGroupThreads) rp[idx] = cbraw[idx >> 5];
-      }
-      named_bar_sync(1 + grp, kGroupThreads);
-      const uint32_t* cb_lane = reinterpret_cast<const uint32_t*>(rep) + lane;
       const XLane xl = make_xlane(xb + (size_t)u->xcol0 * 2, xstride, nullptr, nbp, a.B, lane);
-      if (flags & UF_BITS8) {
-        uint32_t va[16], vb[16];
-        vq_half_words<8, 0>(ra, lane, va); vq_half_words<8, 0>(rbp, lane, vb);
-        vq_pair<8, NB, 0>(va, vb, cb_lane, xl, acca, accb);
-        vq_half_words<8, 1>(ra, lane, va); vq_half_words<8, 1>(rbp, lane, vb);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        vq_pair<8, NB, 1>(va, vb, cb_lane, xl, acca, accb);
-      } else {
-        uint32_t va[12], vb[12];
-        vq_half_words<6, 0>(ra, lane, va); vq_half_words<6, 0>(rbp, lane, vb);
-        vq_pair<6, NB, 0>(va, vb, cb_lane, xl, acca, accb);
-        vq_half_words<6, 1>(ra, lane, va); vq_half_words<6, 1>(rbp, lane, vb);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
-        vq_pair<6, NB, 1>(va, vb, cb_lane, xl, acca, accb);
-      }
+      const uint32_t* cbraw = reinterpret_cast<const uint32_t*>(data + 2 * chb);
+      if (flags & UF_BITS8)
+        vq_unit<8, NB>(ra, rbp, cbraw, rep, w, lane, 1 + grp, &ctrl->empty[slot], xl, acca, accb);
+      else
+        vq_unit<6, NB>(ra, rbp, cbraw, rep, w, lane, 1 + grp, &ctrl->empty[slot], xl, acca, accb);
     }
     if (flags & UF_FLUSH) {
       {
@@ -1378,7 +1381,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   extern __shared__ __align__(128) uint8_t smem[];
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(smem);
   uint8_t* xbufs = smem + kCtrlBytes + (size_t)a.n_slots * a.slot_bytes;
-  uint32_t* mucb = reinterpret_cast<uint32_t*>(xbufs + kXBufTotal);
+  uint32_t* mucb = reinterpret_cast<uint32_t*>(xbufs + XBufs<MIX, NB>::kCount * XBufs<MIX, NB>::kBytes);
   uint8_t* replicas = reinterpret_cast<uint8_t*>(mucb) + kMuScratch;
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.n_slots; ++s) { mbar_init(&ctrl->full[0][s], 1); mbar_init(&ctrl->full[1][s], 1); mbar_init(&ctrl->empty[s], kGroupWarps); }
@@ -1502,7 +1505,8 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   if (has_vq8) data_max = std::max(data_max, 2u * 8u * 2048u + 1024u);
   info->slot_bytes = (128u + data_max + 127u) & ~127u;
   info->replica_bytes = has_vq8 ? 256u * 128u : has_vq6 ? 64u * 128u : 0u;   // per consumer group
-  const uint32_t fixed = kCtrlBytes + kXBufTotal + kMuScratch + (uint32_t)kGroups * info->replica_bytes;
+  const uint32_t xbuf_bytes = xbuf_bytes_of(B <= 8 ? 1 : 2);
+  const uint32_t fixed = kCtrlBytes + XBufs<0, 1>::kCount * xbuf_bytes + kMuScratch + (uint32_t)kGroups * info->replica_bytes;
   int ns = (int)((kSmemLimit - fixed) / info->slot_bytes);
   if (ns > kMaxSlots) ns = kMaxSlots;
   if (ns < 2) return RWKVQ_EUNSUPPORTED;
@@ -1531,7 +1535,6 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;
-  const uint32_t xbuf_bytes = XBufs<0, 1>::kBytes;
   info->mix = any_xform ? 2 : mix ? 1 : 0;      // the kernel's MIX
   const uint32_t nbp = (uint32_t)((B + 1) & ~1);
 
@@ -1627,10 +1630,10 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     // warps, so that the CTAs that get a stage's VQ matrix do not finish last.
     auto cost_of = [&](const HostUnit& h) -> uint64_t {
       const uint64_t recs = (h.u.bytes0 + h.u.bytes1) / h.u.rec_bytes;
-      // in twentieths of an SQ record; the table lookups weigh more the more batch columns a record meets
-      // (whole-step times of all-SQ against all-VQ-64 stacks less the per-stage chain: 1.4 at B = 1,
-      // 1.6 at B = 8, 2.0 at B = 16)
-      const uint64_t vq6 = B > 8 ? 40u : B >= 4 ? 32u : 29u, vq8 = B > 8 ? 34u : B >= 4 ? 28u : 25u;
+      // in twentieths of an SQ record, from stacks of one format and one stage (52 MB a layer, four layers, us: SQ / 64 / 256 entries at batch 1
+      // 88, 121, 128; 8: 99, 135, 143; 16: 146, 177, 189), and the best of 24 to 34 for whole steps (14B-class, batch 16: 24 3416 us, 26 3420, 30 3427,
+      // 34 3475; 7B-class, batch 1: 24 to 28 1153, 30 1162, 33 1185; batch 8: 24 1367, 27 1358, 33 1367)
+      const uint64_t vq6 = B > 8 ? 26u : 27u, vq8 = B > 8 ? 26u : 28u;
       const uint64_t wgt = !(h.u.flags & UF_VQ) ? 20u : (h.u.flags & UF_BITS8) ? vq8 : vq6;
       return recs * wgt * 64u;
     };
