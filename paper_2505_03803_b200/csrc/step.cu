@@ -146,12 +146,16 @@ template <int NB> struct Shape {
 };
 constexpr int groups_of(int NB) { return NB == 2 ? 1 : 2; }
 constexpr int threads_of(int NB) { return NB == 2 ? Shape<2>::kThreads : Shape<1>::kThreads; }
-constexpr int kMaxSlots = 12;
+// Slots of the weight ring: a unit for each consumer group and one on its way.  More are filled while a stage's first inputs are read, and hold those
+// up (7B-class stack, batch 1: two 1257 us, three 1134, four 1144, five 1153; batch 8: 1478, 1355, 1359); above eight rows, with one group, two do
+// as well as four (14B-class stack: 3420 us each).
+constexpr int kMaxSlots = 3;
 constexpr uint32_t kCtrlBytes = 1024, kMuScratch = 1024;
-// Input-segment buffers: two of 32 KB, one in use and one being filled.  Large segments matter more than
-// deep buffering (every hand-over of a segment costs all roles a pass through the barriers): four buffers
-// of a quarter the size, and buffers that cost the weight ring a slot or two, were measured and are slower.
-constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 32768u : 32768u; }
+// Input-segment buffers, one in use and one being filled, as large as the ring leaves: every hand-over of a segment costs all roles a pass through the
+// barriers.  Above eight rows 62 KB hold the 1792 columns of sixteen rows that a CTA's seven units of a 4096-column product read (14B-class stack,
+// batch 16: 32 KB 3420 us, 48 KB 3348, 62 KB 3327); up to eight rows 40 KB hold the 2048 columns of eight (7B-class stack with 256 entries, batch 8:
+// 32 KB 1514 us, 40 KB 1488).
+constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 63488u : 40960u; }
 template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = xbuf_bytes_of(NB); };
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
 constexpr uint32_t kDefaultPollLimit = 1u << 22;

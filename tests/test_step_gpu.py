@@ -434,3 +434,29 @@ def test_step_with_many_products_in_one_stage(Bn):
     torch.cuda.synchronize()
     assert B.rwkvq_device_status() == 0
     _check(ops, Bn)
+
+
+@pytest.mark.parametrize("Bn,ic,bits", [(1, 2560, 3), (2, 2560, 8), (8, 2304, 6), (8, 2560, 3), (8, 2560, 8), (9, 2048, 3), (16, 1792, 8), (16, 2048, 3),
+                                        (16, 2048, 6), (16, 4096, 8)])
+def test_step_inputs_of_one_buffer_and_of_more(Bn, ic, bits):
+    """A row of tiles a CTA: its columns fill an input buffer or go on in the next.  Inputs and decoded weights are exact, so that only the
+    fp32 sums differ (1e-5 of |w| |x|)."""
+    oc, g = 256 * 150, torch.Generator(device="cuda").manual_seed(Bn * ic + bits)
+    desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ if bits == 3 else B.RWKVQ_VQ, bits)
+    w = (torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half()
+    image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    B.rwkvq_quantize_dev_async(w, oc, ic, desc.method, bits, image, ws, kmeans_iters=0, seed=1)
+    x = torch.randn((Bn, ic), generator=g, device="cuda").half()
+    y = torch.full((Bn, oc), float("nan"), device="cuda")
+    ops = B.make_ops([dict(desc=desc, W=image, mu_desc=None, mu=None, x=x, xprev=None, y=y, stage=0)])
+    plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
+    B.rwkvq_step_plan(ops, Bn, plan)
+    B.rwkvq_step_run(plan)
+    decoded = torch.empty((oc, ic), device="cuda")
+    B.rwkvq_dequant(desc, image, decoded)
+    ref = x.double() @ decoded.double().T
+    bound = 1e-5 * x.double().norm(dim=1)[:, None] * decoded.double().norm(dim=1)[None]
+    assert bool(((y.double() - ref).abs() <= bound).all())
+    assert B.rwkvq_device_status() == 0
+    B.rwkvq_step_plan_release(plan)
