@@ -347,8 +347,27 @@ struct VqRecord {
 // Copy one codebook (E half2 entries) into 32 lane-private replicas: entry e of lane l at word
 // e*32 + l, so a lookup by any index pattern is bank-conflict free.
 __device__ __forceinline__ void stage_codebook(uint8_t* dst, const uint32_t* src, int E) {
-  uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  for (int idx = threadIdx.x; idx < E * 32; idx += blockDim.x) d[idx] = __ldg(src + (idx >> 5));
+  uint4* d = reinterpret_cast<uint4*>(dst);
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < E * 8; idx += blockDim.x) {
+    const uint32_t v = __ldg(src + (idx >> 3));
+    d[idx] = make_uint4(v, v, v, v);
+  }
+}
+
+// Entry of index n (0..63) of a lane's VQ stream; `base`: shared address of this lane's replica of entry 0.  The index is shifted to where it counts
+// entries of 128 bytes, so that mask and base follow at once; through an index and a pointer it took half as many integer instructions again (stacks of
+// 64 / 256 entries, one stage: batch 1 140 -> 121, 147 -> 128 us; batch 16 204 -> 177, 210 -> 189).
+template <int BITS, int NW>
+__device__ __forceinline__ uint32_t vq_entry(const uint32_t (&w)[NW], int n, uint32_t base) {
+  constexpr uint32_t mask = ((1u << BITS) - 1u) << 7;
+  const int bit = BITS * n, wi = bit >> 5, sh = bit & 31;
+  uint32_t v;
+  if (sh + BITS > 32) v = __funnelshift_r(w[wi], w[wi + 1 < NW ? wi + 1 : wi], sh - 7);
+  else v = sh >= 7 ? w[wi] >> (sh - 7) : w[wi] << (7 - sh);
+  uint32_t r;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r) : "r"((v & mask) + base));
+  return r;
 }
 
 // One VQ record: every fragment register is one codebook lookup (a 2-D vector is exactly the
@@ -356,11 +375,12 @@ __device__ __forceinline__ void stage_codebook(uint8_t* dst, const uint32_t* src
 template <int BITS, int NB, int JBEG = 0, int JEND = 16>
 __device__ __forceinline__ void vq_record_mma(const uint32_t (&w)[2 * BITS], const uint32_t* cb_lane, const XLane& xl,
                                               float (&acc)[NB][4]) {
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(cb_lane);
 #pragma unroll
   for (int j = JBEG; j < JEND; ++j) {
     uint32_t afrag[4];
 #pragma unroll
-    for (int R = 0; R < 4; ++R) afrag[R] = cb_lane[vq_index<BITS, 2 * BITS>(w, 4 * j + R) * 32u];
+    for (int R = 0; R < 4; ++R) afrag[R] = vq_entry<BITS, 2 * BITS>(w, 4 * j + R, base);
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       const uint2 bf = *reinterpret_cast<const uint2*>(xl.x[n] + j * 32);
@@ -387,21 +407,6 @@ __device__ __forceinline__ void vq_half_words(const uint8_t* rec, int lane, uint
     const uint4 q = *reinterpret_cast<const uint4*>(rec + 1024 + lane * 16);
     w[6] = p.x; w[7] = p.y; w[8] = q.x; w[9] = q.y; w[10] = q.z; w[11] = q.w;
   }
-}
-
-// Entry of index n (0..63) of a lane's VQ stream; `base`: shared address of this lane's replica of entry 0.  The index is shifted to where it counts
-// entries of 128 bytes, so that mask and base follow at once; through an index and a pointer it took half as many integer instructions again (stacks of
-// 64 / 256 entries, one stage: batch 1 140 -> 121, 147 -> 128 us; batch 16 204 -> 177, 210 -> 189).
-template <int BITS, int NW>
-__device__ __forceinline__ uint32_t vq_entry(const uint32_t (&w)[NW], int n, uint32_t base) {
-  constexpr uint32_t mask = ((1u << BITS) - 1u) << 7;
-  const int bit = BITS * n, wi = bit >> 5, sh = bit & 31;
-  uint32_t v;
-  if (sh + BITS > 32) v = __funnelshift_r(w[wi], w[wi + 1 < NW ? wi + 1 : wi], sh - 7);
-  else v = sh >= 7 ? w[wi] >> (sh - 7) : w[wi] << (7 - sh);
-  uint32_t r;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r) : "r"((v & mask) + base));
-  return r;
 }
 
 // Eight tensor-core steps (HALF of the tile's columns) of two VQ records of one tile (rows r and
