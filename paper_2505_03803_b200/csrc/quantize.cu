@@ -19,6 +19,13 @@ namespace {
 
 constexpr int kFlagNonFinite = 1, kFlagTimeout = 2;
 
+// Every kernel here is launched while the one before it still runs, lets the next one be, and touches memory behind this: a call of short kernels
+// otherwise waits 2 us for each to start (five vectors of 4096 with 128 samples, ten kernels: 303 -> 288 us; a layer of 512 columns 284 -> 270).
+__device__ __forceinline__ void after_the_kernel_before() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+}
+
 // The first block of a quantizer kernel also writes the image's header and clears the alignment padding behind its last section
 // (a launch and a memset of their own took as long as quantizing a small matrix).
 __device__ __forceinline__ void write_header(const rwkvq_image_header& h, uint8_t* image) {
@@ -75,6 +82,7 @@ __global__ void __launch_bounds__(32 * kSqWarps, 20 / kSqWarps) sq_quantize_kern
                                                              const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
   __shared__ __align__(16) uint8_t codes_all[kSqWarps][16 * kSqRowStride];
   __shared__ float4 code_all[kSqWarps][2][16];                     // [warp][group][row]: -s, 1/s, z / 8, 1.5 * 2^20 (+ 1/8 for an odd z)
+  after_the_kernel_before();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (blockIdx.x == 0) write_header(head, image);
   const unsigned record = blockIdx.x * kSqWarps + warp, chunk = record >> 3;
@@ -442,7 +450,7 @@ struct TileSeeds {
   uint32_t pick;
 };
 __global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqArgs a) {
-  asm volatile("griddepcontrol.launch_dependents;");
+  after_the_kernel_before();
   extern __shared__ __align__(16) uint8_t smem[];
   TileSeeds& sh = *reinterpret_cast<TileSeeds*>(smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, E = a.E;
@@ -521,7 +529,7 @@ struct SeedShared {
 };
 template <bool kVector>
 __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) {
-  asm volatile("griddepcontrol.launch_dependents;");
+  after_the_kernel_before();
   extern __shared__ __align__(16) uint8_t smem[];
   uint32_t* vec = reinterpret_cast<uint32_t*>(smem);
   const int n = kVector ? a.n_vec : kVqMaxVec, E = a.E, threads = kVector ? (int)blockDim.x : kVqThreads;
@@ -796,6 +804,7 @@ __global__ void __launch_bounds__(LloydOf<kBlocks>::kThreads, kBlocks == 1 ? 1 :
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t rank = cluster_rank();
   const int tile = blockIdx.x / kBlocks, tr = tile / a.TC, tc = tile % a.TC;
+  asm volatile("griddepcontrol.launch_dependents;");      // the kernel of the seeds has seen the one before it end: weights and image may be touched
   if (blockIdx.x == 0) write_header(head, image);
   uint32_t pos[kVec / kThreads / 2];         // numbers of the vectors tid, tid + kThreads, ..., two to a word
   {
@@ -1365,6 +1374,8 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   const float2* wgt = reinterpret_cast<const float2*>(a.elem_w);
   const uint32_t rank = cluster_rank();
   const bool lead = rank == 0u;
+  if (n <= kVecSeeds) asm volatile("griddepcontrol.wait;" ::: "memory");      // else the kernel of the seeds has waited
+  asm volatile("griddepcontrol.launch_dependents;");
   if (lead) write_header(head, image);
   // this block's vectors: [begin, begin + 32 * groups), those below n
   const int groups = (n + 32 * kVecCluster - 1) / (32 * kVecCluster), begin = (int)rank * groups * 32;
@@ -1622,6 +1633,7 @@ __global__ void __launch_bounds__(256) representative_kernel(const RepArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   float* tile = reinterpret_cast<float*>(smem);      // [S][9]
   const int j0 = blockIdx.x * 8, S = a.S, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  after_the_kernel_before();
   for (int i = threadIdx.x; i < S * 8; i += 256) {
     const int s = i >> 3, c = i & 7;
     tile[s * 9 + c] = (j0 + c < a.n) ? __ldg(a.samples + (size_t)s * a.n + j0 + c) : 0.f;
@@ -1693,17 +1705,16 @@ constexpr unsigned kSpreadTiles = 100;
 // enough: 33 clusters of four fit one block an SM, 66 two (36 tiles: 308 us as they come, 252 so).
 constexpr int kSmemAlone = 118 * 1024, kSmemTwo = 80 * 1024;
 size_t smem_to_spread(unsigned tiles) { return tiles <= 33 ? kSmemAlone : tiles <= 66 ? kSmemTwo : 0; }
-// `early`: may start while the kernel before it runs, which this library launched in the same call.
 template <class... Args>
-cudaError_t launch_cluster(void (*fn)(Args...), unsigned blocks, unsigned cluster, unsigned threads, size_t smem, bool early, cudaStream_t s, const Args&... args) {
+cudaError_t launch(void (*fn)(Args...), unsigned blocks, unsigned cluster, unsigned threads, size_t smem, cudaStream_t s, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = early ? 2 : 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 template <int E, bool kWeighted>
@@ -1711,7 +1722,7 @@ cudaError_t launch_vector(const VqArgs& a, const rwkvq_image_header& h, uint8_t*
   static SmemOptIn opt_in(true);
   const cudaError_t e = opt_in((const void*)vq_vector_kernel<E, kWeighted>, (int)sizeof(VecShared<E>));
   if (e != cudaSuccess) return e;
-  return launch_cluster(vq_vector_kernel<E, kWeighted>, kVecCluster, kVecCluster, kVecThreads, sizeof(VecShared<E>), a.n_vec > kVecSeeds, s, a, h, img);
+  return launch(vq_vector_kernel<E, kWeighted>, kVecCluster, kVecCluster, kVecThreads, sizeof(VecShared<E>), s, a, h, img);
 }
 template <int EW, int kBlocks>
 cudaError_t launch_lloyd(const VqArgs& a, const rwkvq_image_header& h, uint8_t* img, unsigned tiles, cudaStream_t s) {
@@ -1720,7 +1731,7 @@ cudaError_t launch_lloyd(const VqArgs& a, const rwkvq_image_header& h, uint8_t* 
   const cudaError_t e = opt_in((const void*)vq_lloyd_kernel<EW, kBlocks>, kBlocks == 1 ? (int)sizeof(Shared) : kSmemAlone);
   if (e != cudaSuccess) return e;
   const size_t smem = kBlocks == 1 ? sizeof(Shared) : std::max(sizeof(Shared), smem_to_spread(tiles));
-  return launch_cluster(vq_lloyd_kernel<EW, kBlocks>, tiles * kBlocks, kBlocks, LloydOf<kBlocks>::kThreads, smem, true, s, a, h, img);
+  return launch(vq_lloyd_kernel<EW, kBlocks>, tiles * kBlocks, kBlocks, LloydOf<kBlocks>::kThreads, smem, s, a, h, img);
 }
 
 }  // namespace
@@ -1760,7 +1771,9 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
   }
   if (d.method == RWKVQ_SQ) {
     const int MB = d.oc_pad / 128, KT = d.ic_pad / 256;
-    sq_quantize_kernel<<<MB * KT * (8 / kSqWarps), 32 * kSqWarps, 0, s>>>(static_cast<const uint16_t*>(w_dev), oc, ic, KT, img + h.off_payload, flags, h, img);
+    e = launch(sq_quantize_kernel, (unsigned)(MB * KT * (8 / kSqWarps)), 1, 32 * kSqWarps, 0, s, static_cast<const uint16_t*>(w_dev), oc, ic, KT, img + h.off_payload, flags,
+               (const rwkvq_image_header)h, img);
+    if (e != cudaSuccess) return cuda_status(e);
   } else {
     VqArgs a;
     a.w = static_cast<const uint16_t*>(w_dev);
@@ -1779,7 +1792,8 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
         const int seed_threads = (a.n_vec + 2047) / 2048 * 32;
         e = opt_in_seed((const void*)vq_seed_kernel<true>, kVqMaxVec * 4 + (int)sizeof(SeedShared));
         if (e != cudaSuccess) return cuda_status(e);
-        vq_seed_kernel<true><<<1, seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s>>>(a);
+        e = launch(vq_seed_kernel<true>, 1, 1, (unsigned)seed_threads, (size_t)seed_threads * kVqPerThread * 4 + sizeof(SeedShared), s, (const VqArgs)a);
+        if (e != cudaSuccess) return cuda_status(e);
       }
       e = d.entries == 64 ? (a.elem_w ? launch_vector<64, true>(a, h, img, s) : launch_vector<64, false>(a, h, img, s))
                           : (a.elem_w ? launch_vector<256, true>(a, h, img, s) : launch_vector<256, false>(a, h, img, s));
@@ -1789,12 +1803,12 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
       if (spread) {
         static SmemOptIn opt_in_seed;
         e = opt_in_seed((const void*)vq_tile_seed_kernel, kSmemAlone);
-        if (e == cudaSuccess) e = launch_cluster(vq_tile_seed_kernel, tiles * kTileBlocks, kTileBlocks, kSeedThreads, std::max(sizeof(TileSeeds), smem_to_spread(tiles)), false, s, (const VqArgs)a);
+        if (e == cudaSuccess) e = launch(vq_tile_seed_kernel, tiles * kTileBlocks, kTileBlocks, kSeedThreads, std::max(sizeof(TileSeeds), smem_to_spread(tiles)), s, (const VqArgs)a);
       } else {
         static SmemOptIn opt_in_seed;
         constexpr size_t seed_smem = (size_t)kVqMaxVec * 4 + sizeof(SeedShared);
         e = opt_in_seed((const void*)vq_seed_kernel<false>, (int)seed_smem);
-        if (e == cudaSuccess) vq_seed_kernel<false><<<tiles, kVqThreads, seed_smem, s>>>(a);
+        if (e == cudaSuccess) e = launch(vq_seed_kernel<false>, tiles, 1, kVqThreads, seed_smem, s, (const VqArgs)a);
       }
       if (e == cudaSuccess) e = d.entries == 64 ? (spread ? launch_lloyd<2, 4>(a, h, img, tiles, s) : launch_lloyd<2, 1>(a, h, img, tiles, s))
                                              : (spread ? launch_lloyd<8, 4>(a, h, img, tiles, s) : launch_lloyd<8, 1>(a, h, img, tiles, s));
@@ -1851,15 +1865,16 @@ rwkvq_status rwkvq_calib_representative(const float* samples_dev, int n_samples,
   a.k_hi = (int)v_hi; a.g_hi = v_hi - (double)a.k_hi;
   if (a.k_hi > n_samples - 1) { a.k_hi = n_samples - 1; a.g_hi = 0.0; }
   const size_t smem = (size_t)n_samples * 9 * sizeof(float);       // at most 36 KB
-  const dim3 grid((n + 7) / 8);
+  const unsigned grid = (unsigned)((n + 7) / 8);
+  cudaError_t e;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (n_samples <= 32) representative_kernel<1><<<grid, 256, smem, st>>>(a);
-  else if (n_samples <= 64) representative_kernel<2><<<grid, 256, smem, st>>>(a);
-  else if (n_samples <= 128) representative_kernel<4><<<grid, 256, smem, st>>>(a);
-  else if (n_samples <= 256) representative_kernel<8><<<grid, 256, smem, st>>>(a);
-  else if (n_samples <= 512) representative_kernel<16><<<grid, 256, smem, st>>>(a);
-  else representative_kernel<32><<<grid, 256, smem, st>>>(a);
-  return cuda_status(cudaGetLastError());
+  if (n_samples <= 32) e = launch(representative_kernel<1>, grid, 1, 256, smem, st, (const RepArgs)a);
+  else if (n_samples <= 64) e = launch(representative_kernel<2>, grid, 1, 256, smem, st, (const RepArgs)a);
+  else if (n_samples <= 128) e = launch(representative_kernel<4>, grid, 1, 256, smem, st, (const RepArgs)a);
+  else if (n_samples <= 256) e = launch(representative_kernel<8>, grid, 1, 256, smem, st, (const RepArgs)a);
+  else if (n_samples <= 512) e = launch(representative_kernel<16>, grid, 1, 256, smem, st, (const RepArgs)a);
+  else e = launch(representative_kernel<32>, grid, 1, 256, smem, st, (const RepArgs)a);
+  return cuda_status(e == cudaSuccess ? cudaGetLastError() : e);
 }
 
 }  // extern "C"

@@ -467,3 +467,31 @@ def test_vq_tiles_alike_in_one_block_and_in_a_cluster(few, bits):
     for t in range(min(few, 3)):
         v = w16[:, t * 256:(t + 1) * 256].astype(np.float64).reshape(-1, 2)
         assert np.array_equal(index[1][:, t * 128:(t + 1) * 128].reshape(-1), orc._nearest(v, books[1][t].astype(np.float64)))
+
+
+@pytest.mark.parametrize("oc,ic,bits", [(128, 256, 3), (2048, 1024, 3), (256, 512, 6), (2816, 2816, 6), (1, 1024, 6), (1, 10240, 8)])
+def test_quantizers_start_behind_what_writes_their_inputs(oc, ic, bits):
+    """Kernels that write the weights, quantize them, read the image and write other weights, one behind the other without a wait of the host."""
+    method = B.RWKVQ_SQ if bits == 3 else B.RWKVQ_VQ
+    desc = B.rwkvq_desc_for(oc, ic, method, bits)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(oc + ic)
+    src = [(torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half() for _ in range(4)]
+    samples = [torch.randn((40, ic), generator=g, device="cuda") for _ in range(4)]
+    w, image = torch.zeros((oc, ic), dtype=torch.float16, device="cuda"), torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+    rep, out = torch.zeros(ic, device="cuda"), torch.empty((oc, ic), device="cuda")
+
+    def one(i, wait):
+        for step in (lambda: w.copy_(src[i]), lambda: B.rwkvq_calib_representative(samples[i], 1.0, rep_sq=rep),
+                     lambda: B.rwkvq_quantize_dev_async(w, oc, ic, method, bits, image, ws, elem_weight=rep if oc == 1 else None, kmeans_iters=2, seed=i),
+                     lambda: B.rwkvq_dequant(desc, image, out)):
+            step()
+            if wait:
+                torch.cuda.synchronize()
+        return out.clone()
+
+    want = [one(i, True) for i in range(4)]
+    got = [one(i % 4, False) for i in range(16)]
+    assert B.rwkvq_quantize_check(ws) == 0
+    for i, y in enumerate(got):
+        assert torch.equal(y, want[i % 4])
