@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(1024, 1) proxy_reduce_kernel(const uint8_t* ws
   __shared__ __align__(16) uint32_t bm[kPatternWords];
   __shared__ SetShared<1024> sh;
   const uint2* all = reinterpret_cast<const uint2*>(ws + (size_t)blockIdx.x * kMatrixBytes);
+  fill_log_table(sh.logs);
   reinterpret_cast<uint2*>(bm)[threadIdx.x] = __ldcg(all + threadIdx.x);
   __syncthreads();
   const double n = (double)(a.n[blockIdx.x] - 1ull);

@@ -79,21 +79,30 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_set_kernel(const uint16
   __syncthreads();
   const uint16_t* src = w + (size_t)r0 * ic + c0;
   if (wide) {
-    const int per_row = nc >> 3, total = nr * per_row;
-    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * T) {
-      uint4 v[4];
-      bool in[4];
+    // the next vectors, or the table of logarithms, are on their way while these are marked
+    const int per_row = nc >> 3, total = nr * per_row, step_r = T / per_row, step_c = T % per_row;
+    int r = threadIdx.x / per_row, c = threadIdx.x % per_row;
+    uint4 v[4], next[4];
+    auto fetch = [&](uint4 (&to)[4], int i0) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * T;
-        in[u] = i < total;
-        if (in[u]) v[u] = ldg_stream(src + (size_t)(i / per_row) * ic + 8 * (i % per_row));
+        if (i0 + u * T < total) to[u] = ldg_stream(src + (size_t)r * ic + 8 * c);
+        r += step_r; c += step_c;
+        if (c >= per_row) { c -= per_row; ++r; }
       }
+    };
+    fetch(v, threadIdx.x);
+    fill_log_table(sh.logs);
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * T) {
+      fetch(next, i0 + 4 * T);
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (in[u]) { mark_pair(bm, v[u].x); mark_pair(bm, v[u].y); mark_pair(bm, v[u].z); mark_pair(bm, v[u].w); }
+      for (int u = 0; u < 4; ++u) {
+        if (i0 + u * T < total) { mark_pair(bm, v[u].x); mark_pair(bm, v[u].y); mark_pair(bm, v[u].z); mark_pair(bm, v[u].w); }
+        v[u] = next[u];
+      }
     }
   } else {
+    fill_log_table(sh.logs);
     const int total = nr * nc;
     for (int i = threadIdx.x; i < total; i += T) mark_pattern(bm, src[(size_t)(i / nc) * ic + i % nc]);
   }
