@@ -1630,16 +1630,16 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           units.push_back(h);
         }
     }
-    // The cost of a unit is its record count weighted by what a record of its format costs the consumer
-    // warps, so that the CTAs that get a stage's VQ matrix do not finish last.
+    // The cost of a unit is what a record of its format costs the consumer warps, so that the CTAs that get a stage's VQ matrix do not finish
+    // last.  A unit of the last 128 rows of an odd number takes the warps as long as a whole one (d 3712, batch 1, twelve layers: 403 us so, 572 when it
+    // counted half; d 2944, batch 12, twenty layers: 793, 955).
     auto cost_of = [&](const HostUnit& h) -> uint64_t {
-      const uint64_t recs = (h.u.bytes0 + h.u.bytes1) / h.u.rec_bytes;
       // in twentieths of an SQ record, from stacks of one format and one stage (52 MB a layer, four layers, us: SQ / 64 / 256 entries at batch 1
       // 88, 121, 128; 8: 99, 135, 143; 16: 146, 177, 189), and the best of 24 to 34 for whole steps (14B-class, batch 16: 24 3416 us, 26 3420, 30 3427,
       // 34 3475; 7B-class, batch 1: 24 to 28 1153, 30 1162, 33 1185; batch 8: 24 1367, 27 1358, 33 1367)
       const uint64_t vq6 = B > 8 ? 26u : 27u, vq8 = B > 8 ? 26u : 28u;
       const uint64_t wgt = !(h.u.flags & UF_VQ) ? 20u : (h.u.flags & UF_BITS8) ? vq8 : vq6;
-      return recs * wgt * 64u;
+      return 16u * wgt * 64u;
     };
     // Units are dealt WHOLE (a consumer group spends about the same time on a piece of a unit as on a whole one, the warps
     // without a record idle), in runs of neighbouring units, by the smallest estimated time of the slowest CTA.  The estimate
