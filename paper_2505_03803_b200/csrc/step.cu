@@ -1538,7 +1538,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   const bool mix = any_xform || (n_ops <= 65535 && share > stages * (B > 8 ? 5600u : 3000u));
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
-  const uint64_t kRunCost = mix ? 32u : 64u, kOddCost = 32u;
+  const uint64_t kRunCost = mix ? 16u : 64u, kOddCost = 32u;
   info->mix = any_xform ? 2 : mix ? 1 : 0;      // the kernel's MIX
   const uint32_t nbp = (uint32_t)((B + 1) & ~1);
 
