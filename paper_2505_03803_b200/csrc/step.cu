@@ -153,9 +153,10 @@ constexpr int kMaxSlots = 3;
 constexpr uint32_t kCtrlBytes = 1024, kMuScratch = 1024;
 // Input-segment buffers, one in use and one being filled, as large as the ring leaves: every hand-over of a segment costs all roles a pass through the
 // barriers.  Above eight rows 62 KB hold the 1792 columns of sixteen rows that a CTA's seven units of a 4096-column product read (14B-class stack,
-// batch 16: 32 KB 3420 us, 48 KB 3348, 62 KB 3327); up to eight rows 40 KB hold the 2048 columns of eight (7B-class stack with 256 entries, batch 8:
-// 32 KB 1514 us, 40 KB 1488).
-constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 63488u : 40960u; }
+// batch 16: 32 KB 3420 us, 48 KB 3348, 62 KB 3327).  Up to eight rows 31 KB hold the 1792 columns of eight and leave the ring three slots beside the
+// copies of two codebooks of 256 entries (7B-class stack with them: batch 1 1276 -> 1154 us, batch 8 1471 -> 1362; without them, batch 8: 40 KB 1345,
+// 30 KB 1350; a size that the plan chooses costs more, 1.6B-class batch 1 414.7 -> 417.3, 14B-class batch 16 3332 -> 3352).
+constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 63488u : 31488u; }
 template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = xbuf_bytes_of(NB); };
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
 constexpr uint32_t kDefaultPollLimit = 1u << 22;
