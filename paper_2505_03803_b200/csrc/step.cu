@@ -97,7 +97,7 @@ struct StepEvent {           // 64 bytes
   uint32_t barrier;          // segment: index + 1 of the stage barrier to pass first; arrival: index of the barrier
   uint32_t xstride_sums;     // segment: xstride | sums << 31
   uint16_t mu_off16;         // segment: offset / 16 of the decoded mu row inside the buffer
-  uint16_t reserved;
+  uint16_t squares;          // 1: of a stage whose inputs every CTA squares for itself (see kSquaresShare); arrival: the stage that begins
 };
 static_assert(sizeof(StepEvent) == 64, "event descriptor size");
 
@@ -893,6 +893,59 @@ __device__ void mix_slice(const StepArgs& a, const StepEvent& ev, int stid, cons
   }
 }
 
+// The sums of a half-warp's 128-column group of row b, from the eight columns a lane has just staged (vector c8 of the row).
+__device__ __forceinline__ void segment_sums(float* gs, const uint4 r, int c8, int b, int nbp, int lane) {
+  const int o = (8 * c8) & 63;
+  const float pa = pair_sum(r.x) + pair_sum(r.z), pb = pair_sum(r.y) + pair_sum(r.w);
+  float sx = pa + pb;
+  float t0 = fmaf((float)rwkvq_sq_bias(o, 0), pa, (float)rwkvq_sq_bias(o + 2, 0) * pb);
+  float t1 = fmaf((float)rwkvq_sq_bias(o, 1), pa, (float)rwkvq_sq_bias(o + 2, 1) * pb);
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) {
+    sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
+    t0 += __shfl_xor_sync(0xFFFFFFFFu, t0, d);
+    t1 += __shfl_xor_sync(0xFFFFFFFFu, t1, d);
+  }
+  if ((lane & 15) == 0) {
+    const int grp = c8 >> 4;
+    gs[(grp * 3 + 0) * nbp + b] = sx;
+    gs[(grp * 3 + 1) * nbp + b] = t0;
+    gs[(grp * 3 + 2) * nbp + b] = t1;
+  }
+}
+
+// A segment of max(src, 0)^2, rounded to fp16, and its sums, by the CTA that reads it.
+template <int NB>
+__device__ __forceinline__ void stage_squares(const StepArgs& a, const StepEvent& ev, uint8_t* xb, int stid) {
+  constexpr int kThreads = Shape<NB>::kStagerThreads, kAhead = 2;
+  const float* src = reinterpret_cast<const float*>(ev.seg.x);
+  const int ic = (int)ev.segd.ic, col0 = (int)ev.segd.col0, nvr = (int)ev.segd.ncols >> 3, total = a.B * nvr, nbp = (a.B + 1) & ~1;
+  const uint32_t xstride = ev.xstride_sums & 0x7FFFFFFFu;
+  const bool sums = (ev.xstride_sums >> 31) != 0;
+  float* gs = reinterpret_cast<float*>(xb + (size_t)a.B * xstride);
+  for (int v0 = stid; v0 < total; v0 += kThreads * kAhead) {
+    float4 lo[kAhead], hi[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int v = v0 + u * kThreads, b = v / nvr, col = col0 + 8 * (v - b * nvr);
+      lo[u] = hi[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (v < total && col < ic) {
+        const float4* at = reinterpret_cast<const float4*>(src + (size_t)b * ic + col);
+        lo[u] = __ldcg(at); hi[u] = __ldcg(at + 1);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int v = v0 + u * kThreads, b = v / nvr, c8 = v - b * nvr;
+      if (v >= total) break;                      // warp-uniform: total is a multiple of 32
+      auto two = [](float x, float y) { x = fmaxf(x, 0.f); y = fmaxf(y, 0.f); return pack_half2(x * x, y * y); };
+      const uint4 r = make_uint4(two(lo[u].x, lo[u].y), two(lo[u].z, lo[u].w), two(hi[u].x, hi[u].y), two(hi[u].z, hi[u].w));
+      *reinterpret_cast<uint4*>(xb + (size_t)b * xstride + (size_t)c8 * 16) = r;
+      if (sums) segment_sums(gs, r, c8, b, nbp, threadIdx.x & 31);
+    }
+  }
+}
+
 // Stagers walk the CTA's event list.
 //  EV_ARRIVE: clear this CTA's slice of the next stage's outputs, then report the stage as done on
 //    the stagers' side (stage_report: the last of the consumer warps and the stagers to report
@@ -912,6 +965,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
   // The grid barriers are polled by the whole first warp (one request per poll, no divergence to leave): c2 B = 1 453 -> 447 us, c3
   // B = 8 1589 -> 1577; by one lane with two batch blocks, where it costs a little (c4 B = 16 4212 -> 4242 us).
   constexpr int kPollLanes = NB == 1 ? 32 : 1;
+  constexpr bool kSquares = MIX == 2 && NB == 1;      // plans with stages whose inputs every CTA squares for itself
   volatile int* abortp = &ctrl->abort_flag;
   uint32_t nseg = 0;          // segments staged so far
   uint32_t passed2 = 0xFFFFFFFFu;   // second-stage barrier this CTA has already passed
@@ -920,7 +974,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
     const StepEvent ev = *reinterpret_cast<const StepEvent*>(reinterpret_cast<const uint8_t*>(a.events) + (size_t)ei * 64);
     if (ev.kind == EV_ARRIVE) {
       if constexpr (MIX) {
-        if (ev.barrier < (uint32_t)a.n_stages) mix_warm<NB>(a, ev, stid);
+        if (ev.barrier < (uint32_t)a.n_stages && !(kSquares && ev.squares)) mix_warm<NB>(a, ev, stid);
       }
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
@@ -943,7 +997,8 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         if (ev.barrier < (uint32_t)a.n_stages) {
           MixSlot* const slots = reinterpret_cast<MixSlot*>(mucb);      // the codebook copy of stagers that mix themselves
           static_assert(sizeof(MixSlot) * Shape<NB>::kStagerWarps <= kMuScratch, "pre-pass slots");
-          const MixPrep prep = mix_prepare<NB, MIX == 2>(a, ev, stid, slots, ctrl->mix_at);
+          MixPrep prep;
+          if (!(kSquares && ev.squares)) prep = mix_prepare<NB, MIX == 2>(a, ev, stid, slots, ctrl->mix_at);
           if (ok && stid < kPollLanes) {
             uint32_t it = 0;
             while ((int)(ld_acquire_gpu(a.counter + ev.barrier) - (a.target + a.wait_skew)) < 0) {
@@ -964,6 +1019,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           }
           ok = named_bar_and(6, kStagerThreads, ok);   // thread 0's acquire precedes every thread's loads of x
           if (!ok) break;
+          if (kSquares && ev.squares) continue;
           mix_slice<NB, MIX == 2>(a, ev, stid, prep, slots, ctrl->mix_at);
           named_bar_sync(4, kStagerThreads);           // every thread's pre-pass stores precede thread 0's release
           if (stid == 0) red_release_gpu(a.counter + (uint32_t)a.n_stages + 1u + ev.barrier, 1u);
@@ -975,6 +1031,16 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
     // uniform verdict over all stager threads: the named barriers below must be reached by all or none
     ok = named_bar_and(7, kStagerThreads, mbar_wait_warp(&ctrl->xempty[buf], ((nseg / XBufs<MIX, NB>::kCount) & 1u) ^ 1u, abortp, a.status) && ok);
     uint8_t* xb = xbufs + (size_t)buf * XBufs<MIX, NB>::kBytes;
+    if constexpr (kSquares) {
+      if (ev.squares) {                    // the stage's barrier has been passed with its arrival event
+        if (ok) stage_squares<NB>(a, ev, xb, stid);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctrl->xfull[buf]);
+        ++nseg;
+        if (!ok) break;
+        continue;
+      }
+    }
     if constexpr (MIX) {
       // The segment is a rectangle of the stage's pre-pass output: pass the stage's second barrier
       // (once per stage), then fetch B rows and the block of sums with bulk copies.
@@ -1093,25 +1159,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
             r.z = mix2(r.z, pr.z, mr.z); r.w = mix2(r.w, pr.w, mr.w);
           }
           *reinterpret_cast<uint4*>(dst) = r;
-          if (sums) {
-            const int o = (8 * c8) & 63;
-            const float pa = pair_sum(r.x) + pair_sum(r.z), pb = pair_sum(r.y) + pair_sum(r.w);
-            float sx = pa + pb;
-            float t0 = fmaf((float)rwkvq_sq_bias(o, 0), pa, (float)rwkvq_sq_bias(o + 2, 0) * pb);
-            float t1 = fmaf((float)rwkvq_sq_bias(o, 1), pa, (float)rwkvq_sq_bias(o + 2, 1) * pb);
-#pragma unroll
-            for (int d = 8; d > 0; d >>= 1) {
-              sx += __shfl_xor_sync(0xFFFFFFFFu, sx, d);
-              t0 += __shfl_xor_sync(0xFFFFFFFFu, t0, d);
-              t1 += __shfl_xor_sync(0xFFFFFFFFu, t1, d);
-            }
-            if ((lane & 15) == 0) {
-              const int grp = c8 >> 4;
-              gs[(grp * 3 + 0) * nbp + b] = sx;
-              gs[(grp * 3 + 1) * nbp + b] = t0;
-              gs[(grp * 3 + 2) * nbp + b] = t1;
-            }
-          }
+          if (sums) segment_sums(gs, r, c8, b, nbp, lane);
         }
       }
     }
@@ -1555,6 +1603,31 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   info->n_stages = n_stages;
   info->n_barriers = ((uint32_t)n_stages + 1) * (mix ? 2u : 1u);   // the pre-pass has a barrier of its own per stage
 
+  // Stages of squared inputs alone (no token shift, no gain): up to kSquaresShare inputs a CTA it squares what it reads itself, behind the stage's
+  // barrier, and the stage needs neither the pre-pass nor its barrier.  Blocks, pre-pass / so, us, at `inputs a CTA`: d 512, batch 1, 256, 101.4 / 94.7;
+  // d 2048, batch 2, 1024, 128.2 / 123.5; batch 4, 2048, 129.4 / 125.7; d 3072, batch 3, 3072, 125.7 / 123.4; d 4096, batch 2, 3584, 194.2 / 194.8;
+  // d 2048, batch 8, 4096, 152.7 / 148.3; d 4096, batch 4, 7168, 213.8 / 215.2.
+  constexpr uint64_t kSquaresShare = 4200u;
+  std::vector<char> squares(n_stages, 0);
+  for (int s = 0; s < n_stages && any_xform && B <= 8; ++s) {
+    uint64_t n = 0;
+    bool all = true;
+    for (int o = stage_ranges[s].first; o < stage_ranges[s].second; ++o) {
+      const rwkvq_gemv_op& op = ops[o];
+      n += (uint64_t)((op.W_desc.oc_pad + 255) / 256) * (uint64_t)(op.W_desc.ic_pad / 256);
+      all = all && op.in.kind == RWKVQ_IN_RELU2 && !op.mu_image_dev && !op.in.xprev_out_fp16 && !op.in.scale_f32;
+    }
+    squares[s] = all && (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B <= kSquaresShare;
+    // a CTA that has staged its inputs clears the next stage's outputs: they must not be what others still read
+    if (squares[s] && s + 1 < n_stages)
+      for (int o = stage_ranges[s].first; o < stage_ranges[s].second; ++o)
+        for (int q = stage_ranges[s + 1].first; q < stage_ranges[s + 1].second; ++q) {
+          const uint64_t src = (uint64_t)(uintptr_t)ops[o].in.src_f32, src_end = src + (uint64_t)B * (uint64_t)ops[o].W_desc.ic * 4u;
+          const uint64_t y = (uint64_t)(uintptr_t)ops[q].y_dev, y_end = y + (uint64_t)B * (uint64_t)ops[q].W_desc.oc * 4u;
+          if (src < y_end && y < src_end) squares[s] = 0;
+        }
+  }
+
   std::vector<std::vector<HostUnit>> cta_units(P);
   std::vector<std::vector<StepEvent>> cta_arrivals(P);      // arrival events, one per barrier
   bool too_many_ranges = false;
@@ -1581,7 +1654,9 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
         base += n;
       }
     }
-    if (mix && barrier < n_stages) {
+    if (mix && barrier < n_stages && squares[barrier]) {
+      ev.squares = 1;
+    } else if (mix && barrier < n_stages) {
       // this CTA's share of the pre-pass of stage `barrier`
       uint64_t G = 0;
       for (int o = stage_ranges[barrier].first; o < stage_ranges[barrier].second; ++o) G += (uint64_t)B * (ops[o].W_desc.ic_pad / 128);
@@ -1817,7 +1892,10 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
         ev.xstride_sums = xstride | (sums ? 0x80000000u : 0u);
         ev.mu_off16 = (uint16_t)(xseg_mu_off(B, ncols, sums) / 16u);
         ev.barrier = (uint32_t)s + 1u;   // stage s reads its inputs after barrier s
-        if (mix) {
+        if (squares[s]) {
+          ev.squares = 1;
+          ev.seg.x = (uint64_t)(uintptr_t)o.in.src_f32;
+        } else if (mix) {
           ev.seg.x = mix_x_off[op] + (uint64_t)kmin * 512u;
           ev.seg.xprev = mix_sums_off[op] + (uint64_t)(kmin * 2) * 3u * nbp * 4u;
           ev.segd.ic = (uint32_t)o.W_desc.ic_pad * 2u;

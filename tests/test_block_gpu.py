@@ -217,3 +217,35 @@ def test_reciprocal_of_the_sigmoids_is_the_rounded_division(exponents):
     B.rwkvq_step_reciprocal(ends, out)
     got = out.cpu().numpy()
     assert got[1] == 0.0 and np.isnan(got[2]) and np.array_equal(got[[0, 3, 4, 5]], np.float32(1.0) / ends.cpu().numpy()[[0, 3, 4, 5]])
+
+
+@pytest.mark.parametrize("Bn,oc,bits", [(1, 256, 3), (3, 512, 6), (8, 384, 3), (8, 1024, 8), (9, 512, 6)])
+def test_squared_inputs_of_one_stage(Bn, oc, bits):
+    """y1 = W1 relu(y0)^2 of y0 = W0 x: squared by every CTA for itself up to eight rows, in the pre-pass above."""
+    ic, g = 1024, torch.Generator(device="cuda").manual_seed(Bn + oc)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+
+    def matrix(rows, cols, b):
+        desc = B.rwkvq_desc_for(rows, cols, B.RWKVQ_SQ if b == 3 else B.RWKVQ_VQ, b)
+        image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+        B.rwkvq_quantize_dev_async((torch.randn((rows, cols), generator=g, device="cuda") * 0.02).half(), rows, cols, desc.method, b, image, ws, kmeans_iters=1, seed=1)
+        decoded = torch.empty((rows, cols), device="cuda")
+        B.rwkvq_dequant(desc, image, decoded)
+        return desc, image, decoded.double()
+
+    (d0, w0, m0), (d1, w1, m1) = matrix(1280, ic, 3), matrix(oc, 1280, bits)
+    x = torch.randn((Bn, ic), generator=g, device="cuda").half()
+    y0, y1 = torch.zeros((Bn, 1280), device="cuda"), torch.zeros((Bn, oc), device="cuda")
+    ops = B.make_ops([dict(desc=d0, W=w0, mu_desc=None, mu=None, x=x, xprev=None, y=y0, stage=0),
+                      dict(desc=d1, W=w1, mu_desc=None, mu=None, x=None, xprev=None, y=y1, stage=1, **{"in": dict(kind=B.RWKVQ_IN_RELU2, src=y0)})])
+    plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
+    B.rwkvq_step_plan(ops, Bn, plan)
+    for _ in range(20):
+        B.rwkvq_step_run(plan)
+    torch.cuda.synchronize()
+    assert B.rwkvq_device_status() == 0
+    k = y0.double()
+    assert bool(((k - x.double() @ m0.T).abs() <= 2e-3 * x.double().norm(dim=1)[:, None] * m0.norm(dim=1)[None]).all())
+    squares = k.clamp_min(0.0) ** 2
+    assert bool(((y1.double() - squares @ m1.T).abs() <= 2e-3 * squares.norm(dim=1)[:, None] * m1.norm(dim=1)[None]).all())
+    B.rwkvq_step_plan_release(plan)
