@@ -1386,7 +1386,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   auto summands = [&](int i, int dim) -> Sums {
     const uint32_t v = __ldg(a.w + 2 * i + dim);
     if constexpr (kWeighted) {
-      const double w = (double)__ldg(a.elem_w + 2 * i + dim);
+      const double w = (double)__ldcg(a.elem_w + 2 * i + dim);        // written by the kernel before, which this one need not have started behind
       return Sums{w * (double)h2f_bits(v), w};                     // the product of 24 and 11 bits is exact
     } else {
       return Sums{half_fixed(v), 1};
@@ -1402,7 +1402,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   auto fetch = [&](int i0) {
     const int i = min(i0 + in_round, n - 1);
     f = vec_of(__ldg(vec + i));
-    if (kWeighted) w = __ldg(wgt + i);
+    if (kWeighted) w = __ldcg(wgt + i);
   };
   fetch(begin);
   if (tid == 0)

@@ -25,7 +25,8 @@
 // the squared ReLU and output gate of Eq. 27, optionally a root-mean-square normalisation), the
 // inputs of a stage are not built per CTA: after the stage barrier all CTAs together compute the
 // stage's x_mix once (mix_slice: a quarter-warp per 128-column group of a plain input, a warp where an operator is in front)
-// into a scratch region of the plan, publish it through a second barrier, and every CTA fetches its segments with bulk copies.
+// into a scratch region of the plan, publish it through a second barrier, and every CTA fetches its segments with bulk copies.  (Squared inputs
+// alone, few to a CTA, are staged by the CTAs that read them: stage_squares.)
 //
 // The host plans the step once: every stage's units are dealt WHOLE to the CTAs, in runs of neighbouring units by the
 // smallest estimated time of the slowest CTA, along rows of tiles where that is no worse; the plan is a per-CTA
