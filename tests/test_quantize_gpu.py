@@ -495,3 +495,37 @@ def test_quantizers_start_behind_what_writes_their_inputs(oc, ic, bits):
     assert B.rwkvq_quantize_check(ws) == 0
     for i, y in enumerate(got):
         assert torch.equal(y, want[i % 4])
+
+
+@pytest.mark.parametrize("oc,ic,bits", [(256, 512, 3), (512, 512, 6), (2816, 2816, 8), (1, 1024, 6), (1, 10240, 6)])
+def test_captured_quantizers(oc, ic, bits):
+    """A graph of the weights' copy, the representative and the quantizer gives the images of the calls made one by one."""
+    method = B.RWKVQ_SQ if bits == 3 else B.RWKVQ_VQ
+    desc = B.rwkvq_desc_for(oc, ic, method, bits)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(oc * 7 + ic)
+    src = [(torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half() for _ in range(3)]
+    samples = torch.randn((33, ic), generator=g, device="cuda")
+    fresh, w, rep = torch.zeros_like(src[0]), torch.zeros_like(src[0]), torch.zeros(ic, device="cuda")
+    image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+
+    def calls():
+        w.copy_(fresh)
+        B.rwkvq_calib_representative(samples, 1.0, rep_sq=rep)
+        B.rwkvq_quantize_dev_async(w, oc, ic, method, bits, image, ws, elem_weight=rep if oc == 1 else None, kmeans_iters=2, seed=5)
+
+    want = []
+    for s in src:
+        fresh.copy_(s)
+        calls()
+        want.append(image.clone())
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for s, ref in list(zip(src, want)) * 2:
+        fresh.copy_(s)
+        image.zero_()
+        graph.replay()
+        assert torch.equal(image, ref)
+    assert B.rwkvq_quantize_check(ws) == 0
