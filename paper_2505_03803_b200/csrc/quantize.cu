@@ -1272,6 +1272,10 @@ __device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n,
       if (lane >= off) incl += v;
     }
     if (lane == 31) sh.tot[warp] = incl;
+    // the sums in front of this thread: added up, not the difference of `incl` and its own sum, which is off by roundings of that sum, and it may be far
+    // larger than the target
+    float front = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+    if (lane == 0) front = 0.f;
     sync();
     float t[kSeedWarps];                           // zeros behind the last warp
 #pragma unroll
@@ -1287,7 +1291,7 @@ __device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n,
 #pragma unroll
       for (int w = 0; w < h; ++w) { t[w] += t[w + h]; before[w] += before[w + h]; }
     const float target = u01 * t[0], margin = target * (320.f / 16777216.f);
-    const float rest = target - (before[0] + (incl - sum[kSeedPer]));
+    const float rest = target - (before[0] + front);
     const float under = rest - margin, over = rest + margin;
     if (sum[0] <= under && sum[kSeedPer] > over) {
       // the last that begins at or below, by halves

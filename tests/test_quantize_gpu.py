@@ -327,6 +327,19 @@ def test_mu_seeds_are_the_draws_of_the_definition(ic, bits, kind):
     assert np.array_equal(got, _drawn_seeds(mu16.reshape(-1, 2), 1 << bits, 7).view(np.uint16))
 
 
+@pytest.mark.parametrize("seed", [661793, 867062, 1253589])
+def test_mu_seeds_where_one_vector_is_far_from_all_others(seed):
+    """A thread's own sum of distances is thousands of times the target of the draw, which falls next to the boundary between two vectors."""
+    i = np.arange(2048)
+    v = np.stack([0.25 + (37 * i % 32) / 4096, 0.25 + (53 * i % 29) / 4096], axis=1)
+    v[31] = 1.0
+    v16 = v.astype(np.float16)
+    _, img = quantize_dev(v16.reshape(-1), B.RWKVQ_VQ, 6, seed=seed, iters=0)
+    _, codes = B.rwkvq_image_unpack(img.cpu().numpy())
+    got = np.asarray(codes["codebook"]).reshape(64, 2).view(np.uint16)
+    assert np.array_equal(got, _drawn_seeds(v16, 64, seed).view(np.uint16))
+
+
 def test_quantize_dev_error_paths():
     w = torch.zeros((256, 256), dtype=torch.float16, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
