@@ -21,6 +21,8 @@ constexpr int kFlagNonFinite = 1, kFlagTimeout = 2;
 
 // Every kernel here is launched while the one before it still runs, lets the next one be, and touches memory behind this: a call of short kernels
 // otherwise waits 2 us for each to start (five vectors of 4096 with 128 samples, ten kernels: 303 -> 288 us; a layer of 512 columns 284 -> 270).
+// What the kernel before may still write while this one is resident is not read through the read-only path, whose data has to stay as it is for the
+// whole life of the reading kernel: __ldcg, or an ordinary load where it is read again.
 __device__ __forceinline__ void after_the_kernel_before() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
@@ -77,7 +79,7 @@ __device__ __forceinline__ float h2f_bits(uint32_t h) { return __half2float(__us
 __device__ __forceinline__ __half2 as_h2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
 __device__ __forceinline__ uint32_t as_u32(__half2 v) { return *reinterpret_cast<uint32_t*>(&v); }
 
-__global__ void __launch_bounds__(32 * kSqWarps, 20 / kSqWarps) sq_quantize_kernel(const uint16_t* __restrict__ w, int oc, int ic, int KT,
+__global__ void __launch_bounds__(32 * kSqWarps, 20 / kSqWarps) sq_quantize_kernel(const uint16_t* w, int oc, int ic, int KT,
                                                              uint8_t* __restrict__ payload, int* __restrict__ flags,
                                                              const __grid_constant__ rwkvq_image_header head, uint8_t* image) {
   __shared__ __align__(16) uint8_t codes_all[kSqWarps][16 * kSqRowStride];
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(32 * kSqWarps, 20 / kSqWarps) sq_quantize_kern
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
     v[r] = make_uint4(0, 0, 0, 0);
-    if (col_in && r0 + r < oc) v[r] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)r * ic));
+    if (col_in && r0 + r < oc) v[r] = __ldcg(reinterpret_cast<const uint4*>(src + (size_t)r * ic));
   }
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
@@ -427,7 +429,7 @@ __device__ __forceinline__ void load_rows(uint32_t* vec, const uint16_t* src, in
   bool bad = false;
 #pragma unroll 4
   for (int r = threadIdx.x >> 5; r < rows; r += warps) {
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(src + (size_t)r * ic) + lane);
+    const uint4 q = __ldcg(reinterpret_cast<const uint4*>(src + (size_t)r * ic) + lane);
     const uint32_t v[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) bad |= ((v[k] & 0x7C00u) == 0x7C00u) | ((v[k] & 0x7C000000u) == 0x7C000000u);
@@ -540,7 +542,7 @@ __global__ void __launch_bounds__(kVqThreads, 1) vq_seed_kernel(const VqArgs a) 
     const uint32_t* src = reinterpret_cast<const uint32_t*>(a.w);
     bool bad = false;
     for (int i = tid; i < threads * kVqPerThread; i += threads) {
-      const uint32_t v = i < n ? __ldg(src + i) : 0u;
+      const uint32_t v = i < n ? __ldcg(src + i) : 0u;
       bad |= ((v & 0x7C00u) == 0x7C00u) | ((v & 0x7C000000u) == 0x7C000000u);
       vec[vq_slot(i)] = v;
     }
@@ -1388,7 +1390,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   const uint32_t sums_here = shared_address(&sh.sums_here), centres_here = shared_address(&sh.centres_here);
   // summands of vector i in one dimension
   auto summands = [&](int i, int dim) -> Sums {
-    const uint32_t v = __ldg(a.w + 2 * i + dim);
+    const uint32_t v = a.w[2 * i + dim];
     if constexpr (kWeighted) {
       const double w = (double)__ldcg(a.elem_w + 2 * i + dim);        // written by the kernel before, which this one need not have started behind
       return Sums{w * (double)h2f_bits(v), w};                     // the product of 24 and 11 bits is exact
@@ -1405,7 +1407,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   float2 f, w = make_float2(1.f, 1.f);
   auto fetch = [&](int i0) {
     const int i = min(i0 + in_round, n - 1);
-    f = vec_of(__ldg(vec + i));
+    f = vec_of(vec[i]);
     if (kWeighted) w = __ldcg(wgt + i);
   };
   fetch(begin);
@@ -1415,7 +1417,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     const int warps = (n + 32 * kSeedPer - 1) / (32 * kSeedPer);
     bool bad = false;
     for (int i = tid; i < warps * 32 * kSeedPer; i += kVecThreads) {
-      const uint32_t v = i < n ? __ldg(vec + i) : 0u;
+      const uint32_t v = i < n ? __ldcg(vec + i) : 0u;
       bad |= ((v & 0x7C00u) == 0x7C00u) | ((v & 0x7C000000u) == 0x7C000000u);
       sh.s.vec[i] = v;
     }
@@ -1640,7 +1642,7 @@ __global__ void __launch_bounds__(256) representative_kernel(const RepArgs a) {
   after_the_kernel_before();
   for (int i = threadIdx.x; i < S * 8; i += 256) {
     const int s = i >> 3, c = i & 7;
-    tile[s * 9 + c] = (j0 + c < a.n) ? __ldg(a.samples + (size_t)s * a.n + j0 + c) : 0.f;
+    tile[s * 9 + c] = (j0 + c < a.n) ? __ldcg(a.samples + (size_t)s * a.n + j0 + c) : 0.f;
   }
   __syncthreads();
   if (j0 + warp >= a.n) return;

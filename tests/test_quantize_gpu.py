@@ -510,6 +510,44 @@ def test_quantizers_start_behind_what_writes_their_inputs(oc, ic, bits):
         assert torch.equal(y, want[i % 4])
 
 
+@pytest.mark.parametrize("reader,oc", [("samples", 2048), ("scalar", 1024), ("tile", 512), ("tile", 26112), ("vector", 1024), ("vector", 10240)])
+def test_quantizers_behind_products_that_end_late(reader, oc):
+    """What a product writes is quantized at once.  The products' kernels let the next one start when they do, so the quantizer is resident while they
+    write; every call changes all of the buffer."""
+    ic, rows = 512, 1 if reader == "vector" else 256
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(oc)
+    desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ, 3)
+    W = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+    B.rwkvq_quantize_dev_async((torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half(), oc, ic, B.RWKVQ_SQ, 3, W, ws)
+    x = [torch.randn((rows, ic), generator=g, device="cuda").to(torch.float16 if rows == 1 else torch.bfloat16) for _ in range(4)]
+    y = torch.zeros((rows, oc), device="cuda", dtype=torch.float16 if rows == 1 else torch.float32 if reader == "samples" else torch.bfloat16)
+    pws = torch.zeros(max(256, B.rwkvq_gemv_workspace_bytes(desc, 1), B.rwkvq_prefill_workspace_bytes(desc, rows, False)), dtype=torch.uint8, device="cuda")
+    method, bits = (B.RWKVQ_SQ, 3) if reader == "scalar" else (B.RWKVQ_VQ, 6)
+    image_desc = None if reader == "samples" else B.rwkvq_desc_for(rows, oc, method, bits)
+    image = torch.zeros(oc * 4 if image_desc is None else int(image_desc.image_bytes), dtype=torch.uint8, device="cuda")
+
+    def one(i, wait):
+        if rows == 1:
+            B.rwkvq_gemv(desc, W, None, None, x[i], None, 1, y, pws)
+        else:
+            B.rwkvq_gemm_prefill(desc, W, None, None, x[i], None, rows, y, pws)
+        if wait:
+            torch.cuda.synchronize()
+        if reader == "samples":
+            B.rwkvq_calib_representative(y, 1.0, rep=image.view(torch.float32))
+        else:       # the bit patterns of bf16 results of this size are finite fp16 numbers
+            B.rwkvq_quantize_dev_async(y.view(torch.float16), rows, oc, method, bits, image, ws, kmeans_iters=1, seed=i)
+        return image.clone()
+
+    want = [one(i, True) for i in range(4)]
+    got = [one(i % 4, False) for i in range(24)]
+    assert B.rwkvq_quantize_check(ws) == 0
+    assert not torch.equal(want[0], want[1])
+    for i, z in enumerate(got):
+        assert torch.equal(z, want[i % 4])
+
+
 @pytest.mark.parametrize("oc,ic,bits", [(256, 512, 3), (512, 512, 6), (2816, 2816, 8), (1, 1024, 6), (1, 10240, 6)])
 def test_captured_quantizers(oc, ic, bits):
     """A graph of the weights' copy, the representative and the quantizer gives the images of the calls made one by one."""
