@@ -1221,8 +1221,10 @@ static_assert(sizeof(VecShared<256>) <= 232448, "shared memory of a block");
 // Draws E seeds; a draw is defined as in vq_seed_kernel: distances summed in fp32 over runs of 64 vectors in order, run sums by a scan over the lanes
 // of a warp, and the last vector whose running sum begins at or below the target.  Those chains are 64 additions long, twice a draw.  So the
 // sums are taken in a tree first: with u = 2^-24, the chains' running sums are off by at most 148 u of themselves and their target by 84 u, the
-// tree's by 23 u and 20 u (its differences from the target by three more), so a vector whose running sums begin and end at least 320 u of the target away from it (and on either side)
-// is the one that the chains give.  Otherwise (one draw in 25 for 2048 vectors) the chains are walked.
+// tree's by 23 u and 20 u (its differences from the target by three more), and the sum in front of a thread, the scan less the thread's own sum, by five u of
+// the scan besides, which may be thousands of times the target.  So a vector whose running sums begin and end at least 320 u of the target and 8 u of the
+// scan away from the target (and on either side) is the one that the chains give.  Otherwise (one draw in 25 for 2048 vectors) the chains are
+// walked.  (The sum in front by a shuffle from the neighbour needs no second term, and took 2 us longer for a vector of 4096.)
 // Called by the first `threads` threads, which hold sixteen vectors each.
 __device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n, int E, uint64_t seed, int threads) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, base = kSeedPer * tid;
@@ -1274,10 +1276,6 @@ __device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n,
       if (lane >= off) incl += v;
     }
     if (lane == 31) sh.tot[warp] = incl;
-    // the sums in front of this thread: added up, not the difference of `incl` and its own sum, which is off by roundings of that sum, and it may be far
-    // larger than the target
-    float front = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-    if (lane == 0) front = 0.f;
     sync();
     float t[kSeedWarps];                           // zeros behind the last warp
 #pragma unroll
@@ -1292,8 +1290,8 @@ __device__ __forceinline__ void draw_seeds(VecSeeds& sh, uint32_t* seeds, int n,
     for (int h = kSeedWarps / 2; h > 0; h >>= 1)
 #pragma unroll
       for (int w = 0; w < h; ++w) { t[w] += t[w + h]; before[w] += before[w + h]; }
-    const float target = u01 * t[0], margin = target * (320.f / 16777216.f);
-    const float rest = target - (before[0] + front);
+    const float target = u01 * t[0], margin = fmaf(incl, 8.f / 16777216.f, target * (320.f / 16777216.f));
+    const float rest = target - (before[0] + (incl - sum[kSeedPer]));
     const float under = rest - margin, over = rest + margin;
     if (sum[0] <= under && sum[kSeedPer] > over) {
       // the last that begins at or below, by halves
