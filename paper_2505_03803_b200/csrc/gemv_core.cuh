@@ -190,10 +190,10 @@ struct SqRecord {
     sz = *reinterpret_cast<const uint4*>(rec + RWKVQ_SQ_CODE_BYTES + (lane >> 2) * 16);
   }
   __device__ __forceinline__ void load(const uint8_t* rec, int lane) {
-    p0 = ldg_stream(rec + lane * 16);
-    p1 = ldg_stream(rec + 512 + lane * 16);
-    p2 = ldg_stream(rec + 1024 + lane * 16);
-    sz = ldg_stream(rec + RWKVQ_SQ_CODE_BYTES + (lane >> 2) * 16);
+    p0 = ld_stream(rec + lane * 16);
+    p1 = ld_stream(rec + 512 + lane * 16);
+    p2 = ld_stream(rec + 1024 + lane * 16);
+    sz = ld_stream(rec + RWKVQ_SQ_CODE_BYTES + (lane >> 2) * 16);
   }
   __device__ __forceinline__ void words(uint32_t (&w)[12]) const {
     w[0] = p0.x; w[1] = p0.y; w[2] = p0.z; w[3] = p0.w;
@@ -338,7 +338,7 @@ struct VqRecord {
   __device__ __forceinline__ void load(const uint8_t* rec, int lane) {
 #pragma unroll
     for (int p = 0; p < NW / 4; ++p) {
-      const uint4 v = ldg_stream(rec + p * 512 + lane * 16);
+      const uint4 v = ld_stream(rec + p * 512 + lane * 16);
       w[4 * p] = v.x; w[4 * p + 1] = v.y; w[4 * p + 2] = v.z; w[4 * p + 3] = v.w;
     }
   }
@@ -350,7 +350,7 @@ __device__ __forceinline__ void stage_codebook(uint8_t* dst, const uint32_t* src
   uint4* d = reinterpret_cast<uint4*>(dst);
 #pragma unroll 4
   for (int idx = threadIdx.x; idx < E * 8; idx += blockDim.x) {
-    const uint32_t v = __ldg(src + (idx >> 3));
+    const uint32_t v = __ldcg(src + (idx >> 3));
     d[idx] = make_uint4(v, v, v, v);
   }
 }

@@ -548,6 +548,40 @@ def test_quantizers_behind_products_that_end_late(reader, oc):
         assert torch.equal(z, want[i % 4])
 
 
+@pytest.mark.parametrize("oc,ic,bits", [(512, 512, 3), (4096, 4096, 3), (512, 512, 6), (512, 512, 8), (2816, 2816, 6), (1, 512, 6), (1, 10240, 8)])
+def test_products_behind_quantizers(oc, ic, bits):
+    """A product reads the image that the quantizer in front of it is still writing when it starts: one image buffer, other weights every time."""
+    method = B.RWKVQ_SQ if bits == 3 else B.RWKVQ_VQ
+    desc = B.rwkvq_desc_for(oc, ic, method, bits)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(oc + 3 * ic)
+    src = [(torch.rand((oc, ic), generator=g, device="cuda") - 0.5).half() for _ in range(4)]
+    image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+    pdesc, pimage, rows = desc, image, oc
+    if oc == 1:      # a token-shift vector: the product's matrix stays as it is
+        rows = 512
+        pdesc = B.rwkvq_desc_for(rows, ic, B.RWKVQ_SQ, 3)
+        pimage = torch.zeros(int(pdesc.image_bytes), dtype=torch.uint8, device="cuda")
+        B.rwkvq_quantize_dev_async((torch.randn((rows, ic), generator=g, device="cuda") * 0.02).half(), rows, ic, B.RWKVQ_SQ, 3, pimage, ws)
+    x, xprev = torch.randn((3, ic), generator=g, device="cuda").half(), torch.randn((3, ic), generator=g, device="cuda").half()
+    y, pws = torch.zeros((3, rows), device="cuda"), torch.zeros(max(256, B.rwkvq_gemv_workspace_bytes(pdesc, 3)), dtype=torch.uint8, device="cuda")
+
+    def one(i, wait):
+        B.rwkvq_quantize_dev_async(src[i], oc, ic, method, bits, image, ws, kmeans_iters=1, seed=i)
+        if wait:
+            torch.cuda.synchronize()
+        mu = (desc, image, x, xprev) if oc == 1 else (None, None, x, None)
+        B.rwkvq_gemv(pdesc, pimage, *mu, 3, y, pws)
+        return y.clone()
+
+    want = [one(i, True) for i in range(4)]
+    got = [one(i % 4, False) for i in range(24)]
+    assert B.rwkvq_quantize_check(ws) == 0
+    assert not torch.equal(want[0], want[1])
+    for i, z in enumerate(got):
+        assert torch.equal(z, want[i % 4])
+
+
 @pytest.mark.parametrize("oc,ic,bits", [(256, 512, 3), (512, 512, 6), (2816, 2816, 8), (1, 1024, 6), (1, 10240, 6)])
 def test_captured_quantizers(oc, ic, bits):
     """A graph of the weights' copy, the representative and the quantizer gives the images of the calls made one by one."""
