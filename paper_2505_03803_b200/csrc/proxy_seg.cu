@@ -282,7 +282,11 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
   double acc[kMaxK];
 #pragma unroll
   for (int i = 0; i < kMaxK; ++i) acc[i] = 0.0;
-  for (int i = tid; i + 1 < count; i += T) gap_terms(logs, (value_of_key32(keys[i + 1]) - value_of_key32(keys[i])) * inv_R, n, K, acc);
+  for (int i = tid; i + 1 < count; i += T) {
+    // gap / R by its reciprocal with one correction: a tile of two weights has a gap of one, exactly, and proxies of zero
+    const double gap = value_of_key32(keys[i + 1]) - value_of_key32(keys[i]), q = gap * inv_R;
+    gap_terms(logs, fma(fma(-q, R, gap), inv_R, q), n, K, acc);
+  }
 #pragma unroll
   for (int i = 0; i < kMaxK; ++i) {
     if (i >= K) break;

@@ -113,6 +113,21 @@ def _close_arr(a, b, rel):
 
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
+def test_proxy_segments_of_two_weights_are_zero(dtype):
+    """One gap, R itself: g' = 1, P_c = P_f = 0 exactly, so that thresholds of zero choose VQ by the strict comparison.  (Gaps of 16-bit types are
+    multiplied by 1 / R: powers of two there.)"""
+    rng = np.random.default_rng(5)
+    w = rng.standard_normal((64, 256)).astype(np.float32)
+    if dtype != torch.float32:
+        w[:, 0::2] = 0.0
+        w[:, 1::2] = rng.choice([-1.0, 1.0], (64, 128)) * 2.0 ** rng.integers(-10, 10, (64, 128))
+    v64, dev = _typed(w, dtype)
+    for K in (2, 8):
+        pc, pf, phi = B.rwkvq_proxy_segments(dev, 1, 2, K, 0.0, math.inf)
+        assert (pc == 0.0).all() and (pf == 0.0).all() and (phi == B.RWKVQ_VQ).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("shape,seg", [((40, 300), (1, 300)), ((40, 300), (16, 128)), ((512, 512), (256, 256)),
                                        ((33, 70), (8, 64)), ((3, 5000), (1, 5000))])
 def test_proxy_segments_match_oracle_per_tile(dtype, shape, seg):
