@@ -121,14 +121,19 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_set_kernel(const uint16
 // fp32: one block of T threads, KPT keys each, per segment: tile (blockIdx.y, blockIdx.x) of seg_rows x seg_cols elements, ragged at the
 // right and bottom edges.  The keys are sorted in shared memory in one pass: counted in buckets by sign, exponent and the leading 23 - SHIFT
 // mantissa bits (sixteen octaves below the tile's largest magnitude, the rest in one bucket a sign), put into their buckets, and then every key
-// counts the smaller ones of its own bucket: in the densest octave of a Gaussian tile four.  A tile with more than 255 keys in one
-// (many equal weights, or all of them close together around a number other than zero) is sorted by a bitonic network instead, as every tile
-// was before.  Bound by instructions (about 300 a key and warp, 66 % of the issue slots).  4096^2 weights, tiles of 128 x 128: 852 -> 219 us,
-// of 128 x 256: 1000 -> 249, of 1 x 4096: 964 -> 217.
+// counts the smaller ones of its own bucket: in the densest octave of a Gaussian tile four.  A tile with more than 255 keys in one bucket, or
+// more comparisons a key than kMostCompared (many equal weights, or all of them close together around a number other than zero), is sorted by a
+// bitonic network instead, as every tile was before, unless it has one value only.  Bound by instructions (about 300 a key and warp, 66 % of the issue
+// slots).  Calls of 4096^2 weights, us, tiles of 128 x 256, 128 x 128 and 1 x 4096, by the network -> by this:
+// Gaussian 1054 -> 290, 907 -> 254, 1039 -> 260; of bf16 numbers 1073 -> 389, 931 -> 318, 1066 -> 263; half of them zero 1026 -> 947, 881 -> 809, 1028 -> 605;
+// around one 1071 -> 971, 918 -> 826, 1038 -> 624; one value 865 -> 156, 731 -> 155, 752 -> 155; 256 values alike often 1034 -> 805, 902 -> 491, 1058 -> 333.
 template <int T, int KPT, int SHIFT, int CTAS>
 struct TileSort {
   static constexpr int kSide = 16 << (23 - SHIFT);       // buckets of a sign
   static constexpr int kKeys = T * KPT;
+  // From there the network is faster: by ranks, 64 / 128 comparisons a key, tiles of 128 x 256 525 / 805 us and by the network 920; of 128 x 128 491 / 739
+  // and 790; of 1 x 4096, 32 / 43 / 64 comparisons, 393 / 463 / 546 and 593.
+  static constexpr uint32_t kMostCompared = T == 1024 ? 140 : 72;
   static constexpr size_t kSmem = (size_t)(kKeys + 4) * 4 + (size_t)kSide * 8;     // four keys of padding
 };
 template <int T, int KPT, int SHIFT, int CTAS>
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
   uint32_t* starts = keys + S::kKeys + 4;        // of the buckets; counts at first
   __shared__ LogTable logs;
   __shared__ double red[kWarps][kMaxK], total[kMaxK];
-  __shared__ uint32_t warp_sum[kWarps], s_max;
+  __shared__ uint32_t warp_sum[kWarps], s_max, s_compared;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r0 = blockIdx.y * seg_rows, c0 = blockIdx.x * seg_cols;
   const int nr = min(seg_rows, oc - r0), nc = min(seg_cols, ic - c0);
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
   SegResult* res = out + (size_t)blockIdx.y * gridDim.x + blockIdx.x;
   fill_log_table(logs);
   for (int i = tid; i < S::kSide / 2; i += T) reinterpret_cast<uint4*>(starts)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid == 0) s_max = 0u;
+  if (tid == 0) s_max = s_compared = 0u;
   __syncthreads();
   uint32_t b[KPT];
   uint32_t top = 0u;
@@ -194,13 +199,14 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
   __syncthreads();
   bool many = false;
   {
-    uint32_t sum = 0u;
+    uint32_t sum = 0u, compared = 0u;
     uint4* const mine = reinterpret_cast<uint4*>(starts + tid * kPer);
 #pragma unroll
     for (int i = 0; i < kPer / 4; ++i) {
       const uint4 v = mine[i];
       sum += v.x + v.y + v.z + v.w;
       many |= max(max(v.x, v.y), max(v.z, v.w)) > 255u;
+      compared += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;      // 2^30 at most
     }
     uint32_t incl = sum;
 #pragma unroll
@@ -209,7 +215,10 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
       if (lane >= d) incl += v;
     }
     if (lane == 31) warp_sum[warp] = incl;
+    compared = __reduce_add_sync(0xFFFFFFFFu, compared);
+    if (lane == 0) atomicAdd(&s_compared, compared);
     __syncthreads();
+    many |= s_compared > S::kMostCompared * (uint32_t)count;
     uint32_t at = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? warp_sum[lane] : 0u) + incl - sum;
 #pragma unroll
     for (int i = 0; i < kPer / 4; ++i) {
@@ -232,18 +241,12 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
       if (p >= count) continue;
       const uint32_t k = keys[p];
       const int bk = bucket(k), first = (int)starts[bk], stop = bk + 1 < 2 * S::kSide ? (int)starts[bk + 1] : count;
-      // the buckets behind hold larger keys, so steps of four may overshoot
-      uint32_t smaller = 0u, equal = 0u;
+      // the buckets behind hold larger keys, so steps of four may overshoot; equal ones keep the order of their places
+      uint32_t smaller = 0u;
       for (int q = first; q < stop; q += 4) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t o = keys[q + i];
-          smaller += o < k ? 1u : 0u;
-          equal += o == k ? 1u : 0u;
-        }
+        for (int i = 0; i < 4; ++i) smaller += keys[q + i] < k + (q + i < p ? 1u : 0u) ? 1u : 0u;
       }
-      if (equal > 1u)                              // equal ones keep the order of their places
-        for (int q = first; q < p; ++q) smaller += keys[q] == k ? 1u : 0u;
       b[j] = k;
       came[j / 4] |= smaller << (8 * (j % 4));
     }
@@ -253,6 +256,15 @@ __global__ void __launch_bounds__(T, CTAS) proxy_segment_f32_kernel(const uint32
       if (tid + j * T < count) keys[starts[bucket(b[j])] + ((came[j / 4] >> (8 * (j % 4))) & 0xFFu)] = b[j];
     __syncthreads();
   } else {
+    // all equal (every bit of a key the same, or zeros of either sign): nothing to sort
+    const float one = __uint_as_float(__ldg(src + (size_t)r0 * ic + c0));
+    bool same = true;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) same &= tid + j * T >= count || __uint_as_float(bits_of_key32(b[j])) == one;
+    if (__syncthreads_and(same)) {
+      if (tid == 0) { res->pc = INFINITY; res->pf = INFINITY; res->count = (unsigned)count; res->nonfinite = 0; }
+      return;
+    }
     // bitonic sorting network, ascending; the padding keys are the largest and end up behind the data
 #pragma unroll
     for (int j = 0; j < KPT; ++j)

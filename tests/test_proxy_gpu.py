@@ -257,3 +257,19 @@ def test_proxy_fp32_tiles_at_the_edges_of_the_sort(count, kind):
     assert np.all(np.abs(pf - rpf) <= 1e-8 * np.maximum(1.0, np.abs(rpf)))
     again = B.rwkvq_proxy_segments(dev, 1, count, 4, 3.0, 1e30)
     assert np.array_equal(pc, again[0]) and np.array_equal(pf, again[1])
+
+
+@pytest.mark.parametrize("count", [300, 4096, 16384, 32768])
+@pytest.mark.parametrize("levels", [1, 2, 100, 300])
+def test_proxy_fp32_tiles_of_many_equal_weights(count, levels):
+    """Few values, each many times: ranks among equal keys, the network behind crowded buckets, tiles of one value (zeros of either sign among them)."""
+    rng = np.random.default_rng(count + levels)
+    a = ((rng.integers(0, levels, (3, count)) - levels // 2) * 0.01).astype(np.float32)
+    if levels == 1:
+        a[1], a[2] = -1.5, np.where(rng.random(count) < 0.5, -0.0, 0.0)
+    vals, dev = _typed(a, torch.float32)
+    pc, pf, phi = B.rwkvq_proxy_segments(dev, 1, count, 4, 3.0, 1e30)
+    rpc, rpf = orc.proxy_segments(vals, 1, count, K=4)
+    _close_arr(pc, rpc, 1e-9)
+    _close_arr(pf, rpf, 1e-8)
+    assert levels > 1 or (phi == B.RWKVQ_VQ).all()
