@@ -97,7 +97,8 @@ struct SymbolAddress {
 // Page-locked host memory of the calling thread that a kernel writes a call's results to, for calls that wait for their stream before they return:
 // a copy of a few kilobytes to pageable memory behind the kernel took as long as a short kernel (256 x 256 tiles of 4096^2 bf16: 58.7 us the call, 49.0 so, four of them in the Python binding).
 // A buffer per thread, device and context, up to 1 MB, freed when the thread ends; nullptr where more is asked for or there is none to be had (the
-// caller then copies).  Each call's results are read before the thread makes another call, so no two calls meet in it.
+// caller then copies).  Each call's results are read before the thread makes another call, so no two calls meet in it; a call that ends with an error
+// first waits for what it has enqueued (cuda_status_behind).
 void* pinned_results(size_t bytes);
 
 void set_last_cuda_error(cudaError_t e);
@@ -105,6 +106,11 @@ inline rwkvq_status cuda_status(cudaError_t e) {
   if (e == cudaSuccess) return RWKVQ_OK;
   set_last_cuda_error(e);
   return RWKVQ_ECUDA;
+}
+// The same for a call that has put work on `s`, which may still be writing its results to the thread's page-locked memory.
+inline rwkvq_status cuda_status_behind(cudaError_t e, cudaStream_t s) {
+  if (e != cudaSuccess) cudaStreamSynchronize(s);
+  return cuda_status(e);
 }
 
 }  // namespace rwkvq

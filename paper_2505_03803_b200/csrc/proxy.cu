@@ -152,11 +152,11 @@ static rwkvq_status run_proxy(const void* const* w, const int* oc, const int* ic
     proxy_reduce_kernel<<<a.count, 1024, 0, s>>>(part, a, res + m0, K, bf16);
   }
   e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status_behind(e, s);
   out->resize(n_mats);
   if (!pinned) e = cudaMemcpyAsync(out->data(), res, (size_t)n_mats * sizeof(ProxyResult), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status_behind(e, s);
   if (pinned) std::copy(pinned, pinned + n_mats, out->begin());
   for (int m = 0; m < n_mats; ++m)
     if ((*out)[m].nonfinite) return RWKVQ_ENONFINITE;

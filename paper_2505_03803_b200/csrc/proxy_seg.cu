@@ -436,7 +436,7 @@ rwkvq_status rwkvq_proxy_segments(const void* w, int dtype, int oc, int ic, int 
     else pseg::proxy_segment_set_kernel<512, 2><<<grid, 512, 0, s>>>(w16, oc, ic, seg_rows, seg_cols, wide, bf16, K, res);
   }
   e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status_behind(e, s);
   std::vector<pseg::SegResult> copy;
   const pseg::SegResult* host = pinned;
   if (!pinned) {
@@ -445,7 +445,7 @@ rwkvq_status rwkvq_proxy_segments(const void* w, int dtype, int oc, int ic, int 
     host = copy.data();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status_behind(e, s);
   rwkvq_status st = RWKVQ_OK;
   for (size_t i = 0; i < nseg; ++i) {
     Pc[i] = host[i].pc; Pf[i] = host[i].pf;

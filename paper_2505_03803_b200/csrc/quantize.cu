@@ -1834,7 +1834,7 @@ rwkvq_status rwkvq_quantize_check(void* workspace_dev, void* stream) {
   cudaError_t e = cudaMemcpyAsync(pinned ? (void*)pinned : &copy, workspace_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(workspace_dev, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status_behind(e, s);
   const int host_flags = pinned ? *pinned : copy;
   return (host_flags & kFlagTimeout) ? RWKVQ_ETIMEOUT : (host_flags & kFlagNonFinite) ? RWKVQ_ENONFINITE : RWKVQ_OK;
 }

@@ -55,6 +55,42 @@ def test_results_up_to_and_beyond_the_buffer(rows):
     assert np.allclose(pc[pick], rpc, rtol=1e-9, atol=1e-9) and np.allclose(pf[pick], rpf, rtol=1e-8, atol=1e-8)
 
 
+@pytest.mark.parametrize("what", ["segments", "whole"])
+def test_a_call_that_fails_has_ended_its_work(what):
+    """An error that an earlier call of the program left behind is reported after the kernels are enqueued: they have ended when the call returns, and the
+    thread's next call, on another stream, gets the buffer to itself."""
+    import ctypes as C
+
+    import torch
+    from paper_2505_03803_b200 import binding as B
+    w = torch.randn((256, 512), generator=torch.Generator(device="cuda").manual_seed(8), device="cuda").half()
+    ws = torch.empty(max(B.rwkvq_proxy_workspace_bytes(1), B.lib().rwkvq_proxy_segments_workspace_bytes(256, 512, 16, 128)), dtype=torch.uint8, device="cuda")
+
+    def call(stream):      # without torch, whose allocator would report the error
+        pc, pf, phi = np.zeros(64), np.zeros(64), np.zeros(64, np.int32)
+        if what == "segments":
+            status = B.lib().rwkvq_proxy_segments(w.data_ptr(), B.RWKVQ_F16, 256, 512, 16, 128, 4, 3.0, math.inf, pc.ctypes.data, pf.ctypes.data,
+                                                  phi.ctypes.data, ws.data_ptr(), ws.nbytes, stream.cuda_stream)
+        else:
+            mat, oc, ic, dbl = (C.c_void_p * 1)(w.data_ptr()), (C.c_int * 1)(256), (C.c_int * 1)(512), C.POINTER(C.c_double)
+            status = B.lib().rwkvq_proxy_select(mat, oc, ic, 1, 4, 3.0, math.inf, pc.ctypes.data_as(dbl), pf.ctypes.data_as(dbl),
+                                                phi.ctypes.data_as(C.POINTER(C.c_int)), ws.data_ptr(), ws.nbytes, stream.cuda_stream)
+        return status, pc, pf, phi
+
+    busy, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    want = call(other)
+    assert want[0] == 0
+    rt, p = C.CDLL("libcudart.so.12"), C.c_void_p()
+    with torch.cuda.stream(busy):
+        torch.cuda._sleep(100_000_000)
+    assert rt.cudaMalloc(C.byref(p), C.c_size_t(1 << 60)) != 0
+    status = call(busy)[0]
+    idle = busy.query()
+    assert status == 6 and idle
+    assert all(np.array_equal(a, b) for a, b in zip(call(other), want))
+
+
 def test_a_thread_may_end_while_another_captures():
     import torch
     from paper_2505_03803_b200 import binding as B
