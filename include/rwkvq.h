@@ -297,7 +297,8 @@ typedef struct {
  * from run to run.  rwkvq_step_plan builds the schedule on
  * the host and copies it into plan_dev (rwkvq_step_plan_bytes() bytes, caller-owned); the plan
  * embeds the pointers of `ops`, so the buffers must stay where they are.  rwkvq_step_run launches
- * it.  ops must be sorted by stage (non-decreasing).  A run may be captured into a graph, which may be launched any number of times, runs
+ * it.  ops must be sorted by stage (non-decreasing).  Outputs may lie where inputs of earlier stages were (y0 -> y1 -> y0), but outputs of
+ * neighbouring stages must not overlap.  A run may be captured into a graph, which may be launched any number of times, runs
  * outside it in between (one after the other, as all runs of a plan).  Errors as rwkvq_gemv plus ETIMEOUT through
  * rwkvq_device_status.
  */

@@ -98,8 +98,11 @@ struct StepEvent {           // 64 bytes
   uint32_t barrier;          // segment: index + 1 of the stage barrier to pass first; arrival: index of the barrier
   uint32_t xstride_sums;     // segment: xstride | sums << 31
   uint16_t mu_off16;         // segment: offset / 16 of the decoded mu row inside the buffer
-  uint16_t squares;          // 1: of a stage whose inputs every CTA squares for itself (see kSquaresShare); arrival: the stage that begins
+  uint16_t flags;            // EF_*
 };
+// EF_SQUARES: of a stage whose inputs every CTA squares for itself (see kSquaresShare); arrival: the stage that begins.  EF_READ_FIRST: arrival; the
+// outputs to clear are inputs of the stage that ends, which every CTA has read when that stage's second barrier opens.
+enum { EF_SQUARES = 1, EF_READ_FIRST = 2 };
 static_assert(sizeof(StepEvent) == 64, "event descriptor size");
 
 // One product's share of a stage's pre-pass: where its inputs are and where x_mix (fp16 rows of
@@ -975,7 +978,20 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
     const StepEvent ev = *reinterpret_cast<const StepEvent*>(reinterpret_cast<const uint8_t*>(a.events) + (size_t)ei * 64);
     if (ev.kind == EV_ARRIVE) {
       if constexpr (MIX) {
-        if (ev.barrier < (uint32_t)a.n_stages && !(kSquares && ev.squares)) mix_warm<NB>(a, ev, stid);
+        if (ev.barrier < (uint32_t)a.n_stages && !(kSquares && (ev.flags & EF_SQUARES))) mix_warm<NB>(a, ev, stid);
+      }
+      if constexpr (MIX == 2) {      // plans with such stages take this kernel: the test alone cost the other 0.2 %
+        if (ev.flags & EF_READ_FIRST) {
+          const uint32_t b2 = (uint32_t)a.n_stages + ev.barrier;      // the second barrier of the stage that ends
+          if (ok && stid < kPollLanes) {
+            uint32_t it = 0;
+            while ((int)(ld_acquire_gpu(a.counter + b2) - (a.target + a.wait_skew)) < 0) {
+              if (++it >= (a.poll_limit << 2) || *abortp) { *abortp = 1; atomicExch(a.status, (int)RWKVQ_ETIMEOUT); ok = false; break; }
+            }
+          }
+          ok = named_bar_and(6, kStagerThreads, ok);
+          if (!ok) break;
+        }
       }
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
@@ -999,7 +1015,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           MixSlot* const slots = reinterpret_cast<MixSlot*>(mucb);      // the codebook copy of stagers that mix themselves
           static_assert(sizeof(MixSlot) * Shape<NB>::kStagerWarps <= kMuScratch, "pre-pass slots");
           MixPrep prep;
-          if (!(kSquares && ev.squares)) prep = mix_prepare<NB, MIX == 2>(a, ev, stid, slots, ctrl->mix_at);
+          if (!(kSquares && (ev.flags & EF_SQUARES))) prep = mix_prepare<NB, MIX == 2>(a, ev, stid, slots, ctrl->mix_at);
           if (ok && stid < kPollLanes) {
             uint32_t it = 0;
             while ((int)(ld_acquire_gpu(a.counter + ev.barrier) - (a.target + a.wait_skew)) < 0) {
@@ -1020,7 +1036,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           }
           ok = named_bar_and(6, kStagerThreads, ok);   // thread 0's acquire precedes every thread's loads of x
           if (!ok) break;
-          if (kSquares && ev.squares) continue;
+          if (kSquares && (ev.flags & EF_SQUARES)) continue;
           mix_slice<NB, MIX == 2>(a, ev, stid, prep, slots, ctrl->mix_at);
           named_bar_sync(4, kStagerThreads);           // every thread's pre-pass stores precede thread 0's release
           if (stid == 0) red_release_gpu(a.counter + (uint32_t)a.n_stages + 1u + ev.barrier, 1u);
@@ -1033,7 +1049,7 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
     ok = named_bar_and(7, kStagerThreads, mbar_wait_warp(&ctrl->xempty[buf], ((nseg / XBufs<MIX, NB>::kCount) & 1u) ^ 1u, abortp, a.status) && ok);
     uint8_t* xb = xbufs + (size_t)buf * XBufs<MIX, NB>::kBytes;
     if constexpr (kSquares) {
-      if (ev.squares) {                    // the stage's barrier has been passed with its arrival event
+      if (ev.flags & EF_SQUARES) {                    // the stage's barrier has been passed with its arrival event
         if (ok) stage_squares<NB>(a, ev, xb, stid);
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctrl->xfull[buf]);
@@ -1568,6 +1584,15 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   info->smem_bytes = fixed + (uint32_t)ns * info->slot_bytes;
   info->P = P; info->B = B; info->NB = B <= 8 ? 1 : 2;
   info->poll_limit = kDefaultPollLimit; info->wait_skew = 0;
+  std::vector<std::pair<int, int>> stage_ranges;  // [first op, last op) per distinct stage value
+  for (int i = 0; i < n_ops;) {
+    int j = i;
+    while (j < n_ops && ops[j].stage == ops[i].stage) ++j;
+    stage_ranges.push_back({i, j});
+    i = j;
+  }
+  const int n_stages = (int)stage_ranges.size();
+  if ((uint32_t)n_stages + 1u > kMaxBarriers) return RWKVQ_EUNSUPPORTED;   // per-barrier counts in the control block
   bool any_xform = false;
   for (int i = 0; i < n_ops; ++i) any_xform = any_xform || ops[i].in.kind != RWKVQ_IN_BUFFER || ops[i].in.xprev_out_fp16 != nullptr;
   // Inputs per CTA and stage: batch rows x columns of an even share of the units, averaged over the stages.
@@ -1579,28 +1604,53 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     share += (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B;
     i = j;
   }
+  // A CTA clears its slice of a stage's outputs when it has done its part of the stage before, whose inputs others may still be reading.  Where the two
+  // overlap (outputs reused in turn: y0 -> y1 -> y0), the inputs are read by the stage's pre-pass alone and the clearing waits for its barrier.
+  std::vector<char> read_first(n_stages, 0);      // the stage's inputs are outputs of the next one
+  bool any_read_first = false;
+  for (int s = 0; s + 1 < n_stages; ++s) {
+    std::vector<std::pair<uint64_t, uint64_t>> y;      // the next stage's outputs, by address
+    for (int q = stage_ranges[s + 1].first; q < stage_ranges[s + 1].second; ++q) {
+      const uint64_t at = (uint64_t)(uintptr_t)ops[q].y_dev;
+      y.push_back({at, at + (uint64_t)B * (uint64_t)ops[q].W_desc.oc * 4u});
+    }
+    std::sort(y.begin(), y.end());
+    auto written = [&](const void* p, uint64_t bytes) {
+      const uint64_t lo = (uint64_t)(uintptr_t)p;
+      if (!p || lo >= y.back().second || lo + bytes <= y.front().first) return false;
+      for (const auto& range : y)
+        if (lo < range.second && range.first < lo + bytes) return true;
+      return false;
+    };
+    for (int o = stage_ranges[s].first; o < stage_ranges[s].second && !read_first[s]; ++o) {
+      const rwkvq_input_xform& in = ops[o].in;
+      const uint64_t n = (uint64_t)ops[o].W_desc.ic, rows = (uint64_t)B * n;
+      bool hit = written(ops[o].mu_image_dev ? ops[o].xprev_fp16_dev : nullptr, rows * 2u) || written(in.xprev_out_fp16, rows * 2u);
+      if (in.kind == RWKVQ_IN_BUFFER) hit = hit || written(ops[o].x_fp16_dev, rows * 2u);
+      else hit = hit || written(in.src_f32, rows * 4u) || written(in.scale_f32, 4u);
+      if (in.kind == RWKVQ_IN_F32) hit = hit || written(in.gate_f32, rows * 4u);
+      if (in.kind == RWKVQ_IN_WKV) {
+        for (const void* p : {(const void*)in.k_f32, (const void*)in.v_f32, (const void*)in.state_a, (const void*)in.state_b, (const void*)in.state_p})
+          hit = hit || written(p, rows * 4u);
+        hit = hit || written(in.u_f32, n * 4u) || written(in.w_f32, n * 4u);
+      }
+      read_first[s] = hit;
+    }
+    any_read_first = any_read_first || read_first[s];
+  }
   // A stage pre-pass (StepArgs::mix) costs a second barrier, about 2 us per stage whatever the sizes; without it every CTA mixes the
   // columns it reads itself.  The line was measured with stacks of 1024 to 4096 columns and batches of 2 to 16 (pre-pass / without, us, at
   // `share / stages` inputs): B=6, 2688, 319 / 286 and B=3, 2688, 262 / 250; B=2, 3072, 335 / 341; B=8, 3584, 328 / 339; B=3, 4608, 338 / 370;
   // with seven stager warps B=10, 4480, 385 / 377; B=16, 5120, 353 / 335; B=16, 7168, 406 / 443; B=12, 8448, 305 / 346.  The
   // element-wise operators exist in the pre-pass only.
-  if (any_xform && n_ops > 65535) return RWKVQ_EUNSUPPORTED;      // the events count products in 16 bits
-  const bool mix = any_xform || (n_ops <= 65535 && share > stages * (B > 8 ? 5600u : 3000u));
+  if ((any_xform || any_read_first) && n_ops > 65535) return RWKVQ_EUNSUPPORTED;      // the events count products in 16 bits
+  const bool mix = any_xform || any_read_first || (n_ops <= 65535 && share > stages * (B > 8 ? 5600u : 3000u));
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 16u : 64u, kOddCost = 32u;
-  info->mix = any_xform ? 2 : mix ? 1 : 0;      // the kernel's MIX
+  info->mix = any_xform || any_read_first ? 2 : mix ? 1 : 0;      // the kernel's MIX
   const uint32_t nbp = (uint32_t)((B + 1) & ~1);
 
-  std::vector<std::pair<int, int>> stage_ranges;  // [first op, last op) per distinct stage value
-  for (int i = 0; i < n_ops;) {
-    int j = i;
-    while (j < n_ops && ops[j].stage == ops[i].stage) ++j;
-    stage_ranges.push_back({i, j});
-    i = j;
-  }
-  const int n_stages = (int)stage_ranges.size();
-  if ((uint32_t)n_stages + 1u > kMaxBarriers) return RWKVQ_EUNSUPPORTED;   // per-barrier counts in the control block
   info->n_stages = n_stages;
   info->n_barriers = ((uint32_t)n_stages + 1) * (mix ? 2u : 1u);   // the pre-pass has a barrier of its own per stage
 
@@ -1618,15 +1668,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       n += (uint64_t)((op.W_desc.oc_pad + 255) / 256) * (uint64_t)(op.W_desc.ic_pad / 256);
       all = all && op.in.kind == RWKVQ_IN_RELU2 && !op.mu_image_dev && !op.in.xprev_out_fp16 && !op.in.scale_f32;
     }
-    squares[s] = all && (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B <= kSquaresShare;
-    // a CTA that has staged its inputs clears the next stage's outputs: they must not be what others still read
-    if (squares[s] && s + 1 < n_stages)
-      for (int o = stage_ranges[s].first; o < stage_ranges[s].second; ++o)
-        for (int q = stage_ranges[s + 1].first; q < stage_ranges[s + 1].second; ++q) {
-          const uint64_t src = (uint64_t)(uintptr_t)ops[o].in.src_f32, src_end = src + (uint64_t)B * (uint64_t)ops[o].W_desc.ic * 4u;
-          const uint64_t y = (uint64_t)(uintptr_t)ops[q].y_dev, y_end = y + (uint64_t)B * (uint64_t)ops[q].W_desc.oc * 4u;
-          if (src < y_end && y < src_end) squares[s] = 0;
-        }
+    squares[s] = all && !read_first[s] && (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B <= kSquaresShare;
   }
 
   std::vector<std::vector<HostUnit>> cta_units(P);
@@ -1636,6 +1678,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     StepEvent ev;
     std::memset(&ev, 0, sizeof(ev));
     ev.kind = EV_ARRIVE; ev.barrier = (uint32_t)barrier;
+    if (barrier > 0 && barrier < n_stages && read_first[barrier - 1]) ev.flags |= EF_READ_FIRST;
     if (stage_idx_to_clear < n_stages) {
       uint64_t total = 0;
       for (int o = stage_ranges[stage_idx_to_clear].first; o < stage_ranges[stage_idx_to_clear].second; ++o)
@@ -1656,7 +1699,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       }
     }
     if (mix && barrier < n_stages && squares[barrier]) {
-      ev.squares = 1;
+      ev.flags |= EF_SQUARES;
     } else if (mix && barrier < n_stages) {
       // this CTA's share of the pre-pass of stage `barrier`
       uint64_t G = 0;
@@ -1894,7 +1937,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
         ev.mu_off16 = (uint16_t)(xseg_mu_off(B, ncols, sums) / 16u);
         ev.barrier = (uint32_t)s + 1u;   // stage s reads its inputs after barrier s
         if (squares[s]) {
-          ev.squares = 1;
+          ev.flags |= EF_SQUARES;
           ev.seg.x = (uint64_t)(uintptr_t)o.in.src_f32;
         } else if (mix) {
           ev.seg.x = mix_x_off[op] + (uint64_t)kmin * 512u;

@@ -460,3 +460,53 @@ def test_step_inputs_of_one_buffer_and_of_more(Bn, ic, bits):
     assert bool(((y.double() - ref).abs() <= bound).all())
     assert B.rwkvq_device_status() == 0
     B.rwkvq_step_plan_release(plan)
+
+
+@pytest.mark.parametrize("kind", ["relu2", "gate", "plain"])
+@pytest.mark.parametrize("Bn", [1, 3, 9])
+def test_outputs_that_are_inputs_of_the_stage_before(kind, Bn):
+    """Buffers in turn, y0 -> y1 -> y0: the outputs of the third stage are cleared only when all CTAs have read them as inputs of the second, whose
+    matrix is a few units that most CTAs have no part in.  Against the same chain with a buffer for every output."""
+    g = torch.Generator(device="cuda").manual_seed(Bn)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+
+    def matrix(rows, cols):
+        desc = B.rwkvq_desc_for(rows, cols, B.RWKVQ_SQ, 3)
+        image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+        B.rwkvq_quantize_dev_async((torch.randn((rows, cols), generator=g, device="cuda") * 0.05).half(), rows, cols, B.RWKVQ_SQ, 3, image, ws)
+        return dict(desc=desc, W=image, mu_desc=None, mu=None, xprev=None)
+
+    def zeros(cols):
+        return torch.zeros((Bn, cols), device="cuda")
+
+    w0, w1, w2, wg = matrix(1280, 1024), matrix(256, 1280), matrix(1280, 256), matrix(1280, 1024)
+    x, x1 = torch.randn((Bn, 1024), generator=g, device="cuda").half(), torch.randn((Bn, 1280), generator=g, device="cuda").half()
+
+    def chain(apart):
+        y0, y1, gate = zeros(1280), zeros(256), zeros(1280)
+        y2 = zeros(1280) if apart or kind == "plain" else gate if kind == "gate" else y0
+        x1d = x1.clone() if apart else y2.view(torch.float16).view(-1)[:Bn * 1280].view(Bn, 1280)
+        second = dict(x=x1d) if kind == "plain" else dict(x=None, **{"in": dict(kind=B.RWKVQ_IN_F32, src=y0, gate=gate) if kind == "gate" else
+                                                                     dict(kind=B.RWKVQ_IN_RELU2, src=y0)})
+        third = dict(x=x1[:, :256].contiguous()) if kind == "plain" else dict(x=None, **{"in": dict(kind=B.RWKVQ_IN_RELU2, src=y1)})
+        keep = [dict(w0, x=x, y=y0, stage=0)] + ([dict(wg, x=x, y=gate, stage=0)] if kind == "gate" else [])
+        keep += [dict(w1, y=y1, stage=1, **second), dict(w2, y=y2, stage=2, **third)]
+        ops = B.make_ops(keep)
+        plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
+        B.rwkvq_step_plan(ops, Bn, plan)
+        out = []
+        for _ in range(3 if apart else 60):
+            if kind == "plain" and not apart:
+                x1d.copy_(x1)
+            B.rwkvq_step_run(plan)
+            out.append((y1.clone(), y2.clone()))
+        torch.cuda.synchronize()
+        assert B.rwkvq_device_status() == 0
+        B.rwkvq_step_plan_release(plan)
+        return out
+
+    want = chain(True)[0]
+    assert all(bool((w != 0).any()) for w in want)
+    for got in chain(False):
+        for a, b in zip(got, want):      # sums in another order; an input may round to the other fp16 number (2^-11)
+            assert float((a.double() - b.double()).norm()) <= 1e-3 * float(b.double().norm())
