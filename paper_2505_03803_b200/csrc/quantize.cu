@@ -1485,11 +1485,11 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     return best < INFINITY ? group * kCentreGroup + at : 0;
   };
   // Two threads add up the members of centre e in dimension `dim` (one thread, of 256 centres), two words of masks at a time; the block that has
-  // the centre, and its place there:
+  // the centre, and its place there (threads beyond the last centre have none, and address the last block):
   constexpr int kSplit = E == 64 ? 2 : 1;
   const int dim = tid & 1, split = (tid >> 1) % kSplit, e = tid / (2 * kSplit);
   constexpr int kOwn = E / kVecCluster;            // centres a block has
-  const uint32_t owner = (uint32_t)(e / kOwn), my_part = peer_address(shared_address(&sh.part[rank][e % kOwn][dim]), owner), owner_bar = peer_address(sums_here, owner);
+  const uint32_t owner = (uint32_t)min(e / kOwn, kVecCluster - 1), my_part = peer_address(shared_address(&sh.part[rank][e % kOwn][dim]), owner), owner_bar = peer_address(sums_here, owner);
   // ... and kOwn * 2 * kVecCluster of them look after one of this block's centres, for one receiver each
   const int own = tid / (2 * kVecCluster), own_dim = tid / kVecCluster % 2;
   const uint32_t receiver = (uint32_t)(tid % kVecCluster);
