@@ -424,7 +424,9 @@ rwkvq_status rwkvq_desc_for(const rwkvq_quant_cfg* cfg, int oc, int ic, rwkvq_de
  * desc.image_bytes of rwkvq_desc_for), ready for every product call above.
  *  SQ (Eq. 2): codes, scales and zero points are identical to rwkvq_pack's (same rounding rules),
  *      bit for bit.
- *  VQ (Eq. 3): one thread block per 256 x 256 tile (or per vector) runs k-means++ seeding and
+ *  VQ (Eq. 3): one thread block per 256 x 256 tile (a cluster of four where there are no more than
+ *      100 tiles), or one cluster of sixteen blocks per vector, which takes a GPU with sixteen SMs in
+ *      one cluster's reach (ECUDA where there are none), runs k-means++ seeding and
  *      cfg->kmeans_iters Lloyd iterations in fp32 with exact integer cluster sums, rounds the
  *      centres to fp16 and takes the final assignment in fp64 against the rounded centres (lowest
  *      index wins ties).  Random draws come from the library's generator seeded with cfg->seed and
@@ -449,14 +451,22 @@ rwkvq_status rwkvq_quantize_dev(const void* w_fp16_dev, int oc, int ic, const rw
  * a NaN/Inf weight sets a flag in the first word of workspace_dev, which must be zero before the
  * first call and is shared by every call that uses the same workspace.  rwkvq_quantize_check
  * synchronizes `stream`, returns RWKVQ_ENONFINITE if the flag was set by any call since the last
- * check (RWKVQ_OK otherwise) and clears it.  ETIMEOUT: a bounded wait between the blocks of a token-shift
- * vector's kernel ran out; the images since the last check are not to be used.
+ * check (RWKVQ_OK otherwise) and clears it.  ETIMEOUT: a bounded wait between the blocks of a cluster (a
+ * token-shift vector's, or a tile's seeds) ran out; the images since the last check are not to be used.
  */
 rwkvq_status rwkvq_quantize_dev_async(const void* w_fp16_dev, int oc, int ic, const rwkvq_quant_cfg* cfg,
                                       const float* elem_weight_dev, void* image_dev, size_t image_bytes,
                                       rwkvq_desc* desc_out, void* workspace_dev, size_t workspace_bytes,
                                       void* stream);
 rwkvq_status rwkvq_quantize_check(void* workspace_dev, void* stream);
+/*
+ * rwkvq_quantize_dev_async with another limit for those waits (tries; 0 = default) and one block of each cluster,
+ * mute_block, that sends nothing: the waits for it run out.  Exists so that a test can watch them do so.
+ */
+rwkvq_status rwkvq_quantize_dev_lost(const void* w_fp16_dev, int oc, int ic, const rwkvq_quant_cfg* cfg,
+                                     const float* elem_weight_dev, void* image_dev, size_t image_bytes,
+                                     void* workspace_dev, size_t workspace_bytes, uint32_t poll_limit,
+                                     uint32_t mute_block, void* stream);
 
 /*
  * Representative X of a batch of calibration activations (Section 4.2): for each of the n

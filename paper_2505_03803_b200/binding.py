@@ -80,7 +80,7 @@ EXPORTS = [
     "rwkvq_proxy_family", "rwkvq_proxy_select_bf16", "rwkvq_proxy_f32_workspace_bytes", "rwkvq_proxy_select_f32",
     "rwkvq_proxy_segments_workspace_bytes", "rwkvq_proxy_segments", "rwkvq_tau_for_fraction", "rwkvq_tau_largest_gap", "rwkvq_quant_error_workspace_bytes", "rwkvq_quant_error",
     "rwkvq_desc_for", "rwkvq_quantize_workspace_bytes", "rwkvq_quantize_dev", "rwkvq_calib_representative",
-    "rwkvq_quantize_dev_async", "rwkvq_quantize_check",
+    "rwkvq_quantize_dev_async", "rwkvq_quantize_dev_lost", "rwkvq_quantize_check",
 ]
 
 _lib = None
@@ -161,6 +161,7 @@ def lib() -> C.CDLL:
         L.rwkvq_quantize_dev.argtypes = [vp, i32, i32, C.POINTER(QuantCfg), vp, vp, sz, C.POINTER(Desc), vp, sz, vp]
         L.rwkvq_calib_representative.argtypes = [vp, i32, i32, dbl, vp, vp, vp]
         L.rwkvq_quantize_dev_async.argtypes = L.rwkvq_quantize_dev.argtypes
+        L.rwkvq_quantize_dev_lost.argtypes = [vp, i32, i32, C.POINTER(QuantCfg), vp, vp, sz, vp, sz, C.c_uint32, C.c_uint32, vp]
         L.rwkvq_quantize_check.argtypes = [vp, vp]
     _lib = L
     return L
@@ -620,8 +621,16 @@ def rwkvq_quantize_dev_async(w, oc: int, ic: int, method: int, bits: int, image,
     return d
 
 
+def rwkvq_quantize_dev_lost(w, oc: int, ic: int, method: int, bits: int, image, workspace, poll_limit: int, mute_block: int, *, elem_weight=None,
+                            kmeans_iters: int = 10, seed: int = 0, stream=None) -> None:
+    """rwkvq_quantize_dev_lost: rwkvq_quantize_dev_async with a block that sends nothing, for tests."""
+    cfg = QuantCfg(method=method, bits=bits, group=128, vec_dim=2, tile=256, kmeans_iters=kmeans_iters, seed=seed, codes_in=None)
+    _check(lib().rwkvq_quantize_dev_lost(_dev_ptr(w), oc, ic, C.byref(cfg), _dev_ptr(elem_weight), _dev_ptr(image), image.nbytes,
+                                         _dev_ptr(workspace), workspace.nbytes, poll_limit, mute_block, _stream_ptr(stream)), "rwkvq_quantize_dev_lost")
+
+
 def rwkvq_quantize_check(workspace, stream=None) -> int:
-    """rwkvq_quantize_check: status code (0 = OK, 4 = a NaN/Inf weight was seen); synchronizes."""
+    """rwkvq_quantize_check: status code (0 = OK, 4 = a NaN/Inf weight was seen, 8 = a bounded wait ran out); synchronizes."""
     return int(lib().rwkvq_quantize_check(_dev_ptr(workspace), _stream_ptr(stream)))
 
 

@@ -230,13 +230,16 @@ __device__ __forceinline__ int below(uint64_t r, int n) {
   return (int)((unsigned long long)(unit_of(r) * (double)n) % (unsigned long long)n);
 }
 
+constexpr uint32_t kDefaultPollLimit = 1u << 20, kNoBlock = ~0u;      // a try takes up to 4 us
 struct VqArgs {
   const uint16_t* w;        // matrix [oc][ic] or vector [ic]
   const float* elem_w;      // vector mode: X^2 per element, or NULL
   int ic;                   // row length of w
   int TC;                   // tiles per row of tiles (matrix mode)
   int n_vec;                // vectors per codebook
-  int bits, E, iters;
+  int E, iters;
+  uint32_t poll_limit;      // tries of a wait between the blocks of a cluster
+  uint32_t mute;            // block of each cluster that sends nothing, for a test; kNoBlock: none
   uint64_t seed;
   uint8_t* payload;         // matrix: chunk grid; vector: bit stream
   uint32_t* aux;            // codebooks, E half2 each
@@ -350,14 +353,18 @@ __device__ __forceinline__ uint4 peer_load4(uint32_t at) {
   asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
   return v;
 }
-// Waits for a phase of a barrier of this block that stores of the cluster complete; gives up after some seconds.
-__device__ __forceinline__ bool wait_sent(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 24); ++i) {
+// Waits for a phase of a barrier of this block that stores of the cluster complete; gives up after `limit` tries.
+__device__ __forceinline__ bool wait_sent(uint32_t bar, uint32_t parity, uint32_t limit) {
+  for (uint32_t i = 0; i < limit; ++i) {
     uint32_t ok;
     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     if (ok) return true;
   }
   return false;
+}
+// A block that has given up stays for some milliseconds after all others have sent what they will: what is still on its way to it lands.
+__device__ __forceinline__ void stay_behind() {
+  for (int i = 0; i < 8; ++i) __nanosleep(1000000);
 }
 
 // ---- seeds ----
@@ -475,36 +482,39 @@ __global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqA
   uint32_t* aux = a.aux + (size_t)tile * E;
   bool lost = false;
   // the block with vector `at` sends it to all
+  const bool mute = rank == a.mute;
   auto send = [&](int at) {
+    if (mute) return;
     const uint32_t v = sh.vec[vq_slot(at)];
 #pragma unroll
     for (uint32_t r = 0; r < kTileBlocks; ++r) peer_send(peer_address(shared_address(&sh.pick), r), v, peer_address(pick_here, r));
   };
-  auto receive = [&](int e) -> uint32_t {
-    if (tid == 0) expect_sent(pick_here, 4);
-    lost = lost || !wait_sent(pick_here, (uint32_t)e & 1u);
-    return sh.pick;
-  };
+  // a warp whose wait has run out leaves: it neither sends nor expects any more, and the others' waits run out in turn
+  auto wait = [&](uint32_t bar, uint32_t parity) { lost = !__all_sync(0xFFFFFFFFu, wait_sent(bar, parity, a.poll_limit)); };
   const int first = below(splitmix(seed, 0), kVqMaxVec);
   if (tid == 0 && first / kPartVec == (int)rank) send(first % kPartVec);
   for (int e = 0;; ++e) {
     // A block sends its next draw when it has the next sums of all warps, and a warp its next sums when it has this draw; the sums of two draws
     // are under way at once, to places and barriers of their own.
-    const uint32_t cv = receive(e);
+    if (tid == 0) expect_sent(pick_here, 4);
+    wait(pick_here, (uint32_t)e & 1u);
+    if (lost) break;
+    const uint32_t cv = sh.pick;
     if (tid == 0 && rank == 0u) aux[e] = cv;
     if (e + 1 == E) break;
     const float local = nearer(dist, sh.vec, base, cv);
     const float incl = sum_to_lane(local);
     const uint32_t bar = tot_here + 8 * (e & 1);
     if (tid == 0) expect_sent(bar, (int)sizeof(sh.tot[0]));
-    if (lane == 31) {
+    if (lane == 31 && !mute) {
 #pragma unroll
       for (uint32_t r = 0; r < kTileBlocks; ++r)
         peer_send(peer_address(shared_address(&sh.tot[e & 1][tile_warp]), r), __float_as_uint(incl), peer_address(bar, r));
     }
     float excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
     if (lane == 0) excl = 0.f;
-    lost = lost || !wait_sent(bar, (uint32_t)(e >> 1) & 1u);
+    wait(bar, (uint32_t)(e >> 1) & 1u);
+    if (lost) break;
     float before, total;
     warp_sums(sh.tot[e & 1], tile_warp, before, total);
     const float target = sh.u01[e + 1] * total;
@@ -519,6 +529,7 @@ __global__ void __launch_bounds__(kSeedThreads, 4) vq_tile_seed_kernel(const VqA
   if (lost) atomicOr(a.flags, kFlagTimeout);
   cluster_arrive();
   cluster_wait();
+  if (lost) stay_behind();
 }
 
 // One block: a tile, where there are enough of them for every SM (hand-overs cost less inside a block), or a token-shift vector of n vectors, more
@@ -1493,6 +1504,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
   // ... and kOwn * 2 * kVecCluster of them look after one of this block's centres, for one receiver each
   const int own = tid / (2 * kVecCluster), own_dim = tid / kVecCluster % 2;
   const uint32_t receiver = (uint32_t)(tid % kVecCluster);
+  const bool sends = tid < 2 * E * kSplit && split == 0 && rank != a.mute;
   bool lost = false;
   int which = 0;
   for (int it = 0; it < a.iters; ++it) {
@@ -1530,7 +1542,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     }
     if (kSplit == 2) { sum.wv += __shfl_xor_sync(0xFFFFFFFFu, sum.wv, 2); sum.w += __shfl_xor_sync(0xFFFFFFFFu, sum.w, 2); }
     if (tid == 0) { expect_sent(sums_here, (int)sizeof(sh.part)); expect_sent(centres_here, (int)sizeof(sh.sent)); }
-    if (tid < 2 * E * kSplit && split == 0) {
+    if (sends) {
       ulonglong2 bits;
       if constexpr (kWeighted) bits = make_ulonglong2((unsigned long long)__double_as_longlong(sum.wv), (unsigned long long)__double_as_longlong(sum.w));
       else bits = make_ulonglong2((unsigned long long)sum.wv, (unsigned long long)sum.w);
@@ -1539,7 +1551,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     // A block sends its next sums when it has the centres of all blocks, and a block its next centres when it has the next sums of all: neither place is
     // written again before it has been read.
     if (tid < 2 * kOwn * kVecCluster) {
-      lost = lost || !wait_sent(sums_here, (uint32_t)it & 1u);
+      lost = !wait_sent(sums_here, (uint32_t)it & 1u, a.poll_limit);
       Sums s[kVecCluster];
 #pragma unroll
       for (int r = 0; r < kVecCluster; ++r) s[r] = reinterpret_cast<const Sums&>(sh.part[r][own][own_dim]);
@@ -1556,10 +1568,10 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
       peer_send(peer_address(shared_address(&sh.sent[rank * kOwn + own][own_dim]), receiver), (unsigned long long)__double_as_longlong(c), peer_address(centres_here, receiver));
     }
     if (tid < 2 * E) {
-      lost = lost || !wait_sent(centres_here, (uint32_t)it & 1u);
+      lost = lost || !wait_sent(centres_here, (uint32_t)it & 1u, a.poll_limit);
       set_centre(tid >> 1, tid & 1, sh.sent[tid >> 1][tid & 1]);
     }
-    __syncthreads();
+    if (__syncthreads_or(lost)) break;             // the whole block leaves: it neither sends nor expects any more
   }
   cluster_arrive();                                // before the end: no block leaves while another might send to it
   if (lost) atomicOr(a.flags, kFlagTimeout);
@@ -1610,6 +1622,7 @@ __global__ void __launch_bounds__(kVecThreads, 1) vq_vector_kernel(const VqArgs 
     reinterpret_cast<uint32_t*>(a.payload)[wi] = val;
   }
   cluster_wait();
+  if (lost) stay_behind();
 }
 
 // ---- representative activation (Section 4.2) -----------------------------------------------------
@@ -1747,7 +1760,8 @@ size_t rwkvq_quantize_workspace_bytes(void) { return 256; }
 
 static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rwkvq_quant_cfg* cfg, const float* elem_weight_dev,
                                      void* image_dev, size_t image_bytes, rwkvq_desc* desc_out, void* workspace_dev,
-                                     size_t workspace_bytes, void* stream, bool clear_flag) {
+                                     size_t workspace_bytes, void* stream, bool clear_flag, uint32_t poll_limit = rwkvq::kDefaultPollLimit,
+                                     uint32_t mute = rwkvq::kNoBlock) {
   using namespace rwkvq;
   if (!w_dev || !cfg || !image_dev || !workspace_dev || cfg->codes_in) return RWKVQ_EINVAL;
   rwkvq_desc d;
@@ -1785,8 +1799,9 @@ static rwkvq_status quantize_enqueue(const void* w_dev, int oc, int ic, const rw
     a.ic = ic;
     a.TC = is_vector ? 1 : ic / 256;
     a.n_vec = is_vector ? ic / 2 : kVqMaxVec;
-    a.bits = d.bits; a.E = d.entries; a.iters = cfg->kmeans_iters;
+    a.E = d.entries; a.iters = cfg->kmeans_iters;
     a.seed = cfg->seed;
+    a.poll_limit = poll_limit; a.mute = mute;
     a.payload = img + h.off_payload;
     a.aux = reinterpret_cast<uint32_t*>(img + h.off_aux);
     a.flags = flags;
@@ -1844,6 +1859,13 @@ rwkvq_status rwkvq_quantize_dev_async(const void* w_dev, int oc, int ic, const r
                                       size_t workspace_bytes, void* stream) {
   return quantize_enqueue(w_dev, oc, ic, cfg, elem_weight_dev, image_dev, image_bytes, desc_out, workspace_dev,
                           workspace_bytes, stream, false);
+}
+
+rwkvq_status rwkvq_quantize_dev_lost(const void* w_dev, int oc, int ic, const rwkvq_quant_cfg* cfg, const float* elem_weight_dev,
+                                     void* image_dev, size_t image_bytes, void* workspace_dev, size_t workspace_bytes, uint32_t poll_limit,
+                                     uint32_t mute_block, void* stream) {
+  return quantize_enqueue(w_dev, oc, ic, cfg, elem_weight_dev, image_dev, image_bytes, nullptr, workspace_dev, workspace_bytes, stream, false,
+                          poll_limit ? poll_limit : rwkvq::kDefaultPollLimit, mute_block);
 }
 
 rwkvq_status rwkvq_quantize_dev(const void* w_dev, int oc, int ic, const rwkvq_quant_cfg* cfg, const float* elem_weight_dev,

@@ -614,3 +614,21 @@ def test_captured_quantizers(oc, ic, bits):
         graph.replay()
         assert torch.equal(image, ref)
     assert B.rwkvq_quantize_check(ws) == 0
+
+
+@pytest.mark.parametrize("oc,ic,bits,weighted", [(256, 256, 6, False), (512, 768, 8, False), (1, 128, 6, False), (1, 4096, 6, True), (1, 10240, 8, False)])
+@pytest.mark.parametrize("mute", [0, 1, 3])
+def test_waits_between_blocks_run_out(oc, ic, bits, weighted, mute):
+    """A block of every cluster sends nothing: the others give up, the kernels return, the next check reports ETIMEOUT once, and the calls after it are right."""
+    g = torch.Generator(device="cuda").manual_seed(ic + bits)
+    w = (torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half()
+    weight = torch.rand(ic, generator=g, device="cuda") if weighted else None
+    desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_VQ, bits)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    image, again = (torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda") for _ in range(2))
+    B.rwkvq_quantize_dev_async(w, oc, ic, B.RWKVQ_VQ, bits, image, ws, elem_weight=weight, kmeans_iters=3, seed=2)
+    assert B.rwkvq_quantize_check(ws) == 0
+    B.rwkvq_quantize_dev_lost(w, oc, ic, B.RWKVQ_VQ, bits, again, ws, 200, mute, elem_weight=weight, kmeans_iters=3, seed=2)
+    B.rwkvq_quantize_dev_async(w, oc, ic, B.RWKVQ_VQ, bits, again, ws, elem_weight=weight, kmeans_iters=3, seed=2)
+    assert B.rwkvq_quantize_check(ws) == 8 and B.rwkvq_quantize_check(ws) == 0
+    assert torch.equal(image, again)
