@@ -366,8 +366,8 @@ rwkvq_status rwkvq_step_run_host(const void* plan_dev, size_t plan_bytes, const 
  * (X[t-1] - X[t]) (.) mu_hat (Eq. 20), with X[-1] = xprev0 (zeros if NULL); mu NULL = no mix.
  * X_bf16_dev: [M][ic] row-major; Y_dev: [M][oc] row-major, F32 or BF16; all device pointers,
  * 16-byte aligned, owned by the caller.  workspace_dev: rwkvq_prefill_workspace_bytes() bytes,
- * 128-byte aligned; it receives x_mix in the tensor core's operand layout and a scheduling word,
- * and must not be shared by products in flight at the same time.  The call enqueues on `stream`
+ * 128-byte aligned (what that gives for M tokens is enough for any fewer); it receives x_mix in the
+ * tensor core's operand layout, a scheduling word and sums of slices, and must not be shared by products in flight at the same time.  The call enqueues on `stream`
  * and returns; a device-side wait that ran out shows in rwkvq_device_status (ETIMEOUT).
  * Errors: EINVAL (NULL pointer, M <= 0, mu without mu_desc, xprev0 without mu, unknown y_dtype),
  * ESHAPE (oc == 1, ic not a multiple of 8), EUNSUPPORTED (format), EALIGN, ENOMEM (workspace

@@ -798,8 +798,9 @@ struct HostProduct {
 // one 22.8; d 768, 400 tokens (2496): three 24.5, two 20.7; d 2048, 400 tokens (6656): two 62.8, one 56.2; 203 tokens (3328): two 34.9, one 37.2;
 // of twelve chunks they are worth it again (d 896, 400 tokens: three 26.6, two 28.7).  A function of the
 // product and M alone, so that a product gives the same bits in every group.
+constexpr int kMaxSlicedTiles = 64;
 int slices_of(int KT, long long tiles, int NT) {
-  constexpr int kMinChunks = 6, kSliceChunks = 4, kMaxSlicedTiles = 64, kShortChunks = 11, kMaxShortSums = 7000;
+  constexpr int kMinChunks = 6, kSliceChunks = 4, kShortChunks = 11, kMaxShortSums = 7000;
   if (KT < kMinChunks) return 1;
   long long most = kMaxSlicedTiles / tiles;
   if (KT <= kShortChunks) most = std::min(most, kMaxShortSums / (tiles * NT));
@@ -836,7 +837,7 @@ rwkvq_status check_product(const rwkvq_prefill_op& o, int M, HostProduct* out) {
   if (!aligned16(o.W_image_dev) || !aligned16(o.X_bf16_dev) || !aligned16(o.Y_dev) || (o.mu_image_dev && !aligned16(o.mu_image_dev)) ||
       (o.xprev0_bf16_dev && !aligned16(o.xprev0_bf16_dev)))
     return RWKVQ_EALIGN;
-  const size_t need = rwkvq_prefill_workspace_bytes(d, M, o.mu_image_dev != nullptr);
+  const size_t need = layout_of(d, M).bytes;
   if (!o.workspace_dev || o.workspace_bytes < need) return RWKVQ_ENOMEM;
   if ((reinterpret_cast<uintptr_t>(o.workspace_dev) & 127u) != 0) return RWKVQ_EALIGN;
   const uint8_t* img = static_cast<const uint8_t*>(o.W_image_dev);
@@ -891,7 +892,11 @@ extern "C" {
 size_t rwkvq_prefill_workspace_bytes(const rwkvq_desc* d, int M, int has_mu) {
   (void)has_mu;   // the room for operand tiles is there whether or not a token shift is applied
   if (!d || M <= 0 || check_matrix_desc(d) != RWKVQ_OK) return 0;
-  return layout_of(d, M).bytes;
+  // fewer tokens may be cut into more slices: a workspace for M tokens serves every shorter prompt
+  size_t most = layout_of(d, M).bytes;
+  const int sliced = pf::kTileTokens * (kMaxSlicedTiles / (d->oc_pad / 128));
+  for (int m = 16; m < M && m <= sliced; m += 16) most = std::max(most, layout_of(d, m).bytes);      // tokens a tile are a multiple of 16
+  return most;
 }
 
 rwkvq_status rwkvq_gemm_prefill_grouped(const rwkvq_prefill_op* ops, int n_ops, int M, int y_dtype, void* stream) {

@@ -32,6 +32,13 @@ def test_library_exports_every_declared_symbol():
     assert set(B.EXPORTS) == declared
 
 
+@pytest.mark.parametrize("oc,ic", [(256, 2560), (512, 1792), (768, 2688), (2048, 7168), (4096, 4096), (9216, 2048)])
+def test_a_prefill_workspace_serves_every_shorter_prompt(oc, ic):
+    desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ, 3)
+    sizes = [B.rwkvq_prefill_workspace_bytes(desc, m, False) for m in range(1, 2400)]
+    assert sizes[0] > 0 and all(a <= b for a, b in zip(sizes, sizes[1:]))
+
+
 def test_sq_encoder_matches_oracle_codes_exactly():
     for seed, kind in ((0, "gauss"), (1, "student"), (2, "uniform")):
         w = inputs.gen_weight(seed, 64, 512, kind)

@@ -233,3 +233,14 @@ def test_prefill_sliced_contractions_and_even_token_tiles(fmt, oc, ic, M, has_mu
     _check(W, mu, M, seed + 2, y_dtype=y_dtype)
     _, Xd = _bf16(inputs.gen_activation(seed + 4, M, ic, n_outliers=8))
     assert torch.equal(_run(W, mu, Xd, None, M, y_dtype), _run(W, mu, Xd, None, M, y_dtype))
+
+
+@pytest.mark.parametrize("oc,ic,most,tokens", [(256, 2560, 1153, 1057), (512, 1792, 833, 385), (768, 2688, 385, 321)])
+def test_a_workspace_for_more_tokens(oc, ic, most, tokens):
+    """A workspace made for a longer prompt, whose contraction is cut into fewer slices, takes a shorter one, with the result that one of its own gives."""
+    W = H.pack_sq(H.random_sq_codes(oc + tokens, oc, ic))
+    _, X = _bf16(inputs.gen_activation(tokens, tokens, ic, n_outliers=8))
+    ws = torch.full((B.rwkvq_prefill_workspace_bytes(W.desc, most, False),), 0xCD, dtype=torch.uint8, device="cuda")
+    Y = torch.full((tokens, oc), float("nan"), device="cuda")
+    B.rwkvq_gemm_prefill(W.desc, W.dev, None, None, X, None, tokens, Y, ws)
+    assert torch.equal(Y, _run(W, None, X, None, tokens))
