@@ -66,7 +66,7 @@ struct StepUnit {            // 128 bytes, copied into the slot header by the pr
   uint32_t row0, oc;         // first output row of chunk A; rows of the product
   uint64_t y;                // float y[B][oc]
   uint32_t xstride, gs_off;  // geometry of the segment: bytes between batch rows, offset of the sums
-  uint32_t nbp, entries;
+  uint32_t nbp, reserved;
   uint32_t chunk_bytes;      // distance between chunk A and chunk B inside the slot
   uint32_t rec_bytes;
   uint32_t ev_index;         // position of the unit's segment in this CTA's event list
@@ -1741,7 +1741,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           if (2 * tr + 1 < MB) { h.u.src1 = (uint64_t)(uintptr_t)(payload + (size_t)((2 * tr + 1) * KT + kt) * cb); h.u.bytes1 = cb; }
           if (vq) {
             h.u.cb_src = (uint64_t)(uintptr_t)(aux + (size_t)(tr * KT + kt) * d.entries * 4);
-            h.u.cb_bytes = (uint32_t)d.entries * 4u; h.u.entries = (uint32_t)d.entries;
+            h.u.cb_bytes = (uint32_t)d.entries * 4u;
           }
           h.u.chunk_bytes = cb; h.u.rec_bytes = rb;
           h.u.row0 = (uint32_t)tr * 256u; h.u.oc = (uint32_t)d.oc; h.u.y = (uint64_t)(uintptr_t)ops[o].y_dev;
