@@ -261,13 +261,14 @@ __device__ void set_gaps(const uint32_t* bm, bool bf16, double n, int K, SetShar
   }
 }
 
-// P_c of Eq. 9 and P_f of Eq. 17 from the sums; `n` = weights - 1, the n - (distinct - 1) ties have t = -1.
+// P_c of Eq. 9 and P_f of Eq. 17 from the sums; `n` = weights - 1, the n - (distinct - 1) ties have t = -1.  Two weights have one gap, R itself, and
+// proxies of zero: by its reciprocal the gap over R is 1 - 2^-53 for one in nine, and a threshold of zero would choose SQ.
 __device__ __forceinline__ void proxy_from_set(const SetStats& s, double n, int K, double* pc, double* pf) {
   const double ties = n - (double)(s.distinct - 1);
   double f = 0.0;
   for (int k = 2; k <= K; ++k) f += fabs((s.pw[k - 2] + ((k & 1) ? -ties : ties)) / n) / (double)(k * (k - 1));
-  *pc = log(n) + s.sum_glng;
-  *pf = f;
+  *pc = n == 1.0 ? 0.0 : log(n) + s.sum_glng;
+  *pf = n == 1.0 ? 0.0 : f;
 }
 
 }  // namespace rwkvq

@@ -127,6 +127,14 @@ def test_proxy_segments_of_two_weights_are_zero(dtype):
         assert (pc == 0.0).all() and (pf == 0.0).all() and (phi == B.RWKVQ_VQ).all()
 
 
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_proxy_of_two_weights_by_gaps_with_inexact_reciprocals_is_zero(dtype):
+    """49, 98 and 103 times their fp64 reciprocals are 1 - 2^-53."""
+    v64, dev = _typed(np.tile(np.array([[0.0, 49.0, 0.0, 98.0, 0.0, 103.0, 12.0, 115.0]], np.float32), (8, 1)), dtype)
+    pc, pf, phi = B.rwkvq_proxy_segments(dev, 1, 2, 4, 0.0, math.inf)
+    assert (pc == 0.0).all() and (pf == 0.0).all() and (phi == B.RWKVQ_VQ).all()
+
+
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("shape,seg", [((40, 300), (1, 300)), ((40, 300), (16, 128)), ((512, 512), (256, 256)),
                                        ((33, 70), (8, 64)), ((3, 5000), (1, 5000))])
