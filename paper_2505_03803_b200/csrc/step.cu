@@ -1655,9 +1655,11 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   info->n_barriers = ((uint32_t)n_stages + 1) * (mix ? 2u : 1u);   // the pre-pass has a barrier of its own per stage
 
   // Stages of squared inputs alone (no token shift, no gain): up to kSquaresShare inputs a CTA it squares what it reads itself, behind the stage's
-  // barrier, and the stage needs neither the pre-pass nor its barrier.  Blocks, pre-pass / so, us, at `inputs a CTA`: d 512, batch 1, 256, 101.4 / 94.7;
-  // d 2048, batch 2, 1024, 128.2 / 123.5; batch 4, 2048, 129.4 / 125.7; d 3072, batch 3, 3072, 125.7 / 123.4; d 4096, batch 2, 3584, 194.2 / 194.8;
-  // d 2048, batch 8, 4096, 152.7 / 148.3; d 4096, batch 4, 7168, 213.8 / 215.2.
+  // barrier, and the stage needs neither the pre-pass nor its barrier.  Four blocks, pre-pass / so, us, at `inputs a CTA`: d 512, batch 1, 256, 100.1 / 94.3;
+  // d 2048, batch 1, 512, 123.5 / 117.1; batch 2, 1024, 125.0 / 119.1; d 3072, batch 1, 1024, 151.7 / 145.6; d 4096, batch 1, 1792, 190.6 / 186.7; batch 8, 2048,
+  // d 512 106.7 / 103.1, d 1024 115.0 / 112.0, d 1536 125.4 / 121.8; d 3072, batch 3, 3072, 164.3 / 161.9; d 4096, batch 2, 3584, 192.7 / 192.5; d 2048, batch 8,
+  // 4096, 150.4 / 146.1; d 4096, batch 3, 5376, 205.0 / 208.6; batch 4, 7168, 211.6 / 213.0.  (What it takes depends on the rows and on the CTA's columns, too: 3584 is
+  // even and 4096 a gain.)
   constexpr uint64_t kSquaresShare = 4200u;
   std::vector<char> squares(n_stages, 0);
   for (int s = 0; s < n_stages && any_xform && B <= 8; ++s) {
