@@ -795,9 +795,12 @@ struct HostProduct {
 // 48 to 296 and lengths from 3 to 7, 64 to 74 and 4 were the best over 22 layers (d 2048, 203 tokens: 53.6 us with whole tiles, 37 with
 // slices; d 768, 48 tokens: 22.6, 14.4; d 640, 1368 tokens, limit 64: no slices, 32.8 where two each took 36.9).  Short contractions, whose slices
 // are a chunk or two shorter than the whole, not where their sums (tiles x tokens of a tile) are many: d 512, 1000 tokens (4160): two slices 26.8 us,
-// one 22.8; d 768, 400 tokens (2496): three 24.5, two 20.7; d 2048, 400 tokens (6656): two 62.8, one 56.2; 203 tokens (3328): two 34.9, one 37.2;
-// of twelve chunks they are worth it again (d 896, 400 tokens: three 26.6, two 28.7).  A function of the
-// product and M alone, so that a product gives the same bits in every group.
+// one 22.8; d 768, 400 tokens (2496): three 24.5, two 20.7; d 2048, 400 tokens (6656): two 62.8, one 56.2; 203 tokens (3328): two 34.9, one 37.2.
+// Of 63 layers of d 512 to 2816 that this rule cuts otherwise (17 to 1368 tokens), 46 gain by it, up to 1.19 times, and 12 lose, up to 1.11 times: what it comes to
+// is how evenly the layer's units fill the SMs (d 2176, 203 tokens, 3536: two 36.9, one 40.8, but d 2304, 3744: 41.4, 41.2; d 2816, 150 tokens, 3520: 47.1,
+// 49.8, but d 2048, 224 tokens, 3584: 46.2, 44.9), and the mean is 1.04.  Of twelve chunks whole ones lose more than they gain: d 2944, 17 to 203 tokens, two
+// 42.5 to 55.9, one 49.1 to 62.3; d 896, 400 tokens, three 26.9, two 28.9, one 26.8, and only from 500 tokens on one is better (28.9, 26.8).  A function of
+// the product and M alone, so that a product gives the same bits in every group.
 constexpr int kMaxSlicedTiles = 64;
 int slices_of(int KT, long long tiles, int NT) {
   constexpr int kMinChunks = 6, kSliceChunks = 4, kShortChunks = 11, kMaxShortSums = 7000;
