@@ -18,7 +18,8 @@
 //     other waits, flushes or synchronises.  Warp w of a group owns rows
 //     16w..16w+15 of both chunks and runs the m16n8k16 tensor-core steps of gemv_core.cuh with
 //     every input fragment shared by the two records.  Partial sums go to y with fp32 reductions
-//     (16 bytes per lane after a transpose among lanes) at the end of a run along K.
+//     (16 bytes per lane after a transpose among lanes) at the end of a run along K.  In plans of small
+//     stages a group's first unit is unpacked into tensor memory while the inputs are on their way.
 //
 // For larger inputs per CTA, and whenever a product's input is an element-wise operator on
 // earlier outputs (rwkvq_input_xform: the WKV recurrence and sigmoid gate of Appendix A.1 Eqs. 23-24,
@@ -148,6 +149,10 @@ template <int NB> struct Shape {
                 "register re-division exceeds the launch's pool");
   static_assert(kLaunchRegs * kThreads <= 65536, "register file");
 };
+// With units unpacked ahead and inputs that the CTAs mix themselves the consumers' code wants eight more, and the stagers', without a pre-pass, make do with
+// 64 (1.6B-class, twelve layers, batch 1: 180.6 us at 96 each, 179.4).
+__host__ __device__ constexpr int consumer_regs(int NB, int MIX, bool PARK) { return NB == 2 ? 152 : PARK && MIX == 0 ? 104 : 96; }
+__host__ __device__ constexpr int stager_regs(int NB, int MIX, bool PARK) { return NB == 2 ? 104 : PARK && MIX == 0 ? 64 : 96; }
 constexpr int groups_of(int NB) { return NB == 2 ? 1 : 2; }
 constexpr int threads_of(int NB) { return NB == 2 ? Shape<2>::kThreads : Shape<1>::kThreads; }
 // Slots of the weight ring: a unit for each consumer group and one on its way.  More are filled while a stage's first inputs are read, and hold those
@@ -294,6 +299,7 @@ struct Ctrl {
   uint32_t mix_at[8];        // batch row | group << 16 of the item in each stager warp's MixSlot
   int abort_flag;
   int poll_limit;            // must follow abort_flag (poll_limit_of)
+  uint32_t tmem_base;
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block");
 constexpr uint32_t kMaxBarriers = 256;   // barriers that close a stage (8-bit counts in Ctrl::stage_cnt)
@@ -1204,12 +1210,10 @@ __device__ __forceinline__ void sq_group_words(const uint8_t* rec, int lane, uin
   }
 }
 
-// A pair of VQ records.  The tile's codebook is copied 32 times for lookups without bank conflicts by the eight warps of the group, an eighth of its
+// The tile's codebook is copied 32 times for lookups without bank conflicts by the eight warps of the group, an eighth of its
 // entries each, sixteen bytes a lane and store: in steps of four bytes, one behind the other, the copies of 256 entries took a fifth of the time.
-// Bound by the lookups, 1024 of the 1750 reads and writes of shared memory that a unit takes (at batch 1 its pipe is busy 70 to 76 % of the time).
-template <int BITS, int NB>
-__device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, const uint32_t* codebook, uint8_t* rep, int w, int lane, int bar,
-                                        uint64_t* empty, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
+template <int BITS>
+__device__ __forceinline__ void copy_codebook(const uint32_t* codebook, uint8_t* rep, int w, int lane, int bar) {
   constexpr int kStores = (1 << BITS) / 32;        // of a warp, four entries each
   uint32_t entry[kStores];
 #pragma unroll
@@ -1217,9 +1221,16 @@ __device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, co
   named_bar_sync(bar, kGroupThreads);              // the group's previous lookups are done
 #pragma unroll
   for (int i = 0; i < kStores; ++i) *reinterpret_cast<uint4*>(rep + (w * kStores + i) * 512 + lane * 16) = make_uint4(entry[i], entry[i], entry[i], entry[i]);
+  named_bar_sync(bar, kGroupThreads);
+}
+// A pair of VQ records.
+// Bound by the lookups, 1024 of the 1750 reads and writes of shared memory that a unit takes (at batch 1 its pipe is busy 70 to 76 % of the time).
+template <int BITS, int NB>
+__device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, const uint32_t* codebook, uint8_t* rep, int w, int lane, int bar,
+                                        uint64_t* empty, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
+  copy_codebook<BITS>(codebook, rep, w, lane, bar);
   uint32_t va[2 * BITS], vb[2 * BITS];
   vq_half_words<BITS, 0>(ra, lane, va); vq_half_words<BITS, 0>(rb, lane, vb);
-  named_bar_sync(bar, kGroupThreads);
   const uint32_t* cb_lane = reinterpret_cast<const uint32_t*>(rep) + lane;
   // A unit's sums start at zero and are added with a rounding of their own: the tensor core's accumulation cuts off, and its error grows with the chain.
   float ca[NB][4] = {}, cb[NB][4] = {};
@@ -1232,6 +1243,197 @@ __device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, co
   for (int n = 0; n < NB; ++n)
 #pragma unroll
     for (int k = 0; k < 4; ++k) { acca[n][k] += ca[n][k]; accb[n][k] += cb[n][k]; }
+}
+
+// ---- units unpacked ahead of their inputs ---------------------------------------------------------------------------
+// A group's first unit of a stage is in shared memory long before the stage's inputs are.  While the warps would wait for these they unpack it, and what they
+// unpack waits in tensor memory, used as a larger register file: every warp reaches 32 lanes of it and has 128 columns to itself, so 128
+// registers of a lane.  Behind the inputs only the fragments' loads and the tensor-core steps are left: 1770 cycles where the whole unit took 2700
+// (1.6B-class, batch 1, both groups at work; step 418 us before, 363 with this and one instruction a row half for one batch column).  Bound by
+// the chain of a warp then: four trips to tensor memory and sixteen tensor-core steps one behind the other.
+constexpr uint32_t kTmemCols = 512, kParkCols = 128;
+__device__ __forceinline__ void park16(uint32_t at, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+               ::"r"(at), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
+__device__ __forceinline__ void park_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// The registers hold what is fetched only behind fetch_wait on them.
+__device__ __forceinline__ void fetch16(uint32_t at, uint32_t (&r)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                 "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(at) : "memory");
+}
+__device__ __forceinline__ void fetch_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void fetched(uint32_t (&r)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) asm volatile("" : "+r"(r[k]));      // no use is scheduled before the wait
+}
+
+// The three words of triple T of a lane of an SQ record.
+template <int T>
+__device__ __forceinline__ void sq_triple(const uint4& p0, const uint4& p1, const uint4& p2, uint32_t (&r)[16]) {
+  if constexpr (T == 0) sq_unpack_triple(p0.x, p0.y, p0.z, r);
+  else if constexpr (T == 1) sq_unpack_triple(p0.w, p1.x, p1.y, r);
+  else if constexpr (T == 2) sq_unpack_triple(p1.z, p1.w, p2.x, r);
+  else sq_unpack_triple(p2.y, p2.z, p2.w, r);
+}
+// Columns of a warp's share: T * 32 (+ 16: second record) for triple T.
+__device__ __forceinline__ void park_sq(uint32_t at, const uint8_t* ra, const uint8_t* rb, int lane) {
+  const uint4 a0 = *reinterpret_cast<const uint4*>(ra + lane * 16), a1 = *reinterpret_cast<const uint4*>(ra + 512 + lane * 16);
+  const uint4 a2 = *reinterpret_cast<const uint4*>(ra + 1024 + lane * 16);
+  const uint4 b0 = *reinterpret_cast<const uint4*>(rb + lane * 16), b1 = *reinterpret_cast<const uint4*>(rb + 512 + lane * 16);
+  const uint4 b2 = *reinterpret_cast<const uint4*>(rb + 1024 + lane * 16);
+  uint32_t r[16];
+  sq_triple<0>(a0, a1, a2, r); park16(at, r);
+  sq_triple<1>(a0, a1, a2, r); park16(at + 32u, r);
+  sq_triple<2>(a0, a1, a2, r); park16(at + 64u, r);
+  sq_triple<3>(a0, a1, a2, r); park16(at + 96u, r);
+  sq_triple<0>(b0, b1, b2, r); park16(at + 16u, r);
+  sq_triple<1>(b0, b1, b2, r); park16(at + 48u, r);
+  sq_triple<2>(b0, b1, b2, r); park16(at + 80u, r);
+  sq_triple<3>(b0, b1, b2, r); park16(at + 112u, r);
+  park_wait();
+}
+// The products of a parked pair of records.  While a triple's fragments are fetched (a trip of some 200 cycles) the inputs of its tensor-core steps are read
+// and the sums of the group before are scaled.
+template <int NB>
+struct Parked {
+  uint32_t a[16], b[16];
+  uint2 x[4][NB];
+  __device__ __forceinline__ void inputs(const XLane& xl, int T) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int n = 0; n < NB; ++n) x[m][n] = *reinterpret_cast<const uint2*>(xl.x[n] + (4 * T + m) * 32);
+  }
+  __device__ __forceinline__ void ready() { fetch_wait(); fetched(a); fetched(b); }
+  // the steps of triple T; triple T + 1 is asked for as soon as this one's fragments have been taken
+  template <int T>
+  __device__ __forceinline__ void steps(uint32_t at, float (&ca)[NB][4], float (&cb)[NB][4]) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const uint32_t f[4] = {a[4 * m], a[4 * m + 1], a[4 * m + 2], a[4 * m + 3]};
+#pragma unroll
+      for (int n = 0; n < NB; ++n) mma_16816(ca[n], f, x[m][n].x, x[m][n].y);
+    }
+    if constexpr (T < 3) fetch16(at + 32u * (T + 1), a);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const uint32_t f[4] = {b[4 * m], b[4 * m + 1], b[4 * m + 2], b[4 * m + 3]};
+#pragma unroll
+      for (int n = 0; n < NB; ++n) mma_16816(cb[n], f, x[m][n].x, x[m][n].y);
+    }
+    if constexpr (T < 3) fetch16(at + 32u * (T + 1) + 16u, b);
+  }
+};
+// As sq_group_mma2: the chains of a group start at -Bx_h; what they end with is scaled.
+template <int NB>
+__device__ __forceinline__ void parked_start(const XLane& xl, int grp, float (&ca)[NB][4], float (&cb)[NB][4]) {
+  const uint8_t* gsp = xl.gs + (size_t)(grp * 3) * xl.gstride;
+#pragma unroll
+  for (int n = 0; n < NB; ++n) {
+    const float2 b0 = *reinterpret_cast<const float2*>(gsp + xl.gstride + n * 32);
+    const float2 b1 = *reinterpret_cast<const float2*>(gsp + 2 * xl.gstride + n * 32);
+    ca[n][0] = cb[n][0] = -b0.x; ca[n][1] = cb[n][1] = -b0.y;
+    ca[n][2] = cb[n][2] = -b1.x; ca[n][3] = cb[n][3] = -b1.y;
+  }
+}
+template <int NB>
+__device__ __forceinline__ void parked_scale(const XLane& xl, int grp, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, const float (&ca)[NB][4],
+                                             const float (&cb)[NB][4], float (&acca)[NB][4], float (&accb)[NB][4]) {
+  const uint8_t* gsp = xl.gs + (size_t)(grp * 3) * xl.gstride;
+  const float2 sa0 = __half22float2(*reinterpret_cast<const __half2*>(&a_lo)), sa1 = __half22float2(*reinterpret_cast<const __half2*>(&a_hi));
+  const float2 sb0 = __half22float2(*reinterpret_cast<const __half2*>(&b_lo)), sb1 = __half22float2(*reinterpret_cast<const __half2*>(&b_hi));
+#pragma unroll
+  for (int n = 0; n < NB; ++n) {
+    const float2 sx = *reinterpret_cast<const float2*>(gsp + n * 32);
+    acca[n][0] = fmaf(sa0.x, fmaf(-sa0.y, sx.x, ca[n][0]), acca[n][0]);
+    acca[n][1] = fmaf(sa0.x, fmaf(-sa0.y, sx.y, ca[n][1]), acca[n][1]);
+    acca[n][2] = fmaf(sa1.x, fmaf(-sa1.y, sx.x, ca[n][2]), acca[n][2]);
+    acca[n][3] = fmaf(sa1.x, fmaf(-sa1.y, sx.y, ca[n][3]), acca[n][3]);
+    accb[n][0] = fmaf(sb0.x, fmaf(-sb0.y, sx.x, cb[n][0]), accb[n][0]);
+    accb[n][1] = fmaf(sb0.x, fmaf(-sb0.y, sx.y, cb[n][1]), accb[n][1]);
+    accb[n][2] = fmaf(sb1.x, fmaf(-sb1.y, sx.x, cb[n][2]), accb[n][2]);
+    accb[n][3] = fmaf(sb1.x, fmaf(-sb1.y, sx.y, cb[n][3]), accb[n][3]);
+  }
+}
+template <int NB>
+__device__ __forceinline__ void parked_sq(uint32_t at, const uint4 sza, const uint4 szb, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
+  Parked<NB> p;
+  float ca[NB][4], cb[NB][4];
+  fetch16(at, p.a);
+  fetch16(at + 16u, p.b);
+  parked_start<NB>(xl, 0, ca, cb);
+  p.inputs(xl, 0);
+  p.ready();
+  p.template steps<0>(at, ca, cb);
+  p.inputs(xl, 1);
+  p.ready();
+  p.template steps<1>(at, ca, cb);
+  p.inputs(xl, 2);
+  parked_scale<NB>(xl, 0, sza.x, sza.z, szb.x, szb.z, ca, cb, acca, accb);
+  parked_start<NB>(xl, 1, ca, cb);
+  p.ready();
+  p.template steps<2>(at, ca, cb);
+  p.inputs(xl, 3);
+  p.ready();
+  p.template steps<3>(at, ca, cb);
+  parked_scale<NB>(xl, 1, sza.y, sza.w, szb.y, szb.w, ca, cb, acca, accb);
+}
+template <int NB>
+__device__ __forceinline__ void parked_vq(uint32_t at, const XLane& xl, float (&acca)[NB][4], float (&accb)[NB][4]) {
+  Parked<NB> p;
+  float ca[NB][4] = {}, cb[NB][4] = {};
+  fetch16(at, p.a);
+  fetch16(at + 16u, p.b);
+  p.inputs(xl, 0);
+  p.ready();
+  p.template steps<0>(at, ca, cb);
+  p.inputs(xl, 1);
+  p.ready();
+  p.template steps<1>(at, ca, cb);
+  p.inputs(xl, 2);
+  p.ready();
+  p.template steps<2>(at, ca, cb);
+  p.inputs(xl, 3);
+  p.ready();
+  p.template steps<3>(at, ca, cb);
+#pragma unroll
+  for (int n = 0; n < NB; ++n)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { acca[n][k] += ca[n][k]; accb[n][k] += cb[n][k]; }
+}
+template <int BITS, int T>
+__device__ __forceinline__ void vq_triple(const uint32_t (&w)[2 * BITS], uint32_t base, uint32_t (&r)[16]) {
+#pragma unroll
+  for (int e = 0; e < 16; ++e) r[e] = vq_entry<BITS, 2 * BITS>(w, 16 * T + e, base);
+}
+template <int BITS>
+__device__ __forceinline__ void vq_words(const uint8_t* rec, int lane, uint32_t (&w)[2 * BITS]) {
+#pragma unroll
+  for (int p = 0; p < BITS / 2; ++p) {
+    const uint4 v = *reinterpret_cast<const uint4*>(rec + p * 512 + lane * 16);
+    w[4 * p] = v.x; w[4 * p + 1] = v.y; w[4 * p + 2] = v.z; w[4 * p + 3] = v.w;
+  }
+}
+template <int BITS>
+__device__ __forceinline__ void park_vq(uint32_t at, const uint8_t* ra, const uint8_t* rb, const uint32_t* codebook, uint8_t* rep, int w, int lane, int bar) {
+  copy_codebook<BITS>(codebook, rep, w, lane, bar);
+  const uint32_t base = smem_u32(rep) + (uint32_t)lane * 4u;
+  uint32_t v[2 * BITS], r[16];
+  vq_words<BITS>(ra, lane, v);
+  vq_triple<BITS, 0>(v, base, r); park16(at, r);
+  vq_triple<BITS, 1>(v, base, r); park16(at + 32u, r);
+  vq_triple<BITS, 2>(v, base, r); park16(at + 64u, r);
+  vq_triple<BITS, 3>(v, base, r); park16(at + 96u, r);
+  vq_words<BITS>(rb, lane, v);
+  vq_triple<BITS, 0>(v, base, r); park16(at + 16u, r);
+  vq_triple<BITS, 1>(v, base, r); park16(at + 48u, r);
+  vq_triple<BITS, 2>(v, base, r); park16(at + 80u, r);
+  vq_triple<BITS, 3>(v, base, r); park16(at + 112u, r);
+  park_wait();
 }
 
 // c[k] of the four lanes whose row index g differs in its two low bits (lanes 4 apart) -> lane i (= g & 3)
@@ -1248,12 +1450,13 @@ __device__ __forceinline__ void transpose4_lanes(float (&c)[4], int i) {
   c[0] = lo ? p0 : a00;  c[1] = lo ? a01 : p0;
   c[2] = lo ? p1 : a10;  c[3] = lo ? a11 : p1;
 }
+__device__ __forceinline__ void red_add(float* p, float v) { asm volatile("red.global.add.f32 [%0], %1;" :: "l"(p), "f"(v) : "memory"); }
 __device__ __forceinline__ void red_add_v4(float* p, const float (&v)[4]) {
   asm volatile("red.global.v4.f32.add [%0], {%1, %2, %3, %4};" :: "l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
 }
 
 // Consumer warp `w` of group `grp`: units grp, grp + 2, ... of the CTA's list.
-template <int NB, int MIX>
+template <int NB, int MIX, bool PARK>
 __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, const uint8_t* xbufs, uint8_t* replicas,
                               uint32_t unit_base, uint32_t n_units, uint32_t ev_base, uint32_t n_events) {
   bool dead = false;
@@ -1324,15 +1527,42 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     }
   };
   uint8_t* rep = replicas + (size_t)grp * a.replica_bytes;
+  // Tensor memory is the consumer warps' alone: the other roles neither wait for it nor for its return.
+  if constexpr (PARK) {
+    if (warp == 0) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctrl->tmem_base)), "n"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    named_bar_sync(3, Shape<NB>::kConsumerThreads);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  // the warp's share of tensor memory, looked up where it is used: lanes 32 (warp mod 4) and on
+  auto park_at = [&]() { return *(volatile uint32_t*)&ctrl->tmem_base + ((threadIdx.x & 0x60u) << 16) + (threadIdx.x >> 7) * kParkCols; };
   // slot and round of unit i (i % n_slots, i / n_slots), advanced without dividing
   const uint32_t n_slots_u = (uint32_t)a.n_slots;
   uint32_t slot_u = (uint32_t)grp % n_slots_u, round = (uint32_t)grp / n_slots_u;
+  bool fresh = true;          // the unit is the group's first of a stage
   for (uint32_t i = (uint32_t)grp; i < n_units; i += kGroups, slot_u += kGroups) {
     while (slot_u >= n_slots_u) { slot_u -= n_slots_u; ++round; }
     const int slot = (int)slot_u;
     const uint8_t* sl = smem + kCtrlBytes + (size_t)slot * a.slot_bytes;
     const StepUnit* u = reinterpret_cast<const StepUnit*>(sl);
     if (!dead && !mbar_wait_warp(&ctrl->full[grp][slot], slot_uses<NB>(round, n_slots_u) & 1u, abortp, a.status)) dead = true;
+    const bool ahead = PARK && fresh && !dead;
+    if constexpr (PARK) {
+      if (ahead) {
+        const uint32_t park = park_at();
+        const uint32_t f = u->flags, chb = u->chunk_bytes, rb = u->rec_bytes;
+        const uint8_t* data = sl + 128;
+        const uint8_t* ra = data + (size_t)w * rb;
+        const uint8_t* rbp = u->bytes1 ? ra + chb : ra;      // no second record: the first one again, whose results are dropped
+        const uint32_t* cbraw = reinterpret_cast<const uint32_t*>(data + 2 * chb);
+        if (!(f & UF_VQ)) park_sq(park, ra, rbp, lane);
+        else if (f & UF_BITS8) park_vq<8>(park, ra, rbp, cbraw, rep, w, lane, 1 + grp);
+        else park_vq<6>(park, ra, rbp, cbraw, rep, w, lane, 1 + grp);
+      }
+    }
     if (!dead && u->ev_index != cur_ev) {
       const uint32_t target = u->ev_index;
       pass_events(target, u->between_mask, target - cur_ev - 1u <= 32u);
@@ -1347,7 +1577,7 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     if (dead) {
       // A warp that gave up keeps walking the list only to keep the group's named barriers whole
       // (the other warps stop at their next bounded wait); it touches neither slots nor outputs.
-      if (a.units[unit_base + i].flags & UF_VQ) { named_bar_sync(1 + grp, kGroupThreads); named_bar_sync(1 + grp, kGroupThreads); }
+      if (!ahead && (a.units[unit_base + i].flags & UF_VQ)) { named_bar_sync(1 + grp, kGroupThreads); named_bar_sync(1 + grp, kGroupThreads); }
       continue;
     }
     const uint32_t flags = u->flags;
@@ -1361,7 +1591,20 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     float* y = reinterpret_cast<float*>(u->y);
     const uint8_t* ra = data + (size_t)w * rb;
     const uint8_t* rbp = data + chb + (size_t)w * rb;
-    if (!(flags & UF_VQ)) {
+    if (ahead) {
+      const uint32_t park = park_at();
+      const uint32_t col = u->xcol0;
+      const XLane xl = make_xlane(xb + (size_t)col * 2, xstride,
+                                  reinterpret_cast<const float*>(xb + u->gs_off) + (size_t)(col >> 7) * 3 * nbp, nbp, a.B, lane);
+      const uint4 sza = *reinterpret_cast<const uint4*>(ra + RWKVQ_SQ_CODE_BYTES + g * 16);
+      const uint4 szb = *reinterpret_cast<const uint4*>((has_b ? rbp : ra) + RWKVQ_SQ_CODE_BYTES + g * 16);
+      // Not before the inputs are there: a slot handed back at once was filled while they were being read, and held them up (1.6B-class, batch 1: 366 us, 363
+      // so; 7B-class 1225, 1181).
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctrl->empty[slot]);
+      if (flags & UF_VQ) parked_vq<NB>(park, xl, acca, accb);
+      else parked_sq<NB>(park, sza, szb, xl, acca, accb);
+    } else if (!(flags & UF_VQ)) {
       const uint32_t col = u->xcol0;
       const XLane xl = make_xlane(xb + (size_t)col * 2, xstride,
                                   reinterpret_cast<const float*>(xb + u->gs_off) + (size_t)(col >> 7) * 3 * nbp, nbp, a.B, lane);
@@ -1405,7 +1648,14 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         vq_unit<6, NB>(ra, rbp, cbraw, rep, w, lane, 1 + grp, &ctrl->empty[slot], xl, acca, accb);
     }
     if (flags & UF_FLUSH) {
-      {
+      if (NB == 1 && a.B == 1) {
+        // One batch column: the lanes t = 0 hold it, eight consecutive rows an instruction.  The transpose below would move three times as much that nobody
+        // takes, at the end of the chain that the next stage waits for (eight layers, d 512 107.0 -> 104.0 us, d 4096 289.6 -> 285.1).
+        const uint32_t r = row0 + (uint32_t)w * 16u;
+        float* p = y + r + (uint32_t)g;
+        if (t == 0 && r < oc) { red_add(p, acca[0][0]); red_add(p + 8, acca[0][2]); }
+        if (has_b && t == 0 && r + 128u < oc) { red_add(p + 128, accb[0][0]); red_add(p + 136, accb[0][2]); }
+      } else {
         // Four lanes that share t hold a 4 x 4 block (rows 4J .. 4J+3 of one row half x the accumulator's four
         // elements): transposed, every lane owns four consecutive rows of ONE batch column and adds them
         // with a single 16-byte reduction instead of four scattered ones.  The plan accepts only outputs
@@ -1431,11 +1681,17 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         for (int k = 0; k < 4; ++k) acca[n][k] = accb[n][k] = 0.f;
     }
     // the group's last unit of the stage: report the stage as finished without waiting for the next unit
-    if (after_count) pass_events(cur_ev + after_count + 1u, after_mask, true);
+    fresh = after_count != 0u;
+    if (fresh) pass_events(cur_ev + after_count + 1u, after_mask, true);
   }
   if (!dead) {
     release_held();
     pass_events(n_events, 0u, false);     // the rest of the list: later stages this warp has no unit in
+  }
+  if constexpr (PARK) {      // all waits above are bounded, so all consumer warps arrive here
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    named_bar_sync(3, Shape<NB>::kConsumerThreads);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(ctrl->tmem_base), "n"(kTmemCols) : "memory");
   }
 }
 
@@ -1445,7 +1701,7 @@ __global__ void __launch_bounds__(256) reciprocal_kernel(const float* y, float* 
   if (i < n) out[i] = rcp_of(y[i]);
 }
 
-template <int NB, int MIX>
+template <int NB, int MIX, bool PARK>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const StepArgs a) {
   constexpr int kConsumerWarps = Shape<NB>::kConsumerWarps, kStagerWarps = Shape<NB>::kStagerWarps;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -1470,12 +1726,12 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   // in registers.  With one block the shares are those of the launch and nothing moves; the instruction stays for the code the compiler makes of the
   // roles beside it (without it: 1.6B-class B=1 428.3 -> 429.9 us, 7B-class B=1 1209.9 -> 1207.5).
   if (warp < kConsumerWarps) {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kConsumerRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(consumer_regs(NB, MIX, PARK)));
   } else {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(Shape<NB>::kStagerRegs));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(stager_regs(NB, MIX, PARK)));
   }
   if (warp < kConsumerWarps) {
-    consumer_role<NB, MIX>(a, smem, ctrl, xbufs, replicas, u0, u1 - u0, e0, e1 - e0);
+    consumer_role<NB, MIX, PARK>(a, smem, ctrl, xbufs, replicas, u0, u1 - u0, e0, e1 - e0);
   } else if (warp < kConsumerWarps + kStagerWarps) {
     stager_role<MIX, NB>(a, smem, ctrl, xbufs, mucb, e0, e1);
   } else {
@@ -1487,6 +1743,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
 
 struct PlanInfo {
   int P, B, NB, n_slots, n_stages, mix;
+  bool park;            // units unpacked ahead of their inputs
   unsigned runs;        // launches since the counters were last zero
   unsigned abort_epoch; // value of the abort epoch when the counters were last known good
   bool captured;        // some run is part of a graph, which may be launched at any time
@@ -1673,6 +1930,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     squares[s] = all && !read_first[s] && (n + (uint64_t)P - 1) / (uint64_t)P * 256u * (uint64_t)B <= kSquaresShare;
   }
 
+  size_t deepest = 0;      // units of the CTA that has most, over all stages
   std::vector<std::vector<HostUnit>> cta_units(P);
   std::vector<std::vector<StepEvent>> cta_arrivals(P);      // arrival events, one per barrier
   bool too_many_ranges = false;
@@ -1836,6 +2094,9 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
         if (fits) deal.swap(by_row);
       }
     }
+    size_t most = 0;
+    for (const auto& d : deal) most = std::max(most, d.second);
+    deepest += most;
     // start at a CTA that moves with the stage, so that idle CTAs are not always the same SMs
     size_t c = ((size_t)s * 37u) % (size_t)P;
     for (const auto& d : deal) {
@@ -1844,6 +2105,12 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     }
     for (int c = 0; c < P; ++c) make_arrival(c, s + 1, s + 1);
   }
+  // Units unpacked ahead of their inputs (consumer_role): they take about 1000 of the 2700 cycles of a group's first unit out of a stage's chain, and a launch takes
+  // 3 us longer.  It gains where most groups have one unit a stage.  Eight layers (d 2048: twelve), without / with, us, at `units of the CTA that has
+  // most, mean over the stages`: batch 1, d 512, 1, 104.5 / 98.5; d 1536, 1.25, 118.6 / 112.8; d 2048, 1.75, 203.4 / 179.4; d 2304, 2.25, 149.6 / 147.3;
+  // d 2560, 2.75, 172.2 / 176.4; d 3072, 3.75, 199.0 / 199.0; d 4096, 6, 284.0 / 287.1; batch 2, d 2048, 149.7 / 139.4; batch 8, d 2048, 212.0 / 200.7,
+  // d 4096, 336.4 / 343.7.  Above eight rows two warps a scheduler do not hide the trips to tensor memory (14B-class stack, batch 16: 3330 / 3554).
+  info->park = B <= 8 && 4 * deepest <= 9 * (size_t)n_stages;
   if (too_many_ranges) return RWKVQ_EUNSUPPORTED;   // a CTA's slice of a stage's outputs may touch at most three products
 
   // pre-pass outputs: one region, reused by every stage (a stage's pre-pass starts only after the
@@ -2138,9 +2405,10 @@ rwkvq_status launch_run(const void* plan_dev, const PlanInfo& info, cudaStream_t
   a.poll_limit = info.poll_limit; a.wait_skew = info.wait_skew;
   a.in_flag = nullptr; a.in_base = 0; a.in_shift = 0; a.in_lo = 0; a.in_hi = 0;
   if (hr) { a.in_flag = hr->in_flag; a.in_base = hr->in_base; a.in_shift = hr->in_shift; a.in_lo = hr->in_lo; a.in_hi = hr->in_hi; }
-  static const void* const kernels[2][3] = {{(const void*)step_kernel<1, 0>, (const void*)step_kernel<1, 1>, (const void*)step_kernel<1, 2>},
-                                            {(const void*)step_kernel<2, 0>, (const void*)step_kernel<2, 1>, (const void*)step_kernel<2, 2>}};
-  const void* fn = kernels[info.NB - 1][info.mix];
+  static const void* const kernels[3][3] = {{(const void*)step_kernel<1, 0, false>, (const void*)step_kernel<1, 1, false>, (const void*)step_kernel<1, 2, false>},
+                                            {(const void*)step_kernel<2, 0, false>, (const void*)step_kernel<2, 1, false>, (const void*)step_kernel<2, 2, false>},
+                                            {(const void*)step_kernel<1, 0, true>, (const void*)step_kernel<1, 1, true>, (const void*)step_kernel<1, 2, true>}};
+  const void* fn = kernels[info.park ? 2 : info.NB - 1][info.mix];
   void* params[] = {&a};
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
   // Cooperative launch: all CTAs must be resident at once because they meet at the stage barrier.

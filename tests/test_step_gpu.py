@@ -510,3 +510,35 @@ def test_outputs_that_are_inputs_of_the_stage_before(kind, Bn):
     for got in chain(False):
         for a, b in zip(got, want):      # sums in another order; an input may round to the other fp16 number (2^-11)
             assert float((a.double() - b.double()).norm()) <= 1e-3 * float(b.double().norm())
+
+
+@pytest.mark.parametrize("Bn,bits", [(1, 3), (1, 6), (2, 8), (3, 6), (8, 3), (8, 8)])
+@pytest.mark.parametrize("rows", [(16, 32, 37, 32), (16, 37, 48)])
+def test_units_unpacked_ahead_of_their_inputs(rows, Bn, bits):
+    """Stages of one, two and three units a CTA (rows of nine tiles on 148 SMs): plans of small stages unpack a group's first unit of a stage while its
+    inputs are on their way, and go on to the next as before; plans of larger ones do not.  Scalar rows end in half a unit.  Inputs and decoded weights are exact,
+    so that only the fp32 sums differ (1e-5 of |w| |x|)."""
+    ic, g = 2304, torch.Generator(device="cuda").manual_seed(10 * Bn + bits)
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    keep = []
+    for stage, r in enumerate(rows):
+        oc = 256 * r - (112 if bits == 3 else 0)
+        desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ if bits == 3 else B.RWKVQ_VQ, bits)
+        image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+        w = (torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half()
+        B.rwkvq_quantize_dev_async(w, oc, ic, desc.method, bits, image, ws, kmeans_iters=0, seed=1)
+        keep.append(dict(desc=desc, W=image, mu_desc=None, mu=None, x=torch.randn((Bn, ic), generator=g, device="cuda").half(), xprev=None,
+                         y=torch.full((Bn, oc), float("nan"), device="cuda"), stage=stage))
+    ops = B.make_ops(keep)
+    plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
+    B.rwkvq_step_plan(ops, Bn, plan)
+    for _ in range(2):
+        B.rwkvq_step_run(plan)
+    for e in keep:
+        decoded = torch.empty((e["desc"].oc, ic), device="cuda")
+        B.rwkvq_dequant(e["desc"], e["W"], decoded)
+        x = e["x"].double()
+        bound = 1e-5 * x.norm(dim=1)[:, None] * decoded.double().norm(dim=1)[None]
+        assert bool(((e["y"].double() - x @ decoded.double().T).abs() <= bound).all()), e["stage"]
+    assert B.rwkvq_device_status() == 0
+    B.rwkvq_step_plan_release(plan)
