@@ -52,7 +52,8 @@ namespace rwkvq {
 int* device_status_ptr();  // api_misc.cu
 unsigned abort_epoch();     // api_misc.cu: bumped whenever rwkvq_device_status reports a failed wait
 
-enum { UF_FLUSH = 1, UF_VQ = 2, UF_BITS8 = 4 };
+// UF_HEAD: reads the head of its segment, announced by itself (UF_PHASE: in the barrier's second phase); UF_REST: its group's first unit behind the head.
+enum { UF_FLUSH = 1, UF_VQ = 2, UF_BITS8 = 4, UF_HEAD = 8, UF_REST = 16, UF_PHASE = 32 };
 
 struct StepUnit {            // 128 bytes, copied into the slot header by the producer
   uint64_t src0, src1;       // global addresses of chunk A / chunk B (0 = absent)
@@ -103,7 +104,8 @@ struct StepEvent {           // 64 bytes
 };
 // EF_SQUARES: of a stage whose inputs every CTA squares for itself (see kSquaresShare); arrival: the stage that begins.  EF_READ_FIRST: arrival; the
 // outputs to clear are inputs of the stage that ends, which every CTA has read when that stage's second barrier opens.
-enum { EF_SQUARES = 1, EF_READ_FIRST = 2 };
+// EF_HEAD: segment; its first kHeadTiles tiles are announced ahead of the rest.
+enum { EF_SQUARES = 1, EF_READ_FIRST = 2, EF_HEAD = 4 };
 static_assert(sizeof(StepEvent) == 64, "event descriptor size");
 
 // One product's share of a stage's pre-pass: where its inputs are and where x_mix (fp16 rows of
@@ -167,6 +169,8 @@ constexpr uint32_t kCtrlBytes = 1024, kMuScratch = 1024;
 // 30 KB 1350; a size that the plan chooses costs more, 1.6B-class batch 1 414.7 -> 417.3, 14B-class batch 16 3332 -> 3352).
 constexpr uint32_t xbuf_bytes_of(int NB) { return NB == 2 ? 63488u : 31488u; }
 template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u, kBytes = xbuf_bytes_of(NB); };
+// Tiles at the head of a stage's first segment: one for each of two consumer groups' first units.
+constexpr int kHeadTiles = 2;
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
 constexpr uint32_t kDefaultPollLimit = 1u << 22;
 
@@ -290,7 +294,7 @@ __device__ __forceinline__ uint32_t smem_add_acq_rel(uint32_t* p, uint32_t v) {
 // looks like the one the group waits for (waits see the parity of a phase, not its number).
 struct Ctrl {
   uint64_t full[2][kMaxSlots], empty[kMaxSlots];
-  uint64_t xfull[4], xempty[4];
+  uint64_t xfull[4], xempty[4], xhead[2];
   uint32_t stage_cnt[64];    // one 8-bit count per grid barrier (four per word): how many of the parties
                              // of this CTA (every consumer warp, and the stagers as one) have reported the
                              // stage that the barrier closes.  Per barrier, not one running total: consumer
@@ -966,7 +970,7 @@ __device__ __forceinline__ void stage_squares(const StepArgs& a, const StepEvent
 //    shared memory BEFORE the stage barrier, so that only one round of vector loads of x, the
 //    mix and the sums remain behind it.  A thread owns 8 consecutive columns (16 bytes) of one
 //    batch row; a half-warp owns one 128-column group, whose three sums it reduces with shuffles.
-template <int MIX, int NB>
+template <int MIX, int NB, bool HEAD>
 __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_t* xbufs, uint32_t* mucb,
                             uint32_t e0, uint32_t e1) {
   constexpr int kStagerThreads = Shape<NB>::kStagerThreads;
@@ -1183,6 +1187,11 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
           }
           *reinterpret_cast<uint4*>(dst) = r;
           if (sums) segment_sums(gs, r, c8, b, nbp, lane);
+          if (HEAD && u == 0 && (ev.flags & EF_HEAD) && v0 == stid) {      // one row: the threads' first vectors hold the head
+            static_assert(kStagerThreads >= 32 * kHeadTiles, "head of a segment");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctrl->xhead[buf]);
+          }
         }
       }
     }
@@ -1456,9 +1465,10 @@ __device__ __forceinline__ void red_add_v4(float* p, const float (&v)[4]) {
 }
 
 // Consumer warp `w` of group `grp`: units grp, grp + 2, ... of the CTA's list.
-template <int NB, int MIX, bool PARK>
+template <int NB, int MIX, bool PARK, bool ONE>
 __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, const uint8_t* xbufs, uint8_t* replicas,
                               uint32_t unit_base, uint32_t n_units, uint32_t ev_base, uint32_t n_events) {
+  constexpr bool HEAD = ONE && !PARK;
   bool dead = false;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kGroups = Shape<NB>::kGroups;
@@ -1571,8 +1581,15 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         const uint32_t q = seg_next++;
         held = (int)q;
         cur_ev = target;
-        if (!mbar_wait_warp(&ctrl->xfull[q % XBufs<MIX, NB>::kCount], (q / XBufs<MIX, NB>::kCount) & 1u, abortp, a.status)) dead = true;
+        if constexpr (HEAD) {
+          const uint32_t f = u->flags, buf = q % XBufs<MIX, NB>::kCount;
+          if (!mbar_wait_warp(f & UF_HEAD ? &ctrl->xhead[buf] : &ctrl->xfull[buf], f & UF_HEAD ? (f & UF_PHASE ? 1u : 0u) : (q / XBufs<MIX, NB>::kCount) & 1u, abortp, a.status)) dead = true;
+        } else if (!mbar_wait_warp(&ctrl->xfull[q % XBufs<MIX, NB>::kCount], (q / XBufs<MIX, NB>::kCount) & 1u, abortp, a.status)) {
+          dead = true;
+        }
       }
+    } else if (HEAD && !dead && (u->flags & UF_REST)) {
+      if (!mbar_wait_warp(&ctrl->xfull[(uint32_t)held % XBufs<MIX, NB>::kCount], ((uint32_t)held / XBufs<MIX, NB>::kCount) & 1u, abortp, a.status)) dead = true;
     }
     if (dead) {
       // A warp that gave up keeps walking the list only to keep the group's named barriers whole
@@ -1648,7 +1665,7 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         vq_unit<6, NB>(ra, rbp, cbraw, rep, w, lane, 1 + grp, &ctrl->empty[slot], xl, acca, accb);
     }
     if (flags & UF_FLUSH) {
-      if (NB == 1 && a.B == 1) {
+      if (ONE || (NB == 1 && MIX != 0 && a.B == 1)) {
         // One batch column: the lanes t = 0 hold it, eight consecutive rows an instruction.  The transpose below would move three times as much that nobody
         // takes, at the end of the chain that the next stage waits for (eight layers, d 512 107.0 -> 104.0 us, d 4096 289.6 -> 285.1).
         const uint32_t r = row0 + (uint32_t)w * 16u;
@@ -1701,7 +1718,8 @@ __global__ void __launch_bounds__(256) reciprocal_kernel(const float* y, float* 
   if (i < n) out[i] = rcp_of(y[i]);
 }
 
-template <int NB, int MIX, bool PARK>
+// ONE: one batch row, mixed by the CTAs that read it.
+template <int NB, int MIX, bool PARK, bool ONE = false>
 __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const StepArgs a) {
   constexpr int kConsumerWarps = Shape<NB>::kConsumerWarps, kStagerWarps = Shape<NB>::kStagerWarps;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -1712,6 +1730,7 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.n_slots; ++s) { mbar_init(&ctrl->full[0][s], 1); mbar_init(&ctrl->full[1][s], 1); mbar_init(&ctrl->empty[s], kGroupWarps); }
     for (int b = 0; b < 4; ++b) { mbar_init(&ctrl->xfull[b], kStagerWarps); mbar_init(&ctrl->xempty[b], kConsumerWarps); }
+    for (int b = 0; b < 2; ++b) mbar_init(&ctrl->xhead[b], kStagerWarps);
     for (int k = 0; k < 64; ++k) ctrl->stage_cnt[k] = 0u;
     ctrl->abort_flag = 0;
     ctrl->poll_limit = (int)a.poll_limit;
@@ -1731,9 +1750,9 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(stager_regs(NB, MIX, PARK)));
   }
   if (warp < kConsumerWarps) {
-    consumer_role<NB, MIX, PARK>(a, smem, ctrl, xbufs, replicas, u0, u1 - u0, e0, e1 - e0);
+    consumer_role<NB, MIX, PARK, ONE>(a, smem, ctrl, xbufs, replicas, u0, u1 - u0, e0, e1 - e0);
   } else if (warp < kConsumerWarps + kStagerWarps) {
-    stager_role<MIX, NB>(a, smem, ctrl, xbufs, mucb, e0, e1);
+    stager_role<MIX, NB, ONE && !PARK>(a, smem, ctrl, xbufs, mucb, e0, e1);
   } else {
     producer_role<NB>(a, smem, ctrl, u0, u1);
   }
@@ -2175,10 +2194,11 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
       if (!same_run) L[i].u.flags |= UF_FLUSH;
     }
     all_events.push_back(cta_arrivals[c][0]);
-    uint32_t seg_no = 0;
+    uint32_t seg_no = 0, heads[2] = {0, 0};
     size_t i = 0;
     for (int s = 0; s < n_stages; ++s) {
       // segments: maximal runs of units of one product whose column span fits the buffer
+      bool first_of_stage = true;
       while (i < n && L[i].stage == s) {
         const int op = L[i].op;
         const bool sums = ops[op].W_desc.method == RWKVQ_SQ;
@@ -2225,6 +2245,21 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           L[k].u.xcol0 = (uint32_t)(L[k].kt - kmin) * 256u;
           L[k].u.xstride = xstride; L[k].u.gs_off = (uint32_t)B * xstride; L[k].u.nbp = nbp;
         }
+        // One row that the CTA mixes itself, large stages: the head of a stage's first segment, the tiles of its groups' first units, is announced by itself
+        // where at least as many follow, and the rest is mixed while those are at work.  Eight layers, batch 1, without / with, us: d 3072 202.9 / 198.9, d 3584
+        // 246.6 / 239.7, d 4096 287.3 / 274.8.  (Copies of the pre-pass's results gain nothing by it, and what a unit's question for its barrier costs is
+        // lost: batch 8, d 4096, 334 / 338; batch 16 445 / 455.  As a segment of its own the head cost more than it gave: batch 1, d 4096, 304.)
+        bool in_order = first_of_stage && !mix && B == 1 && !info->park && kmax - kmin >= 2 * kHeadTiles && last + 1 - i >= 2 * (size_t)kHeadTiles;
+        for (int k = 0; k < kHeadTiles && in_order; ++k) in_order = L[i + k].kt == kmin + k;
+        if (in_order) {
+          ev.flags |= EF_HEAD;
+          const uint32_t phase = heads[seg_no & 1u]++ & 1u;
+          for (int k = 0; k < kHeadTiles; ++k) {
+            L[i + k].u.flags |= UF_HEAD | (phase ? UF_PHASE : 0u);
+            L[i + kHeadTiles + k].u.flags |= UF_REST;      // every group waits for either
+          }
+        }
+        first_of_stage = false;
         all_events.push_back(ev);
         ++seg_no;
         i = last + 1;
@@ -2408,7 +2443,8 @@ rwkvq_status launch_run(const void* plan_dev, const PlanInfo& info, cudaStream_t
   static const void* const kernels[3][3] = {{(const void*)step_kernel<1, 0, false>, (const void*)step_kernel<1, 1, false>, (const void*)step_kernel<1, 2, false>},
                                             {(const void*)step_kernel<2, 0, false>, (const void*)step_kernel<2, 1, false>, (const void*)step_kernel<2, 2, false>},
                                             {(const void*)step_kernel<1, 0, true>, (const void*)step_kernel<1, 1, true>, (const void*)step_kernel<1, 2, true>}};
-  const void* fn = kernels[info.park ? 2 : info.NB - 1][info.mix];
+  static const void* const one_row[2] = {(const void*)step_kernel<1, 0, false, true>, (const void*)step_kernel<1, 0, true, true>};
+  const void* fn = info.B == 1 && info.mix == 0 ? one_row[info.park] : kernels[info.park ? 2 : info.NB - 1][info.mix];
   void* params[] = {&a};
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)info.smem_bytes);
   // Cooperative launch: all CTAs must be resident at once because they meet at the stage barrier.

@@ -513,11 +513,11 @@ def test_outputs_that_are_inputs_of_the_stage_before(kind, Bn):
 
 
 @pytest.mark.parametrize("Bn,bits", [(1, 3), (1, 6), (2, 8), (3, 6), (8, 3), (8, 8)])
-@pytest.mark.parametrize("rows", [(16, 32, 37, 32), (16, 37, 48)])
+@pytest.mark.parametrize("rows", [(16, 32, 37, 32), (16, 37, 48), (80, 75, 96, 80)])
 def test_units_unpacked_ahead_of_their_inputs(rows, Bn, bits):
-    """Stages of one, two and three units a CTA (rows of nine tiles on 148 SMs): plans of small stages unpack a group's first unit of a stage while its
-    inputs are on their way, and go on to the next as before; plans of larger ones do not.  Scalar rows end in half a unit.  Inputs and decoded weights are exact,
-    so that only the fp32 sums differ (1e-5 of |w| |x|)."""
+    """Stages of one to six units a CTA (rows of nine tiles on 148 SMs): plans of small stages unpack a group's first unit of a stage while its
+    inputs are on their way, and go on to the next as before; plans of larger ones do not, and with one row their stages' first inputs are announced ahead of
+    the rest.  Scalar rows end in half a unit.  Inputs and decoded weights are exact, so that only the fp32 sums differ (1e-5 of |w| |x|)."""
     ic, g = 2304, torch.Generator(device="cuda").manual_seed(10 * Bn + bits)
     ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
     keep = []
