@@ -1916,12 +1916,12 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     any_read_first = any_read_first || read_first[s];
   }
   // A stage pre-pass (StepArgs::mix) costs a second barrier, about 2 us per stage whatever the sizes; without it every CTA mixes the
-  // columns it reads itself.  The line was measured with stacks of 1024 to 4096 columns and batches of 2 to 16 (pre-pass / without, us, at
-  // `share / stages` inputs): B=6, 2688, 319 / 286 and B=3, 2688, 262 / 250; B=2, 3072, 335 / 341; B=8, 3584, 328 / 339; B=3, 4608, 338 / 370;
-  // with seven stager warps B=10, 4480, 385 / 377; B=16, 5120, 353 / 335; B=16, 7168, 406 / 443; B=12, 8448, 305 / 346.  The
-  // element-wise operators exist in the pre-pass only.
+  // columns it reads itself.  The line was measured with stacks of eight layers, 1024 to 4096 columns (pre-pass / without, us, at
+  // `share / stages` inputs): B=6, 1920, 172 / 146; B=3, 2112, 214 / 200; B=5, 2240, 184 / 178; B=2, 2432, 269 / 276; B=8, 2560, 174 / 170; B=6, 2688, 185 / 184;
+  // B=4, 2816, 217 / 226; B=2, 3072, 299 / 331; B=8, 3584, 190 / 222; with seven stager warps B=10, 4480, 232 / 224; B=16, 5120, 213 / 214; B=12, 5376,
+  // 235 / 240; B=9, 6336, 269 / 289.  The element-wise operators exist in the pre-pass only.
   if ((any_xform || any_read_first) && n_ops > 65535) return RWKVQ_EUNSUPPORTED;      // the events count products in 16 bits
-  const bool mix = any_xform || any_read_first || (n_ops <= 65535 && share > stages * (B > 8 ? 5600u : 3000u));
+  const bool mix = any_xform || any_read_first || (n_ops <= 65535 && share > stages * (B > 8 ? 5200u : 2700u));
   // In 64ths of an SQ unit: what a further row of tiles (flush, input segment) costs a CTA, and an odd number of units where two consumer groups
   // take them in turn.  A segment that the CTA mixes itself weighs more.
   const uint64_t kRunCost = mix ? 16u : 64u, kOddCost = 32u;
@@ -2127,10 +2127,11 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   }
   // Units unpacked ahead of their inputs (consumer_role): they take about 1000 of the 2700 cycles of a group's first unit out of a stage's chain, and a launch takes
   // 3 us longer.  It gains where most groups have one unit a stage.  Eight layers (d 2048: twelve), without / with, us, at `units of the CTA that has
-  // most, mean over the stages`: batch 1, d 512, 1, 104.5 / 98.5; d 1536, 1.25, 118.6 / 112.8; d 2048, 1.75, 203.4 / 179.4; d 2304, 2.25, 149.6 / 147.3;
+  // most, mean over the stages`: batch 1, d 512, 1, 104.5 / 98.5; d 1536, 1.25, 118.6 / 112.8; d 2048, 1.75, 203.4 / 179.4; d 2304, 2.25, 149.6 / 147.3, but
+  // batch 4, d 2176, 2.25, twelve layers, 283.6 / 287.9;
   // d 2560, 2.75, 172.2 / 176.4; d 3072, 3.75, 199.0 / 199.0; d 4096, 6, 284.0 / 287.1; batch 2, d 2048, 149.7 / 139.4; batch 8, d 2048, 212.0 / 200.7,
   // d 4096, 336.4 / 343.7.  Above eight rows two warps a scheduler do not hide the trips to tensor memory (14B-class stack, batch 16: 3330 / 3554).
-  info->park = B <= 8 && 4 * deepest <= 9 * (size_t)n_stages;
+  info->park = B <= 8 && deepest <= 2 * (size_t)n_stages;
   if (too_many_ranges) return RWKVQ_EUNSUPPORTED;   // a CTA's slice of a stage's outputs may touch at most three products
 
   // pre-pass outputs: one region, reused by every stage (a stage's pre-pass starts only after the
