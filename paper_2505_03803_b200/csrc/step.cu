@@ -1666,13 +1666,22 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
         vq_unit<6, NB>(ra, rbp, cbraw, rep, w, lane, 1 + grp, &ctrl->empty[slot], xl, acca, accb);
     }
     if (flags & UF_FLUSH) {
-      if (ONE || (NB == 1 && MIX != 0 && a.B == 1)) {
-        // One batch column: the lanes t = 0 hold it, eight consecutive rows an instruction.  The transpose below would move three times as much that nobody
-        // takes, at the end of the chain that the next stage waits for (eight layers, d 512 107.0 -> 104.0 us, d 4096 289.6 -> 285.1).
+      if (ONE || (NB == 1 && (PARK || (MIX != 0 && a.B == 1)))) {
+        // Eight consecutive rows of up to four batch columns an instruction, straight from the accumulators.  With one column the transpose below would move
+        // three times as much that nobody takes, and at the end of a small stage it is a part of the chain that the next one waits for (eight layers, d 512, batch 1
+        // 107.0 -> 104.0 us; d 4096 289.6 -> 285.1; with units unpacked ahead: d 1024, batch 8 142.5 -> 140.1; blocks of d 512, batch 4 90.3 -> 88.3).  Large stages of
+        // more columns gain by the fewer instructions of the other form (d 4096, batch 8 324.0, 322.1).
         const uint32_t r = row0 + (uint32_t)w * 16u;
-        float* p = y + r + (uint32_t)g;
-        if (t == 0 && r < oc) { red_add(p, acca[0][0]); red_add(p + 8, acca[0][2]); }
-        if (has_b && t == 0 && r + 128u < oc) { red_add(p + 128, accb[0][0]); red_add(p + 136, accb[0][2]); }
+        const int b = ONE ? 0 : 2 * t;
+        float* p = y + (size_t)b * oc + r + (uint32_t)g;
+        const bool in = ONE ? t == 0 : b < a.B;
+        if (in && r < oc) { red_add(p, acca[0][0]); red_add(p + 8, acca[0][2]); }
+        if (has_b && in && r + 128u < oc) { red_add(p + 128, accb[0][0]); red_add(p + 136, accb[0][2]); }
+        if constexpr (!ONE) {
+          p += oc;
+          if (b + 1 < a.B && r < oc) { red_add(p, acca[0][1]); red_add(p + 8, acca[0][3]); }
+          if (has_b && b + 1 < a.B && r + 128u < oc) { red_add(p + 128, accb[0][1]); red_add(p + 136, accb[0][3]); }
+        }
       } else {
         // Four lanes that share t hold a 4 x 4 block (rows 4J .. 4J+3 of one row half x the accumulator's four
         // elements): transposed, every lane owns four consecutive rows of ONE batch column and adds them
