@@ -338,6 +338,21 @@ rwkvq_status rwkvq_step_reciprocal(const float* y_dev, float* out_dev, size_t n,
 rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, int n_ctas,
                                    uint32_t* counts_host, size_t n_counts, uint32_t* cta_items_host);
 /*
+ * Host-only: the forms of the schedule rwkvq_step_plan would build for n_ctas CTAs, so that a test can tell which of them it runs.
+ * Errors as rwkvq_step_plan_cover.
+ */
+typedef struct {
+  int32_t pre_pass;           /* 0: CTAs mix the inputs they read; 1: mixed once per stage and copied; 2: the same, with operators */
+  int32_t unpacked_ahead;     /* 1: units are unpacked ahead of their inputs */
+  uint32_t segments;          /* runs of input columns, over all CTAs */
+  uint32_t announced_heads;   /* of these: their first tiles are announced ahead of the rest */
+  uint32_t most_heads;        /* announced heads of the CTA that has most */
+  uint32_t squared;           /* squared by the CTAs that read them */
+  uint32_t behind_squared;    /* copied to a buffer that held squares */
+  uint32_t smem_bytes;        /* dynamic shared memory of a CTA */
+} rwkvq_step_forms;
+rwkvq_status rwkvq_step_plan_forms(const rwkvq_gemv_op* ops, int n_ops, int B, int n_ctas, rwkvq_step_forms* forms_host);
+/*
  * The same step for callers whose activations live in host memory: act_bytes are copied from act_host
  * to act_dev (the device buffer the plan's x / x_prev pointers lie in), the step runs, and y_bytes are
  * copied from y_dev (the buffer the plan's outputs lie in) to y_host.  Everything is ordered behind what

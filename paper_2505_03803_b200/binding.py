@@ -64,6 +64,11 @@ class GemvOp(C.Structure):
                 ("stage", C.c_int32), ("y_dtype", C.c_int32), ("in_", InputXform)]
 
 
+class StepForms(C.Structure):
+    _fields_ = [("pre_pass", C.c_int32), ("unpacked_ahead", C.c_int32), ("segments", C.c_uint32), ("announced_heads", C.c_uint32),
+                ("most_heads", C.c_uint32), ("squared", C.c_uint32), ("behind_squared", C.c_uint32), ("smem_bytes", C.c_uint32)]
+
+
 class PrefillOp(C.Structure):
     _fields_ = [("W_desc", C.POINTER(Desc)), ("W_image_dev", C.c_void_p), ("mu_desc", C.POINTER(Desc)),
                 ("mu_image_dev", C.c_void_p), ("X_bf16_dev", C.c_void_p), ("xprev0_bf16_dev", C.c_void_p),
@@ -75,6 +80,7 @@ EXPORTS = [
     "rwkvq_image_unpack", "rwkvq_blob_free", "rwkvq_proxy_workspace_bytes", "rwkvq_proxy_select",
     "rwkvq_gemv_workspace_bytes", "rwkvq_gemv", "rwkvq_gemv_static", "rwkvq_gemv_static_max_scratch_bytes", "rwkvq_step_plan_bytes", "rwkvq_step_plan", "rwkvq_step_run",
     "rwkvq_step_run_host", "rwkvq_step_plan_release", "rwkvq_step_set_wait", "rwkvq_step_reciprocal", "rwkvq_step_plan_cover",
+    "rwkvq_step_plan_forms",
     "rwkvq_prefill_workspace_bytes", "rwkvq_gemm_prefill", "rwkvq_gemm_prefill_grouped", "rwkvq_dequant", "rwkvq_device_status",
     "rwkvq_status_str", "rwkvq_last_cuda_error",
     "rwkvq_proxy_family", "rwkvq_proxy_select_bf16", "rwkvq_proxy_f32_workspace_bytes", "rwkvq_proxy_select_f32",
@@ -149,6 +155,7 @@ def lib() -> C.CDLL:
         L.rwkvq_step_set_wait.argtypes = [vp, C.c_uint32, C.c_uint32]
         L.rwkvq_step_reciprocal.argtypes = [vp, vp, sz, vp]
         L.rwkvq_step_plan_cover.argtypes = [C.POINTER(GemvOp), i32, i32, i32, C.POINTER(C.c_uint32), sz, C.POINTER(C.c_uint32)]
+        L.rwkvq_step_plan_forms.argtypes = [C.POINTER(GemvOp), i32, i32, i32, C.POINTER(StepForms)]
     if hasattr(L, "rwkvq_gemm_prefill"):
         L.rwkvq_prefill_workspace_bytes.argtypes = [C.POINTER(Desc), i32, i32]
         L.rwkvq_prefill_workspace_bytes.restype = sz
@@ -524,6 +531,13 @@ def rwkvq_step_plan_cover(ops, B: int, n_ctas: int):
     _check(lib().rwkvq_step_plan_cover(ops, len(ops), B, n_ctas, counts.ctypes.data_as(C.POINTER(C.c_uint32)), counts.size,
                                        per_cta.ctypes.data_as(C.POINTER(C.c_uint32))), "rwkvq_step_plan_cover")
     return counts[:n], per_cta
+
+
+def rwkvq_step_plan_forms(ops, B: int, n_ctas: int) -> StepForms:
+    """Host-only: which forms the schedule for n_ctas CTAs takes."""
+    forms = StepForms()
+    _check(lib().rwkvq_step_plan_forms(ops, len(ops), B, n_ctas, C.byref(forms)), "rwkvq_step_plan_forms")
+    return forms
 
 
 def rwkvq_step_run_host(plan, act_host, act_dev, y_dev, y_host, stream=None):

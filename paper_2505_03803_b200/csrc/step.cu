@@ -104,8 +104,9 @@ struct StepEvent {           // 64 bytes
 };
 // EF_SQUARES: of a stage whose inputs every CTA squares for itself (see kSquaresShare); arrival: the stage that begins.  EF_READ_FIRST: arrival; the
 // outputs to clear are inputs of the stage that ends, which every CTA has read when that stage's second barrier opens.
-// EF_HEAD: segment; its first kHeadTiles tiles are announced ahead of the rest.
-enum { EF_SQUARES = 1, EF_READ_FIRST = 2, EF_HEAD = 4 };
+// EF_HEAD: segment; its first kHeadTiles tiles are announced ahead of the rest.  EF_BEHIND_SQUARES: copied segment; its buffer was last filled by
+// stage_squares.
+enum { EF_SQUARES = 1, EF_READ_FIRST = 2, EF_HEAD = 4, EF_BEHIND_SQUARES = 8 };
 static_assert(sizeof(StepEvent) == 64, "event descriptor size");
 
 // One product's share of a stage's pre-pass: where its inputs are and where x_mix (fp16 rows of
@@ -1071,6 +1072,11 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
     if constexpr (MIX) {
       // The segment is a rectangle of the stage's pre-pass output: pass the stage's second barrier
       // (once per stage), then fetch B rows and the block of sums with bulk copies.
+      if constexpr (kSquares) {
+        // What stage_squares stored here (seen through xfull and xempty) precedes what the copy engine writes to the same bytes.  By the warp that asks for the
+        // copies, in front of the poll, whose wait it lies in (1.6B-class blocks, batch 2: 110.0 us without, 109.9 with).
+        if (stid < 32 && (ev.flags & EF_BEHIND_SQUARES)) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      }
       const uint32_t b2 = (uint32_t)a.n_stages + ev.barrier;      // counter of the second barrier of stage ev.barrier - 1
       if (ok && stid < kPollLanes && b2 != passed2) {
         uint32_t it = 0;
@@ -1084,8 +1090,9 @@ __device__ void stager_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, uint8_
         const uint32_t xstride = ev.xstride_sums & 0x7FFFFFFFu;
         const uint32_t row_bytes = ev.segd.ncols * 2u;
         const uint32_t sums_bytes = (ev.xstride_sums >> 31) ? (ev.segd.ncols >> 7) * 3u * (uint32_t)((a.B + 1) & ~1) * 4u : 0u;
-        // What other CTAs wrote with ordinary stores is read below by the copy engine, in global memory alone: a fence of all spaces is half a microsecond slower
-        // in every stage (7B-class stack of eight layers, batch 8: 336.9 us, 325.8 so; 1.6B-class blocks, batch 2: 112.8, 110.6).
+        // What other CTAs wrote to global memory with ordinary stores is read below by the copy engine.  The buffer it is copied to was last filled by the copy engine,
+        // too, or fenced above: here a fence of all spaces is half a microsecond slower in every stage (7B-class stack of eight layers, batch 8: 336.9 us, 325.8
+        // so; 1.6B-class blocks, batch 2: 112.8, 110.6).
         asm volatile("fence.proxy.async.global;" ::: "memory");
         if (lane == 0) mbar_arrive_expect_tx(&ctrl->xfull[buf], (uint32_t)a.B * row_bytes + sums_bytes);
         __syncwarp();
@@ -2206,6 +2213,8 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     }
     all_events.push_back(cta_arrivals[c][0]);
     uint32_t seg_no = 0, heads[2] = {0, 0};
+    bool squared[2] = {false, false};      // the segment last put into the buffer
+    static_assert(XBufs<2, 1>::kCount == 2u, "segments take the buffers in turn");
     size_t i = 0;
     for (int s = 0; s < n_stages; ++s) {
       // segments: maximal runs of units of one product whose column span fits the buffer
@@ -2240,6 +2249,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           ev.flags |= EF_SQUARES;
           ev.seg.x = (uint64_t)(uintptr_t)o.in.src_f32;
         } else if (mix) {
+          if (squared[seg_no & 1u]) ev.flags |= EF_BEHIND_SQUARES;
           ev.seg.x = mix_x_off[op] + (uint64_t)kmin * 512u;
           ev.seg.xprev = mix_sums_off[op] + (uint64_t)(kmin * 2) * 3u * nbp * 4u;
           ev.segd.ic = (uint32_t)o.W_desc.ic_pad * 2u;
@@ -2271,6 +2281,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
           }
         }
         first_of_stage = false;
+        squared[seg_no & 1u] = squares[s] != 0;
         all_events.push_back(ev);
         ++seg_no;
         i = last + 1;
@@ -2546,6 +2557,33 @@ rwkvq_status rwkvq_step_plan_cover(const rwkvq_gemv_op* ops, int n_ops, int B, i
     }
     if (cta_items_host) cta_items_host[c] = items;
   }
+  return RWKVQ_OK;
+}
+
+rwkvq_status rwkvq_step_plan_forms(const rwkvq_gemv_op* ops, int n_ops, int B, int n_ctas, rwkvq_step_forms* forms_host) {
+  if (!forms_host || n_ctas <= 0) return RWKVQ_EINVAL;
+  PlanInfo info;
+  std::vector<uint8_t> image;
+  const rwkvq_status st = build_plan(ops, n_ops, B, n_ctas, &image, &info);
+  if (st != RWKVQ_OK) return st;
+  rwkvq_step_forms f;
+  std::memset(&f, 0, sizeof(f));
+  f.pre_pass = info.mix; f.unpacked_ahead = info.park ? 1 : 0; f.smem_bytes = info.smem_bytes;
+  const uint32_t* event_off = reinterpret_cast<const uint32_t*>(image.data() + info.off_event_off);
+  const StepEvent* events = reinterpret_cast<const StepEvent*>(image.data() + info.off_events);
+  for (int c = 0; c < n_ctas; ++c) {
+    uint32_t heads = 0;
+    for (uint32_t e = event_off[c]; e < event_off[c + 1]; ++e) {
+      if (events[e].kind != EV_SEGMENT) continue;
+      ++f.segments;
+      heads += (events[e].flags & EF_HEAD) != 0;
+      f.squared += (events[e].flags & EF_SQUARES) != 0;
+      f.behind_squared += (events[e].flags & EF_BEHIND_SQUARES) != 0;
+    }
+    f.announced_heads += heads;
+    f.most_heads = std::max(f.most_heads, heads);
+  }
+  *forms_host = f;
   return RWKVQ_OK;
 }
 

@@ -249,3 +249,36 @@ def test_squared_inputs_of_one_stage(Bn, oc, bits):
     squares = k.clamp_min(0.0) ** 2
     assert bool(((y1.double() - squares @ m1.T).abs() <= 2e-3 * squares.norm(dim=1)[:, None] * m1.norm(dim=1)[None]).all())
     B.rwkvq_step_plan_release(plan)
+
+
+@pytest.mark.parametrize("Bn,rows,kinds", [(1, 17, "pspspp"), (1, 70, "spspps"), (3, 33, "psppsspp"), (8, 17, "psppsspp"), (8, 16, "sspps"), (2, 64, "pspsp")])
+def test_copied_inputs_behind_squared_ones(Bn, rows, kinds):
+    """Stages of squared (s) and of plain (p) inputs by turns: the copies of a plain stage land where squares that the CTA stored itself lay before.  Every product
+    has inputs of its own, squares rounded to fp16 as the step rounds them, so that only the fp32 sums differ (1e-5 of |w| |x|)."""
+    ic, g = 2304, torch.Generator(device="cuda").manual_seed(Bn * rows)
+    oc = 256 * rows
+    ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ, 3)
+    image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+    B.rwkvq_quantize_dev_async((torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half(), oc, ic, desc.method, 3, image, ws)
+    decoded = torch.empty((oc, ic), device="cuda")
+    B.rwkvq_dequant(desc, image, decoded)
+    keep, want = [], []
+    for stage, kind in enumerate(kinds):
+        x = torch.randn((Bn, ic), generator=g, device="cuda")
+        e = dict(desc=desc, W=image, mu_desc=None, mu=None, xprev=None, y=torch.zeros((Bn, oc), device="cuda"), stage=stage)
+        e.update(dict(x=None, **{"in": dict(kind=B.RWKVQ_IN_RELU2, src=x)}) if kind == "s" else dict(x=x.half()))
+        keep.append((e, x))
+        want.append((x.clamp_min(0.0).square() if kind == "s" else x).half().double())
+    ops = B.make_ops([e for e, _ in keep])
+    forms = B.rwkvq_step_plan_forms(ops, Bn, torch.cuda.get_device_properties(0).multi_processor_count)
+    assert forms.squared > 0 and forms.behind_squared > 0
+    plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
+    B.rwkvq_step_plan(ops, Bn, plan)
+    for _ in range(10):
+        B.rwkvq_step_run(plan)
+        for (e, _), x in zip(keep, want):
+            bound = 1e-5 * x.norm(dim=1)[:, None] * decoded.double().norm(dim=1)[None]
+            assert bool(((e["y"].double() - x @ decoded.double().T).abs() <= bound).all()), e["stage"]
+    assert B.rwkvq_device_status() == 0
+    B.rwkvq_step_plan_release(plan)

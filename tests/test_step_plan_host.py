@@ -114,3 +114,24 @@ def test_plan_rejects_bad_arguments():
     assert lib.rwkvq_step_set_wait(C.c_void_p(4096), 0, 0) == 1
     with pytest.raises(B.RwkvqError):
         B.rwkvq_step_plan_cover(_ops(512, 1280, 1), 0, 148)
+
+
+@pytest.mark.parametrize("kinds", ["psp", "pspspspp", "sspp", "spps", "pppss", "spsp", "ppssppsspp"])
+@pytest.mark.parametrize("Bn", [1, 8, 9])
+def test_copies_behind_squares_are_marked(kinds, Bn):
+    """One CTA and one tile a stage: segments take the two input buffers in turn.  A plain stage (p) is copied into the buffer that the stage before the last
+    filled: marked where that one held squares (s), which the CTA stored itself.  Above eight rows squares come from the pre-pass, too."""
+    arr = (B.GemvOp * len(kinds))()
+    for k, kind in enumerate(kinds):
+        o = arr[k]
+        o.W_desc = _desc(B.RWKVQ_SQ, 256, 256, 3)
+        o.W_image_dev, o.y_dev, o.stage = (1 << 30) + (k << 26), (1 << 36) + (k << 26), k
+        if kind == "s":
+            o.in_.kind, o.in_.src_f32 = B.RWKVQ_IN_RELU2, (1 << 38) + (k << 26)
+        else:
+            o.x_fp16_dev = (1 << 37) + (k << 26)
+    forms = B.rwkvq_step_plan_forms(arr, Bn, 1)
+    own = Bn <= 8
+    assert forms.pre_pass == 2 and forms.segments == len(kinds)
+    assert forms.squared == (kinds.count("s") if own else 0)
+    assert forms.behind_squared == (sum(kinds[k - 2:k + 1:2] == "sp" for k in range(2, len(kinds))) if own else 0)
