@@ -131,9 +131,9 @@ static_assert(sizeof(StepMixX) == 80, "pre-pass operator descriptor size");
 constexpr int kGroupWarps = 8, kGroupThreads = kGroupWarps * 32;
 // Thread layout of a CTA, by the number of batch blocks NB a record is multiplied with.
 //   NB = 1 (B <= 8): two consumer groups of eight warps, three stager warps, one producer warp: 640 threads,
-//     96 registers each, for all roles (with 104 for the consumers and 64 for the others, which the compiler takes as the limit of these
+//     96 registers each at launch.  They stay so for all roles (with 104 for the consumers and 64 for the others, which the compiler takes as the limit of these
 //     roles' code, the pre-pass of a stage spilled, and behind a barrier's acquire a spilled word is a trip to L2: blocks 136 us where
-//     they take 127).
+//     they took 127), except with units unpacked ahead and no pre-pass (consumer_regs, stager_regs).
 //   NB = 2 (B > 8): the record routine wants about 150 registers, which sixteen consumer warps cannot have,
 //     and eight warps that keep everything in registers outrun sixteen that spill: ONE consumer group,
 //     seven stager warps (the stage pre-pass is theirs), one producer: 512 threads, 128 registers at
@@ -146,10 +146,7 @@ template <int NB> struct Shape {
   static constexpr int kConsumerThreads = kConsumerWarps * 32, kStagerThreads = kStagerWarps * 32;
   static constexpr int kThreads = kConsumerThreads + kStagerThreads + 32;
   static constexpr int kLaunchRegs = NB == 2 ? 128 : 96;
-  static constexpr int kConsumerRegs = NB == 2 ? 152 : 96, kStagerRegs = NB == 2 ? 104 : 96;
   static_assert(kConsumerWarps % 4 == 0 && (kStagerWarps + 1) % 4 == 0, "register re-division works on warpgroups of four warps");
-  static_assert(kConsumerRegs * kConsumerThreads + kStagerRegs * (kStagerThreads + 32) <= kLaunchRegs * kThreads,
-                "register re-division exceeds the launch's pool");
   static_assert(kLaunchRegs * kThreads <= 65536, "register file");
 };
 // With units unpacked ahead and inputs that the CTAs mix themselves the consumers' code wants eight more, and the stagers', without a pre-pass, make do with
@@ -1744,6 +1741,8 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   uint8_t* xbufs = smem + kCtrlBytes + (size_t)a.n_slots * a.slot_bytes;
   uint32_t* mucb = reinterpret_cast<uint32_t*>(xbufs + XBufs<MIX, NB>::kCount * XBufs<MIX, NB>::kBytes);
   uint8_t* replicas = reinterpret_cast<uint8_t*>(mucb) + kMuScratch;
+  static_assert(consumer_regs(NB, MIX, PARK) * Shape<NB>::kConsumerThreads + stager_regs(NB, MIX, PARK) * (Shape<NB>::kStagerThreads + 32) <=
+                    Shape<NB>::kLaunchRegs * Shape<NB>::kThreads, "a re-division above the launch's registers would wait for ever");
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.n_slots; ++s) { mbar_init(&ctrl->full[0][s], 1); mbar_init(&ctrl->full[1][s], 1); mbar_init(&ctrl->empty[s], kGroupWarps); }
     for (int b = 0; b < 4; ++b) { mbar_init(&ctrl->xfull[b], kStagerWarps); mbar_init(&ctrl->xempty[b], kConsumerWarps); }
@@ -1759,8 +1758,9 @@ __global__ void __launch_bounds__(Shape<NB>::kThreads, 1) step_kernel(const Step
   const int warp = threadIdx.x >> 5;
   // With two batch blocks registers are re-divided at entry (see Shape): the warpgroups of stagers and producer hand part of
   // their share back and the consumer warpgroups take it, so that the record routine keeps everything
-  // in registers.  With one block the shares are those of the launch and nothing moves; the instruction stays for the code the compiler makes of the
-  // roles beside it (without it: 1.6B-class B=1 428.3 -> 429.9 us, 7B-class B=1 1209.9 -> 1207.5).
+  // in registers; so they are with one block where units are unpacked ahead over inputs that the CTAs mix themselves.  In the other kernels of one block the shares are
+  // those of the launch and nothing moves; the instruction stays for the code the compiler makes of the roles beside it (without it, before units were unpacked
+  // ahead: 1.6B-class B=1 428.3 -> 429.9 us, 7B-class B=1 1209.9 -> 1207.5).
   if (warp < kConsumerWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(consumer_regs(NB, MIX, PARK)));
   } else {
