@@ -170,6 +170,11 @@ template <int MIX, int NB> struct XBufs { static constexpr uint32_t kCount = 2u,
 // Tiles at the head of a stage's first segment: one for each of two consumer groups' first units.
 constexpr int kHeadTiles = 2;
 constexpr uint32_t kSmemLimit = 232448;  // 227 KB
+// Of a CTA that allocates tensor memory.  tcgen05.alloc waits, without a limit, for columns that another CTA on the SM holds, and beside this kernel's registers
+// (61 440 of 65 536) a small one would fit.  An SM has 228 KB, of which every CTA takes 1 KB for the system: beside this none does (128: the kernels' static
+// shared memory), so the columns are always there.  1.6B-class, batch 1: 347.9 us without and with; 1.6B-class blocks, batch 2: 108.6, 108.7.
+constexpr uint32_t kSmemAlone = kSmemLimit - 128;
+static_assert(233472 - (kSmemAlone + 1024) < 1024, "room for another CTA");
 constexpr uint32_t kDefaultPollLimit = 1u << 22;
 
 struct StepArgs {
@@ -1542,7 +1547,8 @@ __device__ void consumer_role(const StepArgs& a, uint8_t* smem, Ctrl* ctrl, cons
     }
   };
   uint8_t* rep = replicas + (size_t)grp * a.replica_bytes;
-  // Tensor memory is the consumer warps' alone: the other roles neither wait for it nor for its return.
+  // Tensor memory is the consumer warps' alone: the other roles neither wait for it nor for its return.  No other CTA is on the SM (kSmemAlone), so the
+  // allocation does not wait either.
   if constexpr (PARK) {
     if (warp == 0) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctrl->tmem_base)), "n"(kTmemCols) : "memory");
@@ -2148,6 +2154,7 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
   // d 2560, 2.75, 172.2 / 176.4; d 3072, 3.75, 199.0 / 199.0; d 4096, 6, 284.0 / 287.1; batch 2, d 2048, 149.7 / 139.4; batch 8, d 2048, 212.0 / 200.7,
   // d 4096, 336.4 / 343.7.  Above eight rows two warps a scheduler do not hide the trips to tensor memory (14B-class stack, batch 16: 3330 / 3554).
   info->park = B <= 8 && deepest <= 2 * (size_t)n_stages;
+  if (info->park) info->smem_bytes = std::max(info->smem_bytes, kSmemAlone);
   if (too_many_ranges) return RWKVQ_EUNSUPPORTED;   // a CTA's slice of a stage's outputs may touch at most three products
 
   // pre-pass outputs: one region, reused by every stage (a stage's pre-pass starts only after the

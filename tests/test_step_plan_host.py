@@ -135,3 +135,15 @@ def test_copies_behind_squares_are_marked(kinds, Bn):
     assert forms.pre_pass == 2 and forms.segments == len(kinds)
     assert forms.squared == (kinds.count("s") if own else 0)
     assert forms.behind_squared == (sum(kinds[k - 2:k + 1:2] == "sp" for k in range(2, len(kinds))) if own else 0)
+
+
+@pytest.mark.parametrize("vq_every,bits", [(0, 6), (1, 6), (1, 8), (3, 8)])
+@pytest.mark.parametrize("Bn", [1, 8])
+def test_a_cta_with_tensor_memory_is_alone_on_its_sm(vq_every, bits, Bn):
+    """Plans that unpack units ahead allocate all of an SM's tensor memory, which waits for whoever holds some: their CTAs leave no shared memory
+    for another one (228 KB an SM, 1 KB of it reserved for each CTA, 227 KB at most for one)."""
+    forms = B.rwkvq_step_plan_forms(_ops(512, 1280, 2, vq_every=vq_every, bits=bits), Bn, 148)
+    assert forms.unpacked_ahead == 1
+    assert forms.smem_bytes <= 227 << 10 and (228 << 10) - (forms.smem_bytes + 1024) < 1024
+    other = B.rwkvq_step_plan_forms(_ops(4096, 14336, 1, vq_every=vq_every, bits=bits), Bn, 148)
+    assert other.unpacked_ahead == 0 and other.smem_bytes <= 227 << 10
