@@ -42,6 +42,10 @@ def _plan(ops, Bn):
     return plan
 
 
+def _forms(ops, Bn):
+    return B.rwkvq_step_plan_forms(ops, Bn, torch.cuda.get_device_properties(0).multi_processor_count)
+
+
 def _check(ops, Bn):
     worst = 0.0
     for e in ops:
@@ -515,9 +519,9 @@ def test_outputs_that_are_inputs_of_the_stage_before(kind, Bn):
 @pytest.mark.parametrize("Bn,bits", [(1, 3), (1, 6), (2, 8), (3, 6), (8, 3), (8, 8)])
 @pytest.mark.parametrize("rows", [(16, 32, 37, 32), (16, 37, 48), (80, 75, 96, 80)])
 def test_units_unpacked_ahead_of_their_inputs(rows, Bn, bits):
-    """Stages of one to six units a CTA (rows of nine tiles on 148 SMs): plans of small stages unpack a group's first unit of a stage while its
-    inputs are on their way, and go on to the next as before; plans of larger ones do not, and with one row their stages' first inputs are announced ahead of
-    the rest.  Scalar rows end in half a unit.  Inputs and decoded weights are exact, so that only the fp32 sums differ (1e-5 of |w| |x|)."""
+    """Stages of one to six units a CTA (rows of nine tiles on 148 SMs): plans of small stages (the first, of two units on average) unpack a group's first unit
+    of a stage while its inputs are on their way, and go on to the next as before; plans of larger ones do not, and with one row the largest stages' first inputs are announced
+    ahead of the rest.  Scalar rows end in half a unit.  Inputs and decoded weights are exact, so that only the fp32 sums differ (1e-5 of |w| |x|)."""
     ic, g = 2304, torch.Generator(device="cuda").manual_seed(10 * Bn + bits)
     ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
     keep = []
@@ -530,6 +534,8 @@ def test_units_unpacked_ahead_of_their_inputs(rows, Bn, bits):
         keep.append(dict(desc=desc, W=image, mu_desc=None, mu=None, x=torch.randn((Bn, ic), generator=g, device="cuda").half(), xprev=None,
                          y=torch.full((Bn, oc), float("nan"), device="cuda"), stage=stage))
     ops = B.make_ops(keep)
+    forms = _forms(ops, Bn)
+    assert forms.unpacked_ahead == (len(rows) == 4 and rows[0] == 16) and (forms.announced_heads > 0) == (rows[0] == 80 and Bn == 1)
     plan = torch.zeros(B.rwkvq_step_plan_bytes(ops, Bn), dtype=torch.uint8, device="cuda")
     B.rwkvq_step_plan(ops, Bn, plan)
     for _ in range(2):
@@ -542,3 +548,71 @@ def test_units_unpacked_ahead_of_their_inputs(rows, Bn, bits):
         assert bool(((e["y"].double() - x @ decoded.double().T).abs() <= bound).all()), e["stage"]
     assert B.rwkvq_device_status() == 0
     B.rwkvq_step_plan_release(plan)
+
+
+class _Large:
+    """Stages of one scalar product each, rows of `tiles` column tiles, with token shifts where `shift` says so.  The inputs are mixed as the step mixes them and the
+    decoded weights are exact, so that only the fp32 sums differ (1e-5 of |w| |x|)."""
+
+    def __init__(self, Bn, rows, shift=True, tiles=9):
+        self.Bn, self.keep, ic = Bn, [], 256 * tiles
+        g = torch.Generator(device="cuda").manual_seed(100 * Bn + len(rows))
+        ws = torch.zeros(B.rwkvq_quantize_workspace_bytes(), dtype=torch.uint8, device="cuda")
+        for stage, r in enumerate(rows):
+            oc = 256 * r
+            desc = B.rwkvq_desc_for(oc, ic, B.RWKVQ_SQ, 3)
+            image = torch.zeros(int(desc.image_bytes), dtype=torch.uint8, device="cuda")
+            B.rwkvq_quantize_dev_async((torch.randn((oc, ic), generator=g, device="cuda") * 0.02).half(), oc, ic, desc.method, 3, image, ws)
+            decoded = torch.empty((oc, ic), device="cuda")
+            B.rwkvq_dequant(desc, image, decoded)
+            x, xp = (torch.randn((Bn, ic), generator=g, device="cuda").half() for _ in range(2))
+            mu = H.pack_mu(H.random_mu_codes(1500 + stage, ic, 6), 6) if shift else None
+            mixed = x.double()
+            if shift:      # the difference is rounded to fp32, then one fused multiply-add
+                mixed = ((xp.float() - x.float()).double() * torch.from_numpy(mu.w_hat).cuda().double() + x.double()).float().half().double()
+            self.keep.append((dict(desc=desc, W=image, mu_desc=mu.desc if shift else None, mu=mu.dev if shift else None, x=x, xprev=xp if shift else None,
+                                   y=torch.zeros((Bn, oc), device="cuda"), stage=stage), decoded.double(), mixed, mu))
+        self.ops = B.make_ops([e for e, *_ in self.keep])
+        self.forms = _forms(self.ops, Bn)
+        self.plan = torch.zeros(B.rwkvq_step_plan_bytes(self.ops, Bn), dtype=torch.uint8, device="cuda")
+        B.rwkvq_step_plan(self.ops, Bn, self.plan)
+
+    def run_and_check(self):
+        for e, *_ in self.keep:
+            e["y"].fill_(float("nan"))
+        B.rwkvq_step_run(self.plan)
+        assert B.rwkvq_device_status() == 0
+        for e, w, x, _ in self.keep:
+            bound = 1e-5 * x.norm(dim=1)[:, None] * w.norm(dim=1)[None]
+            assert bool(((e["y"].double() - x @ w.T).abs() <= bound).all()), e["stage"]
+
+
+@pytest.mark.parametrize("rows", [(80, 75, 96, 80, 77, 80, 91), (170, 60, 160)])
+@pytest.mark.parametrize("shift", [True, False])
+def test_announced_heads_of_one_row(rows, shift):
+    """One row, large stages: the first tiles of a stage's first segment are announced ahead of the rest, with the previous token's row and mu_hat where
+    there is a token shift.  In seven stages of one segment either buffer's announcements come to a third phase."""
+    large = _Large(1, rows, shift)
+    assert large.forms.pre_pass == 0 and large.forms.unpacked_ahead == 0 and large.forms.announced_heads > 0
+    assert len(rows) < 7 or large.forms.most_heads >= 6
+    for _ in range(3):
+        large.run_and_check()
+    B.rwkvq_step_plan_release(large.plan)
+
+
+@pytest.mark.parametrize("Bn,rows,pre_pass", [(1, (80, 75, 96), 0), (2, (48, 45, 50), 0), (8, (48, 45, 50), 1)])
+def test_bounded_waits_of_large_stages_run_out_and_the_plan_recovers(Bn, rows, pre_pass):
+    """As test_bounded_waits_run_out_and_the_plan_recovers, for plans that do not unpack units ahead; with one row consumers wait for announced heads that
+    never come."""
+    large = _Large(Bn, rows)
+    assert large.forms.pre_pass == pre_pass and large.forms.unpacked_ahead == 0 and (large.forms.announced_heads > 0) == (Bn == 1)
+    large.run_and_check()
+    B.rwkvq_step_set_wait(large.plan, poll_limit=2000, wait_skew=1)
+    B.rwkvq_step_run(large.plan)
+    torch.cuda.synchronize()                                         # the kernel returns by itself
+    assert B.rwkvq_device_status() == 8                              # RWKVQ_ETIMEOUT, and the word is cleared
+    assert B.rwkvq_device_status() == 0
+    B.rwkvq_step_set_wait(large.plan, poll_limit=0, wait_skew=0)     # defaults again
+    for _ in range(2):
+        large.run_and_check()
+    B.rwkvq_step_plan_release(large.plan)
