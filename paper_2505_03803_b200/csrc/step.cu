@@ -150,7 +150,9 @@ template <int NB> struct Shape {
   static_assert(kLaunchRegs * kThreads <= 65536, "register file");
 };
 // With units unpacked ahead and inputs that the CTAs mix themselves the consumers' code wants eight more, and the stagers', without a pre-pass, make do with
-// 64 (1.6B-class, twelve layers, batch 1: 180.6 us at 96 each, 179.4).
+// 64 (1.6B-class, twelve layers, batch 1: 180.6 us at 96 each, 179.4).  The kernels that unpack ahead still spill a few words of the consumers' (<1, 0, true, true> 12 bytes of
+// stores and 44 of loads, <1, 1, true> and <1, 2, true> 12 and 36; the others up to eight rows none).  They cost nothing that can be measured: with values read again where they are
+// rarely wanted (no spills in the first, 4 and 8 bytes in the other two) the steps are no faster (1.6B-class 347.9 us, without 348.5 to 353.7; blocks, batch 2, 108.6, 108.7).
 __host__ __device__ constexpr int consumer_regs(int NB, int MIX, bool PARK) { return NB == 2 ? 152 : PARK && MIX == 0 ? 104 : 96; }
 __host__ __device__ constexpr int stager_regs(int NB, int MIX, bool PARK) { return NB == 2 ? 104 : PARK && MIX == 0 ? 64 : 96; }
 constexpr int groups_of(int NB) { return NB == 2 ? 1 : 2; }
@@ -1268,7 +1270,7 @@ __device__ __forceinline__ void vq_unit(const uint8_t* ra, const uint8_t* rb, co
 // A group's first unit of a stage is in shared memory long before the stage's inputs are.  While the warps would wait for these they unpack it, and what they
 // unpack waits in tensor memory, used as a larger register file: every warp reaches 32 lanes of it and has 128 columns to itself, so 128
 // registers of a lane.  Behind the inputs only the fragments' loads and the tensor-core steps are left: 1770 cycles where the whole unit took 2700
-// (1.6B-class, batch 1, both groups at work; step 418 us before, 363 with this and one instruction a row half for one batch column).  Bound by
+// (1.6B-class, batch 1, both groups at work; step 397 us without, 346 with it).  Bound by
 // the chain of a warp then: four trips to tensor memory and sixteen tensor-core steps one behind the other.
 constexpr uint32_t kTmemCols = 512, kParkCols = 128;
 __device__ __forceinline__ void park16(uint32_t at, const uint32_t (&r)[16]) {
@@ -2147,12 +2149,13 @@ static rwkvq_status build_plan(const rwkvq_gemv_op* ops, int n_ops, int B, int P
     }
     for (int c = 0; c < P; ++c) make_arrival(c, s + 1, s + 1);
   }
-  // Units unpacked ahead of their inputs (consumer_role): they take about 1000 of the 2700 cycles of a group's first unit out of a stage's chain, and a launch takes
-  // 3 us longer.  It gains where most groups have one unit a stage.  Eight layers (d 2048: twelve), without / with, us, at `units of the CTA that has
-  // most, mean over the stages`: batch 1, d 512, 1, 104.5 / 98.5; d 1536, 1.25, 118.6 / 112.8; d 2048, 1.75, 203.4 / 179.4; d 2304, 2.25, 149.6 / 147.3, but
-  // batch 4, d 2176, 2.25, twelve layers, 283.6 / 287.9;
-  // d 2560, 2.75, 172.2 / 176.4; d 3072, 3.75, 199.0 / 199.0; d 4096, 6, 284.0 / 287.1; batch 2, d 2048, 149.7 / 139.4; batch 8, d 2048, 212.0 / 200.7,
-  // d 4096, 336.4 / 343.7.  Above eight rows two warps a scheduler do not hide the trips to tensor memory (14B-class stack, batch 16: 3330 / 3554).
+  // Units unpacked ahead of their inputs (consumer_role): they take about 1000 of the 2700 cycles of a group's first unit out of a stage's chain; a launch takes no
+  // longer by itself (one layer of d 512: 17.5 us either way).  It gains where most groups have one unit a stage.  Eight layers where nothing else is said, without / with, us,
+  // at `units of the CTA that has most, mean over the stages`: batch 1, d 512, 1, 104.3 / 96.3; d 1536, 1.25, 118.3 / 108.7; d 2048, 1.75, twelve layers, 203.0 / 176.5; d 2304,
+  // 2.25, 148.4 / 144.5, but batch 4, d 2176, 2.25, twelve layers, 278.0 / 282.4; batch 1, d 2560, 2.75, 170.2 / 172.2; d 3072, 3.75, 194.7 / 192.5; d 4096, 6, 271.2 / 279.0;
+  // batch 2, d 2048, 149.6 / 136.3; batch 8, d 2048, 200.9 / 189.2, d 4096, 324.7 / 325.7; four blocks of d 2048, batch 2, 114.8 / 108.7.  (One line for all batches
+  // and for the whole plan: d 2304 and 3072 are on the wrong side of it.)  Above eight rows two warps a scheduler do not hide the trips to tensor memory (14B-class stack, batch
+  // 16: 3330 / 3554).
   info->park = B <= 8 && deepest <= 2 * (size_t)n_stages;
   if (info->park) info->smem_bytes = std::max(info->smem_bytes, kSmemAlone);
   if (too_many_ranges) return RWKVQ_EUNSUPPORTED;   // a CTA's slice of a stage's outputs may touch at most three products
